@@ -250,9 +250,10 @@ lvlm_status lvlm_kv_compress(void* Kc, void* Vc, float* acc_score, int32_t* pos,
  * written in the previous decoding step; NOT true right after lvlm_kv_compress or
  * lvlm_merge_compact on the same cache).  The kernel then starts fetching the cache while that
  * operation is still draining; q, k_new, v_new and all writes wait for it as always.
- * Workspace: only used when acc_score is given and the cache is so long that the scaled logits of a CTA's
+ * Workspace: used when acc_score is given and the cache is so long that the scaled logits of a CTA's
  * own keys do not fit in its shared memory (they are then parked there between the pass over the keys and
- * the update of acc_score); its contents need not be zeroed.
+ * the update of acc_score), and for the partial results where few heads with long caches are cut into parts
+ * (two launches then); its contents need not be zeroed.
  * Reads d: B,H,Hkv,D,cap,kv_stride_*.
  * Errors: INVALID_ARG, UNSUPPORTED (D!=128, H/Hkv > 8), ALIGNMENT, WORKSPACE.
  */
@@ -271,10 +272,9 @@ lvlm_status lvlm_decode_attn(const void* q, void* Kc, void* Vc, int32_t* len,
  * outputs are still the caller's.
  *
  * The scratch is a fixed array of LVLM_STATIC_SCRATCH_BYTES inside the library image: every GPU
- * on which the library is loaded carries it until the process exits.  A problem whose
- * lvlm_workspace_bytes(LVLM_OP_DECODE_ATTN, d) exceeds that size is rejected with
- * LVLM_ERR_WORKSPACE and nothing is enqueued (B * H * cap * 4 bytes are needed; B = 8, H = 32,
- * cap = 1152 takes about 1.2 MiB).
+ * on which the library is loaded carries it until the process exits.  A problem that needs more is
+ * rejected with LVLM_ERR_WORKSPACE and nothing is enqueued (B * H * cap * 4 bytes are needed; B = 8, H = 32,
+ * cap = 1152 takes about 1.2 MiB; long caches are cut into parts only where their results fit as well).
  *
  * The first call on each device looks up the array's device address (with that device current)
  * and remembers it; make that first call outside any stream capture.  No call allocates or frees

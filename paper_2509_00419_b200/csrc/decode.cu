@@ -16,6 +16,13 @@
 // distributed shared memory in rank order, each finishing a slice of the output channels and the
 // acc_score entries of its own keys, whose scaled logits it has kept in shared memory (in the
 // workspace when a run is too long for that).
+//
+// Few heads with long caches (a video prompt's first layers: one sequence, 4 KV heads, 32898 rows) leave most of the
+// GPU idle that way: a cluster has at most 8 CTAs.  There the run of a head is cut into as many parts as fill the GPU
+// twice, without clusters; every part leaves its (max, sum, output) in the workspace, and a second, small launch adds
+// the parts in order, finishes acc_score and bumps len.  HBM-bound either way.  That shape, per layer (67 MB):
+// 53.6 us with 8 CTAs a head, 17.8 us as 74 parts a head
+// (3.8 TB/s; the start-up, the merge and the second launch are 6 us of it).
 #include <mutex>
 
 #include "common.cuh"
@@ -36,12 +43,30 @@ constexpr int kRingBytes = kStagesDec * kStageBytes;
 constexpr int kDecTargetCtas = 2 * 148;              // CTAs wanted in flight: two per SM of a 148-SM part
 constexpr int kDecMaxCluster = 8;                    // portable cluster size
 constexpr int kDecMinTiles = 2;                      // a CTA's run is not made shorter than this by splitting
+constexpr int kDecPartTiles = 4;                     // a part's run is not made shorter than this
 constexpr int kDecLogitBytes = 12 * 1024;            // scaled logits of a CTA's own keys kept in shared memory
 constexpr float kLog2e = 1.4426950408889634f;
 
-struct DecodeLayout { int S; size_t off_s, total; };
+// S CTAs a head form a cluster; P > 0: as many independent CTAs a head whose results a second launch adds.
+struct DecodeLayout { int S, P; size_t off_s, off_ml, off_o, off_len, total; };
 
-static bool decode_layout(const lvlm_dims* d, DecodeLayout* L) {
+// Rows of a cache, in tiles, from which the parts are the faster form where a cluster of 8 a head leaves SMs idle (the
+// lengths are only known on the device).  us per layer as cluster / as parts, inside a chain of layers:
+//   from 32 heads the clusters of 8 no longer fit the GPU side by side: 36 heads of 216 rows 10.3 / 7.3, 2000 17.9 / 13.4,
+//   20000 91 / 65; 32 heads of 130 rows 4.9 / 5.4;
+//   without acc_score the cluster's one launch wins while the runs are short: 4 heads of 600 rows 5.4 / 5.5, 1100 6.2 / 5.5,
+//   32898 54.1 / 17.8; 8 heads of 1100 rows 5.5 / 5.4, 8000 15.5 / 11.6; 16 heads of 2000 rows 8.5 / 9.3, 8000 20.4 / 16.2;
+//   28 heads of 4000 rows 15.8 / 16.0, 8000 25.7 / 25.1;
+//   with it the second launch takes the update of acc_score off the cluster's tail: 4 heads of 400 rows 5.65 / 5.64, 600
+//   6.6 / 5.7, 32898 66.8 / 17.8; 20 heads of 600 rows 8.6 / 7.8, 8000 27.9 / 22.6; 28 heads of 2000 rows 11.9 / 13.1.
+static int parts_from_tiles(int64_t heads, bool acc) {
+    if (heads >= 32) return 14;
+    if (acc) return heads <= 20 ? 32 : 384;
+    return heads <= 8 ? 16 * (int)heads : 384;
+}
+
+// may_split: the caller's workspace has room for the parts (lvlm_decode_attn_static's may not).
+static bool decode_layout(const lvlm_dims* d, DecodeLayout* L, bool may_split = true) {
     if (!d || d->B <= 0 || d->H <= 0 || d->Hkv <= 0 || d->H % d->Hkv || d->cap <= 0) return false;
     // cluster size: the power of two that brings the grid closest to the target without going
     // over it, as long as a full cache still gives every CTA a few tiles
@@ -50,8 +75,20 @@ static bool decode_layout(const lvlm_dims* d, DecodeLayout* L) {
     int S = 1;
     while (S < kDecMaxCluster && heads * (2 * S) <= kDecTargetCtas && tiles / (2 * S) >= kDecMinTiles) S *= 2;
     L->S = S;
+    L->P = 0;
+    if (may_split && S == kDecMaxCluster &&
+        (tiles >= parts_from_tiles(heads, false) || tiles >= parts_from_tiles(heads, true))) {
+        const int fill = (int)(kDecTargetCtas / heads), most = tiles / kDecPartTiles;
+        L->P = fill < most ? fill : most;
+    }
     size_t off = 0;
     L->off_s = off; off = align_up(off + (size_t)d->B * d->H * d->cap * 4, 256);
+    L->off_ml = L->off_o = L->off_len = off;
+    if (L->P > 0) {
+        L->off_ml = off;  off = align_up(off + (size_t)d->B * d->H * L->P * 8, 256);
+        L->off_o = off;   off = align_up(off + (size_t)d->B * d->H * L->P * kHeadDim * 4, 256);
+        L->off_len = off; off = align_up(off + (size_t)heads * 4, 256);
+    }
     L->total = off;
     return true;
 }
@@ -120,6 +157,9 @@ struct DecodeArgs {
     int logit_keys;          // keys of a run whose logits fit in shared memory (0: they go to ws_s)
     int64_t kv_sb, kv_sh;
     float scale_log2;
+    float2* part_ml;         // parts: [B*Hkv][S][G] (max, sum), [B*Hkv][S][G][128] output relative to it,
+    float* part_o;           //        and [B*Hkv] length before the append, -1 = nothing was appended
+    int32_t* part_len;
     float* ws_s;             // [B*H][cap] scaled logits (log2 domain), only with acc_score and a long run
     int32_t* dev_status;
 };
@@ -131,11 +171,15 @@ __device__ __forceinline__ uint32_t stage_off(int r, int ch) {
 }
 
 // grid.x = heads * S, clusters of S CTAs along x: cluster = (sequence, KV head), rank = run of tiles.
-// CL = false: one CTA per head and no cluster instruction in the kernel at all.
-template <int G, bool CL>
+// kDecSolo: one CTA per head and no cluster instruction in the kernel at all.  kDecParts: S CTAs that know nothing of
+// each other leave their results in the workspace.
+enum { kDecSolo = 0, kDecCluster = 1, kDecParts = 2 };
+
+template <int G, int MODE>
 __global__ void __launch_bounds__(kDecThreads, 2)
 decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                       const DecodeArgs a) {
+    constexpr bool CL = MODE == kDecCluster;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     float* s_acc = reinterpret_cast<float*>(smem);                      // [slots][G][128]; slot 0 = this CTA's output (the ring, once it is done)
@@ -163,9 +207,9 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     // With a.early the first key/value stages and the length are fetched while the kernel ahead in the
     // stream is still finishing; q, k_new, v_new and every write come after the wait in any case.
     if (!a.early) pdl_enter();
-    const int S = CL ? a.S : 1, H = a.H, cap = a.cap;
+    const int S = MODE == kDecSolo ? 1 : a.S, H = a.H, cap = a.cap;
     const int hd = blockIdx.x / S;
-    const int rank = CL ? (int)cluster_ctarank() : 0;
+    const int rank = MODE == kDecParts ? (int)(blockIdx.x % S) : CL ? (int)cluster_ctarank() : 0;
     const int b = hd / a.Hkv, g = hd % a.Hkv, h0 = g * G;
 
     // ---- this head's length; every CTA of the cluster takes the same decisions ---------------------------
@@ -178,6 +222,11 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     const int lne = ln + (app ? 1 : 0);
     if (lne == 0) {                                                     // no key at all: zeros
         if (a.early) pdl_enter();
+        if (MODE == kDecParts) {
+            if (tid < G) a.part_ml[((int64_t)hd * S + rank) * G + tid] = make_float2(-INFINITY, 0.f);
+            if (rank == 0 && tid == 0) a.part_len[hd] = -1;
+            return;
+        }
         if (rank == 0)
             for (int i = tid; i < G * kHeadDim; i += kDecThreads)
                 a.out[(int64_t)(b * H + h0) * kHeadDim + i] = __float2bfloat16_rn(0.f);
@@ -387,7 +436,8 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
             float v = s_acc[hh * kHeadDim + tid];
 #pragma unroll
             for (int sl = 1; sl < kSlots; ++sl) v += s_acc[sl * (G * kHeadDim) + hh * kHeadDim + tid];
-            s_acc[hh * kHeadDim + tid] = v;
+            if (MODE == kDecParts) a.part_o[(((int64_t)hd * S + rank) * G + hh) * kHeadDim + tid] = v;
+            else s_acc[hh * kHeadDim + tid] = v;
         }
         if (tid < G) {
             float M2 = -INFINITY;
@@ -399,9 +449,14 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
                 const float mw = s_wm[w * 8 + tid];
                 if (mw > -INFINITY) Ls += s_wl[w * 8 + tid] * exp2f(mw - M2);
             }
+            if (MODE == kDecParts) a.part_ml[((int64_t)hd * S + rank) * G + tid] = make_float2(M2, Ls);
             s_M[tid] = M2;
             s_L[tid] = Ls;
         }
+    }
+    if (MODE == kDecParts) {
+        if (rank == 0 && tid == 0) a.part_len[hd] = app ? ln : -1;
+        return;
     }
 
     // ---- combine the CTAs of the cluster in rank order through distributed shared memory ----------------
@@ -506,6 +561,104 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     if (CL) cluster_wait();                               // nobody leaves while its shared memory is still read
 }
 
+// Adds the parts of every head.  grid (G + key slices, heads): CTA y < G finishes the output of query head y of the
+// group, the others add the probabilities of a slice of the keys to acc_score.  Latency-bound (0.3 to 1 MB in all): every
+// weight is worked out first, so that the loads of the parts depend on nothing - a warp takes every 16th part, a lane
+// four channels - and the warps are added in warp order.
+constexpr int kDecCombineThreads = 512;
+constexpr int kDecSliceKeys = 2 * kDecCombineThreads;
+
+template <int G>
+__global__ void __launch_bounds__(kDecCombineThreads) decode_combine_kernel(const DecodeArgs a) {
+    constexpr int kWarps = kDecCombineThreads / 32;
+    __shared__ float s_M[G], s_I[G];
+    __shared__ float s_w[kDecTargetCtas];                  // this query head's weight of every part
+    __shared__ float4 s_o[kWarps][32];
+    pdl_enter();
+    const int hd = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, S = a.S;
+    const float2* ml = a.part_ml + (int64_t)hd * S * G;
+    const int app_at = a.part_len[hd];
+    // every warp takes one of the query heads this CTA needs: (max, 1/sum) over the parts
+    const bool finish = (int)blockIdx.x < G;
+    const int hh_w = finish ? (int)blockIdx.x : warp;
+    if (finish ? warp == 0 : warp < G) {
+        float m[(kDecTargetCtas + 31) / 32], l[(kDecTargetCtas + 31) / 32], M = -INFINITY, Ls = 0.f;
+#pragma unroll
+        for (int u = 0; u < (kDecTargetCtas + 31) / 32; ++u) {
+            const int p = u * 32 + lane;
+            const float2 v = p < S ? ml[p * G + hh_w] : make_float2(-INFINITY, 0.f);
+            m[u] = v.x; l[u] = v.y;
+            M = fmaxf(M, v.x);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
+#pragma unroll
+        for (int u = 0; u < (kDecTargetCtas + 31) / 32; ++u) {
+            const int p = u * 32 + lane;
+            const float w = m[u] > -INFINITY ? exp2f(m[u] - M) : 0.f;
+            Ls += l[u] * w;
+            if (finish && p < S) s_w[p] = w;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) Ls += __shfl_xor_sync(0xFFFFFFFFu, Ls, o);
+        if (lane == 0) { s_M[hh_w] = M; s_I[hh_w] = Ls > 0.f ? 1.0f / Ls : 0.f; }
+    }
+    __syncthreads();
+    const int b = hd / a.Hkv, h0 = (hd % a.Hkv) * G;
+    if (finish) {
+        const int hh = blockIdx.x;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int p0 = warp; p0 < S; p0 += 8 * kWarps) {
+            float4 x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int p = p0 + u * kWarps;
+                x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (p < S && s_w[p] > 0.f)                 // (a part without keys has written no output)
+                    x[u] = __ldcg(reinterpret_cast<const float4*>(a.part_o + (((int64_t)hd * S + p) * G + hh) * kHeadDim) + lane);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int p = p0 + u * kWarps;
+                const float w = p < S ? s_w[p] : 0.f;
+                v.x += x[u].x * w; v.y += x[u].y * w; v.z += x[u].z * w; v.w += x[u].w * w;
+            }
+        }
+        s_o[warp][lane] = v;
+        __syncthreads();
+        if (tid < kHeadDim) {
+            float r = 0.f;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) r += reinterpret_cast<const float*>(s_o[w])[tid];
+            a.out[(int64_t)(b * a.H + h0 + hh) * kHeadDim + tid] = __float2bfloat16_rn(r * s_I[hh]);
+        }
+        if (hh == 0 && tid == 0 && app_at >= 0) a.len[hd] = app_at + 1;
+        return;
+    }
+    // (a.acc_score) where a row was appended another CTA bumps len meanwhile: part_len tells the keys then
+    const int lne = app_at >= 0 ? app_at + 1 : a.len[hd];
+    if (lne < 0 || lne > a.cap) return;                    // this head was skipped
+    float* acc = a.acc_score + (int64_t)hd * a.cap;
+    const int j0 = ((int)blockIdx.x - G) * kDecSliceKeys;
+    float lg[2][G], old[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int j = j0 + u * kDecCombineThreads + tid;
+        old[u] = 0.f;
+#pragma unroll
+        for (int hh = 0; hh < G; ++hh) lg[u][hh] = j < lne ? __ldcg(a.ws_s + (int64_t)(b * a.H + h0 + hh) * a.cap + j) : 0.f;
+        if (j < lne && j != app_at) old[u] = acc[j];       // a new entry starts at zero
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int j = j0 + u * kDecCombineThreads + tid;
+        float pr = 0.f;
+#pragma unroll
+        for (int hh = 0; hh < G; ++hh) pr += exp2f(lg[u][hh] - s_M[hh]) * s_I[hh];
+        if (j < lne) acc[j] = old[u] + pr;
+    }
+}
+
 template <int G>
 static lvlm_status launch_decode(const void* q, void* Kc, void* Vc, int32_t* len, const void* k_new,
                                  const void* v_new, float* acc_score, const lvlm_dims* d, float scale,
@@ -513,16 +666,14 @@ static lvlm_status launch_decode(const void* q, void* Kc, void* Vc, int32_t* len
                                  int64_t kv_sh, int32_t* dev_status, cudaStream_t stream) {
     // scaled logits of a CTA's own keys stay in shared memory when the longest run fits the budget
     const int nt_max = (d->cap + kTileKeys - 1) / kTileKeys;
-    int per = (nt_max + L.S - 1) / L.S;
+    const bool parts = L.P > 0 && nt_max >= parts_from_tiles((int64_t)d->B * d->Hkv, acc_score != nullptr);
+    const int S = parts ? L.P : L.S;
+    int per = (nt_max + S - 1) / S;
     if (per >= kDecWarps) per = (per + kDecWarps - 1) / kDecWarps * kDecWarps;
     const int run_keys = per * kTileKeys;
-    const int logit_keys = acc_score && (size_t)G * run_keys * 4 <= (size_t)kDecLogitBytes ? run_keys : 0;
+    const int logit_keys = acc_score && !parts && (size_t)G * run_keys * 4 <= (size_t)kDecLogitBytes ? run_keys : 0;
     const size_t smem = 1024 + (size_t)kRingBytes + (size_t)(2 * kDecWarps * 8 + 4 * 8 + 2 * 8 * kDecMaxCluster) * 4 +
                         (size_t)(2 * kStagesDec + 1) * 8 + (size_t)G * logit_keys * 4;
-    LVLM_RETURN_IF_CUDA(cudaFuncSetAttribute(decode_cluster_kernel<G, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem));
-    LVLM_RETURN_IF_CUDA(cudaFuncSetAttribute(decode_cluster_kernel<G, false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem));
     CUtensorMap kmap, vmap;
     {
         const uint64_t dims[4] = {(uint64_t)kHeadDim, (uint64_t)d->cap, (uint64_t)d->Hkv, (uint64_t)d->B};
@@ -531,7 +682,7 @@ static lvlm_status launch_decode(const void* q, void* Kc, void* Vc, int32_t* len
         if (!make_tmap_bf16(&kmap, Kc, 4, dims, strides, box) || !make_tmap_bf16(&vmap, Vc, 4, dims, strides, box))
             return LVLM_ERR_CUDA;
     }
-    const int64_t ctas = (int64_t)d->B * d->Hkv * L.S;
+    const int64_t ctas = (int64_t)d->B * d->Hkv * S;
     if (ctas > 0x7FFFFFFFll) return LVLM_ERR_UNSUPPORTED;
     DecodeArgs a;
     a.q = static_cast<const __nv_bfloat16*>(q);
@@ -542,28 +693,30 @@ static lvlm_status launch_decode(const void* q, void* Kc, void* Vc, int32_t* len
     a.v_new = static_cast<const __nv_bfloat16*>(v_new);
     a.acc_score = acc_score;
     a.out = static_cast<__nv_bfloat16*>(out);
-    a.H = d->H; a.Hkv = d->Hkv; a.cap = d->cap; a.S = L.S;
+    a.H = d->H; a.Hkv = d->Hkv; a.cap = d->cap; a.S = S;
     a.early = d->cache_stable != 0 && pdl_enabled();
     a.kv_sb = kv_sb; a.kv_sh = kv_sh; a.scale_log2 = scale * kLog2e;
     a.ws_s = acc_score ? reinterpret_cast<float*>(wsb + L.off_s) : nullptr;
     a.logit_keys = logit_keys;
     a.dev_status = dev_status;
 
-    if (L.S == 1)
-        return launch_kernel(decode_cluster_kernel<G, false>, dim3((unsigned)ctas), dim3(kDecThreads), smem, stream, 1, kmap, vmap, a);
-    return launch_kernel(decode_cluster_kernel<G, true>, dim3((unsigned)ctas), dim3(kDecThreads), smem, stream, L.S, kmap, vmap, a);
+    a.part_ml = reinterpret_cast<float2*>(wsb + L.off_ml);
+    a.part_o = reinterpret_cast<float*>(wsb + L.off_o);
+    a.part_len = reinterpret_cast<int32_t*>(wsb + L.off_len);
+    void (*kernel)(CUtensorMap, CUtensorMap, DecodeArgs) =
+        parts ? decode_cluster_kernel<G, kDecParts> : S == 1 ? decode_cluster_kernel<G, kDecSolo> : decode_cluster_kernel<G, kDecCluster>;
+    LVLM_RETURN_IF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem));
+    const lvlm_status st = launch_kernel(kernel, dim3((unsigned)ctas), dim3(kDecThreads), smem, stream, parts ? 1 : S, kmap, vmap, a);
+    if (st != LVLM_OK || !parts) return st;
+    const int slices = acc_score ? (d->cap + kDecSliceKeys - 1) / kDecSliceKeys : 0;
+    return launch_kernel(decode_combine_kernel<G>, dim3((unsigned)(G + slices), (unsigned)(d->B * d->Hkv)), dim3(kDecCombineThreads),
+                         0, stream, 1, a);
 }
 
-}  // namespace lvlm
-
-extern "C" lvlm_status lvlm_decode_attn(const void* q, void* Kc, void* Vc, int32_t* len,
-                                         const void* k_new, const void* v_new, float* acc_score,
-                                         const lvlm_dims* d, float scale, void* out, void* ws,
-                                         size_t ws_bytes, int32_t* dev_status, void* stream_) {
-    using namespace lvlm;
-    cudaStream_t stream = (cudaStream_t)stream_;
-    DecodeLayout L;
-    if (!q || !Kc || !Vc || !len || !out || !decode_layout(d, &L)) return LVLM_ERR_INVALID_ARG;
+static lvlm_status decode_attn(const void* q, void* Kc, void* Vc, int32_t* len, const void* k_new, const void* v_new,
+                               float* acc_score, const lvlm_dims* d, const DecodeLayout& L, float scale, void* out,
+                               void* ws, size_t ws_bytes, int32_t* dev_status, cudaStream_t stream) {
+    if (!q || !Kc || !Vc || !len || !out) return LVLM_ERR_INVALID_ARG;
     if ((k_new == nullptr) != (v_new == nullptr)) return LVLM_ERR_INVALID_ARG;
     const int G = d->H / d->Hkv;
     if (d->D != kHeadDim || G > kMaxGroup) return LVLM_ERR_UNSUPPORTED;
@@ -583,6 +736,19 @@ extern "C" lvlm_status lvlm_decode_attn(const void* q, void* Kc, void* Vc, int32
     }
 #undef LVLM_DEC_CASE
     return LVLM_ERR_UNSUPPORTED;
+}
+
+}  // namespace lvlm
+
+extern "C" lvlm_status lvlm_decode_attn(const void* q, void* Kc, void* Vc, int32_t* len,
+                                         const void* k_new, const void* v_new, float* acc_score,
+                                         const lvlm_dims* d, float scale, void* out, void* ws,
+                                         size_t ws_bytes, int32_t* dev_status, void* stream_) {
+    using namespace lvlm;
+    DecodeLayout L;
+    if (!decode_layout(d, &L)) return LVLM_ERR_INVALID_ARG;
+    return decode_attn(q, Kc, Vc, len, k_new, v_new, acc_score, d, L, scale, out, ws, ws_bytes, dev_status,
+                       (cudaStream_t)stream_);
 }
 
 // ---- decode attention for callers that cannot allocate ------------------------------------------
@@ -620,10 +786,11 @@ extern "C" lvlm_status lvlm_decode_attn_static(const void* q, void* Kc, void* Vc
     using namespace lvlm;
     DecodeLayout L;
     if (!decode_layout(d, &L)) return LVLM_ERR_INVALID_ARG;
+    if (L.total > (size_t)LVLM_STATIC_SCRATCH_BYTES) decode_layout(d, &L, false);     // without room for parts
     if (L.total > (size_t)LVLM_STATIC_SCRATCH_BYTES) return LVLM_ERR_WORKSPACE;
     void* scratch = nullptr;
     const lvlm_status st = static_scratch_address(&scratch);
     if (st != LVLM_OK) return st;
-    return lvlm_decode_attn(q, Kc, Vc, len, k_new, v_new, acc_score, d, scale, out, scratch,
-                            (size_t)LVLM_STATIC_SCRATCH_BYTES, dev_status, stream);
+    return decode_attn(q, Kc, Vc, len, k_new, v_new, acc_score, d, L, scale, out, scratch,
+                       (size_t)LVLM_STATIC_SCRATCH_BYTES, dev_status, (cudaStream_t)stream);
 }
