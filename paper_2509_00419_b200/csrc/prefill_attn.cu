@@ -458,7 +458,6 @@ extern "C" lvlm_status lvlm_prefill_attn(const void* Q, const void* K, const voi
     if (s0 != LVLM_OK || !score) return s0;
     // the column sums of the window: the second pass of lvlm_score_tokens, fed by the normalisers written above
     const __nv_bfloat16* Qwin = static_cast<const __nv_bfloat16*>(Q) + (int64_t)d->q_lo * st.q_sn;
-    return launch_score_tc(Qwin, K, nullptr, d, st, scale, reinterpret_cast<float*>(wsb + L.off_lse),
-                           reinterpret_cast<float*>(wsb + L.off_partial), reinterpret_cast<int32_t*>(wsb + L.off_cnt),
-                           score, score_head, dev_status, stream, /*normalisers_ready=*/true);
+    return launch_score_tc(Qwin, K, nullptr, d, st, scale, L, wsb, score, score_head, dev_status, stream,
+                           /*normalisers_ready=*/true);
 }

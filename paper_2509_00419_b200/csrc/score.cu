@@ -12,10 +12,13 @@ bool score_layout(const lvlm_dims* d, ScoreLayout* L) {
         d->i0 < 0 || (int64_t)d->i0 + d->n > d->N || d->q_lo < 0 || d->q_lo >= d->q_hi ||
         d->q_hi > d->N || d->cap < d->N)
         return false;
+    const ScoreShape s = L->shape = score_shape(d);
+    const size_t groups = (size_t)d->B * d->Hkv;
     size_t off = 0;
-    L->off_partial = off; off = align_up(off + (size_t)d->B * d->H * d->n * 4, 256);
+    L->off_partial = off; off = align_up(off + groups * s.parts * s.nkt * 128 * 4, 256);
     L->off_lse = off;     off = align_up(off + (size_t)d->B * d->H * (d->q_hi - d->q_lo) * 4, 256);
-    L->off_cnt = off;     off = align_up(off + (size_t)d->B * ((d->n + 127) / 128) * 4, 256);
+    L->off_nlse = off;    off = align_up(off + groups * s.tpg * 128 * 4, 256);
+    L->off_stat = off;    off = align_up(off + (s.ksplit > 1 ? groups * s.tpg * s.ksplit * 128 * 8 : 0), 256);
     L->total = off;
     return true;
 }
@@ -48,9 +51,5 @@ extern "C" lvlm_status lvlm_score_tokens(const void* Q, const void* K, const flo
         st.kv_sh % 8 || st.kv_sb % 8)
         return LVLM_ERR_ALIGNMENT;
     if (!ws || !aligned256(ws) || ws_bytes < L.total) return LVLM_ERR_WORKSPACE;
-    char* wsb = static_cast<char*>(ws);
-    float* partial = reinterpret_cast<float*>(wsb + L.off_partial);
-    float* lse_ws = reinterpret_cast<float*>(wsb + L.off_lse);
-    return launch_score_tc(Q, K, lse, d, st, scale, lse_ws, partial,
-                           reinterpret_cast<int32_t*>(wsb + L.off_cnt), score, score_head, dev_status, stream);
+    return launch_score_tc(Q, K, lse, d, st, scale, L, static_cast<char*>(ws), score, score_head, dev_status, stream);
 }

@@ -57,3 +57,31 @@ def test_decode_in_parts_bad_lengths_are_skipped():
     assert flag.item() == L.DEV_BOUNDS and ln.tolist() == [[cap + 1, -1, cap, 701]]
     assert not out[0, :2].any() and not acc[0, :2].any()
     assert abs(acc[0, 2].sum().item() - 1) < 1e-4 and abs(acc[0, 3, :701].sum().item() - 1) < 1e-4 and not acc[0, 3, 701:].any()
+
+
+# scoring: few and many tiles (small and large shape of the kernel), heads of a group in one query tile or one each, windows
+# whose rows lie several times in a tile, query tiles kept over key tiles or not, splits with remainders, own normalisers
+@pytest.mark.parametrize("case", [        # B, H, Hkv, N, i0, n, T, causal, lse
+    (1, 1, 1, 130, 0, 1, 1, True, False), (1, 2, 2, 700, 3, 640, 32, True, False), (2, 4, 4, 513, 0, 385, 33, True, True),
+    (1, 8, 1, 400, 70, 250, 64, True, False), (1, 14, 2, 1155, 5, 1025, 65, False, False), (1, 28, 4, 3012, 1, 2880, 131, True, False),
+    (3, 24, 4, 1300, 0, 1283, 17, True, True), (16, 8, 2, 1500, 0, 1409, 91, True, False), (8, 12, 4, 2100, 0, 2000, 100, True, True),
+    (1, 6, 2, 1200, 100, 1000, 1200, True, False), (2, 16, 8, 1409, 0, 1409, 1409, True, False), (1, 5, 1, 900, 0, 900, 900, False, True)])
+def test_score_shapes(case):
+    B, H, Hkv, N, i0, n, T, causal, own = case
+    g = torch.Generator(device="cuda").manual_seed(N + H)
+    Q = torch.randn(B, T, H, 128, generator=g, device="cuda").to(torch.bfloat16)
+    K = torch.randn(B, Hkv, N, 128, generator=g, device="cuda").to(torch.bfloat16)
+    k = K.double().repeat_interleave(H // Hkv, dim=1)
+    logits = torch.einsum("bthd,bhnd->bhtn", Q.double(), k) / 128 ** 0.5
+    if causal:
+        hidden = torch.arange(N, device="cuda")[None] > torch.arange(N - T, N, device="cuda")[:, None]
+        logits.masked_fill_(hidden, -torch.inf)
+    lse = torch.logsumexp(logits, dim=-1)
+    s_head = torch.exp(logits - lse[..., None])[..., i0:i0 + n].sum(dim=2)
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(2):                     # the second call finds the workspace as the first one left it
+        score, head = L.score_tokens(Q, K, N=N, i0=i0, n=n, q_lo=N - T, q_hi=N, causal=causal, want_head=True,
+                                     lse=lse.float() if own else None, dev_status=flag)
+    assert flag.item() == 0
+    assert_scores_close(f64(score), f64(s_head.mean(dim=1)), what="score")
+    assert_scores_close(f64(head), f64(s_head.view(B, Hkv, H // Hkv, n).sum(dim=2)), what="score_head")
