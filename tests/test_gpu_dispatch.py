@@ -85,3 +85,30 @@ def test_score_shapes(case):
     assert flag.item() == 0
     assert_scores_close(f64(score), f64(s_head.mean(dim=1)), what="score")
     assert_scores_close(f64(head), f64(s_head.view(B, Hkv, H // Hkv, n).sum(dim=2)), what="score_head")
+
+
+# attention: pairs of heads, pairs of query tiles of the odd head, a lone last tile; the key tiles of one query tile split
+# between the halves of a CTA (few tiles); one key tile, ragged ends, rows that see one key
+@pytest.mark.parametrize("case", [        # B, H, Hkv, N, causal
+    (1, 1, 1, 1, True), (1, 2, 2, 128, True), (1, 3, 1, 129, False), (1, 7, 1, 257, True), (2, 8, 2, 384, True),
+    (1, 28, 4, 1025, True), (6, 12, 4, 900, True), (3, 9, 3, 1300, False), (1, 48, 8, 1409, True), (13, 8, 8, 515, True)])
+def test_attention_shapes(case):
+    B, H, Hkv, N, causal = case
+    g = torch.Generator(device="cuda").manual_seed(N + H)
+    Q = (3 * torch.randn(B, N, H, 128, generator=g, device="cuda")).to(torch.bfloat16)
+    K = torch.randn(B, Hkv, N, 128, generator=g, device="cuda").to(torch.bfloat16)
+    V = torch.randn(B, Hkv, N, 128, generator=g, device="cuda").to(torch.bfloat16)
+    out, lse = torch.full_like(Q, 9.0), torch.empty(B, H, N, device="cuda")
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    first = None
+    for _ in range(4):
+        L.prefill_attn(Q, K, V, N=N, causal=causal, out=out, lse=lse, dev_status=flag)
+        first = out.clone() if first is None else first
+        assert torch.equal(out, first)
+    logits = torch.einsum("bthd,bhnd->bhtn", Q.double(), K.double().repeat_interleave(H // Hkv, dim=1)) / 128 ** 0.5
+    if causal:
+        logits.masked_fill_(torch.ones(N, N, dtype=torch.bool, device="cuda").triu(1), -torch.inf)
+    want = torch.einsum("bhtn,bhnd->bthd", torch.softmax(logits, dim=-1), V.double().repeat_interleave(H // Hkv, dim=1))
+    assert flag.item() == 0
+    assert_rows_close(f64(out), f64(want), what="attention output")
+    np.testing.assert_allclose(f64(lse), f64(torch.logsumexp(logits, dim=-1)), rtol=1e-5, atol=1e-5)   # fp32 sums
