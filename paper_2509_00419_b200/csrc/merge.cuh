@@ -18,6 +18,7 @@ struct StreamKv { const void* K; const void* V; int64_t kv_sb, kv_sh; int Hkv, k
 // Reads every input row of `hidden` once.  dst_map[b][i] >= 0: the row is copied to that row of
 // hidden_out; == -1: it is added, times wgt, to the merged row P_new at row i0+k (wgt != NULL);
 // <= -2: it is copied to row -dst-2 of `scratch` (scratch != NULL).  Strides in elements.
+// inv_norm (without wgt): [B][k], 1 / |x| of the kept image rows (1 for a zero row), by output row.
 // hidden_out == NULL: nothing is stored, only the merged rows are read and one fp32 partial row per cluster
 // is left in `partial` ([B][*partials_out][C]) for the in-place compaction that follows.  L gives the launch
 // shape at most: fewer CTAs are used when the device cannot run that many clusters at a time.
@@ -25,7 +26,8 @@ lvlm_status launch_hidden_rows(const void* hidden, void* hidden_out, int64_t hid
                                const lvlm_dims* d, const HiddenGrid& L, const int32_t* dst_map,
                                const float* wgt, int32_t* meta, float* partial, void* scratch,
                                int64_t scr_sb, cudaStream_t stream, const StreamKv* kv = nullptr,
-                               int32_t* dev_status = nullptr, int* partials_out = nullptr);
+                               int32_t* dev_status = nullptr, int* partials_out = nullptr,
+                               float* inv_norm = nullptr);
 
 // lvlm_merge_compact in mode LVLM_W_NEAREST_KEPT (nearest_kept.cu).
 size_t nearest_kept_workspace(const lvlm_dims* d);

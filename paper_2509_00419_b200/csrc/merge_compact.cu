@@ -324,6 +324,7 @@ struct StreamArgs {
     const char* K; const char* Vc; int64_t kv_sb, kv_sh; // bytes
     int Hkv, kvP, kvL, kvT;
     float* kv_partial;
+    float* inv_norm;                                     // [B][k], without wgt: 1 / |x| of the kept image rows
     int32_t* dev_status;
 };
 
@@ -557,6 +558,24 @@ __global__ void __launch_bounds__(kStreamThreads, 1) row_stream_kernel(const Str
                     }
                 }
             }
+            if (ok && a.inv_norm) {
+                // 1 / |x| of the kept image rows: a warp a row, fixed order of summation
+                for (int l = warp; l < t.cnt; l += kHidThreads / 32) {
+                    const int q = td[l] - a.i0;
+                    if (q < 0 || q >= a.k) continue;
+                    const uint4* rowp = reinterpret_cast<const uint4*>(sbase + (size_t)l * a.rowB);
+                    float s = 0.f;
+                    for (int c = lane; c < a.V; c += 32) {
+                        const uint4 x = rowp[c];
+                        const float e0 = bf16_lo(x.x), e1 = bf16_hi(x.x), e2 = bf16_lo(x.y), e3 = bf16_hi(x.y);
+                        const float e4 = bf16_lo(x.z), e5 = bf16_hi(x.z), e6 = bf16_lo(x.w), e7 = bf16_hi(x.w);
+                        s += (e0 * e0 + e1 * e1) + (e2 * e2 + e3 * e3) + (e4 * e4 + e5 * e5) + (e6 * e6 + e7 * e7);
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+                    if (lane == 0) a.inv_norm[(int64_t)b * a.k + q] = s > 0.f ? rsqrtf(s) : 1.f;
+                }
+            }
             __syncwarp();
             if (lane == 0) sm100::mbar_arrive(&s_empty[slot]);
             if (t.kv && t.item_end) {
@@ -667,7 +686,7 @@ lvlm_status launch_hidden_rows(const void* hidden, void* hidden_out, int64_t hid
                                const lvlm_dims* d, const HiddenGrid& L, const int32_t* dst_map,
                                const float* wgt, int32_t* meta, float* partial, void* scratch,
                                int64_t scr_sb, cudaStream_t stream, const StreamKv* kv, int32_t* dev_status,
-                               int* partials_out) {
+                               int* partials_out, float* inv_norm) {
     const int chunks = (L.V + kHidThreads - 1) / kHidThreads;
     if (chunks > kHidMaxChunks || L.nstage < 3) return LVLM_ERR_UNSUPPORTED;  // more than 8192 channels
     // No more clusters than the device runs at a time: a second wave would double the time.  Clusters are placed
@@ -710,6 +729,7 @@ lvlm_status launch_hidden_rows(const void* hidden, void* hidden_out, int64_t hid
         a.kvT = L.slotB / kKvRowBytes >= 64 ? 64 : (L.slotB / kKvRowBytes) / 16 * 16;
         a.kv_partial = kv->kv_partial;
     }
+    a.inv_norm = inv_norm;
     a.dev_status = dev_status;
     switch (chunks) {
         case 1: return launch_row_stream<1>(a, cps, cl_run, d->B, stream);

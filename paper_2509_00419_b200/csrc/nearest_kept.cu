@@ -4,32 +4,34 @@
 // (lower kept index wins ties); masses make repeated merging a true mean.
 //
 // Launches, all on the caller's stream:
-//   plan      one CTA per sequence: kept / dropped token lists, row maps, position ids, new length
-//   rows      the streaming kernel of the hidden states: kept rows to their place in the output,
+//   plan      a cluster per sequence: kept / dropped token lists, row map, position ids, new length
+//   rows      the streaming kernel of the hidden states: kept rows to their place in the output, with 1 / |x_t| on the way,
 //             dropped rows side by side into scratch
-//   norms     1 / |x_t| of every kept row
 //   sim       dropped x kept similarity on the tensor cores (tcgen05, accumulators in TMEM, operands by
 //             TMA), arg-max per dropped row in the epilogue, merged over column splits with atomicMax
 //             on (similarity, ~index) keys
-//   group     dropped tokens sorted by (kept token, own index) by rank counting -> segments
+//   group     dropped tokens by kept token: counts, places, and the tokens of a kept token in ascending order
 //   merge     every kept row becomes the mass-weighted mean of itself and its segment, in token order
-//   K, V      the same mean per KV head into scratch, text rows shifted down in place, means stored
+//   K, V      the same mean per KV head, and the rows behind the image, into scratch; then stored in place
 //   mass      token masses compacted in place
+// us at 16384 + 256 tokens of 6144 channels, 4096 kept, before -> now: plan 39 -> 10, norms 8 -> 0, similarity 523 -> 452 (618
+// GFLOP: 1370 TFLOP/s), group 92 -> 22, K and V 60 -> 35; rows 64 and merge 46 run at the copy rate.
 #include "common.cuh"
-#include "compact.cuh"
 #include "merge.cuh"
 #include "sm100.cuh"
-#include "rank_count.cuh"
 
 namespace lvlm {
 
 using namespace sm100;
 
+constexpr int kMaxDropped = 65536;
+
 struct NkLayout {
     int r, Nout, V;
     HiddenGrid grid;
-    size_t off_assign, off_src, off_dst, off_kept, off_drop, off_inv, off_best, off_order, off_sorted, off_seg,
-           off_meta, off_newmass, off_scratch, off_kvtmp, total;
+    int rest;                           // rows behind the image
+    size_t off_assign, off_dst, off_kept, off_drop, off_inv, off_best, off_place, off_order, off_seg, off_newmass,
+           off_scratch, off_kvtmp, total;
 };
 
 static bool nk_layout(const lvlm_dims* d, NkLayout* L) {
@@ -43,20 +45,19 @@ static bool nk_layout(const lvlm_dims* d, NkLayout* L) {
     L->grid = hidden_grid(d);
     size_t off = 0;
     L->off_assign = off;  off = align_up(off + B * (r ? r : 1) * 4, 256);   // first: callers may read it
-    L->off_src = off;     off = align_up(off + B * d->N * 4, 256);
+    L->rest = d->N - d->i0 - d->n;
     L->off_dst = off;     off = align_up(off + B * d->N * 4, 256);
     L->off_kept = off;    off = align_up(off + B * (k ? k : 1) * 4, 256);
     L->off_drop = off;    off = align_up(off + B * (r ? r : 1) * 4, 256);
     L->off_inv = off;     off = align_up(off + B * (k ? k : 1) * 4, 256);
     L->off_best = off;    off = align_up(off + B * (r ? r : 1) * 8, 256);
-    L->off_order = off;   off = align_up(off + B * (r ? r : 1) * 4, 256);
-    L->off_sorted = off;  off = align_up(off + B * (r ? r : 1) * 4, 256);
+    L->off_place = off;   off = align_up(off + B * (r ? r : 1) * 4, 256);
+    L->off_order = off;   off = align_up(off + B * (r ? r : 1) * 8, 256);
     L->off_seg = off;     off = align_up(off + B * (k + 1) * 4, 256);
-    L->off_meta = off;    off = align_up(off + B * kMetaInts * 4, 256);
     L->off_newmass = off; off = align_up(off + B * (k ? k : 1) * 4, 256);
     L->off_scratch = off; off = align_up(off + B * (r ? r : 1) * (size_t)d->C * 2, 256);
     L->off_kvtmp = off;
-    if (d->Hkv > 0) off = align_up(off + B * d->Hkv * 2 * (k ? k : 1) * (size_t)kHeadDim * 2, 256);
+    if (d->Hkv > 0) off = align_up(off + B * d->Hkv * 2 * (k + L->rest + 1) * (size_t)kHeadDim * 2, 256);
     L->total = off;
     return true;
 }
@@ -67,135 +68,188 @@ size_t nearest_kept_workspace(const lvlm_dims* d) {
 }
 
 // ---- plan ------------------------------------------------------------------------------------------
-// One CTA per sequence.  kept[q] / drop[q]: image-token indices in ascending order.
-// dst[i]: output row of input row i, or -2-q for the q-th dropped token.  src[o]: input row of
-// output row o.  Position ids are compacted in place (tile by tile, sources lie at or after
-// their destination).
+__device__ __forceinline__ uint32_t nk_cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void nk_cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n"
+                 "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ int nk_ld_cluster(const int* my_smem, uint32_t rank) {
+    uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+    int v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
+    return v;
+}
+
+// A cluster of P CTAs per sequence (grid (P, B)), CTA c the c-th run of the image tokens: it counts its kept tokens, learns
+// from the lower ranks how many came before, then writes its run tile by tile (thread = token, coalesced; one CTA with
+// a run of tokens per thread took 39 us for 16384 tokens).  kept[q] / drop[q]: image-token indices in ascending
+// order.  dst[i]: output row of input row i, or -2-q for the q-th dropped token.  Position ids are compacted in place in
+// rounds (sources lie at or after their destination): every CTA loads its rows of the round, a barrier, then stores.
 __global__ void __launch_bounds__(1024)
 nk_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int i0, int n, int k,
-               int32_t* __restrict__ src_map, int32_t* __restrict__ dst_map, int32_t* __restrict__ kept,
-               int32_t* __restrict__ drop, unsigned long long* __restrict__ best, int32_t* __restrict__ meta,
-               int32_t* new_len, int32_t* dev_status) {
+               int32_t* __restrict__ dst_map, int32_t* kept, int32_t* __restrict__ drop,
+               unsigned long long* __restrict__ best, int32_t* __restrict__ seg, int32_t* new_len, int32_t* dev_status) {
     __shared__ int scan_scratch[33];
+    __shared__ int s_total;
     pdl_enter();
-    const int b = blockIdx.x, r = n - k, Nout = N - r;
+    const int b = blockIdx.y, r = n - k, Nout = N - r, P = (int)gridDim.x, cr = (int)nk_cluster_rank();
     const int32_t* rk = rank + (int64_t)b * n;
-    int32_t* src = src_map + (int64_t)b * N;
     int32_t* dst = dst_map + (int64_t)b * N;
-    const int per = (n + blockDim.x - 1) / blockDim.x;
-    const int j0 = min(n, (int)threadIdx.x * per), j1 = min(n, j0 + per);
-    int cnt = 0;
+    int32_t* kp = kept + (int64_t)b * k;
+    const int chunk = (n + P - 1) / P;
+    const int c_lo = min(n, cr * chunk), c_hi = min(n, c_lo + chunk);
+    if (threadIdx.x == 0) s_total = 0;
+    __syncthreads();
     bool bad = false;
-    for (int j = j0; j < j1; ++j) {
+    int mine = 0;
+    for (int j = c_lo + threadIdx.x; j < c_hi; j += blockDim.x) {
         const int rj = rk[j];
         if (rj < 0 || rj >= n) bad = true;
-        cnt += rj < k;
+        mine += rj < k;
     }
-    int total;
-    int kq = block_exclusive_scan(cnt, scan_scratch, &total);      // kept tokens before j0
-    if (total != k) bad = true;
-    int dq = j0 - kq;                                              // dropped tokens before j0
-    for (int j = j0; j < j1; ++j) {
-        if (rk[j] < k) {
-            if (kq < k) { kept[(int64_t)b * k + kq] = j; src[i0 + kq] = i0 + j; dst[i0 + j] = i0 + kq; }
-            else dst[i0 + j] = -2 - min(dq, max(r - 1, 0));
-            ++kq;
-        } else {
-            if (dq < r) { drop[(int64_t)b * r + dq] = j; best[(int64_t)b * r + dq] = 0ull; dst[i0 + j] = -2 - dq; }
-            else dst[i0 + j] = i0;                                 // inconsistent rank: flagged below
-            ++dq;
+    mine = warp_sum(mine);
+    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&s_total, mine);
+    nk_cluster_barrier();
+    int kq = 0, all = 0;
+    for (int c = 0; c < P; ++c) {
+        const int t = nk_ld_cluster(&s_total, c);
+        kq += c < cr ? t : 0;
+        all += t;
+    }
+    if (all != k) bad = true;
+    for (int t0 = c_lo; t0 < c_hi; t0 += blockDim.x) {
+        const int j = t0 + threadIdx.x;
+        const int is_kept = j < c_hi && rk[j] < k;
+        int total;
+        const int q = kq + block_exclusive_scan(is_kept, scan_scratch, &total);         // kept tokens before mine
+        if (j < c_hi) {
+            const int dq = j - q;                                                       // dropped tokens before mine
+            if (is_kept) {
+                if (q < k) kp[q] = j;
+                dst[i0 + j] = q < k ? i0 + q : -2 - min(dq, max(r - 1, 0));              // (inconsistent rank: flagged below)
+            } else {
+                if (dq < r) { drop[(int64_t)b * r + dq] = j; best[(int64_t)b * r + dq] = 0ull; }
+                dst[i0 + j] = dq < r ? -2 - dq : i0;
+            }
         }
+        kq += total;
     }
-    for (int o = threadIdx.x; o < Nout; o += blockDim.x) {
-        if (o < i0) { src[o] = o; dst[o] = o; }
-        else if (o >= i0 + k) { src[o] = o + r; dst[o + r] = o; }
-    }
+    const int first = cr * blockDim.x + threadIdx.x, step = P * blockDim.x;
+    for (int o = first; o < i0; o += step) dst[o] = o;
+    for (int o = i0 + k + first; o < Nout; o += step) dst[o + r] = o;
+    for (int t = first; t <= k; t += step) seg[(int64_t)b * (k + 1) + t] = 0;            // counts, to begin with
     if (bad && dev_status) atomicOr(dev_status, LVLM_DEV_BOUNDS);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        meta[b * kMetaInts + 0] = i0;                               // first row of K, V that changes
-        meta[b * kMetaInts + 1] = 0;
-        if (new_len) new_len[b] = Nout;
-    }
+    if (cr == 0 && threadIdx.x == 0 && new_len) new_len[b] = Nout;
+    nk_cluster_barrier();                                                               // the kept list is complete
     if (pos_ids) {
         int32_t* pid = pos_ids + (int64_t)b * N;
-        for (int o0 = 0; o0 < Nout; o0 += blockDim.x) {
-            const int o = o0 + threadIdx.x;
+        for (int o0 = i0; o0 < Nout; o0 += step) {
+            const int o = o0 + first;
             int val = 0;
-            __syncthreads();
-            if (o < Nout) val = pid[src[o]];
-            __syncthreads();
+            if (o < Nout) val = pid[o < i0 + k ? i0 + (all == k ? kp[o - i0] : o - i0) : o + r];
+            nk_cluster_barrier();
             if (o < Nout) pid[o] = val;
         }
     }
-}
-
-// ---- norms -----------------------------------------------------------------------------------------
-// One warp per kept row of the output: 1 / |x| in fp32 (1 for a zero row), fixed summation order.
-__global__ void __launch_bounds__(256)
-nk_norm_kernel(const uint4* __restrict__ out, int64_t out_stride_b, int V, int i0, int k,
-               float* __restrict__ inv_norm) {
-    pdl_enter();
-    const int b = blockIdx.y, lane = threadIdx.x & 31;
-    const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (t >= k) return;
-    const uint4* row = out + (int64_t)b * out_stride_b + (int64_t)(i0 + t) * V;
-    float s = 0.f;
-    for (int c = lane; c < V; c += 32) {
-        const uint4 x = __ldg(row + c);
-        const float e0 = bf16_lo(x.x), e1 = bf16_hi(x.x), e2 = bf16_lo(x.y), e3 = bf16_hi(x.y);
-        const float e4 = bf16_lo(x.z), e5 = bf16_hi(x.z), e6 = bf16_lo(x.w), e7 = bf16_hi(x.w);
-        s += (e0 * e0 + e1 * e1) + (e2 * e2 + e3 * e3) + (e4 * e4 + e5 * e5) + (e6 * e6 + e7 * e7);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-    if (lane == 0) inv_norm[(int64_t)b * k + t] = s > 0.f ? rsqrtf(s) : 1.f;
+    nk_cluster_barrier();                                  // nobody leaves while its shared memory may still be read
 }
 
 // ---- group -----------------------------------------------------------------------------------------
-// Dropped tokens sorted by (kept token they go to, own order), by counting ranks: grid (blocks of 256
-// dropped tokens, S, B), clusters (1, S, 1).  Writes the assignment, the sorted order and the kept
-// token at every place of that order; a second kernel finds where every kept token's segment starts.
-__global__ void __launch_bounds__(kRankThreads)
-nk_group_kernel(const unsigned long long* __restrict__ best, int r, int k, int S, int slice_len, int jt,
-                int32_t* __restrict__ assign, int32_t* __restrict__ order, int32_t* __restrict__ sorted_t) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_cnt[kRankMaxJT * kRankThreads];
+// Dropped tokens by the kept token they go to.  count: the assignment, how many go to every kept token (in seg) and a
+// place among them, in order of arrival.  place: where every kept token's segment starts, and every dropped token into
+// its segment.  sort: the segments, a few tokens each, in ascending token order - so the order of arrival does not matter.
+// (Ranking all tokens against each other took 92 us for 12288 of them.)
+__global__ void __launch_bounds__(256)
+nk_count_kernel(const unsigned long long* __restrict__ best, int r, int k, int32_t* __restrict__ assign,
+                int32_t* __restrict__ place, int32_t* seg) {
     pdl_enter();
-    const int b = blockIdx.z;
-    const unsigned long long* bb = best + (int64_t)b * r;
-    auto key_of = [&](int q) {
-        const uint32_t t = 0xFFFFFFFFu - (uint32_t)(bb[q] & 0xFFFFFFFFull);
-        return ((uint64_t)(t < (uint32_t)k ? t : 0u) << 32) | (uint32_t)q;     // nothing won: kept token 0
-    };
-    int p[kRankMaxJT];
-    if (rank_by_counting(key_of, r, S, slice_len, jt, reinterpret_cast<uint64_t*>(smem_raw), s_cnt, p)) {
+    const int b = blockIdx.y, q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= r) return;
+    uint32_t t = 0xFFFFFFFFu - (uint32_t)(__ldcg(best + (int64_t)b * r + q) & 0xFFFFFFFFull);
+    t = t < (uint32_t)k ? t : 0u;                          // nothing won: kept token 0
+    assign[(int64_t)b * r + q] = (int)t;
+    place[(int64_t)b * r + q] = atomicAdd(seg + (int64_t)b * (k + 1) + t, 1);
+}
+
+// One CTA per sequence.  order[p] = (dropped token q, its image-token index).
+__global__ void __launch_bounds__(1024)
+nk_place_kernel(int32_t* seg, int r, int k, const int32_t* __restrict__ assign, const int32_t* __restrict__ place,
+                const int32_t* __restrict__ drop, int2* __restrict__ order) {
+    __shared__ int scan_scratch[33];
+    pdl_enter();
+    const int b = blockIdx.x;
+    int32_t* sg = seg + (int64_t)b * (k + 1);
+    int before = 0;
+    for (int t0 = 0; t0 < k + 1; t0 += 4 * blockDim.x) {   // four consecutive counts a thread
+        int c[4], sum = 0, total;
 #pragma unroll
-        for (int u = 0; u < kRankMaxJT; ++u) {
-            const int q = rank_key_index(jt, u);
-            if (u < jt && q < r) {
-                const int t = (int)(key_of(q) >> 32);
-                assign[(int64_t)b * r + q] = t;
-                order[(int64_t)b * r + p[u]] = q;
-                sorted_t[(int64_t)b * r + p[u]] = t;
-            }
+        for (int u = 0; u < 4; ++u) {
+            const int t = t0 + threadIdx.x * 4 + u;
+            c[u] = t < k ? sg[t] : 0;
+            sum += c[u];
         }
+        int run = before + block_exclusive_scan(sum, scan_scratch, &total);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = t0 + threadIdx.x * 4 + u;
+            if (t <= k) sg[t] = run;
+            run += c[u];
+        }
+        before += total;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < r; q += blockDim.x) {
+        const int64_t i = (int64_t)b * r + q;
+        order[(int64_t)b * r + sg[assign[i]] + place[i]] = make_int2(q, drop[i]);
     }
 }
 
-// seg[t] = first place of the sorted order whose kept token is >= t (t = 0..k).
-__global__ void __launch_bounds__(256)
-nk_seg_kernel(const int32_t* __restrict__ sorted_t, int r, int k, int32_t* __restrict__ seg) {
+// A warp per kept token; the segments with more than 32 tokens are sorted by the CTA, through a bitmap of the dropped tokens.
+constexpr int kSortWarps = 8;
+__global__ void __launch_bounds__(kSortWarps * 32)
+nk_sort_kernel(const int32_t* __restrict__ seg, int r, int k, const int32_t* __restrict__ drop, int2* __restrict__ order) {
+    __shared__ uint32_t bits[kMaxDropped / 32];
+    __shared__ int scan_scratch[33];
+    __shared__ int s_long[kSortWarps];
     pdl_enter();
-    const int b = blockIdx.y, t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t > k) return;
-    const int32_t* st = sorted_t + (int64_t)b * r;
-    int lo = 0, hi = r;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (st[mid] < t) lo = mid + 1; else hi = mid;
+    const int b = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int t = blockIdx.x * kSortWarps + warp;
+    const int32_t* sg = seg + (int64_t)b * (k + 1);
+    int2* ord = order + (int64_t)b * r;
+    const int p0 = t < k ? sg[t] : 0, len = t < k ? sg[t + 1] - p0 : 0;
+    if (lane == 0) s_long[warp] = len > 32;
+    if (len > 1 && len <= 32) {
+        const int2 mine = lane < len ? ord[p0 + lane] : make_int2(0x7FFFFFFF, 0);
+        int at = 0;
+        for (int i = 0; i < len; ++i) at += __shfl_sync(0xFFFFFFFFu, mine.x, i) < mine.x;
+        __syncwarp();
+        if (lane < len) ord[p0 + at] = mine;
     }
-    seg[(int64_t)b * (k + 1) + t] = lo;
+    __syncthreads();
+    for (int w = 0; w < kSortWarps; ++w) {
+        if (!s_long[w]) continue;
+        const int tw = blockIdx.x * kSortWarps + w, q0 = sg[tw], q1 = sg[tw + 1];
+        const int words = (r + 31) / 32, per = (words + (int)blockDim.x - 1) / (int)blockDim.x;
+        for (int i = threadIdx.x; i < words; i += blockDim.x) bits[i] = 0u;
+        __syncthreads();
+        for (int p = q0 + threadIdx.x; p < q1; p += blockDim.x) { const int q = ord[p].x; atomicOr(&bits[q >> 5], 1u << (q & 31)); }
+        __syncthreads();
+        const int w0 = min(words, (int)threadIdx.x * per), w1 = min(words, w0 + per);
+        int cnt = 0, total;
+        for (int i = w0; i < w1; ++i) cnt += __popc(bits[i]);
+        int p = q0 + block_exclusive_scan(cnt, scan_scratch, &total);
+        for (int i = w0; i < w1; ++i)
+            for (uint32_t m = bits[i]; m; m &= m - 1) {
+                const int q = i * 32 + __ffs((int)m) - 1;
+                ord[p++] = make_int2(q, drop[(int64_t)b * r + q]);
+            }
+        __syncthreads();
+    }
 }
 
 // ---- merge of the hidden rows ------------------------------------------------------------------------
@@ -208,19 +262,17 @@ template <int CH>
 __global__ void __launch_bounds__(kNkThreads)
 nk_merge_kernel(uint4* __restrict__ out, int64_t out_stride_b, const uint4* __restrict__ scratch,
                 int64_t scr_stride_b, int V, int N, int i0, int k, int r,
-                const int32_t* __restrict__ kept, const int32_t* __restrict__ drop,
-                const int32_t* __restrict__ order, const int32_t* __restrict__ seg,
+                const int32_t* __restrict__ kept, const int2* __restrict__ order, const int32_t* __restrict__ seg,
                 const float* __restrict__ mass, float* __restrict__ newmass) {
     pdl_enter();
     const int b = blockIdx.y, tid = threadIdx.x;
     uint4* orow = out + (int64_t)b * out_stride_b + (int64_t)i0 * V;
     const uint4* srow = scratch + (int64_t)b * scr_stride_b;
-    const int32_t* ord = order + (int64_t)b * r;
-    const int32_t* dr = drop + (int64_t)b * r;
+    const int2* ord = order + (int64_t)b * r;
     const float* ms = mass ? mass + (int64_t)b * N + i0 : nullptr;
     for (int t = blockIdx.x; t < k; t += gridDim.x) {
         const int p0 = seg[(int64_t)b * (k + 1) + t], p1 = seg[(int64_t)b * (k + 1) + t + 1];
-        const float mt = ms ? ms[kept[(int64_t)b * k + t]] : 1.f;
+        const float mt = ms ? ms[min(max(kept[(int64_t)b * k + t], 0), k + r - 1)] : 1.f;
         float den = mt;
         float acc[CH][8];
 #pragma unroll
@@ -238,8 +290,9 @@ nk_merge_kernel(uint4* __restrict__ out, int64_t out_stride_b, const uint4* __re
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int p = pb + u;
-                const int q = p < p1 ? ord[p] : 0;
-                md[u] = p < p1 ? (ms ? ms[dr[q]] : 1.f) : 0.f;
+                const int2 e = p < p1 ? ord[p] : make_int2(0, 0);
+                const int q = e.x;
+                md[u] = p < p1 ? (ms ? ms[min(max(e.y, 0), k + r - 1)] : 1.f) : 0.f;
 #pragma unroll
                 for (int ci = 0; ci < CH; ++ci) {
                     const int c = tid + ci * kNkThreads;
@@ -279,71 +332,96 @@ nk_merge_kernel(uint4* __restrict__ out, int64_t out_stride_b, const uint4* __re
 }
 
 // ---- K and V ---------------------------------------------------------------------------------------------
-// The same mean per (sequence, KV head, tensor), read from the cache as it stands before compaction and
-// parked in scratch: 16 threads per 256-byte row, 16 kept rows per CTA.
+// The same mean per (sequence, KV head, tensor), read from the cache as it stands, and the rows behind the image as they
+// are, parked in scratch (a row of the cache may be the source of a row before it): 16 threads per 256-byte row, 16
+// rows per CTA.  Then stored.
+// A thread has the row in kKvSeqs of the Hkv * 2 sequences: they share the segment, whose look-up is a chain of loads.
+constexpr int kKvSeqs = 4;
 __global__ void __launch_bounds__(kNkThreads)
 nk_kv_merge_kernel(const uint4* __restrict__ Kc, const uint4* __restrict__ Vc, int64_t kv_sb, int64_t kv_sh,
-                   int Hkv, int N, int i0, int k, int r, const int32_t* __restrict__ kept,
-                   const int32_t* __restrict__ drop, const int32_t* __restrict__ order,
-                   const int32_t* __restrict__ seg, const float* __restrict__ mass, uint4* __restrict__ kvtmp) {
+                   int Hkv, int N, int i0, int n, int k, int r, int rest, const int32_t* __restrict__ kept,
+                   const int2* __restrict__ order, const int32_t* __restrict__ seg, const float* __restrict__ mass,
+                   uint4* __restrict__ kvtmp) {
     pdl_enter();
-    const int b = blockIdx.z, g = blockIdx.y >> 1, which = blockIdx.y & 1;
+    const int b = blockIdx.z, s0 = blockIdx.y * kKvSeqs;
     const int c = threadIdx.x & 15, t = blockIdx.x * 16 + (threadIdx.x >> 4);
-    if (t >= k) return;
-    const uint4* rows = (which ? Vc : Kc) + (int64_t)b * kv_sb + (int64_t)g * kv_sh + (int64_t)i0 * 16;
-    const float* ms = mass ? mass + (int64_t)b * N + i0 : nullptr;
-    const int32_t* ord = order + (int64_t)b * r;
-    const int32_t* dr = drop + (int64_t)b * r;
-    const int jt = kept[(int64_t)b * k + t];
-    const int p0 = seg[(int64_t)b * (k + 1) + t], p1 = seg[(int64_t)b * (k + 1) + t + 1];
-    const float mt = ms ? ms[jt] : 1.f;
-    float den = mt, acc[8];
-    {
-        const uint4 x = rows[(int64_t)jt * 16 + c];
-        acc[0] = mt * bf16_lo(x.x); acc[1] = mt * bf16_hi(x.x); acc[2] = mt * bf16_lo(x.y); acc[3] = mt * bf16_hi(x.y);
-        acc[4] = mt * bf16_lo(x.z); acc[5] = mt * bf16_hi(x.z); acc[6] = mt * bf16_lo(x.w); acc[7] = mt * bf16_hi(x.w);
+    if (t >= k + rest) return;
+    const uint4* rows[kKvSeqs];
+    uint4* to = kvtmp + (((int64_t)b * Hkv * 2 + s0) * (k + rest) + t) * 16 + c;
+    const int64_t to_step = (int64_t)(k + rest) * 16;
+#pragma unroll
+    for (int s = 0; s < kKvSeqs; ++s) {                           // (past the last sequence: the last one again, not stored)
+        const int sq = min(s0 + s, Hkv * 2 - 1);
+        rows[s] = ((sq & 1) ? Vc : Kc) + (int64_t)b * kv_sb + (int64_t)(sq >> 1) * kv_sh + (int64_t)i0 * 16 + c;
     }
-    for (int pb = p0; pb < p1; pb += 4) {
-        float md[4];
-        uint4 x[4];
+    const int p0 = t < k ? seg[(int64_t)b * (k + 1) + t] : 0, p1 = t < k ? seg[(int64_t)b * (k + 1) + t + 1] : 0;
+    // (a rank that is no permutation leaves gaps in the list)
+    const int jt = t < k ? min(max(kept[(int64_t)b * k + t], 0), n - 1) : n + t - k;
+    uint4 own[kKvSeqs];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int p = pb + u;
-            const int jd = p < p1 ? dr[ord[p]] : 0;
-            md[u] = p < p1 ? (ms ? ms[jd] : 1.f) : 0.f;
-            x[u] = p < p1 ? rows[(int64_t)jd * 16 + c] : make_uint4(0, 0, 0, 0);
+    for (int s = 0; s < kKvSeqs; ++s) own[s] = rows[s][(int64_t)jt * 16];
+    if (p1 > p0) {                                                // (otherwise: the row as it is)
+        const float* ms = mass ? mass + (int64_t)b * N + i0 : nullptr;
+        const int2* ord = order + (int64_t)b * r;
+        const float mt = ms ? ms[jt] : 1.f;
+        float den = mt, acc[kKvSeqs][8];
+#pragma unroll
+        for (int s = 0; s < kKvSeqs; ++s) {
+            acc[s][0] = mt * bf16_lo(own[s].x); acc[s][1] = mt * bf16_hi(own[s].x); acc[s][2] = mt * bf16_lo(own[s].y); acc[s][3] = mt * bf16_hi(own[s].y);
+            acc[s][4] = mt * bf16_lo(own[s].z); acc[s][5] = mt * bf16_hi(own[s].z); acc[s][6] = mt * bf16_lo(own[s].w); acc[s][7] = mt * bf16_hi(own[s].w);
         }
+        for (int pb = p0; pb < p1; pb += 2) {
+            float md[2];
+            uint4 x[2][kKvSeqs];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (pb + u < p1) {
-                den += md[u];
-                acc[0] = fmaf(md[u], bf16_lo(x[u].x), acc[0]); acc[1] = fmaf(md[u], bf16_hi(x[u].x), acc[1]);
-                acc[2] = fmaf(md[u], bf16_lo(x[u].y), acc[2]); acc[3] = fmaf(md[u], bf16_hi(x[u].y), acc[3]);
-                acc[4] = fmaf(md[u], bf16_lo(x[u].z), acc[4]); acc[5] = fmaf(md[u], bf16_hi(x[u].z), acc[5]);
-                acc[6] = fmaf(md[u], bf16_lo(x[u].w), acc[6]); acc[7] = fmaf(md[u], bf16_hi(x[u].w), acc[7]);
+            for (int u = 0; u < 2; ++u) {
+                const int p = pb + u;
+                const int jd = p < p1 ? min(max(ord[p].y, 0), n - 1) : 0;
+                md[u] = p < p1 ? (ms ? ms[jd] : 1.f) : 0.f;
+#pragma unroll
+                for (int s = 0; s < kKvSeqs; ++s) x[u][s] = p < p1 ? rows[s][(int64_t)jd * 16] : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (pb + u < p1) {
+                    den += md[u];
+#pragma unroll
+                    for (int s = 0; s < kKvSeqs; ++s) {
+                        const uint4 v = x[u][s];
+                        acc[s][0] = fmaf(md[u], bf16_lo(v.x), acc[s][0]); acc[s][1] = fmaf(md[u], bf16_hi(v.x), acc[s][1]);
+                        acc[s][2] = fmaf(md[u], bf16_lo(v.y), acc[s][2]); acc[s][3] = fmaf(md[u], bf16_hi(v.y), acc[s][3]);
+                        acc[s][4] = fmaf(md[u], bf16_lo(v.z), acc[s][4]); acc[s][5] = fmaf(md[u], bf16_hi(v.z), acc[s][5]);
+                        acc[s][6] = fmaf(md[u], bf16_lo(v.w), acc[s][6]); acc[s][7] = fmaf(md[u], bf16_hi(v.w), acc[s][7]);
+                    }
+                }
             }
         }
+        const float inv = 1.0f / den;
+#pragma unroll
+        for (int s = 0; s < kKvSeqs; ++s) {
+            own[s].x = pack_bf16(acc[s][0] * inv, acc[s][1] * inv); own[s].y = pack_bf16(acc[s][2] * inv, acc[s][3] * inv);
+            own[s].z = pack_bf16(acc[s][4] * inv, acc[s][5] * inv); own[s].w = pack_bf16(acc[s][6] * inv, acc[s][7] * inv);
+        }
     }
-    const float inv = 1.0f / den;
-    uint4 o;
-    if (p1 > p0) {
-        o.x = pack_bf16(acc[0] * inv, acc[1] * inv); o.y = pack_bf16(acc[2] * inv, acc[3] * inv);
-        o.z = pack_bf16(acc[4] * inv, acc[5] * inv); o.w = pack_bf16(acc[6] * inv, acc[7] * inv);
-    } else {
-        o = rows[(int64_t)jt * 16 + c];                           // nothing merged in: the row as it is
-    }
-    kvtmp[((((int64_t)b * Hkv + g) * 2 + which) * k + t) * 16 + c] = o;
+#pragma unroll
+    for (int s = 0; s < kKvSeqs; ++s)
+        if (s0 + s < Hkv * 2) to[s * to_step] = own[s];
 }
 
+// grid (CTAs, Hkv * 2, B): four 16-byte words a thread.
 __global__ void __launch_bounds__(kNkThreads)
 nk_kv_store_kernel(uint4* __restrict__ Kc, uint4* __restrict__ Vc, int64_t kv_sb, int64_t kv_sh, int Hkv,
-                   int i0, int k, const uint4* __restrict__ kvtmp) {
+                   int i0, int rows_out, const uint4* __restrict__ kvtmp) {
     pdl_enter();
-    const int b = blockIdx.z, g = blockIdx.y >> 1, which = blockIdx.y & 1;
-    const int c = threadIdx.x & 15, t = blockIdx.x * 16 + (threadIdx.x >> 4);
-    if (t >= k) return;
-    uint4* rows = (which ? Vc : Kc) + (int64_t)b * kv_sb + (int64_t)g * kv_sh + (int64_t)i0 * 16;
-    rows[(int64_t)t * 16 + c] = kvtmp[((((int64_t)b * Hkv + g) * 2 + which) * k + t) * 16 + c];
+    const int b = blockIdx.z, g = blockIdx.y >> 1, which = blockIdx.y & 1, words = rows_out * 16;
+    uint4* to = (which ? Vc : Kc) + (int64_t)b * kv_sb + (int64_t)g * kv_sh + (int64_t)i0 * 16;
+    const uint4* from = kvtmp + (((int64_t)b * Hkv + g) * 2 + which) * words;
+    const int c = blockIdx.x * 4 * kNkThreads + threadIdx.x;
+    uint4 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) if (c + u * kNkThreads < words) x[u] = __ldcg(from + c + u * kNkThreads);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) if (c + u * kNkThreads < words) to[c + u * kNkThreads] = x[u];
 }
 
 // Token masses, in place: the kept tokens take their new mass, the rows behind the image move up.
@@ -363,30 +441,50 @@ nk_mass_kernel(float* mass, int N, int i0, int k, int r, const float* __restrict
 }
 
 // ---- similarity on the tensor cores --------------------------------------------------------------------
-// S = X_dropped X_kept^T, 128 dropped rows x 256 kept columns per accumulator, K = channels in chunks
-// of 64.  grid (row tiles, column splits, B).  Warp 0 feeds a ring of shared-memory stages by TMA,
-// warp 1 issues the MMAs into two TMEM accumulators in turn, eight epilogue warps scale the columns by
-// 1/|x_t| and keep the best (value, kept index) of their row while the next accumulator fills.
-constexpr int kSimM = 128, kSimN = 256, kSimK = 64, kSimStages = 4;
+// S = X_dropped X_kept^T, K = channels in chunks of 64.  The operands come from L2 faster than it can deliver them: a
+// 128x256 tile a time (48 KB a chunk, 424 cycles of MMAs) asked for 30 TB/s over all SMs and got 14.  So a CTA multiplies
+// TWO row tiles of 128 with a column tile of 256 at a time (64 KB for twice the work; the two accumulators fill the
+// tensor memory).  The kernel is persistent: the (column tile, row tile) units are shared out evenly, a CTA takes its run
+// of them in pairs, so that no last wave is left (1536 units on 148 SMs: 11 turns where CTAs of four took 12.75).  Warp 0
+// feeds a ring of shared-memory stages by TMA across units, warp 1 issues the MMAs, eight epilogue warps scale the columns
+// by 1/|x_t| and find the best (value, kept index) of every row.
+constexpr int kSimM = 128, kSimN = 256, kSimK = 64, kSimStages = 3;
 constexpr int kSimABytes = kSimM * kSimK * 2, kSimBBytes = kSimN * kSimK * 2;
-constexpr int kSimStageBytes = kSimABytes + kSimBBytes;
+constexpr int kSimStageBytes = 2 * kSimABytes + kSimBBytes;
 constexpr int kSimThreads = 320, kSimEpi = 256;
 constexpr uint32_t kSimTmemCols = 512;
 
 struct SimArgs {
-    int r, k, nkc, nct, cps;
+    int r, k, nkc, nrt, nct, units;
     const float* inv_norm;          // [B][k]
     unsigned long long* best;       // [B][r] (orderable similarity << 32) | ~kept index, zero before
     int32_t* dev_status;
 };
 
 struct SimSmem {
-    uint64_t full[kSimStages], empty[kSimStages], tmem_full[2], tmem_empty[2];
+    uint64_t full[kSimStages], empty[kSimStages], tmem_full, tmem_empty;
     uint32_t tmem_base;
     volatile int abort;
-    float inv_s[8][2][128];         // per epilogue warp and accumulator: 1/|x_t| of its 128 columns
-    float xv[kSimM];                // upper column half's best, handed to the lower half
-    int xt[kSimM];
+    float inv_s[2][kSimN];          // 1/|x_t| of the columns, per column half (written by its warps for themselves)
+    float xv[2][kSimM];             // upper column half's best, handed to the lower half
+    int xt[2][kSimM];
+};
+
+// The units of a CTA: (sequence, column tile, row tile), row tiles fastest; one or two row tiles of a column at a time.
+struct SimUnits {
+    int u, end, b, ct, rt, n;
+    __device__ explicit SimUnits(const SimArgs& a)
+        : u((int)((int64_t)a.units * blockIdx.x / gridDim.x)), end((int)((int64_t)a.units * (blockIdx.x + 1) / gridDim.x)), n(0) {}
+    __device__ bool next(const SimArgs& a) {
+        u += n;
+        if (u >= end) return false;
+        rt = u % a.nrt;
+        const int c = u / a.nrt;
+        ct = c % a.nct;
+        b = c / a.nct;
+        n = min(2, min(end - u, a.nrt - rt));
+        return true;
+    }
 };
 
 __device__ __forceinline__ bool sim_wait(uint64_t* bar, uint32_t parity, SimSmem* sm, int32_t* dev_status) {
@@ -404,13 +502,11 @@ nk_sim_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
         (reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
     SimSmem* sm = reinterpret_cast<SimSmem*>(base + kSimStageBytes * kSimStages);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rt = blockIdx.x, split = blockIdx.y, b = blockIdx.z;
-    const int ct0 = split * a.cps, ct1 = min(a.nct, ct0 + a.cps);
-    const int ntile = max(0, ct1 - ct0);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kSimStages; ++s) { mbar_init(&sm->full[s], 1); mbar_init(&sm->empty[s], 1); }
-        for (int s = 0; s < 2; ++s) { mbar_init(&sm->tmem_full[s], 1); mbar_init(&sm->tmem_empty[s], kSimEpi); }
+        mbar_init(&sm->tmem_full, 1);
+        mbar_init(&sm->tmem_empty, kSimEpi);
         sm->abort = 0;
         fence_barrier_init();
         fence_proxy_async();
@@ -424,105 +520,115 @@ nk_sim_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
     const uint32_t tmem_base = sm->tmem_base;
     pdl_enter();
 
+    SimUnits w(a);
     if (warp == 0) {
         if (lane == 0) {
-            int it = 0;
-            for (int j = 0; j < ntile; ++j) {
-                for (int kc = 0; kc < a.nkc; ++kc, ++it) {
-                    const int st = it % kSimStages;
-                    if (it >= kSimStages && !sim_wait(&sm->empty[st], ((it / kSimStages) - 1) & 1, sm, a.dev_status)) { j = ntile; break; }
+            uint32_t st = 0, phase = 1;                        // (the first lap finds every stage empty)
+            bool ok = true;
+            while (ok && w.next(a)) {
+                for (int kc = 0; kc < a.nkc; ++kc) {
+                    if (!(ok = sim_wait(&sm->empty[st], phase, sm, a.dev_status))) break;
                     unsigned char* dst = base + st * kSimStageBytes;
-                    mbar_arrive_expect_tx(&sm->full[st], kSimStageBytes);
-                    tma_load_3d(dst, &amap, &sm->full[st], kc * kSimK, rt * kSimM, b);
-                    tma_load_3d(dst + kSimABytes, &bmap, &sm->full[st], kc * kSimK, (ct0 + j) * kSimN, b);
+                    mbar_arrive_expect_tx(&sm->full[st], (uint32_t)(w.n * kSimABytes + kSimBBytes));
+                    for (int i = 0; i < w.n; ++i)
+                        tma_load_3d(dst + i * kSimABytes, &amap, &sm->full[st], kc * kSimK, (w.rt + i) * kSimM, w.b);
+                    tma_load_3d(dst + 2 * kSimABytes, &bmap, &sm->full[st], kc * kSimK, w.ct * kSimN, w.b);
+                    if (++st == kSimStages) { st = 0; phase ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
         // all lanes run the loop (uniform operands), one elected lane issues
-        {
-            constexpr uint32_t idesc = idesc_bf16_f32(kSimM, kSimN);
-            int it = 0;
-            bool ok = true;
-            for (int j = 0; ok && j < ntile; ++j) {
-                const int buf = j & 1;
-                if (j >= 2) ok = __all_sync(0xFFFFFFFFu, sim_wait(&sm->tmem_empty[buf], ((j / 2) - 1) & 1, sm, a.dev_status));
-                for (int kc = 0; ok && kc < a.nkc; ++kc, ++it) {
-                    const int st = it % kSimStages;
-                    const uint32_t a_addr = smem_u32(base + st * kSimStageBytes);
-                    const uint32_t b_addr = a_addr + kSimABytes;
-                    const uint32_t d_tmem = tmem_base + buf * kSimN;
-                    uint64_t ad[4], bd[4];
+        constexpr uint32_t idesc = idesc_bf16_f32(kSimM, kSimN);
+        const uint64_t d0 = smem_desc_sw128(smem_u32(base));
+        uint32_t st = 0, phase = 0, it = 0;
+        bool ok = true;
+        while (ok && w.next(a)) {
+            if (it > 0) ok = __all_sync(0xFFFFFFFFu, sim_wait(&sm->tmem_empty, (it - 1) & 1, sm, a.dev_status));
+            for (int kc = 0; ok && kc < a.nkc; ++kc) {
+                const uint64_t ad = d0 + st * (uint32_t)(kSimStageBytes >> 4), bd = ad + (uint32_t)(2 * kSimABytes >> 4);
+                ok = __all_sync(0xFFFFFFFFu, sim_wait(&sm->full[st], phase, sm, a.dev_status));
+                if (!ok) break;
+                tc_fence_after();
+                if (elect_one()) {
+                    for (int i = 0; i < w.n; ++i)
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) { ad[kk] = smem_desc_sw128(a_addr + kk * 32); bd[kk] = smem_desc_sw128(b_addr + kk * 32); }
-                    ok = __all_sync(0xFFFFFFFFu, sim_wait(&sm->full[st], (it / kSimStages) & 1, sm, a.dev_status));
-                    if (!ok) break;
-                    tc_fence_after();
-                    if (elect_one()) {
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) mma_bf16_ss(d_tmem, ad[kk], bd[kk], idesc, (kc > 0 || kk > 0) ? 1u : 0u);
-                        mma_commit(&sm->empty[st]);
-                    }
-                    __syncwarp();
+                        for (int kk = 0; kk < 4; ++kk)
+                            mma_bf16_ss(tmem_base + i * kSimN, ad + (uint32_t)(i * (kSimABytes >> 4) + kk * 2), bd + (uint32_t)(kk * 2), idesc,
+                                        (kc > 0 || kk > 0) ? 1u : 0u);
+                    mma_commit(&sm->empty[st]);
+                    if (kc == a.nkc - 1) mma_commit(&sm->tmem_full);
                 }
-                if (ok && elect_one()) mma_commit(&sm->tmem_full[buf]);
                 __syncwarp();
+                if (++st == kSimStages) { st = 0; phase ^= 1u; }
             }
+            ++it;
         }
     } else {
         const int quarter = warp & 3, half = (warp - 2) >> 2;
         const int row = quarter * 32 + lane;
-        const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
-        const float* inv = a.inv_norm + (int64_t)b * a.k;
-        float best_v = -INFINITY;
-        int best_t = -1;
-        float inv_next[4];
-        auto fetch_inv = [&](int j) {
+        const uint32_t my_tmem = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * 128;
+        bool ok = true;
+        // (every epilogue thread goes through every unit, also after a wait has given up: the barriers count them all)
+        for (uint32_t it = 0; w.next(a); ++it) {
+            // 1/|x_t| of my half's columns, while the unit is being multiplied (the four warps write the same values)
+            const int t0 = w.ct * kSimN + half * 128;
+            const float* inv = a.inv_norm + (int64_t)w.b * a.k;
+            asm volatile("bar.sync 1, 256;" ::: "memory");       // the unit before has been read
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int t = (ct0 + j) * kSimN + half * 128 + u * 32 + lane;
-                inv_next[u] = t < a.k ? __ldg(inv + t) : 0.f;
+                const int t = t0 + u * 32 + lane;
+                sm->inv_s[half][u * 32 + lane] = t < a.k ? __ldg(inv + t) : 0.f;
             }
-        };
-        if (ntile > 0) fetch_inv(0);
-        for (int j = 0; j < ntile; ++j) {
-            const int buf = j & 1;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) sm->inv_s[warp - 2][buf][u * 32 + lane] = inv_next[u];
-            if (j + 1 < ntile) fetch_inv(j + 1);
             __syncwarp();
-            if (!sim_wait(&sm->tmem_full[buf], (j / 2) & 1, sm, a.dev_status)) break;
-            tc_fence_after();
-#pragma unroll 1
-            for (int c4 = 0; c4 < 4; ++c4) {
-                float v[32];
-                tmem_ld32(lane_addr + buf * kSimN + half * 128 + c4 * 32, v);
-                tmem_ld_wait();
-                const int tb = (ct0 + j) * kSimN + half * 128 + c4 * 32;
-                const float* is = &sm->inv_s[warp - 2][buf][c4 * 32];
+            ok = __all_sync(0xFFFFFFFFu, ok && sim_wait(&sm->tmem_full, it & 1, sm, a.dev_status));
+            float best_v[2] = {-INFINITY, -INFINITY};
+            int best_t[2] = {-1, -1};
+            if (ok) {
+                tc_fence_after();
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
-                    const float val = v[c] * is[c];
-                    if (tb + c < a.k && val > best_v) { best_v = val; best_t = tb + c; }
+                for (int i = 0; i < 2; ++i) {
+                    if (i >= w.n) break;
+                    // (a chunk is read while the one before is worked on)
+                    float v[2][32];
+                    tmem_ld32(my_tmem + i * kSimN, v[0]);
+#pragma unroll
+                    for (int c4 = 0; c4 < 4; ++c4) {
+                        tmem_ld_wait();
+                        if (c4 < 3) tmem_ld32(my_tmem + i * kSimN + (c4 + 1) * 32, v[(c4 + 1) & 1]);
+                        const int tb = t0 + c4 * 32;
+                        const float* is = &sm->inv_s[half][c4 * 32];
+#pragma unroll
+                        for (int c = 0; c < 32; ++c) {
+                            const float val = v[c4 & 1][c] * is[c];
+                            if (tb + c < a.k && val > best_v[i]) { best_v[i] = val; best_t[i] = tb + c; }
+                        }
+                    }
                 }
+                tc_fence_before();
             }
-            tc_fence_before();
-            mbar_arrive(&sm->tmem_empty[buf]);
-        }
-        // the two column halves of a row meet in shared memory (on equal similarity the lower kept index
-        // wins, whichever half and column tile it sits in); every epilogue thread comes here, also after a timeout
-        if (half == 1) { sm->xv[row] = best_v; sm->xt[row] = best_t; }
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (half == 0) {
-            const float ov = sm->xv[row];
-            const int ot = sm->xt[row];
-            if (ot >= 0 && (best_t < 0 || ov > best_v || (ov == best_v && ot < best_t))) { best_v = ov; best_t = ot; }
-            const int q = rt * kSimM + row;
-            if (!sm->abort && q < a.r && best_t >= 0) {
-                uint32_t u = __float_as_uint(best_v);
-                u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);         // ascending in the value
-                const unsigned long long key = ((unsigned long long)u << 32) | (0xFFFFFFFFu - (uint32_t)best_t);
-                atomicMax(a.best + (int64_t)b * a.r + q, key);
+            mbar_arrive(&sm->tmem_empty);
+            // the two column halves of a row meet in shared memory (on equal similarity the lower kept index
+            // wins, whichever half and column tile it sits in)
+            if (half == 1) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) { sm->xv[i][row] = best_v[i]; sm->xt[i][row] = best_t[i]; }
+            }
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+            if (half == 0 && ok && !sm->abort) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int q = (w.rt + i) * kSimM + row;
+                    if (i >= w.n || q >= a.r) continue;
+                    const float ov = sm->xv[i][row];
+                    const int ot = sm->xt[i][row];
+                    if (ot >= 0 && (best_t[i] < 0 || ov > best_v[i])) { best_v[i] = ov; best_t[i] = ot; }
+                    if (best_t[i] < 0) continue;
+                    uint32_t u = __float_as_uint(best_v[i]);
+                    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);         // ascending in the value
+                    const unsigned long long key = ((unsigned long long)u << 32) | (0xFFFFFFFFu - (uint32_t)best_t[i]);
+                    atomicMax(a.best + (int64_t)w.b * a.r + q, key);
+                }
             }
         }
     }
@@ -540,13 +646,13 @@ nk_sim_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
 
 template <int CH>
 static lvlm_status launch_nk_merge(void* out, int64_t out_sb, const void* scratch, int64_t scr_sb, const lvlm_dims* d,
-                                   const NkLayout& L, const int32_t* kept, const int32_t* drop, const int32_t* order,
-                                   const int32_t* seg, const float* mass, float* newmass, cudaStream_t stream) {
+                                   const NkLayout& L, const int32_t* kept, const int2* order, const int32_t* seg,
+                                   const float* mass, float* newmass, cudaStream_t stream) {
     int ctas = (4 * 148) / d->B;
     ctas = ctas < 1 ? 1 : (ctas > d->k ? d->k : ctas);
     return launch_kernel(nk_merge_kernel<CH>, dim3(ctas, d->B), dim3(kNkThreads), 0, stream, 1,
                          static_cast<uint4*>(out), out_sb / 8, static_cast<const uint4*>(scratch), scr_sb / 8, L.V,
-                         d->N, d->i0, d->k, L.r, kept, drop, order, seg, mass, newmass);
+                         d->N, d->i0, d->k, L.r, kept, order, seg, mass, newmass);
 }
 
 lvlm_status launch_nearest_kept(const void* hidden, void* hidden_out, void* Kc, void* Vc, int32_t* pos_ids,
@@ -555,7 +661,7 @@ lvlm_status launch_nearest_kept(const void* hidden, void* hidden_out, void* Kc, 
     NkLayout L;
     if (!nk_layout(d, &L) || d->k < 1) return LVLM_ERR_INVALID_ARG;
     if (!hidden_out || hidden_out == hidden) return LVLM_ERR_UNSUPPORTED;     // out of place only
-    if (L.r > kRankMaxKeys) return LVLM_ERR_UNSUPPORTED;       // the slices of the keys have to fit in shared memory
+    if (L.r > kMaxDropped) return LVLM_ERR_UNSUPPORTED;        // the bitmap of the sort
     if (!ws || !aligned256(ws) || ws_bytes < L.total) return LVLM_ERR_WORKSPACE;
     const int64_t hid_sb = d->hid_stride_b ? d->hid_stride_b : (int64_t)d->N * d->C;
     const int64_t out_sb = d->out_stride_b ? d->out_stride_b : (int64_t)L.Nout * d->C;
@@ -564,30 +670,27 @@ lvlm_status launch_nearest_kept(const void* hidden, void* hidden_out, void* Kc, 
     const int64_t scr_sb = (int64_t)L.r * d->C;
     char* wsb = static_cast<char*>(ws);
     int32_t* assign = reinterpret_cast<int32_t*>(wsb + L.off_assign);
-    int32_t* src_map = reinterpret_cast<int32_t*>(wsb + L.off_src);
     int32_t* dst_map = reinterpret_cast<int32_t*>(wsb + L.off_dst);
     int32_t* kept = reinterpret_cast<int32_t*>(wsb + L.off_kept);
     int32_t* drop = reinterpret_cast<int32_t*>(wsb + L.off_drop);
     float* inv_norm = reinterpret_cast<float*>(wsb + L.off_inv);
     unsigned long long* best = reinterpret_cast<unsigned long long*>(wsb + L.off_best);
-    int32_t* order = reinterpret_cast<int32_t*>(wsb + L.off_order);
-    int32_t* sorted_t = reinterpret_cast<int32_t*>(wsb + L.off_sorted);
+    int32_t* place = reinterpret_cast<int32_t*>(wsb + L.off_place);
+    int2* order = reinterpret_cast<int2*>(wsb + L.off_order);
     int32_t* seg = reinterpret_cast<int32_t*>(wsb + L.off_seg);
-    int32_t* meta = reinterpret_cast<int32_t*>(wsb + L.off_meta);
     float* newmass = reinterpret_cast<float*>(wsb + L.off_newmass);
     void* scratch = wsb + L.off_scratch;
     uint4* kvtmp = reinterpret_cast<uint4*>(wsb + L.off_kvtmp);
 
     lvlm_status st;
     const int plan_threads = d->n >= 1024 ? 1024 : (d->n <= 128 ? 128 : ((d->n + 31) / 32) * 32);
-    st = launch_kernel(nk_plan_kernel, dim3(d->B), dim3(plan_threads), 0, stream, 1, rank, pos_ids, d->N, d->i0,
-                       d->n, d->k, src_map, dst_map, kept, drop, best, meta, new_len, dev_status);
+    int P = (d->n + 2047) / 2048;                        // CTAs per sequence: about two tiles of tokens each
+    P = P < 1 ? 1 : (P > 8 ? 8 : P);
+    st = launch_kernel(nk_plan_kernel, dim3(P, d->B), dim3(plan_threads), 0, stream, P, rank, pos_ids, d->N, d->i0,
+                       d->n, d->k, dst_map, kept, drop, best, seg, new_len, dev_status);
     if (st != LVLM_OK) return st;
-    st = launch_hidden_rows(hidden, hidden_out, hid_sb, out_sb, d, L.grid, dst_map, nullptr, meta, nullptr,
-                            scratch, scr_sb, stream);
-    if (st != LVLM_OK) return st;
-    st = launch_kernel(nk_norm_kernel, dim3((d->k + 7) / 8, d->B), dim3(256), 0, stream, 1,
-                       static_cast<const uint4*>(hidden_out), out_sb / 8, L.V, d->i0, d->k, inv_norm);
+    st = launch_hidden_rows(hidden, hidden_out, hid_sb, out_sb, d, L.grid, dst_map, nullptr, nullptr, nullptr,
+                            scratch, scr_sb, stream, nullptr, dev_status, nullptr, inv_norm);
     if (st != LVLM_OK) return st;
     {
         CUtensorMap amap, bmap;
@@ -602,61 +705,43 @@ lvlm_status launch_nearest_kept(const void* hidden, void* hidden_out, void* Kc, 
         if (!make_tmap_bf16(&bmap, bbase, 3, bdims, bstr, bbox)) return LVLM_ERR_CUDA;
         SimArgs a;
         a.r = L.r; a.k = d->k; a.nkc = (d->C + kSimK - 1) / kSimK; a.nct = (d->k + kSimN - 1) / kSimN;
-        const int row_tiles = (L.r + kSimM - 1) / kSimM;
-        // column splits: one CTA per SM at a time, so the kernel takes waves x (column tiles per CTA + a
-        // little for the set-up of a CTA); take the split with the smallest product
-        int nsplit = 1;
-        double best_est = 1e30;
-        for (int ns = 1; ns <= a.nct; ++ns) {
-            const int cps = (a.nct + ns - 1) / ns, used = (a.nct + cps - 1) / cps;
-            const int64_t ctas = (int64_t)row_tiles * d->B * used;
-            const double est = (double)((ctas + 147) / 148) * (cps + 0.25);
-            if (est < best_est - 1e-9) { best_est = est; nsplit = used; a.cps = cps; }
-        }
+        a.nrt = (L.r + kSimM - 1) / kSimM;
+        const int64_t units = (int64_t)d->B * a.nct * a.nrt;
+        if (units > 0x7FFFFFFFll) return LVLM_ERR_UNSUPPORTED;
+        a.units = (int)units;
         a.inv_norm = inv_norm; a.best = best; a.dev_status = dev_status;
         const size_t smem = 1024 + (size_t)kSimStageBytes * kSimStages + sizeof(SimSmem);
         LVLM_RETURN_IF_CUDA(cudaFuncSetAttribute(nk_sim_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)smem));
-        st = launch_kernel(nk_sim_kernel, dim3(row_tiles, nsplit, d->B), dim3(kSimThreads), smem, stream, 1,
+        st = launch_kernel(nk_sim_kernel, dim3((unsigned)(units < 148 ? units : 148)), dim3(kSimThreads), smem, stream, 1,
                            amap, bmap, a);
         if (st != LVLM_OK) return st;
     }
-    {
-        int S, slice_len, jt;
-        rank_shape(L.r, d->B, &S, &slice_len, &jt);
-        LVLM_RETURN_IF_CUDA(cudaFuncSetAttribute(nk_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 kMaxDynSmem));
-        st = launch_kernel_cluster(nk_group_kernel, dim3((L.r + kRankThreads * jt - 1) / (kRankThreads * jt), S, d->B),
-                                   dim3(kRankThreads), rank_smem_bytes(slice_len), stream, dim3(1, S, 1),
-                                   best, L.r, d->k, S, slice_len, jt, assign, order, sorted_t);
-        if (st != LVLM_OK) return st;
-        st = launch_kernel(nk_seg_kernel, dim3((d->k + 1 + 255) / 256, d->B), dim3(256), 0, stream, 1,
-                           sorted_t, L.r, d->k, seg);
-        if (st != LVLM_OK) return st;
-    }
+    st = launch_kernel(nk_count_kernel, dim3((L.r + 255) / 256, d->B), dim3(256), 0, stream, 1, best, L.r, d->k, assign, place, seg);
+    if (st != LVLM_OK) return st;
+    st = launch_kernel(nk_place_kernel, dim3(d->B), dim3(1024), 0, stream, 1, seg, L.r, d->k, assign, place, drop, order);
+    if (st != LVLM_OK) return st;
+    st = launch_kernel(nk_sort_kernel, dim3((d->k + kSortWarps - 1) / kSortWarps, d->B), dim3(kSortWarps * 32), 0, stream, 1,
+                       seg, L.r, d->k, drop, order);
+    if (st != LVLM_OK) return st;
     const int chunks = (L.V + kNkThreads - 1) / kNkThreads;
     switch (chunks) {
-        case 1: st = launch_nk_merge<1>(hidden_out, out_sb, scratch, scr_sb, d, L, kept, drop, order, seg, mass, newmass, stream); break;
-        case 2: st = launch_nk_merge<2>(hidden_out, out_sb, scratch, scr_sb, d, L, kept, drop, order, seg, mass, newmass, stream); break;
-        case 3: st = launch_nk_merge<3>(hidden_out, out_sb, scratch, scr_sb, d, L, kept, drop, order, seg, mass, newmass, stream); break;
-        case 4: st = launch_nk_merge<4>(hidden_out, out_sb, scratch, scr_sb, d, L, kept, drop, order, seg, mass, newmass, stream); break;
+        case 1: st = launch_nk_merge<1>(hidden_out, out_sb, scratch, scr_sb, d, L, kept, order, seg, mass, newmass, stream); break;
+        case 2: st = launch_nk_merge<2>(hidden_out, out_sb, scratch, scr_sb, d, L, kept, order, seg, mass, newmass, stream); break;
+        case 3: st = launch_nk_merge<3>(hidden_out, out_sb, scratch, scr_sb, d, L, kept, order, seg, mass, newmass, stream); break;
+        case 4: st = launch_nk_merge<4>(hidden_out, out_sb, scratch, scr_sb, d, L, kept, order, seg, mass, newmass, stream); break;
         default: return LVLM_ERR_UNSUPPORTED;
     }
     if (st != LVLM_OK) return st;
     if (Kc) {
-        const dim3 grid((d->k + 15) / 16, d->Hkv * 2, d->B);
-        st = launch_kernel(nk_kv_merge_kernel, grid, dim3(kNkThreads), 0, stream, 1, static_cast<const uint4*>(Kc),
-                           static_cast<const uint4*>(Vc), kv_sb / 8, kv_sh / 8, d->Hkv, d->N, d->i0, d->k, L.r, kept,
-                           drop, order, seg, mass, kvtmp);
+        const int rows_out = d->k + L.rest;
+        st = launch_kernel(nk_kv_merge_kernel, dim3((rows_out + 15) / 16, (d->Hkv * 2 + kKvSeqs - 1) / kKvSeqs, d->B), dim3(kNkThreads), 0,
+                           stream, 1, static_cast<const uint4*>(Kc), static_cast<const uint4*>(Vc), kv_sb / 8, kv_sh / 8, d->Hkv, d->N,
+                           d->i0, d->n, d->k, L.r, L.rest, kept, order, seg, mass, kvtmp);
         if (st != LVLM_OK) return st;
-        CompactJob cj;
-        cj.base0 = Kc; cj.base1 = Vc; cj.stride_b = kv_sb * 2; cj.stride_g = kv_sh * 2; cj.B = d->B; cj.G = d->Hkv;
-        cj.V = kHeadDim / 8; cj.src_map = src_map; cj.map_stride = d->N; cj.meta = meta; cj.meta_stride = kMetaInts;
-        cj.Nout = L.Nout; cj.N = d->N;
-        st = launch_inplace_compact(cj, stream);
-        if (st != LVLM_OK) return st;
-        st = launch_kernel(nk_kv_store_kernel, grid, dim3(kNkThreads), 0, stream, 1, static_cast<uint4*>(Kc),
-                           static_cast<uint4*>(Vc), kv_sb / 8, kv_sh / 8, d->Hkv, d->i0, d->k, kvtmp);
+        st = launch_kernel(nk_kv_store_kernel, dim3((rows_out * 16 + 4 * kNkThreads - 1) / (4 * kNkThreads), d->Hkv * 2, d->B),
+                           dim3(kNkThreads), 0, stream, 1, static_cast<uint4*>(Kc), static_cast<uint4*>(Vc), kv_sb / 8,
+                           kv_sh / 8, d->Hkv, d->i0, rows_out, kvtmp);
         if (st != LVLM_OK) return st;
     }
     if (mass)

@@ -112,3 +112,36 @@ def test_attention_shapes(case):
     assert flag.item() == 0
     assert_rows_close(f64(out), f64(want), what="attention output")
     np.testing.assert_allclose(f64(lse), f64(torch.logsumexp(logits, dim=-1)), rtol=1e-5, atol=1e-5)   # fp32 sums
+
+
+# nearest-kept grouping: every dropped token to one kept token (one long segment), segments around a warp's 32 tokens, none
+# at all for most; text rows that are the source of rows before them; runs over several CTAs of the plan's cluster
+@pytest.mark.parametrize("case", [        # B, C, Hkv, i0, n, T, k, kept tokens that attract the dropped ones
+    (1, 64, 1, 0, 40, 5, 7, 1), (2, 128, 2, 3, 300, 20, 33, 1), (1, 256, 1, 0, 700, 600, 20, 20), (1, 64, 2, 17, 4500, 31, 2500, 60),
+    (3, 72, 1, 2, 2100, 300, 100, 3), (1, 64, 1, 0, 9000, 10, 1030, 1030)])
+def test_nearest_kept_groups(case):
+    B, C, Hkv, i0, n, T, k, attract = case
+    r = np.random.default_rng(n + k)
+    N = i0 + n + T
+    rank = np.stack([r.permutation(n) for _ in range(B)]).astype(np.int32)
+    hidden = r.normal(size=(B, N, C)).astype(np.float32)
+    for b in range(B):
+        by_rank = np.argsort(rank[b])
+        to = by_rank[:attract][r.integers(0, attract, size=n - k)]
+        hidden[b, i0 + by_rank[k:]] = hidden[b, i0 + to] + 0.05 * hidden[b, i0 + by_rank[k:]]
+    hid = torch.from_numpy(hidden).to(torch.bfloat16)
+    K, V = (torch.from_numpy(r.normal(size=(B, Hkv, N, 128)).astype(np.float32)).to(torch.bfloat16) for _ in range(2))
+    pos = np.tile(np.arange(N, dtype=np.int32), (B, 1))
+    mass = (r.integers(1, 5, size=(B, N))).astype(np.float32)
+    want = O.nearest_kept_merge(f64(hid), rank, i0, n, k, Kc=f64(K), Vc=f64(V), pos_ids=pos, mass=mass)
+    Kd, Vd, pd, md = K.cuda(), V.cuda(), torch.from_numpy(pos).cuda(), torch.from_numpy(mass).cuda()
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out, new_len = L.merge_compact(hid.cuda(), torch.from_numpy(rank).cuda(), i0=i0, k=k, mode=L.W_NEAREST_KEPT, Kc=Kd, Vc=Vd,
+                                   pos_ids=pd, mass=md, dev_status=flag)
+    Nout = N - (n - k)
+    assert flag.item() == 0 and new_len.tolist() == [Nout] * B
+    assert_rows_close(f64(out), want["hidden"], what="hidden")
+    assert_rows_close(f64(Kd)[:, :, :Nout], want["Kc"], what="K")
+    assert_rows_close(f64(Vd)[:, :, :Nout], want["Vc"], what="V")
+    assert np.array_equal(i32(pd)[:, :Nout], want["pos_ids"])
+    np.testing.assert_allclose(md.cpu().numpy()[:, :Nout], want["mass"], rtol=1e-6)                 # small whole numbers
