@@ -17,6 +17,14 @@
 // acc_score entries of its own keys, whose scaled logits it has kept in shared memory (in the
 // workspace when a run is too long for that).
 //
+// Inside a chain of layers the fetches of a layer start while the one ahead finishes; what counts is the time from the
+// end of the layer ahead: query, one lap of products, merge of the warps, cluster barrier, output.  So: a warp parks its
+// output where its own rows of the last stage lay (one block barrier), no releasing barrier waits for stores (the
+// appended row is written last), and few registers live across the loop (they spilled).  us per layer, before -> now:
+// 4 heads of 216 rows 4.5 -> 4.0, with acc_score 5.65 -> 4.9; 64 heads of 1100 rows 12.1 -> 11.3 (acc_score), 216 rows 7.3 -> 6.2;
+// 128 heads of 1100 rows 19.9 -> 17.5.  Tried and slower: 8 or 16 compute warps a CTA (5.7 to 20 us), acc_score
+// fetched ahead of the cluster barrier (5.2 -> 5.6).
+//
 // Few heads with long caches (a video prompt's first layers: one sequence, 4 KV heads, 32898 rows) leave most of the
 // GPU idle that way: a cluster has at most 8 CTAs.  There the run of a head is cut into as many parts as fill the GPU
 // twice, without clusters; every part leaves its (max, sum, output) in the workspace, and a second, small launch adds
@@ -52,17 +60,18 @@ struct DecodeLayout { int S, P; size_t off_s, off_ml, off_o, off_len, total; };
 
 // Rows of a cache, in tiles, from which the parts are the faster form where a cluster of 8 a head leaves SMs idle (the
 // lengths are only known on the device).  us per layer as cluster / as parts, inside a chain of layers:
-//   from 32 heads the clusters of 8 no longer fit the GPU side by side: 36 heads of 216 rows 10.3 / 7.3, 2000 17.9 / 13.4,
-//   20000 91 / 65; 32 heads of 130 rows 4.9 / 5.4;
-//   without acc_score the cluster's one launch wins while the runs are short: 4 heads of 600 rows 5.4 / 5.5, 1100 6.2 / 5.5,
-//   32898 54.1 / 17.8; 8 heads of 1100 rows 5.5 / 5.4, 8000 15.5 / 11.6; 16 heads of 2000 rows 8.5 / 9.3, 8000 20.4 / 16.2;
-//   28 heads of 4000 rows 15.8 / 16.0, 8000 25.7 / 25.1;
-//   with it the second launch takes the update of acc_score off the cluster's tail: 4 heads of 400 rows 5.65 / 5.64, 600
-//   6.6 / 5.7, 32898 66.8 / 17.8; 20 heads of 600 rows 8.6 / 7.8, 8000 27.9 / 22.6; 28 heads of 2000 rows 11.9 / 13.1.
+//   from 32 heads the clusters of 8 no longer fit the GPU side by side: 36 heads of 216 rows 9.3 / 6.9, 2500 18.0 / 14.0,
+//   9000 45 / 33; 32 heads of 216 rows 6.5 / 5.7, 9000 32 / 29;
+//   without acc_score the cluster's one launch wins while the runs are short: 4 heads of 600 rows 4.8 / 5.4, 1100 5.5 / 5.4,
+//   9000 17.2 / 10.2; 8 heads of 2500 rows 6.9 / 7.3, 4000 9.3 / 8.3; 16 heads of 4000 rows 11.8 / 11.9, 6000 16.0 / 14.0;
+//   28 heads of 9000 rows 26.0 / 26.9;
+//   with it the second launch takes the update of acc_score off the cluster's tail: 4 heads of 400 rows 4.9 / 5.6, 600
+//   5.7 / 5.5, 9000 20 / 9.8; 8 heads of 600 rows 5.2 / 5.0; 16 heads of 2500 rows 9.3 / 10.4, 4000 13.2 / 12.1; 28 heads of
+//   9000 rows 31 / 32.
 static int parts_from_tiles(int64_t heads, bool acc) {
     if (heads >= 32) return 14;
-    if (acc) return heads <= 20 ? 32 : 384;
-    return heads <= 8 ? 16 * (int)heads : 384;
+    if (acc) return heads <= 8 ? 36 : heads <= 20 ? 192 : 800;
+    return heads <= 4 ? 64 : heads <= 8 ? 192 : heads <= 20 ? 320 : 800;
 }
 
 // may_split: the caller's workspace has room for the parts (lvlm_decode_attn_static's may not).
@@ -110,8 +119,10 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n"
                  "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
-__device__ __forceinline__ void cluster_arrive() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+// Execution only: what I have read from other CTAs has been used, nothing is published (a releasing arrive would wait for
+// the stores to global memory before it, about 1200 cycles).
+__device__ __forceinline__ void cluster_arrive_exec() {
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
     asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
@@ -125,9 +136,9 @@ __device__ __forceinline__ uint32_t dsmem_addr(uint32_t saddr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ float dsmem_ld(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+__device__ __forceinline__ float2 dsmem_ld2(uint32_t addr) {
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
     return v;
 }
 
@@ -182,19 +193,16 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     constexpr bool CL = MODE == kDecCluster;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    float* s_acc = reinterpret_cast<float*>(smem);                      // [slots][G][128]; slot 0 = this CTA's output (the ring, once it is done)
-    float* s_wm = reinterpret_cast<float*>(smem + kRingBytes);          // [4 warps][8 heads] running max
-    float* s_wl = s_wm + kDecWarps * 8;                                 // [4 warps][8 heads] running sum
-    float* s_M = s_wl + kDecWarps * 8;                                  // [8] this CTA's max per head
-    float* s_L = s_M + 8;                                               // [8] this CTA's sum per head
-    float* s_FM = s_L + 8;                                              // [8] cluster-wide max
+    float2* s_wml = reinterpret_cast<float2*>(smem + kRingBytes);       // [4 warps][8 heads] (max, sum)
+    float2* s_ML = s_wml + kDecWarps * 8;                               // [8] this CTA's (max, sum) per head
+    float* s_FM = reinterpret_cast<float*>(s_ML + 8);                   // [8] cluster-wide max
     float* s_FI = s_FM + 8;                                             // [8] 1 / cluster-wide sum
-    float* s_rm = s_FI + 8;                                             // [S][8] max of every CTA of the cluster
-    float* s_rl = s_rm + 8 * kDecMaxCluster;                            // [S][8] sum of every CTA
-    uint64_t* s_full = reinterpret_cast<uint64_t*>(s_rl + 8 * kDecMaxCluster);   // [kStagesDec]
+    float2* s_res = reinterpret_cast<float2*>(smem + 2 * kBoxBytes);    // [G][64] this CTA's output (the ring, once it is done)
+    uint64_t* s_full = reinterpret_cast<uint64_t*>(s_FI + 8);                    // [kStagesDec]
     uint64_t* s_empty = s_full + kStagesDec;                            // [kStagesDec]
     float* s_logit = reinterpret_cast<float*>(s_empty + kStagesDec + 1);          // [G][logit_keys]
     __shared__ int s_abort;
+    __shared__ __align__(16) uint4 s_app[32];                          // the appended row: K, then V
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 32) { prefetch_tmap(&kmap); prefetch_tmap(&vmap); }     // the descriptors start their way first
@@ -252,6 +260,12 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     for (int i = 0; i < 16; ++i) o[i][0] = o[i][1] = 0.f;
     float m_run = -INFINITY, l_run = 0.f;      // of head `row`; l_run is this lane's share of the sum
     const int row = lane >> 2, qd = lane & 3;
+    // the warp of this CTA whose tile takes the appended row, or -1
+    const int app_warp = app && ln / kTileKeys >= t_lo && ln / kTileKeys < t_hi ? (ln / kTileKeys - t_lo) % kDecWarps : -1;
+    auto store_appended = [&]() {
+        if (warp == app_warp)
+            *reinterpret_cast<uint4*>((lane < 16 ? a.Kc : a.Vc) + (int64_t)b * a.kv_sb + (int64_t)g * a.kv_sh + (int64_t)ln * kHeadDim + (lane & 15) * 8) = s_app[lane];
+    };
 
     if (warp == kDecWarps) {
         // ---- producer: four tile copies per stage ---------------------------------------------------------
@@ -281,11 +295,14 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
             for (int j = j_lo + tid * 32; j < j_hi; j += kDecWarps * 32 * 32) prefetch_l2(acc + j);
         }
         if (a.early) pdl_enter();
-        const int64_t kv_off = (int64_t)b * a.kv_sb + (int64_t)g * a.kv_sh;
-        __nv_bfloat16* Kseq = a.Kc + kv_off;
-        __nv_bfloat16* Vseq = a.Vc + kv_off;
         const __nv_bfloat16* kn = app ? a.k_new + (int64_t)hd * kHeadDim : nullptr;
         const __nv_bfloat16* vn = app ? a.v_new + (int64_t)hd * kHeadDim : nullptr;
+        // the appended row: fetched now, patched into its tile below, written to the cache at the very end (a store
+        // before the cluster barrier would be waited for there)
+        if (app_warp == warp) {
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(&s_app[lane])),
+                         "l"((lane < 16 ? kn : vn) + (lane & 15) * 8) : "memory");
+        }
         // query fragments: heads of the group are rows 0..G-1 of a 16-row A tile
         uint32_t qa[8][2];
 #pragma unroll
@@ -305,12 +322,12 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
                 const int r0 = warp * kTileKeys;                               // my rows of the stage
                 const int j0 = t * kTileKeys;
                 if (app && ln >= j0 && ln < j0 + kTileKeys) {
-                    // the appended row: into its place of the tile and into the cache
+                    // the appended row: into its place of the tile
                     const int rr = r0 + ln - j0, ch = lane & 15;
-                    const uint4 x = *reinterpret_cast<const uint4*>((lane < 16 ? kn : vn) + ch * 8);
                     const uint32_t off = (lane < 16 ? 0 : 2 * kBoxBytes) + stage_off(rr, ch);
+                    asm volatile("cp.async.wait_all;\n" ::: "memory");
+                    const uint4 x = s_app[lane];             // (copied by this very lane)
                     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(st + off), "r"(x.x), "r"(x.y), "r"(x.z), "r"(x.w) : "memory");
-                    *reinterpret_cast<uint4*>((lane < 16 ? Kseq : Vseq) + (int64_t)ln * kHeadDim + ch * 8) = x;
                 }
                 if (j0 + kTileKeys > lne) {
                     // V rows past the last key hold whatever the cache holds: zero them, their weight is zero
@@ -394,166 +411,134 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
             if (lane == 0) mbar_arrive(&s_empty[s % kStagesDec]);
         }
     }
-    // every copy issued has landed: the compute warps have waited for each stage; the ring is free
+    // ---- merge the four warps in warp order ------------------------------------------------------------
+    // A warp parks its output where its own K rows of the last stage lay (nobody else reads those, and nothing is fetched there
+    // any more): heads 0..3 in the box of the low channels, heads 4..7 in the other; pairs of channels, XOR-swizzled by head.
+    l_run += __shfl_xor_sync(0xFFFFFFFFu, l_run, 1);
+    l_run += __shfl_xor_sync(0xFFFFFFFFu, l_run, 2);
+    const uint32_t last = (uint32_t)((nstage > 0 ? nstage - 1 : 0) % kStagesDec) * kStageBytes;
+    auto slot_of = [&](int w, int hh, int pair) {
+        return reinterpret_cast<float2*>(smem + last + (hh >> 2) * kBoxBytes + w * kTileKeys * 128 + (hh & 3) * 512) + (pair ^ ((hh & 3) * 4));
+    };
+    if (warp < kDecWarps && row < G) {
+        if (qd == 0) s_wml[warp * 8 + row] = make_float2(m_run, l_run);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) *slot_of(warp, row, i * 4 + qd) = make_float2(o[i][0], o[i][1]);
+    }
     __syncthreads();
     if (s_abort) {                             // a wait gave up: copies may still be in flight, let them land
 #pragma unroll 1
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
         __syncthreads();
     }
-
-    // ---- merge the four warps in warp order ------------------------------------------------------------
-    l_run += __shfl_xor_sync(0xFFFFFFFFu, l_run, 1);
-    l_run += __shfl_xor_sync(0xFFFFFFFFu, l_run, 2);
-    if (warp < kDecWarps && row < G && qd == 0) { s_wm[warp * 8 + row] = m_run; s_wl[warp * 8 + row] = l_run; }
-    __syncthreads();
-    {
-        // kSlots warps write side by side, the others add to them in warp order; the slots are added
-        // in slot order when they are folded into slot 0
-        constexpr int kSlots = G <= 4 ? 4 : 2;
-        float Mh = -INFINITY;
-        if (row < G) {
+    for (int idx = tid; idx < G * (kHeadDim / 2); idx += kDecThreads) {
+        const int hh = idx >> 6, pair = idx & 63;
+        float2 ml[kDecWarps], x[kDecWarps];
 #pragma unroll
-            for (int w = 0; w < kDecWarps; ++w) Mh = fmaxf(Mh, s_wm[w * 8 + row]);
+        for (int w = 0; w < kDecWarps; ++w) { ml[w] = s_wml[w * 8 + hh]; x[w] = *slot_of(w, hh, pair); }
+        float M2 = -INFINITY, Ls = 0.f;
+#pragma unroll
+        for (int w = 0; w < kDecWarps; ++w) M2 = fmaxf(M2, ml[w].x);
+        float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int w = 0; w < kDecWarps; ++w) {
+            const float f = ml[w].x > -INFINITY ? exp2f(ml[w].x - M2) : 0.f;
+            v.x += x[w].x * f; v.y += x[w].y * f; Ls += ml[w].y * f;
         }
-        const float f = (row < G && m_run > -INFINITY) ? exp2f(m_run - Mh) : 0.f;
-#pragma unroll
-        for (int rnd = 0; rnd < kDecWarps / kSlots; ++rnd) {
-            if (warp / kSlots == rnd && row < G) {
-                float* slot = s_acc + (warp % kSlots) * (G * kHeadDim);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    float2* dst = reinterpret_cast<float2*>(slot + row * kHeadDim + i * 8 + qd * 2);
-                    float2 v = make_float2(o[i][0] * f, o[i][1] * f);
-                    if (rnd > 0) { const float2 old = *dst; v.x += old.x; v.y += old.y; }
-                    *dst = v;
-                }
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int hh = 0; hh < G && tid < kHeadDim; ++hh) {  // thread = channel
-            float v = s_acc[hh * kHeadDim + tid];
-#pragma unroll
-            for (int sl = 1; sl < kSlots; ++sl) v += s_acc[sl * (G * kHeadDim) + hh * kHeadDim + tid];
-            if (MODE == kDecParts) a.part_o[(((int64_t)hd * S + rank) * G + hh) * kHeadDim + tid] = v;
-            else s_acc[hh * kHeadDim + tid] = v;
-        }
-        if (tid < G) {
-            float M2 = -INFINITY;
-#pragma unroll
-            for (int w = 0; w < kDecWarps; ++w) M2 = fmaxf(M2, s_wm[w * 8 + tid]);
-            float Ls = 0.f;
-#pragma unroll
-            for (int w = 0; w < kDecWarps; ++w) {
-                const float mw = s_wm[w * 8 + tid];
-                if (mw > -INFINITY) Ls += s_wl[w * 8 + tid] * exp2f(mw - M2);
-            }
-            if (MODE == kDecParts) a.part_ml[((int64_t)hd * S + rank) * G + tid] = make_float2(M2, Ls);
-            s_M[tid] = M2;
-            s_L[tid] = Ls;
+        if (MODE == kDecParts) reinterpret_cast<float2*>(a.part_o)[((int64_t)hd * S + rank) * (G * 64) + idx] = v;
+        else s_res[idx] = v;
+        if (pair == 0) {
+            if (MODE == kDecParts) a.part_ml[((int64_t)hd * S + rank) * G + hh] = make_float2(M2, Ls);
+            s_ML[hh] = make_float2(M2, Ls);
         }
     }
     if (MODE == kDecParts) {
         if (rank == 0 && tid == 0) a.part_len[hd] = app ? ln : -1;
+        store_appended();
         return;
     }
 
     // ---- combine the CTAs of the cluster in rank order through distributed shared memory ----------------
     if (CL) cluster_sync_all(); else __syncthreads();
-    // my slice of the output channels: element (hh, d) with hh*128 + d = rank*128 + tid (+ S*128 ...).
-    // A thread fetches what it needs from every CTA in one go (max, sum and its channel) and
-    // works out the weights itself, so there is one round trip and no block barrier on this path.
-    for (int idx = rank * kDecThreads + tid; idx < G * kHeadDim; idx += S * kDecThreads) {
-        const int hh = idx >> 7;
-        const uint32_t a_o = (uint32_t)__cvta_generic_to_shared(s_acc + idx);
-        const uint32_t a_m = (uint32_t)__cvta_generic_to_shared(s_M + hh);
-        const uint32_t a_l = (uint32_t)__cvta_generic_to_shared(s_L + hh);
-        float x[kDecMaxCluster], m[kDecMaxCluster], l[kDecMaxCluster];
+    // my slice of the output: pairs of channels rank * kDecThreads + tid (+ S * kDecThreads ...) of the G heads.  A thread fetches
+    // what it needs from every CTA in one go (max, sum and its channels) and works out the weights itself, so there is one
+    // round trip and no block barrier on this path.
+    for (int idx = rank * kDecThreads + tid; idx < G * (kHeadDim / 2); idx += S * kDecThreads) {
+        const int hh = idx >> 6;
+        const uint32_t a_o = (uint32_t)__cvta_generic_to_shared(s_res + idx), a_ml = (uint32_t)__cvta_generic_to_shared(s_ML + hh);
+        float2 x[kDecMaxCluster], ml[kDecMaxCluster];
 #pragma unroll
         for (int r = 0; r < kDecMaxCluster; ++r) {
-            x[r] = 0.f; m[r] = -INFINITY; l[r] = 0.f;
+            x[r] = make_float2(0.f, 0.f); ml[r] = make_float2(-INFINITY, 0.f);
             if (r < S) {
                 if (CL) {
-                    x[r] = dsmem_ld(dsmem_addr(a_o, r));
-                    m[r] = dsmem_ld(dsmem_addr(a_m, r));
-                    l[r] = dsmem_ld(dsmem_addr(a_l, r));
+                    x[r] = dsmem_ld2(dsmem_addr(a_o, r));
+                    ml[r] = dsmem_ld2(dsmem_addr(a_ml, r));
                 } else {                       // a head with one CTA: its own shared memory, read directly
-                    x[r] = s_acc[idx]; m[r] = s_M[hh]; l[r] = s_L[hh];
+                    x[r] = s_res[idx]; ml[r] = s_ML[hh];
                 }
             }
         }
         float FM = -INFINITY;
 #pragma unroll
-        for (int r = 0; r < kDecMaxCluster; ++r) FM = fmaxf(FM, m[r]);
-        float v = 0.f, Ls = 0.f;
+        for (int r = 0; r < kDecMaxCluster; ++r) FM = fmaxf(FM, ml[r].x);
+        float2 v = make_float2(0.f, 0.f);
+        float Ls = 0.f;
 #pragma unroll
         for (int r = 0; r < kDecMaxCluster; ++r) {
-            const float w = m[r] > -INFINITY ? exp2f(m[r] - FM) : 0.f;
-            v += x[r] * w;
-            Ls += l[r] * w;
+            const float w = ml[r].x > -INFINITY ? exp2f(ml[r].x - FM) : 0.f;
+            v.x += x[r].x * w; v.y += x[r].y * w;
+            Ls += ml[r].y * w;
         }
-        a.out[(int64_t)(b * H + h0) * kHeadDim + idx] = __float2bfloat16_rn(Ls > 0.f ? v / Ls : 0.f);
+        const float inv = Ls > 0.f ? 1.0f / Ls : 0.f;
+        reinterpret_cast<uint32_t*>(a.out + (int64_t)(b * H + h0) * kHeadDim)[idx] = pack_bf16(v.x * inv, v.y * inv);
     }
-    if (CL && a.acc_score && tid < 8 * S) {    // (max, sum) of every CTA and head, for the acc_score update
-        const int r = tid >> 3, hh = tid & 7;
-        float m = -INFINITY, l = 0.f;
-        if (hh < G) {
-            m = dsmem_ld(dsmem_addr((uint32_t)__cvta_generic_to_shared(s_M + hh), r));
-            l = dsmem_ld(dsmem_addr((uint32_t)__cvta_generic_to_shared(s_L + hh), r));
-        }
-        s_rm[tid] = m;
-        s_rl[tid] = l;
+    if (a.acc_score && tid < 64) {             // cluster-wide (max, 1 / sum) of every head: thread = (head, CTA)
+        const int hh = tid >> 3, r = tid & 7;
+        float2 ml = make_float2(-INFINITY, 0.f);
+        if (hh < G && r < S) ml = CL ? dsmem_ld2(dsmem_addr((uint32_t)__cvta_generic_to_shared(s_ML + hh), r)) : s_ML[hh];
+        float FM = ml.x;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) FM = fmaxf(FM, __shfl_xor_sync(0xFFFFFFFFu, FM, o));
+        float Ls = ml.x > -INFINITY ? ml.y * exp2f(ml.x - FM) : 0.f;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) Ls += __shfl_xor_sync(0xFFFFFFFFu, Ls, o);
+        if (r == 0) { s_FM[hh] = FM; s_FI[hh] = Ls > 0.f ? 1.0f / Ls : 0.f; }
     }
-    if (CL) cluster_arrive();                  // my reads of the other CTAs' shared memory are done
+    if (CL) cluster_arrive_exec();             // my reads of the other CTAs' shared memory are done
+    store_appended();
     // the probabilities of my own keys go to acc_score
     if (a.acc_score) {
-        if (!CL) {                             // one CTA: its own (max, sum) are the head's
-            if (tid < G) { s_FM[tid] = s_M[tid]; s_FI[tid] = s_L[tid] > 0.f ? 1.0f / s_L[tid] : 0.f; }
-        } else {
-            __syncthreads();
-        }
-        if (CL && tid < G) {
-            float FM = -INFINITY;
-            for (int r = 0; r < S; ++r) FM = fmaxf(FM, s_rm[r * 8 + tid]);
-            float Ls = 0.f;
-            for (int r = 0; r < S; ++r) {
-                const float m = s_rm[r * 8 + tid];
-                if (m > -INFINITY) Ls += s_rl[r * 8 + tid] * exp2f(m - FM);
-            }
-            s_FM[tid] = FM;
-            s_FI[tid] = Ls > 0.f ? 1.0f / Ls : 0.f;
-        }
         __syncthreads();
         float* acc = a.acc_score + (int64_t)hd * cap;
         float il[G], mx[G];
 #pragma unroll
         for (int hh = 0; hh < G; ++hh) { mx[hh] = s_FM[hh]; il[hh] = s_FI[hh]; }
         const int j_lo = t_lo * kTileKeys, j_hi = min(lne, t_hi * kTileKeys);
-        // four keys per thread per round: 4 (G + 1) independent loads in flight
+        // four keys per thread per round (past the end: the last key again, not stored): 4 (G + 1) independent loads in flight
+        const float* ws = a.ws_s + (int64_t)(b * H + h0) * cap;
         for (int j0 = j_lo + tid; j0 < j_hi; j0 += 4 * kDecThreads) {
             float lg[4][G], old[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int j = j0 + u * kDecThreads;
-                old[u] = 0.f;
-                if (j < j_hi) {
+            for (int u = 0; u < 4; ++u) old[u] = __ldcg(acc + min(j0 + u * kDecThreads, j_hi - 1));
+            if (a.logit_keys) {
 #pragma unroll
-                    for (int hh = 0; hh < G; ++hh)
-                        lg[u][hh] = a.logit_keys ? s_logit[hh * a.logit_keys + (j - j_lo)]
-                                                 : __ldcg(a.ws_s + (int64_t)(b * H + h0 + hh) * cap + j);
-                    if (!(app && j == ln)) old[u] = acc[j];                  // a new entry starts at zero
-                }
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int hh = 0; hh < G; ++hh) lg[u][hh] = s_logit[hh * a.logit_keys + min(j0 + u * kDecThreads, j_hi - 1) - j_lo];
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int hh = 0; hh < G; ++hh) lg[u][hh] = __ldcg(ws + (int64_t)hh * cap + min(j0 + u * kDecThreads, j_hi - 1));
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int j = j0 + u * kDecThreads;
-                if (j < j_hi) {
-                    float pr = 0.f;
+                float pr = 0.f;
 #pragma unroll
-                    for (int hh = 0; hh < G; ++hh) pr += exp2f(lg[u][hh] - mx[hh]) * il[hh];
-                    acc[j] = old[u] + pr;
-                }
+                for (int hh = 0; hh < G; ++hh) pr += exp2f(lg[u][hh] - mx[hh]) * il[hh];
+                if (j < j_hi) acc[j] = (app && j == ln ? 0.f : old[u]) + pr;         // a new entry starts at zero
             }
         }
     }
@@ -672,7 +657,7 @@ static lvlm_status launch_decode(const void* q, void* Kc, void* Vc, int32_t* len
     if (per >= kDecWarps) per = (per + kDecWarps - 1) / kDecWarps * kDecWarps;
     const int run_keys = per * kTileKeys;
     const int logit_keys = acc_score && !parts && (size_t)G * run_keys * 4 <= (size_t)kDecLogitBytes ? run_keys : 0;
-    const size_t smem = 1024 + (size_t)kRingBytes + (size_t)(2 * kDecWarps * 8 + 4 * 8 + 2 * 8 * kDecMaxCluster) * 4 +
+    const size_t smem = 1024 + (size_t)kRingBytes + (size_t)(2 * kDecWarps * 8 + 4 * 8) * 4 +
                         (size_t)(2 * kStagesDec + 1) * 8 + (size_t)G * logit_keys * 4;
     CUtensorMap kmap, vmap;
     {
