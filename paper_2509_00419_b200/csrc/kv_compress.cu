@@ -35,59 +35,49 @@ __device__ __forceinline__ long long score_units(float s) {
     return __float2ll_rn(s * 16777216.0f);               // exact: a power of two (beyond 2^104 both saturate)
 }
 
-// ceil(a * b / c) for a, b < 2^63, c = 10^6, in 128-bit arithmetic.
-__device__ __forceinline__ unsigned long long ceil_muldiv(unsigned long long a, unsigned long long b,
-                                                          unsigned long long c) {
-    unsigned long long hi = __umul64hi(a, b), lo = a * b;
-    // long division of (hi:lo) by c, 64 steps; hi < c holds because a < c (beta < 1) ... not
-    // assumed: reduce hi first.
-    unsigned long long rem = hi % c;
-    unsigned long long q = 0;
-#pragma unroll 1
-    for (int bit = 63; bit >= 0; --bit) {
-        rem = (rem << 1) | ((lo >> bit) & 1ull);        // rem < 2c < 2^63, no overflow
-        q <<= 1;
-        if (rem >= c) { rem -= c; q |= 1ull; }
-    }
-    // the quotient's high word (hi / c) is zero whenever a <= c, which the caller guarantees
-    return q + (rem != 0);
+// ceil(beta_ppm * total / 10^6) for beta_ppm < 10^6, total < 2^63: with total = 10^6 q + r it is beta_ppm q + ceil(beta_ppm r / 10^6).
+// (Divisions by a constant; a 128-bit long division took 7 us.)
+__device__ __forceinline__ unsigned long long beta_of_total(unsigned long long beta_ppm, unsigned long long total) {
+    const unsigned long long q = total / 1000000ull, r = total - q * 1000000ull;
+    return beta_ppm * q + (beta_ppm * r + 999999ull) / 1000000ull;
 }
 
-// Sums over the first `nwarp` warps of the block of a count and a 64-bit mass (one barrier: the scratch rows
-// alternate with `turn`).
-struct PlanScratch { int c[2][32]; unsigned long long m[2][32]; };
-__device__ __forceinline__ void block_sum2(int* c, unsigned long long* ms, PlanScratch* sc, int turn, int nwarp) {
-    int cc = *c;
-    unsigned long long mm = *ms;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        cc += __shfl_xor_sync(0xFFFFFFFFu, cc, o);
-        mm += __shfl_xor_sync(0xFFFFFFFFu, mm, o);
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) { sc->c[turn][warp] = cc; sc->m[turn][warp] = mm; }
-    asm volatile("bar.sync 1, %0;" ::"r"(nwarp * 32) : "memory");       // the warps that hold entries
-    cc = 0; mm = 0;
-    for (int wv = 0; wv < nwarp; ++wv) { cc += sc->c[turn][wv]; mm += sc->m[turn][wv]; }
-    *c = cc; *ms = mm;
+__device__ __forceinline__ unsigned long long redux_add_u64(unsigned long long v) {
+    // three limbs of 22 bits: 32 of them still fit a word (v < 2^63)
+    const uint32_t l0 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)v & 0x3FFFFFu);
+    const uint32_t l1 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(v >> 22) & 0x3FFFFFu);
+    const uint32_t l2 = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(v >> 44));
+    return (unsigned long long)l0 + ((unsigned long long)l1 << 22) + ((unsigned long long)l2 << 44);
 }
 
-// One CTA per (sequence, KV head).  A thread holds KPT consecutive evictable entries as 64-bit keys (order-
-// preserving image of the score above the index: ascending key = descending score, lower index first).  Nothing
-// is sorted: the entry at which the accumulated score reaches the threshold, and the entry that closes the budget,
-// are found by building the key bit by bit from the top - "do the entries up to this key reach the target?" is one
-// sum over the block - and only over the bits in which the keys differ at all.  All sums are integers, so the
-// result does not depend on the order of summation.
-template <int KPT>
-__global__ void __launch_bounds__(1024)
+// The score units behind a key.
+__device__ __forceinline__ unsigned long long units_of_key(uint32_t dk) {
+    if (dk == 0xFFFFFFFFu) return 0ull;
+    const uint32_t asc = ~dk;
+    return score_units(__uint_as_float((asc & 0x80000000u) ? (asc & 0x7FFFFFFFu) : ~asc));
+}
+
+// One CTA per (sequence, KV head).  A warp has 32 * KPT consecutive evictable entries, lane l of it l, l + 32, ..., as 32-bit
+// keys (order-preserving image of the score: ascending key = descending score; among equal scores the lower index comes
+// first).  Nothing is sorted: the score at which the accumulated score reaches the threshold, and the one that closes
+// the budget, are found from the top, 11 bits a pass, at most three passes: a histogram in shared memory (of the count, or
+// of the score in limbs of 18 bits, so that 16384 of them fit a word), a scan, and only the entries of the bucket that
+// crosses the target go on.  88 heads of 3008 rows: 42 us a bit a time over 64-bit keys (a block-wide sum and a barrier
+// each), 22 with two bits a time, now 16.  All sums are integers, so the result does not depend on the order of summation.
+constexpr int kPlanDigit = 11, kPlanBuckets = 1 << kPlanDigit, kPlanLimb = 18, kPlanLimbs = 4;
+constexpr int kPlanHist = kPlanBuckets + kPlanBuckets / 8;         // a word of padding every 8: a thread scans 8 buckets (or 2)
+__device__ __forceinline__ uint32_t plan_bucket(uint32_t i) { return i + (i >> 3); }
+
+template <int KPT, int MAXT>
+__global__ void __launch_bounds__(MAXT)
 kv_plan_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t* __restrict__ e_lo,
                const int32_t* __restrict__ e_hi, int Hkv, int cap, int recent, int min_m,
                unsigned long long beta_ppm, int budget, int32_t* __restrict__ src_map,
                int32_t* __restrict__ meta, int32_t* __restrict__ nout, float* __restrict__ acc_new,
                int32_t* __restrict__ pos_new, int32_t* dev_status) {
-    __shared__ PlanScratch sc;
-    __shared__ unsigned long long s_and[32], s_or[32];
-    __shared__ int scan_scratch[33];
+    __shared__ __align__(16) uint32_t s_hist[kPlanLimbs][kPlanHist];
+    __shared__ unsigned long long s_sum[32], s_before;
+    __shared__ uint32_t s_and[32], s_or[32], s_digit;
     __shared__ int s_first_drop;
 
     pdl_enter();
@@ -113,6 +103,7 @@ kv_plan_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t* __re
     // only the warps that hold entries stay: every barrier below counts them alone
     const int nwarp = max(1, (m + 32 * KPT - 1) / (32 * KPT)), nthr = nwarp * 32;
     if ((int)threadIdx.x >= nthr) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto sync_active = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory"); };
     if (threadIdx.x == 0) s_first_drop = m;
     // compacted acc_score and pos go beside the map; the kernel that moves the K and V rows copies them back
@@ -121,118 +112,180 @@ kv_plan_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t* __re
     int32_t* pn = pos_new + (int64_t)m_idx * cap;
 
     // ---- my keys -------------------------------------------------------------------------------------
-    const int j0 = threadIdx.x * KPT;
-    uint64_t key[KPT];
+    const int j0 = warp * (32 * KPT) + lane;             // my entries: j0, j0 + 32, ...
+    float sv[KPT];
+    uint32_t key[KPT];
     unsigned long long un[KPT];                          // the scores in integer units
     bool nonfinite = false;
-    uint64_t k_and = ~0ull, k_or = 0ull;
-    unsigned long long total = 0;
-    int turn = 0;
+    uint32_t k_and = ~0u, k_or = 0u;
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) sv[u] = j0 + 32 * u < m ? acc[lo + j0 + 32 * u] : 0.f;
 #pragma unroll
     for (int u = 0; u < KPT; ++u) {
-        key[u] = ~0ull;                                  // past the end: above every real key
+        key[u] = ~0u;                                    // past the end: the top value, no score
         un[u] = 0ull;
-        if (j0 + u < m) {
-            const float sv = acc[lo + j0 + u];
-            key[u] = ((uint64_t)desc_key(sv, &nonfinite) << 32) | (uint32_t)(j0 + u);
+        if (j0 + 32 * u < m) {
+            key[u] = desc_key(sv[u], &nonfinite);
             k_and &= key[u]; k_or |= key[u];
-            un[u] = (unsigned long long)score_units(sv);
-            total += un[u];
+            un[u] = (unsigned long long)score_units(sv[u]);
         }
     }
     if (nonfinite && dev_status) atomicOr(dev_status, LVLM_DEV_NONFINITE);
-    {   // bits in which the keys differ, and the total score
+    k_and = __reduce_and_sync(0xFFFFFFFFu, k_and);       // bits in which the keys differ
+    k_or = __reduce_or_sync(0xFFFFFFFFu, k_or);
+    if (lane == 0) { s_and[warp] = k_and; s_or[warp] = k_or; }
+    sync_active();
+    k_and = __reduce_and_sync(0xFFFFFFFFu, lane < nwarp ? s_and[lane] : ~0u);
+    k_or = __reduce_or_sync(0xFFFFFFFFu, lane < nwarp ? s_or[lane] : 0u);
+    const uint32_t diff = m > 0 ? (k_and ^ k_or) : 0u;
+
+    // Exclusive prefix sum over the block's threads, in thread order, and the total.
+    auto block_scan = [&](unsigned long long x, unsigned long long* total) -> unsigned long long {
+        unsigned long long incl = x;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            k_and &= __shfl_xor_sync(0xFFFFFFFFu, k_and, o);
-            k_or |= __shfl_xor_sync(0xFFFFFFFFu, k_or, o);
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += t;
         }
-        if ((threadIdx.x & 31) == 0) { s_and[threadIdx.x >> 5] = k_and; s_or[threadIdx.x >> 5] = k_or; }
-        int dummy = 0;
-        block_sum2(&dummy, &total, &sc, turn, nwarp); turn ^= 1;            // (its barrier also publishes s_and / s_or)
-        k_and = ~0ull; k_or = 0ull;
-        for (int wv = 0; wv < nwarp; ++wv) { k_and &= s_and[wv]; k_or |= s_or[wv]; }
-    }
-    const uint64_t diff = m > 0 ? (k_and ^ k_or) : 0ull;
-    // Smallest key T such that the entries with key <= T hold at least `target` (their count, or their score when
-    // by_mass).  The caller guarantees that all entries together reach the target.
-    auto search = [&](unsigned long long target, bool by_mass) -> uint64_t {
-        uint64_t ans = k_and;
-        uint64_t todo = diff;
-        while (todo) {
-            const int bit = 63 - __clzll((long long)todo);
-            todo &= ~(1ull << bit);
-            const uint64_t cand = (ans & ~(1ull << bit)) | ((1ull << bit) - 1ull);
-            int cnt = 0;
-            unsigned long long ms = 0;
+        sync_active();                                   // s_sum may still be read from a call before
+        if (lane == 31) s_sum[warp] = incl;
+        sync_active();
+        const unsigned long long w = lane < nwarp ? s_sum[lane] : 0ull;
+        *total = redux_add_u64(w);
+        return redux_add_u64(lane < warp ? w : 0ull) + incl - x;
+    };
+    // Smallest score key T such that the entries with key <= T hold at least `target` (their count, or their score when
+    // by_mass, in `limbs` limbs); *before: what the entries with a strictly better score hold.  The caller guarantees
+    // that all entries together reach the target.
+    auto search = [&](unsigned long long target, bool by_mass, int limbs, unsigned long long* before) -> uint32_t {
+        unsigned long long below = 0ull;
+        uint32_t prefix = k_and;                         // T, as far as it is known: the bits from `shift` up
+        int shift = 32 - __clz((int)diff);               // (the bits from here up do not differ)
+        const int per = (kPlanBuckets + nthr - 1) / nthr, b0 = min(kPlanBuckets, (int)threadIdx.x * per), b1 = min(kPlanBuckets, b0 + per);
+        while (shift > 0) {
+            const int hi_shift = shift;
+            shift = max(0, shift - kPlanDigit);
+            for (int i = threadIdx.x; i < limbs * (kPlanHist / 4); i += nthr)
+                reinterpret_cast<uint4*>(s_hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+            sync_active();
 #pragma unroll
             for (int u = 0; u < KPT; ++u) {
-                if (key[u] <= cand) { ++cnt; ms += un[u]; }
-            }
-            block_sum2(&cnt, &ms, &sc, turn, nwarp); turn ^= 1;
-            const unsigned long long have = by_mass ? ms : (unsigned long long)cnt;
-            if (have >= target) ans &= ~(1ull << bit); else ans |= 1ull << bit;
-        }
-        return ans;
-    };
-    auto count_upto = [&](uint64_t T) -> int {
-        int cnt = 0;
-        unsigned long long ms = 0;
+                // (shifts of 32 are not defined: two steps)
+                if (j0 + 32 * u >= m || ((key[u] ^ prefix) >> (hi_shift - 1)) >> 1) continue;
+                const uint32_t d = plan_bucket((key[u] >> shift) & (kPlanBuckets - 1));
+                if (!by_mass) { atomicAdd(&s_hist[0][d], 1u); continue; }
 #pragma unroll
-        for (int u = 0; u < KPT; ++u) cnt += key[u] <= T;
-        block_sum2(&cnt, &ms, &sc, turn, nwarp); turn ^= 1;
-        return cnt;
+                for (int l = 0; l < kPlanLimbs; ++l) {
+                    const uint32_t x = (uint32_t)(un[u] >> (l * kPlanLimb)) & ((1u << kPlanLimb) - 1u);
+                    if (x) atomicAdd(&s_hist[l][d], x);
+                }
+            }
+            sync_active();
+            unsigned long long mine = 0ull, total;
+#pragma unroll
+            for (int l = 0; l < kPlanLimbs; ++l) {       // (a limb summed over all entries fits a word)
+                uint32_t x = 0u;
+                if (l < limbs) {
+#pragma unroll 8
+                    for (int i = b0; i < b1; ++i) x += s_hist[l][plan_bucket(i)];
+                }
+                mine += (unsigned long long)x << (l * kPlanLimb);
+            }
+            unsigned long long run = below + block_scan(mine, &total);
+            if (run < target && run + mine >= target) {  // the bucket that crosses the target is one of mine
+                unsigned long long b = run;
+                int d = b0;
+#pragma unroll 4
+                for (int i = b0; i < b1; ++i) {          // (no early exit: the loads overlap)
+                    unsigned long long x = 0ull;
+#pragma unroll
+                    for (int l = 0; l < kPlanLimbs; ++l)
+                        if (l < limbs) x += (unsigned long long)s_hist[l][plan_bucket(i)] << (l * kPlanLimb);
+                    run += x;
+                    if (run < target) { b = run; d = i + 1; }
+                }
+                s_digit = (uint32_t)d;
+                s_before = b;
+            }
+            sync_active();
+            below = s_before;
+            // (the digit may reach above the bits that differ: those bits are the same in every key)
+            prefix = (prefix & ~((kPlanBuckets - 1u) << shift)) | (s_digit << shift);
+        }
+        *before = below;
+        return prefix;
     };
 
     // ---- how many entries of E reach the threshold, how many the budget allows ---------------------------
-    int k_beta = m;
-    uint64_t T = ~0ull;                                  // keys <= T survive
+    int k_beta = m, need = 0;
+    uint32_t T = ~0u;                                    // survivors: score key < T, and the first `need` entries of key T
     bool have_T = false;
+    unsigned long long before = 0ull;
     if (beta_ppm < 1000000ull && m > 0) {
-        const unsigned long long thr = ceil_muldiv(beta_ppm, total, 1000000ull);
+        unsigned long long mine = 0ull, total;
+#pragma unroll
+        for (int u = 0; u < KPT; ++u) mine += un[u];
+        block_scan(mine, &total);
+        const unsigned long long thr = beta_of_total(beta_ppm, total);
         if (thr == 0) k_beta = 1;
         else {
-            T = search(thr, true);
-            k_beta = count_upto(T);
+            const int limbs = min(kPlanLimbs, (63 - __clzll((long long)total)) / kPlanLimb + 1);     // (no entry holds more than all)
+            T = search(thr, true, limbs, &before);
+            const unsigned long long each = units_of_key(T);             // > 0: the entries of key T are needed
+            need = (int)((thr - before + each - 1ull) / each);
             have_T = true;
         }
     }
+    // Entries better than T and of score T, in the warps before mine (16 bits each), and of all warps.
+    auto count_T = [&](int* all) -> int {
+        int better = 0, equal = 0;
+#pragma unroll
+        for (int u = 0; u < KPT; ++u) {
+            better += __popc(__ballot_sync(0xFFFFFFFFu, j0 + 32 * u < m && key[u] < T));
+            equal += __popc(__ballot_sync(0xFFFFFFFFu, j0 + 32 * u < m && key[u] == T));
+        }
+        sync_active();
+        if (lane == 0) s_sum[warp] = (unsigned long long)(uint32_t)(better | (equal << 16));
+        sync_active();
+        const uint32_t w = lane < nwarp ? (uint32_t)s_sum[lane] : 0u;
+        *all = (int)__reduce_add_sync(0xFFFFFFFFu, w);
+        return (int)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? w : 0u);
+    };
+    int all = 0, before_me = 0;
+    if (have_T) { before_me = count_T(&all); k_beta = (all & 0xFFFF) + need; }
     int kc = k_beta;
     if (budget > 0) kc = min(kc, budget - (ln - m));
     kc = min(max(kc, 0), m);
-    if (kc < m && kc > 0 && !(have_T && kc == k_beta)) T = search((unsigned long long)kc, false);
+    if (kc < m && kc > 0 && !(have_T && kc == k_beta)) {
+        T = search((unsigned long long)kc, false, 1, &before);
+        need = kc - (int)before;
+        before_me = count_T(&all);
+    }
 
-    // ---- survivor map: my entries are consecutive, so a scan of the counts gives their places ------------------
+    // ---- survivor map, in index order: a warp's entries 32 at a time, places by ballot --------------------------
     {
-        int cnt = 0, first_drop = m;
+        int eq = before_me >> 16;                        // entries of score T in the warps before mine
+        int off = kc >= m ? warp * (32 * KPT) : kc == 0 ? 0 : (before_me & 0xFFFF) + min(eq, need);
+        const uint32_t lt = (1u << lane) - 1u;
+        int first_drop = m;
 #pragma unroll
         for (int u = 0; u < KPT; ++u) {
-            if (j0 + u < m) {
-                const bool kept = kc >= m || (kc > 0 && key[u] <= T);
-                if (kept) ++cnt; else if (first_drop == m) first_drop = j0 + u;
+            const int j = j0 + 32 * u;
+            const bool valid = j < m, is_eq = valid && key[u] == T;
+            const uint32_t beq = __ballot_sync(0xFFFFFFFFu, is_eq);
+            const bool kept = valid && (kc >= m || (kc > 0 && (key[u] < T || (is_eq && eq + __popc(beq & lt) < need))));
+            const uint32_t bk = __ballot_sync(0xFFFFFFFFu, kept), bd = __ballot_sync(0xFFFFFFFFu, valid && !kept);
+            if (kept) {
+                const int o = lo + off + __popc(bk & lt);
+                src[o] = lo + j;
+                an[o] = KPT > 4 && MAXT > 256 ? acc[lo + j] : sv[u];     // (1024 threads: 16 scores more do not fit the registers)
+                if (ps) pn[o] = ps[lo + j];
             }
+            if (first_drop == m && bd) first_drop = j - lane + __ffs((int)bd) - 1;
+            off += __popc(bk);
+            eq += __popc(beq);
         }
-        // exclusive scan of the counts over the active warps
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) scan_scratch[warp] = incl;
-        sync_active();
-        int off = incl - cnt;
-        for (int wv = 0; wv < warp; ++wv) off += scan_scratch[wv];
-        if (first_drop < m) atomicMin(&s_first_drop, first_drop);
-#pragma unroll
-        for (int u = 0; u < KPT; ++u)
-            if (j0 + u < m && (kc >= m || (kc > 0 && key[u] <= T))) {
-                src[lo + off] = lo + j0 + u;
-                an[lo + off] = acc[lo + j0 + u];
-                if (ps) pn[lo + off] = ps[lo + j0 + u];
-                ++off;
-            }
+        if (lane == 0 && first_drop < m) atomicMin(&s_first_drop, first_drop);
     }
     const int new_len = lo + kc + (ln - hi);
     for (int o = threadIdx.x; o < new_len; o += nthr) {
@@ -326,12 +379,6 @@ kv_plan_warp_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t*
         k_or |= __shfl_xor_sync(0xFFFFFFFFu, k_or, o);
     }
     const uint32_t diff = m > 0 ? (k_and ^ k_or) : 0u;
-    auto units_of = [](uint32_t dk) -> unsigned long long {      // the score units behind a key
-        if (dk == 0xFFFFFFFFu) return 0ull;
-        const uint32_t asc = ~dk;
-        const uint32_t bits = (asc & 0x80000000u) ? (asc & 0x7FFFFFFFu) : ~asc;
-        return (unsigned long long)score_units(__uint_as_float(bits));
-    };
     // Score units of the entries with key <= cand (or < cand), summed over the warp.
     auto mass_upto = [&](uint32_t cand, bool strict) -> unsigned long long {
         unsigned long long ms = 0;
@@ -339,11 +386,9 @@ kv_plan_warp_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t*
         for (int u = 0; u < KPL; ++u) {
             uint32_t h = hk[u];
             if (KPL > 32) asm volatile("" : "+r"(h));    // worked out again at every use: 64 more registers would not fit
-            if (strict ? h < cand : h <= cand) ms += units_of(h);
+            if (strict ? h < cand : h <= cand) ms += units_of_key(h);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ms += __shfl_xor_sync(0xFFFFFFFFu, ms, o);
-        return ms;
+        return redux_add_u64(ms);
     };
     // Smallest score key T such that the entries with key <= T are at least `target` many (by_count) or hold at
     // least `target` units of score: built bit by bit from the top, over the bits in which the keys differ.
@@ -360,7 +405,7 @@ kv_plan_warp_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t*
                 int cnt = 0;
 #pragma unroll
                 for (int u = 0; u < KPL; ++u) cnt += hk[u] <= cand;
-                have = (unsigned long long)warp_sum(cnt);
+                have = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)cnt);
             } else {
                 have = mass_upto(cand, false);
             }
@@ -372,7 +417,7 @@ kv_plan_warp_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t*
         int c = 0;
 #pragma unroll
         for (int u = 0; u < KPL; ++u) c += hk[u] < T;
-        return warp_sum(c);
+        return (int)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)c);
     };
 
     // ---- how many entries reach the threshold, how many the budget allows --------------------------------------
@@ -382,13 +427,13 @@ kv_plan_warp_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t*
     bool have_T = false;
     if (MASS && m > 0) {
         const unsigned long long total = mass_upto(~0u, false);
-        const unsigned long long thr = ceil_muldiv(beta_ppm, total, 1000000ull);
+        const unsigned long long thr = beta_of_total(beta_ppm, total);
         if (thr == 0) k_beta = 1;
         else {
             T = search(thr, false);
             const int c = count_below(T);
             const unsigned long long below = mass_upto(T, true);
-            const unsigned long long each = units_of(T);                 // > 0: the entries of key T are needed
+            const unsigned long long each = units_of_key(T);                 // > 0: the entries of key T are needed
             need = (int)((thr - below + each - 1ull) / each);
             k_beta = c + need;
             have_T = true;
@@ -491,9 +536,8 @@ extern "C" lvlm_status lvlm_kv_compress(void* Kc, void* Vc, float* acc_score, in
     // With enough heads to fill the GPU with one warp each, a warp per head (no barrier in the searches); a CTA per
     // head otherwise, and for the heads whose entries do not fit a warp's registers.
     const bool many = heads >= 4 * 148;
-    const int kpt = d->cap <= 4096 ? 4 : 16;
+    const int kpt = d->cap <= 1024 ? 4 : 16;             // entries a thread: at most 8 warps up to 4096 rows
     int threads = ((d->cap + kpt - 1) / kpt + 31) / 32 * 32;
-    threads = threads < 64 ? 64 : threads;
     int min_m = 0;                                       // heads the CTA kernel leaves to the warp kernel
     bool cta_kernel = true;
     if (many) {
@@ -507,13 +551,10 @@ extern "C" lvlm_status lvlm_kv_compress(void* Kc, void* Vc, float* acc_score, in
         min_m = 32 * 32 + 1;
     }
     if (cta_kernel) {
-        // a CTA per head, a thread holds 4 entries (caches up to 4096 rows) or 16; warps without entries leave at once
-        st = kpt == 4 ? launch_kernel(kv_plan_kernel<4>, dim3(d->Hkv, d->B), dim3(threads), 0, stream, 1, acc_score, pos,
-                                      len, e_lo, e_hi, d->Hkv, d->cap, d->recent, min_m, beta_ppm, budget, src_map,
-                                      meta, nout, acc_new, pos_new, dev_status)
-                      : launch_kernel(kv_plan_kernel<16>, dim3(d->Hkv, d->B), dim3(threads), 0, stream, 1, acc_score, pos,
-                                      len, e_lo, e_hi, d->Hkv, d->cap, d->recent, min_m, beta_ppm, budget, src_map,
-                                      meta, nout, acc_new, pos_new, dev_status);
+        // a CTA per head; warps without entries leave at once
+        auto kernel = kpt == 4 ? kv_plan_kernel<4, 256> : threads <= 256 ? kv_plan_kernel<16, 256> : kv_plan_kernel<16, 1024>;
+        st = launch_kernel(kernel, dim3(d->Hkv, d->B), dim3(threads), 0, stream, 1, acc_score, pos, len, e_lo, e_hi, d->Hkv, d->cap,
+                           d->recent, min_m, beta_ppm, budget, src_map, meta, nout, acc_new, pos_new, dev_status);
     }
 #undef LVLM_PLAN_WARP
 #undef LVLM_PLAN_WARP_

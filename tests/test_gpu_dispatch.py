@@ -145,3 +145,26 @@ def test_nearest_kept_groups(case):
     assert_rows_close(f64(Vd)[:, :, :Nout], want["Vc"], what="V")
     assert np.array_equal(i32(pd)[:, :Nout], want["pos_ids"])
     np.testing.assert_allclose(md.cpu().numpy()[:, :Nout], want["mass"], rtol=1e-6)                 # small whole numbers
+
+
+# cache compression, a CTA per head: scores that tie in one or a few values, keys that differ in one bit, in few bits or in
+# all, entries that outweigh all others by 2^40, caches at the ends of a thread's 4 and 16 entries
+@pytest.mark.parametrize("cap", [1, 31, 4096, 4097, 16384])
+@pytest.mark.parametrize("kind", ["one_value", "two_neighbours", "four_values", "wide"])
+def test_kv_threshold_search(cap, kind):
+    r = np.random.default_rng(cap)
+    acc = {"one_value": np.full((1, 3, cap), 0.3), "two_neighbours": 0.5 + (r.random((1, 3, cap)) < 0.5) * 2.0 ** -24,
+           "four_values": r.integers(0, 4, size=(1, 3, cap)) * 0.125,
+           "wide": 2.0 ** r.uniform(-24, 16, size=(1, 3, cap))}[kind].astype(np.float32)
+    ln = np.array([[cap, max(1, cap - 5), (cap + 1) // 2]], np.int32)
+    Kc = torch.from_numpy(r.normal(size=(1, 3, cap, 128)).astype(np.float32)).to(torch.bfloat16)
+    for beta, budget in ((0.5, 0), (0.999, 0), (0.9, cap // 3), (1.0, max(1, cap // 2))):
+        want = O.kv_compress(f64(Kc), f64(Kc), acc, ln, beta=beta, budget=budget or None)
+        Kd, Vd, ad, ld = Kc.cuda(), Kc.cuda(), torch.from_numpy(acc).cuda(), torch.from_numpy(ln).cuda()
+        flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+        L.kv_compress(Kd, Vd, ad, ld, beta=beta, budget=budget, dev_status=flag)
+        assert flag.item() == 0 and np.array_equal(i32(ld), want["len"]), (beta, budget)
+        for g in range(3):
+            m = want["len"][0, g]
+            assert np.array_equal(ad[0, g, :m].cpu().numpy(), want["acc_score"][0, g, :m]), (beta, budget, g)
+            assert np.array_equal(f64(Kd)[0, g, :m], want["Kc"][0, g, :m].astype(np.float64)), (beta, budget, g)
