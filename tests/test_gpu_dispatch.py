@@ -168,3 +168,22 @@ def test_kv_threshold_search(cap, kind):
             m = want["len"][0, g]
             assert np.array_equal(ad[0, g, :m].cpu().numpy(), want["acc_score"][0, g, :m]), (beta, budget, g)
             assert np.array_equal(f64(Kd)[0, g, :m], want["Kc"][0, g, :m].astype(np.float64)), (beta, budget, g)
+
+
+# selection by bins: 1, 2, 4 and 8 slices, 1, 2 and 4 tokens a thread, last slices that are shorter; bins as deep as they may be
+# and one key deeper, one bin for all but one key, one value
+@pytest.mark.parametrize("B,n", [(1, 511), (1, 512), (1, 1023), (1, 1025), (1, 2049), (1, 14337), (2, 34817), (37, 3001), (140, 1100)])
+@pytest.mark.parametrize("kind", ["random", "deep", "outlier", "one_value"])
+def test_select_bins(B, n, kind):
+    r = np.random.default_rng(n)
+    s = {"random": r.random((B, n)), "deep": (np.arange(n) * 4 // (n + n % 2)) * 0.25 + np.zeros((B, 1)),
+         "outlier": np.where(np.arange(n) == n // 2, 1e30, 1.0 + r.random((B, n)) * 1e-3), "one_value": np.full((B, n), -0.5)}[kind]
+    s = s.astype(np.float32)
+    if kind != "deep":
+        s[0] = s[0, r.permutation(n)]
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rank, _, _ = L.select_topk(torch.from_numpy(s).cuda(), n // 3, want_kept=False, dev_status=flag)
+    order = np.argsort(-s, axis=1, kind="stable")                # whole numbers: nothing to tolerate
+    want = np.empty_like(order)
+    np.put_along_axis(want, order, np.arange(n)[None].repeat(B, 0), axis=1)
+    assert flag.item() == 0 and np.array_equal(i32(rank), want)
