@@ -148,31 +148,39 @@ __device__ __forceinline__ int plan_ld_cluster(const int* my_smem, uint32_t rank
     return v;
 }
 
-// A cluster of P CTAs per sequence (grid (P, B)): source map, destination map, weights, position ids,
-// new length.  CTA r takes the r-th run of the image tokens: it counts its kept tokens, learns from the
-// lower ranks how many came before, then writes the maps of its run (tile by tile, thread = token,
-// coalesced).  The position ids are compacted in place in rounds of P x blockDim output rows: every CTA
-// loads its rows of the round, a cluster barrier, then it stores them (a row's source lies at or behind it,
-// so nothing a later round needs is overwritten).
+// A cluster of P CTAs per sequence (grid (P, B)): source map, destination map, weights, position ids, new length.
+// A chain of latencies, so everything is loaded once, at the start, and the CTAs meet once a round: in a round each
+// warp takes 32 T consecutive image tokens (a lane every 32nd, up to four, ranks and position ids in registers),
+// counts its kept ones by ballots, learns what the warps and the CTAs ahead have, and writes the maps and - in place -
+// the position ids.  (All reads of a round come before the barrier and all writes behind it, and a row never moves up: no
+// round overwrites what a later one reads.)  The rows behind the image span, if more than P x blockDim, go in rounds
+// of their own.  One round up to 32768 tokens.
+// us between the launches around it: 32767 tokens 25 -> 13, 17400 tokens 14 -> 9; one token a thread: 7 -> 4.8 (2880 tokens).
+constexpr int kPlanTokens = 4;                            // tokens of a thread in a round
 __global__ void __launch_bounds__(1024)
 merge_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int i0, int n, int k,
                   int mode, float inv_sum, const float* __restrict__ w_custom,
                   int32_t* __restrict__ src_map, int32_t* __restrict__ dst_map,
                   float* __restrict__ wgt, int32_t* __restrict__ meta, int32_t* new_len,
-                  int32_t* dev_status) {
-    __shared__ int scan_scratch[33];
+                  int32_t* dev_status, int T) {
     __shared__ float fsum_scratch[33];
-    __shared__ int s_total, s_first_drop, s_merged_tok;
+    __shared__ int s_warp[2][32];                         // kept tokens of every warp, of two rounds
+    __shared__ int s_cta[2][3];                           // ... of the CTA; first dropped token; the token that gives P_new its place
     pdl_enter();
     const int b = blockIdx.y, P = (int)gridDim.x, cr = (int)plan_cluster_rank();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const int r1 = n - k, r = r1 - 1, Nout = N - r;
     const int32_t* rk = rank + (int64_t)b * n;
     int32_t* src = src_map + (int64_t)b * N;
     int32_t* dst = dst_map + (int64_t)b * N;      // output row of every input row, -1 = merged away
     float* w = wgt + (int64_t)b * n;
-    const int chunk = (n + P - 1) / P;
-    const int c_lo = min(n, cr * chunk), c_hi = min(n, c_lo + chunk);
-    if (threadIdx.x == 0) { s_total = 0; s_first_drop = n; s_merged_tok = -1; }
+    int32_t* pid = pos_ids ? pos_ids + (int64_t)b * N : nullptr;
+    // the first rows behind the image span: their position ids move by r rows
+    const int tail0 = i0 + k + 1, me = cr * (int)blockDim.x + (int)threadIdx.x;
+    int tail_pos = 0, pos_new = 0;
+    bool is_new = false;
+    if (pid && tail0 + me < Nout) tail_pos = pid[tail0 + me + r];
+    if (threadIdx.x < 2) { s_cta[threadIdx.x][0] = 0; s_cta[threadIdx.x][1] = n; s_cta[threadIdx.x][2] = -1; }
 
     if (mode == LVLM_W_CUSTOM) {
         float part = 0.f;
@@ -182,66 +190,87 @@ merge_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int
     }
     __syncthreads();
 
-    // kept tokens of my run
     bool bad = false;
-    int mine = 0;
-    for (int t0 = c_lo; t0 < c_hi; t0 += blockDim.x) {
-        const int j = t0 + threadIdx.x;
-        const int rj = j < c_hi ? rk[j] : n;
-        if (j < c_hi && (rj < 0 || rj >= n)) bad = true;
-        mine += j < c_hi && rj < k;
-    }
-    mine = warp_sum(mine);
-    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&s_total, mine);
-    plan_cluster_barrier();
-    int kept_before = 0, kept_all = 0;
-    for (int q = 0; q < P; ++q) {
-        const int t = plan_ld_cluster(&s_total, q);
-        kept_before += q < cr ? t : 0;
-        kept_all += t;
-    }
-    if (kept_all != k) bad = true;
-
-    // the maps of my run
-    for (int t0 = c_lo; t0 < c_hi; t0 += blockDim.x) {
-        const int j = t0 + threadIdx.x;
-        const int rj = j < c_hi ? rk[j] : n;              // past the end: counts as dropped, writes nothing
-        const int is_kept = j < c_hi && rj < k;
-        int total;
-        const int off = kept_before + block_exclusive_scan(is_kept, scan_scratch, &total);
-        if (j < c_hi) {
-            float wj = 0.f;
-            if (is_kept) {
-                if (off < k) src[i0 + off] = i0 + j;
-                dst[i0 + j] = off < k ? i0 + off : -1;
-            } else {
-                dst[i0 + j] = -1;
-                if (rj == k) s_merged_tok = j;
-                int p = rj - k;
-                p = p < 0 ? 0 : (p >= r1 ? r1 - 1 : p);
-                wj = merge_weight(mode, p, r1, inv_sum, w_custom);
-            }
-            w[j] = wj;
-        }
-        int fd = (j < c_hi && !is_kept) ? j : n;           // first dropped token: one atomic per warp
+    int kept_before = 0, first_drop = n, merged_tok = 0, round = 0;
+    const int per_round = P * (int)blockDim.x * T;
+    for (int base = 0; base < n; base += per_round, ++round) {
+        const int pb = round & 1;
+        const int j0 = base + (cr * nwarp + warp) * 32 * T + lane;
+        int rj[kPlanTokens], pv[kPlanTokens];
+        unsigned kept[kPlanTokens];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) fd = min(fd, __shfl_xor_sync(0xFFFFFFFFu, fd, o));
-        if ((threadIdx.x & 31) == 0 && fd < n) atomicMin(&s_first_drop, fd);
-        kept_before += total;
+        for (int t = 0; t < kPlanTokens; ++t) {
+            const int j = j0 + 32 * t;
+            const bool on = t < T && j < n;
+            rj[t] = on ? rk[j] : n;                       // past the end: counts as dropped, writes nothing
+            pv[t] = on && pid ? pid[i0 + j] : 0;
+        }
+        int mine = 0;
+#pragma unroll
+        for (int t = 0; t < kPlanTokens; ++t) {
+            const int j = j0 + 32 * t;
+            const bool on = t < T && j < n;
+            if (on && (rj[t] < 0 || rj[t] >= n)) bad = true;
+            kept[t] = __ballot_sync(0xFFFFFFFFu, on && rj[t] < k);
+            mine += __popc(kept[t]);
+            const unsigned drop = __ballot_sync(0xFFFFFFFFu, on && rj[t] >= k);
+            if (lane == 0 && drop) atomicMin(&s_cta[pb][1], j + __ffs(drop) - 1);
+            if (on && rj[t] == k) { s_cta[pb][2] = j; is_new = true; pos_new = pv[t]; }     // P_new takes this token's place
+        }
+        if (lane == 0) { s_warp[pb][warp] = mine; atomicAdd(&s_cta[pb][0], mine); }
+        if (P > 1) plan_cluster_barrier(); else __syncthreads();
+        int c = 0, d = n, m = -1;                         // lane q asks CTA q
+        if (lane < P) {
+            c = plan_ld_cluster(&s_cta[pb][0], lane);
+            d = plan_ld_cluster(&s_cta[pb][1], lane);
+            m = plan_ld_cluster(&s_cta[pb][2], lane);
+        }
+        first_drop = min(first_drop, __reduce_min_sync(0xFFFFFFFFu, d));
+        m = __reduce_max_sync(0xFFFFFFFFu, m);
+        if (m >= 0) merged_tok = m;
+        int off = kept_before + __reduce_add_sync(0xFFFFFFFFu, lane < cr ? c : 0) +
+                  __reduce_add_sync(0xFFFFFFFFu, lane < warp ? s_warp[pb][lane] : 0);
+        kept_before += __reduce_add_sync(0xFFFFFFFFu, c);
+        const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+        for (int t = 0; t < kPlanTokens; ++t) {
+            const int j = j0 + 32 * t;
+            if (t < T && j < n) {
+                float wj = 0.f;
+                int to = -1;
+                if (kept[t] & (1u << lane)) {
+                    const int o = off + __popc(kept[t] & lt);
+                    if (o < k) { to = i0 + o; src[to] = i0 + j; if (pid) pid[to] = pv[t]; }
+                } else {
+                    const int p = min(max(rj[t] - k, 0), r1 - 1);
+                    wj = merge_weight(mode, p, r1, inv_sum, w_custom);
+                }
+                dst[i0 + j] = to;
+                w[j] = wj;
+            }
+            off += __popc(kept[t]);
+        }
+        if (base + per_round < n && round >= 1) {         // (everybody has read the exchange of the round before)
+            if (threadIdx.x == 0) { s_cta[pb ^ 1][0] = 0; s_cta[pb ^ 1][1] = n; s_cta[pb ^ 1][2] = -1; }
+            __syncthreads();
+        }
     }
+    if (kept_before != k) bad = true;
     // rows outside the image span, shared out over the CTAs
-    for (int o = cr * blockDim.x + threadIdx.x; o < Nout; o += P * blockDim.x) {
+    for (int o = me; o < Nout; o += P * blockDim.x) {
         if (o < i0) { src[o] = o; dst[o] = o; }
         else if (o == i0 + k) src[o] = -1;
         else if (o > i0 + k) { src[o] = o + r; dst[o + r] = o; }
     }
-    if (bad && dev_status) atomicOr(dev_status, LVLM_DEV_BOUNDS);
-    plan_cluster_barrier();                               // the maps are complete, every CTA's findings are in place
-    int first_drop = n, merged_tok = 0;
-    for (int q = 0; q < P; ++q) {
-        first_drop = min(first_drop, plan_ld_cluster(&s_first_drop, q));
-        const int mt = plan_ld_cluster(&s_merged_tok, q);
-        if (mt >= 0) merged_tok = mt;
+    if (pid) {
+        if (is_new) pid[i0 + k] = pos_new;
+        if (tail0 + me < Nout) pid[tail0 + me] = tail_pos;
+        for (int o0 = tail0 + P * (int)blockDim.x; o0 < Nout; o0 += P * (int)blockDim.x) {
+            const bool on = o0 + me < Nout;
+            if (on) tail_pos = pid[o0 + me + r];
+            plan_cluster_barrier();
+            if (on) pid[o0 + me] = tail_pos;
+        }
     }
     if (cr == 0 && threadIdx.x == 0) {
         meta[b * kMetaInts + 0] = i0 + first_drop;       // first row whose content changes
@@ -249,18 +278,8 @@ merge_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int
         meta[b * kMetaInts + 2] = merged_tok;
         if (new_len) new_len[b] = Nout;
     }
-    if (pos_ids) {
-        int32_t* pid = pos_ids + (int64_t)b * N;
-        const int pos_new = pid[i0 + merged_tok];         // read before any CTA stores (first store: after a barrier)
-        for (int o0 = 0; o0 < Nout; o0 += P * blockDim.x) {
-            const int o = o0 + cr * blockDim.x + threadIdx.x;
-            int val = 0;
-            if (o < Nout) { const int sidx = src[o]; val = sidx >= 0 ? pid[sidx] : pos_new; }
-            plan_cluster_barrier();
-            if (o < Nout) pid[o] = val;
-        }
-    }
-    plan_cluster_barrier();                               // nobody leaves while its shared memory may still be read
+    if (bad && dev_status) atomicOr(dev_status, LVLM_DEV_BOUNDS);
+    if (P > 1) plan_cluster_barrier();                   // nobody leaves while its shared memory may still be read
 }
 
 __global__ void identity_len_kernel(int32_t* new_len, int B, int N) {
@@ -807,11 +826,13 @@ extern "C" lvlm_status lvlm_merge_compact(void* hidden, void* hidden_out, void* 
     else if (mode == LVLM_W_UNIFORM) inv_sum = (float)(1.0 / (double)L.r1);
     const int plan_threads = d->n >= 1024 ? 1024 : (d->n <= 128 ? 128 : ((d->n + 31) / 32) * 32);
     {
-        int P = (d->n + 2047) / 2048;                    // CTAs per sequence: about two tiles of tokens each
-        P = P < 1 ? 1 : (P > 8 ? 8 : P);
+        int P = (d->n + 1023) / 1024;                    // CTAs per sequence: a token a thread while they last
+        P = P > 8 ? 8 : P;
+        int T = (d->n + P * plan_threads - 1) / (P * plan_threads);
+        T = T > kPlanTokens ? kPlanTokens : T;
         const lvlm_status st = launch_kernel(merge_plan_kernel, dim3(P, d->B), dim3(plan_threads), 0, stream, P,
                                              rank, pos_ids, d->N, d->i0, d->n, d->k, (int)mode, inv_sum, w_custom,
-                                             src_map, dst_map, wgt, meta, new_len, dev_status);
+                                             src_map, dst_map, wgt, meta, new_len, dev_status, T);
         if (st != LVLM_OK) return st;
     }
 

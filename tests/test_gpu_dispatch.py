@@ -187,3 +187,25 @@ def test_select_bins(B, n, kind):
     want = np.empty_like(order)
     np.put_along_axis(want, order, np.arange(n)[None].repeat(B, 0), axis=1)
     assert flag.item() == 0 and np.array_equal(i32(rank), want)
+
+
+# the plan of a merge: 1 to 8 CTAs of 1 to 4 tokens a thread, more than one round (a lone wide batch keeps rows short), image spans
+# that end inside a warp, text behind the image of less and more than one round of rows, the first and the last token on top
+@pytest.mark.parametrize("case", [        # N, i0, n, k
+    (40, 0, 33, 1), (1100, 3, 1025, 700), (3000, 0, 2049, 100), (9000, 7, 8193, 8000), (33500, 0, 32769, 20000),
+    (70000, 5, 65530, 3), (100040, 3, 100000, 40000), (30000, 2, 300, 200), (13000, 1, 3000, 0)])
+@pytest.mark.parametrize("order", ["random", "first", "last"])
+def test_merge_plan_rounds(case, order):
+    N, i0, n, k = case
+    r = np.random.default_rng(N)
+    rank = {"random": r.permutation(n), "first": np.arange(n), "last": np.arange(n)[::-1].copy()}[order].astype(np.int32)
+    hid = torch.from_numpy(r.normal(size=(1, N, 8)).astype(np.float32)).to(torch.bfloat16)
+    pos = r.integers(0, 1 << 30, size=(1, N)).astype(np.int32)
+    pd, flag = torch.from_numpy(pos.copy()).cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    out, new_len = L.merge_compact(hid.cuda(), torch.from_numpy(rank[None]).cuda(), i0=i0, k=k, pos_ids=pd, dev_status=flag)
+    kept = i0 + np.flatnonzero(rank < k)
+    src = np.concatenate([np.arange(i0), kept, [i0 + int(np.flatnonzero(rank == k)[0])], np.arange(i0 + n, N)])
+    assert flag.item() == 0 and new_len.item() == src.size
+    assert np.array_equal(i32(pd)[0, :src.size], pos[0, src])            # whole numbers and rows that move: nothing to tolerate
+    stay = np.arange(src.size) != i0 + k
+    assert np.array_equal(f64(out)[0, stay], f64(hid)[0, src[stay]])
