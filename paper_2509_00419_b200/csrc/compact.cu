@@ -14,7 +14,11 @@
 //
 // The merged row of lvlm_merge_compact is not computed here: the kernel that streams the rows
 // before this one leaves fp32 partial sums, and the CTA that owns the merged position adds them in
-// a fixed order and writes the row.
+// a fixed order and writes the row, as soon as the sums are there and while its first rows come in.
+// (One thread a column group waited for up to 80 partial rows, four at a time, at the end of the last super-tile.  us of a whole
+// merge: 32933 rows of 7 KB and 4 heads' K and V 143.8 -> 111.1, 9075 rows 66.8 -> 39.6, 3008 rows 26.6 -> 21.6, 640 rows of
+// 2 KB and 8 heads 21.6 -> 19.7, 16 sequences of 1888 119.3 -> 118.6.  The scratch for it lies in the second buffer: 8 KB of
+// its own made the last of these 128.)
 #include "compact.cuh"
 
 namespace lvlm {
@@ -53,23 +57,43 @@ __device__ __forceinline__ void cluster_barrier_exec() {
                  "barrier.cluster.wait.aligned;\n" ::: "memory");
 }
 
-// Sum of P fp32 partial rows (pp[p*row_floats + c*8 ...], p = 0..P-1 in that order) for 16-byte group c, rounded once.
-__device__ __forceinline__ uint4 sum_partials(const float* pp, int P, int64_t row_floats, int c) {
+// Sum of P fp32 partial rows (pp[p*row_floats + c*8 ...]) for 16-byte group c, rounded once.  `lanes` threads (256 /
+// lanes apart) take every lanes-th row, four in flight, and the first of them adds up what they have, in a fixed
+// order: one thread for all of up to 80 rows waits for 20 loads one after the other.  Called by every thread of the CTA;
+// the result is the first lane's.  red: [kCompactThreads][8] floats of shared memory (8 KB; the smallest buffer has 12).
+__device__ __forceinline__ uint4 sum_partials(const float* pp, int P, int64_t row_floats, int c, bool on, int lanes, float (*red)[8]) {
+    const int step = kCompactThreads / lanes, lane = threadIdx.x / step;
     float t[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int p0 = 0; p0 < P; p0 += 4) {
-        float4 x0[4], x1[4];
+    if (on) {
+        for (int p0 = lane; p0 < P; p0 += 4 * lanes) {
+            float4 x0[4], x1[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            x0[u] = x1[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (p0 + u < P) {
-                const float4* q = reinterpret_cast<const float4*>(pp + (int64_t)(p0 + u) * row_floats + c * 8);
-                x0[u] = __ldcg(q); x1[u] = __ldcg(q + 1);
+            for (int u = 0; u < 4; ++u) {
+                x0[u] = x1[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (p0 + u * lanes < P) {
+                    const float4* q = reinterpret_cast<const float4*>(pp + (int64_t)(p0 + u * lanes) * row_floats + c * 8);
+                    x0[u] = __ldcg(q); x1[u] = __ldcg(q + 1);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                t[0] += x0[u].x; t[1] += x0[u].y; t[2] += x0[u].z; t[3] += x0[u].w;
+                t[4] += x1[u].x; t[5] += x1[u].y; t[6] += x1[u].z; t[7] += x1[u].w;
             }
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            t[0] += x0[u].x; t[1] += x0[u].y; t[2] += x0[u].z; t[3] += x0[u].w;
-            t[4] += x1[u].x; t[5] += x1[u].y; t[6] += x1[u].z; t[7] += x1[u].w;
+    }
+    if (lanes > 1) {
+        __syncthreads();                                 // `red` may still be read from a call before
+        *reinterpret_cast<float4*>(red[threadIdx.x]) = make_float4(t[0], t[1], t[2], t[3]);
+        *reinterpret_cast<float4*>(red[threadIdx.x] + 4) = make_float4(t[4], t[5], t[6], t[7]);
+        __syncthreads();
+        if (lane == 0) {
+            for (int l = 1; l < lanes; ++l) {
+                const float4 y0 = *reinterpret_cast<const float4*>(red[threadIdx.x + l * step]);
+                const float4 y1 = *reinterpret_cast<const float4*>(red[threadIdx.x + l * step] + 4);
+                t[0] += y0.x; t[1] += y0.y; t[2] += y0.z; t[3] += y0.w;
+                t[4] += y1.x; t[5] += y1.y; t[6] += y1.z; t[7] += y1.w;
+            }
         }
     }
     uint4 o;
@@ -89,8 +113,12 @@ __global__ void __launch_bounds__(kCompactThreads) inplace_compact_kernel(const 
         const int b = blockIdx.z;
         const float* pp = a.fin_partial + (int64_t)b * a.fin_P * a.fin_V * 8;
         uint4* out = reinterpret_cast<uint4*>(a.fin_base + (int64_t)b * a.fin_stride_b) + (int64_t)a.fin_row * a.fin_V;
-        for (int c = blockIdx.x * kCompactThreads + threadIdx.x; c < a.fin_V; c += gridDim.x * kCompactThreads)
-            out[c] = sum_partials(pp, a.fin_P, (int64_t)a.fin_V * 8, c);
+        const int lanes = a.fin_P > 8 ? 8 : 1, step = kCompactThreads / lanes;
+        for (int c0 = blockIdx.x * step; c0 < a.fin_V; c0 += gridDim.x * step) {
+            const int c = c0 + (int)threadIdx.x % step;
+            const uint4 v = sum_partials(pp, a.fin_P, (int64_t)a.fin_V * 8, c, c < a.fin_V, lanes, reinterpret_cast<float (*)[8]>(tile));
+            if ((int)threadIdx.x < step && c < a.fin_V) out[c] = v;
+        }
         return;
     }
     const int S = a.S;
@@ -166,6 +194,21 @@ __global__ void __launch_bounds__(kCompactThreads) inplace_compact_kernel(const 
     }
     load_tile(0, buf[0]);
     if (a.early) pdl_enter();                         // the partial rows and every write come after the kernel ahead
+    // The merged row, if it falls to this CTA: summed while the first rows come in, written in its round (until then it may be
+    // a row that somebody reads).  Thread c of the first 256 / lanes has column groups c, c + 256, ... (lanes > 1: one).
+    uint4 mrow[MAXC];
+    const bool has_merged = a.partial && a.merged_row >= o_start && a.merged_row < Nout && (a.merged_row - o_start) % Rc / R == rank;
+    if (has_merged) {
+        const float* pp = a.partial + (int64_t)((b * a.G + g) * a.T + which) * a.P * V * 8 + (int64_t)c0 * 8;
+        int lanes = 1;
+        while (lanes < 16 && 4 * lanes < a.P && vw * 2 * lanes <= kCompactThreads) lanes *= 2;
+#pragma unroll
+        for (int ci = 0; ci < MAXC; ++ci) {
+            const int c = ci * kCompactThreads + (int)threadIdx.x % (kCompactThreads / lanes);
+            if (ci * kCompactThreads < vw) mrow[ci] = sum_partials(pp, a.P, (int64_t)V * 8, c, c < vw, lanes, reinterpret_cast<float (*)[8]>(buf[1]));
+        }
+        if (lanes > 1) __syncthreads();               // (the buffer is free now)
+    }
     int k = 0;
     for (int t0 = o_start; t0 < Nout; t0 += Rc, ++k) {
         if (t0 + Rc < Nout) load_tile((k + 1) % 3, buf[(k + 1) & 1]);
@@ -187,11 +230,12 @@ __global__ void __launch_bounds__(kCompactThreads) inplace_compact_kernel(const 
                 }
             }
         }
-        if (a.partial && a.merged_row >= lo && a.merged_row < lo + R && a.merged_row < Nout) {
-            // the merged row: partial sums added in their order, rounded once
-            const float* pp = a.partial + (int64_t)((b * a.G + g) * a.T + which) * a.P * V * 8 + (int64_t)c0 * 8;
-            for (int c = threadIdx.x; c < vw; c += kCompactThreads)
-                rows[(int64_t)a.merged_row * V + c] = sum_partials(pp, a.P, (int64_t)V * 8, c);
+        if (has_merged && a.merged_row >= lo && a.merged_row < lo + R) {
+#pragma unroll
+            for (int ci = 0; ci < MAXC; ++ci) {
+                const int c = ci * kCompactThreads + (int)threadIdx.x;
+                if (c < vw) rows[(int64_t)a.merged_row * V + c] = mrow[ci];
+            }
         }
         put_idx((k + 2) % 3, reg);
         __syncthreads();                              // buffer and index slot are reused in the next round
@@ -209,8 +253,8 @@ lvlm_status launch_inplace_compact(const CompactJob& j, cudaStream_t stream) {
         if (!fin) return LVLM_ERR_INVALID_ARG;
         a.fin_y = 0; a.S = 1; a.G = 1; a.T = 1;
         const int ctas = (j.fin_V + kCompactThreads - 1) / kCompactThreads;
-        return launch_kernel(inplace_compact_kernel<1>, dim3((unsigned)ctas, 1, (unsigned)j.B), dim3(kCompactThreads), 0,
-                             stream, 1, a);
+        return launch_kernel(inplace_compact_kernel<1>, dim3((unsigned)ctas, 1, (unsigned)j.B), dim3(kCompactThreads),
+                             kCompactThreads * 32, stream, 1, a);
     }
     if (!j.src_map || !j.meta || j.B <= 0 || j.G <= 0 || j.V <= 0 || j.N <= 0) return LVLM_ERR_INVALID_ARG;
     if (j.partial && (j.P <= 0 || j.merged_row < 0)) return LVLM_ERR_INVALID_ARG;

@@ -209,3 +209,28 @@ def test_merge_plan_rounds(case, order):
     assert np.array_equal(i32(pd)[0, :src.size], pos[0, src])            # whole numbers and rows that move: nothing to tolerate
     stay = np.arange(src.size) != i0 + k
     assert np.array_equal(f64(out)[0, stay], f64(hid)[0, src[stay]])
+
+
+# the merged rows, from few and from many partial sums of the passes over the rows (1 to 16 threads add up a column group), of
+# narrow rows and of rows wider than a column group per thread
+@pytest.mark.parametrize("case", [        # B, N, i0, n, C, Hkv, k
+    (1, 1000, 2, 900, 64, 1, 300), (1, 2500, 0, 2450, 8192, 1, 1000), (1, 9600, 0, 9500, 1024, 2, 4000), (6, 2100, 5, 2000, 512, 3, 700)])
+@pytest.mark.parametrize("in_place", [False, True])
+def test_merge_partial_sums(case, in_place):
+    B, N, i0, n, C, Hkv, k = case
+    r = np.random.default_rng(N)
+    hid, Kc, Vc = (torch.from_numpy(r.normal(size=s).astype(np.float32)).to(torch.bfloat16)
+                   for s in ((B, N, C), (B, Hkv, N, 128), (B, Hkv, N, 128)))
+    rank = np.stack([r.permutation(n) for _ in range(B)]).astype(np.int32)
+    want = O.merge_compact(f64(hid), rank, i0, n, k, Kc=f64(Kc), Vc=f64(Vc))
+    Kd, Vd, flag = Kc.cuda(), Vc.cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    out, _ = L.merge_compact(hid.cuda(), torch.from_numpy(rank).cuda(), i0=i0, k=k, Kc=Kd, Vc=Vd, in_place=in_place, dev_status=flag)
+    assert flag.item() == 0
+    Nout = L.merged_rows(N, n, k)
+    # a unit in the last place of bf16 (2^-7) where the two sums round apart, and fp32 sums of up to 300 terms in a row, whose
+    # weights add up to one: 300 x 2^-24 x the largest |x| (below 6) < 1.1e-4
+    for got, w, what in ((out[:, None], want["hidden"][:, None], "hidden"), (Kd, want["Kc"], "K"), (Vd, want["Vc"], "V")):
+        got, w = f64(got)[:, :, :Nout], w.astype(np.float64)[:, :, :Nout]
+        assert_rows_close(got[:, :, i0 + k], w[:, :, i0 + k], rtol=2.0 ** -7, atol=1.1e-4, what=what)
+        got[:, :, i0 + k] = w[:, :, i0 + k]
+        assert np.array_equal(got, w), what
