@@ -39,10 +39,18 @@ HiddenGrid hidden_grid(const lvlm_dims* d) {
     g.V = d->C / 8;
     const int rowB = d->C * 2;
     int rpt = kStreamTileBytes / rowB;
-    rpt = rpt < 1 ? 1 : (rpt > 32 ? 32 : rpt);
+    rpt = rpt > 32 ? 32 : rpt;
+    rpt = rpt < 1 ? 1 : rpt;
+    // Short sequences, where that would leave most SMs without rows: two smaller tiles for every SM (a chain of a dozen tiles in a
+    // few CTAs is the time).  us of a merge, 34 KB tiles / this: 640 rows of 2 KB and 8 heads 19.5 / 13.6, 220 rows 19.9 / 11.4;
+    // 1060 rows of 7 KB, where 132 CTAs have rows, 14.2 / 15.1.
+    if ((int64_t)d->N * d->B < (int64_t)148 * rpt) {
+        const int few = (int)(((int64_t)d->N * d->B) / (2 * 148));
+        rpt = few < 1 ? 1 : few;
+    }
     g.rpt = rpt;
     g.slotB = rpt * rowB;
-    if (g.slotB < 16 * kKvRowBytes) g.slotB = 16 * kKvRowBytes;    // room for a tile of K or V rows
+    if (g.slotB < 64 * kKvRowBytes) g.slotB = 64 * kKvRowBytes;    // room for a tile of K or V rows
     g.slotB = (g.slotB + 127) / 128 * 128;
     int ns = kStreamRingBytes / g.slotB;
     g.nstage = ns > kStreamMaxStages ? kStreamMaxStages : ns;
@@ -60,11 +68,12 @@ HiddenGrid hidden_grid(const lvlm_dims* d) {
 }
 
 // Chunks the image span of every K and V sequence is cut into when the merged rows are summed: about four
-// work items per CTA of the sequence's batch element (the CTAs take them in turn), not shorter than 128 rows.
+// work items per CTA of the sequence's batch element (the CTAs take them in turn), not shorter than 128 rows
+// (64, a tile, where that makes an item a CTA at most: 330 rows of 7 KB and 4 heads 13.3 -> 12.5 us; with more items it is slower).
 static int kv_chunks(const lvlm_dims* d, const HiddenGrid& g) {
     if (d->Hkv <= 0) return 1;
     int p = (4 * g.cps + d->Hkv * 2 - 1) / (d->Hkv * 2);
-    const int by_rows = d->n / 128;
+    const int by_rows = d->n / (d->Hkv * 2 * (int64_t)(d->n / 64) <= g.cps ? 64 : 128);
     p = p > by_rows ? by_rows : p;
     p = p < 1 ? 1 : p;
     while (p > 1 && (int64_t)(p - 1) * ((d->n + p - 1) / p) >= d->n) --p;      // no chunk is empty
