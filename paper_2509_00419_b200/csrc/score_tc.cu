@@ -22,7 +22,7 @@
 // a pair of them serves four keys); rows that a query tile does not have.
 // us a call, before -> now: all rows of 8448 x 48 heads, pass 2: 1105 -> 553; 22 layers of 3008 keys x 28 heads x 128 rows,
 // pass 2: 134 -> 91, both: 215 -> 178; 16 sequences of 1888 keys x 32 heads x 96 rows, both: 114 -> 80; 32933 keys x 28 heads
-// x 131 rows, both: 178 -> 101; 640 keys x 8 heads x 64 rows: 12.9 -> 13.0 (start-up and hand-overs).  Of a tile's 1300 to 2000 cycles the special-function unit is busy for 1024; a polynomial on
+// x 131 rows, both: 178 -> 100; 640 keys x 8 heads x 64 rows: 12.9 -> 13.0 (start-up and hand-overs).  Of a tile's 1300 to 2000 cycles the special-function unit is busy for 1024; a polynomial on
 // the FMA pipe for a quarter of the exponentials made it 2 to 6 % slower.
 // Small launches add the parked sums: normalisers (large shape, where items share a query tile's keys), scores.
 #include <type_traits>
@@ -275,21 +275,26 @@ __device__ __forceinline__ float minus_normaliser(const ScoreTcArgs& a, int qt, 
     return -(M + log2f(Ls));
 }
 
-// The (max, sum) of the ksplit items of a query tile, added in key order: minus the normalisers of four rows from `r` on.
+// (max, sum) M, Ls and m, l of two sets of keys added.
+__device__ __forceinline__ void add_stat(float& M, float& Ls, float m, float l) {
+    const float m_new = fmaxf(M, m);
+    if (m_new > -INFINITY) { Ls = Ls * exp2f(M - m_new) + l * exp2f(m - m_new); M = m_new; }
+}
+
+// The (max, sum) of every `step`-th item of a query tile from `first` on, added in key order, for four rows from `r` on.
 // DEEP items' loads are in flight at a time.
 template <int DEEP>
-__device__ __forceinline__ void norm_of_stat(const ScoreTcArgs& a, int64_t tile, int r, float* out) {
+__device__ __forceinline__ void add_stats(const ScoreTcArgs& a, int64_t tile, int r, int first, int step, float* M, float* Ls) {
     const float2* st = a.stat + tile * a.s.ksplit * kTile + r;
-    float M[4], Ls[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) { M[u] = -INFINITY; Ls[u] = 0.f; }
-    for (int k0 = 0; k0 < a.s.ksplit; k0 += DEEP) {
+    for (int k0 = first; k0 < a.s.ksplit; k0 += DEEP * step) {
         float4 v[DEEP][2];
 #pragma unroll
         for (int k = 0; k < DEEP; ++k) {
             v[k][0] = v[k][1] = make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
-            if (k0 + k < a.s.ksplit) {
-                const float4* x = reinterpret_cast<const float4*>(st + (int64_t)(k0 + k) * kTile);
+            if (k0 + k * step < a.s.ksplit) {
+                const float4* x = reinterpret_cast<const float4*>(st + (int64_t)(k0 + k * step) * kTile);
                 v[k][0] = __ldcg(x); v[k][1] = __ldcg(x + 1);
             }
         }
@@ -298,11 +303,17 @@ __device__ __forceinline__ void norm_of_stat(const ScoreTcArgs& a, int64_t tile,
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const float4& x = v[k][u >> 1];
-                const float m = (u & 1) ? x.z : x.x, l = (u & 1) ? x.w : x.y, m_new = fmaxf(M[u], m);
-                if (m_new > -INFINITY) { Ls[u] = Ls[u] * exp2f(M[u] - m_new) + l * exp2f(m - m_new); M[u] = m_new; }
+                add_stat(M[u], Ls[u], (u & 1) ? x.z : x.x, (u & 1) ? x.w : x.y);
             }
         }
     }
+}
+
+// Minus the normalisers of four rows of a query tile from all its items.
+template <int DEEP>
+__device__ __forceinline__ void norm_of_stat(const ScoreTcArgs& a, int64_t tile, int r, float* out) {
+    float M[4], Ls[4];
+    add_stats<DEEP>(a, tile, r, 0, 1, M, Ls);
     const int qt = (int)(tile % a.s.tpg);
 #pragma unroll
     for (int u = 0; u < 4; ++u) out[u] = minus_normaliser(a, qt, r + u, M[u], Ls[u]);
@@ -714,14 +725,37 @@ score_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant_
     }
 }
 
-// Large shape: the normalisers of every query tile, from stat or lse, for the bulk copies of pass 2.  A warp per tile.
-constexpr int kNormThreads = 128;
+// Large shape: the normalisers of every query tile, from stat or lse, for the bulk copies of pass 2.  A warp per tile; where a
+// tile has more items than a warp loads at a time, the four warps of a CTA share it (us of a whole call,
+// one warp / four: 4 heads of 7 x 9000 keys x 64 rows, 18 items, 35.4 / 32.3; 8 of 4 x 20000 x 20, 32 items, 41.0 / 37.6).
+constexpr int kNormThreads = 128, kNormWarps = kNormThreads / 32, kNormDeep = 8;
+template <bool SHARE>
 __global__ void __launch_bounds__(kNormThreads) score_norm_kernel(const ScoreTcArgs a, int tiles) {
+    __shared__ float4 s_m[kNormWarps][32], s_l[kNormWarps][32];
     pdl_enter();
-    const int tile = blockIdx.x * (kNormThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (tile >= tiles) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tile = SHARE ? (int)blockIdx.x : (int)blockIdx.x * kNormWarps + warp;
     float v[4];
-    if (a.from_stat) norm_of_stat<8>(a, tile, lane * 4, v); else norm_of_lse(a, tile, lane * 4, v);
+    if (SHARE) {
+        float M[4], Ls[4];
+        add_stats<kNormDeep>(a, tile, lane * 4, warp, kNormWarps, M, Ls);
+        s_m[warp][lane] = make_float4(M[0], M[1], M[2], M[3]);
+        s_l[warp][lane] = make_float4(Ls[0], Ls[1], Ls[2], Ls[3]);
+        __syncthreads();
+        if (warp > 0) return;
+#pragma unroll
+        for (int q = 1; q < kNormWarps; ++q) {
+            const float4 m = s_m[q][lane], l = s_l[q][lane];
+            add_stat(M[0], Ls[0], m.x, l.x); add_stat(M[1], Ls[1], m.y, l.y);
+            add_stat(M[2], Ls[2], m.z, l.z); add_stat(M[3], Ls[3], m.w, l.w);
+        }
+        const int qt = tile % a.s.tpg;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = minus_normaliser(a, qt, lane * 4 + u, M[u], Ls[u]);
+    } else {
+        if (tile >= tiles) return;
+        if (a.from_stat) norm_of_stat<kNormDeep>(a, tile, lane * 4, v); else norm_of_lse(a, tile, lane * 4, v);
+    }
     reinterpret_cast<float4*>(a.nlse + (int64_t)tile * kTile)[lane] = make_float4(v[0], v[1], v[2], v[3]);
 }
 
@@ -794,8 +828,9 @@ ScoreShape score_shape(const lvlm_dims* d) {
     };
     s.small1 = groups * s.tpg * max_kt <= kSmallTiles1;
     s.small2 = groups * s.nkt * s.tpg <= kSmallTiles2;
-    // (large shape, pass 1: items that share a query tile need a launch that adds their results, about five tiles' time)
-    s.ksplit = s.small1 ? split(s.tpg, max_kt, 16, 2 * kSmCount, 1, 4.0, 0.5, 0.3) : split(s.tpg, max_kt, 32, kSmCount, 2, 1.0, 2.5, 0.05);
+    // (large shape, pass 1: items that share a query tile need a launch that adds their results, about five tiles' time: 16 x 8 heads
+    // of 4 x 1230 keys x 96 rows, whole call, without 59.1 us, with three items a tile 63.4)
+    s.ksplit = s.small1 ? split(s.tpg, max_kt, 16, 2 * kSmCount, 1, 4.0, 0.5, 0.3) : split(s.tpg, max_kt, 32, kSmCount, 2, 1.0, 4.5, 0.02);
     s.parts = s.small2 ? split(s.nkt, s.tpg, 16, 2 * kSmCount, 1, 4.0, 0.0, 0.02) : split(s.nkt, s.tpg, 16, kSmCount, 2, 1.0, 0.0, 0.02);
     return s;
 }
@@ -853,8 +888,10 @@ lvlm_status launch_score_tc(const void* Q, const void* K, const float* lse, cons
     if (r == LVLM_OK && (s.small2 ? a.from_stat && !s.small1 && s.ksplit > 4 : a.from_stat || a.lse)) {
         const int64_t tiles = groups * s.tpg;
         if (tiles > 0x7FFFFFFFll) return LVLM_ERR_UNSUPPORTED;
-        r = launch_kernel(score_norm_kernel, dim3((unsigned)((tiles + kNormThreads / 32 - 1) / (kNormThreads / 32))), dim3(kNormThreads), 0,
-                          stream, 1, a, (int)tiles);
+        r = a.from_stat && s.ksplit > kNormDeep
+                ? launch_kernel(score_norm_kernel<true>, dim3((unsigned)tiles), dim3(kNormThreads), 0, stream, 1, a, (int)tiles)
+                : launch_kernel(score_norm_kernel<false>, dim3((unsigned)((tiles + kNormWarps - 1) / kNormWarps)), dim3(kNormThreads), 0,
+                                stream, 1, a, (int)tiles);
         a.from_stat = 0; a.lse = nullptr;
     }
     if (r != LVLM_OK) return r;

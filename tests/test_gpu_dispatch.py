@@ -65,6 +65,7 @@ def test_decode_in_parts_bad_lengths_are_skipped():
     (1, 1, 1, 130, 0, 1, 1, True, False), (1, 2, 2, 700, 3, 640, 32, True, False), (2, 4, 4, 513, 0, 385, 33, True, True),
     (1, 8, 1, 400, 70, 250, 64, True, False), (1, 14, 2, 1155, 5, 1025, 65, False, False), (1, 28, 4, 3012, 1, 2880, 131, True, False),
     (3, 24, 4, 1300, 0, 1283, 17, True, True), (16, 8, 2, 1500, 0, 1409, 91, True, False), (8, 12, 4, 2100, 0, 2000, 100, True, True),
+    (1, 14, 2, 16000, 7, 15900, 64, True, False),          # more than eight items to a query tile
     (1, 6, 2, 1200, 100, 1000, 1200, True, False), (2, 16, 8, 1409, 0, 1409, 1409, True, False), (1, 5, 1, 900, 0, 900, 900, False, True)])
 def test_score_shapes(case):
     B, H, Hkv, N, i0, n, T, causal, own = case
