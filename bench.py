@@ -345,9 +345,9 @@ class FullPass:
     @property
     def launches(self):
         w = self.w
-        # reduction stages; 2 scoring kernels per compressed layer + plan and compaction; one decode
+        # reduction stages; 3 scoring kernels (at least) per group of compressed layers + plan and compaction; one decode
         # kernel per layer
-        return self.pre.launches + 2 * len(self.groups) + 2 + w.L
+        return self.pre.launches + 3 * len(self.groups) + 2 + w.L
 
 
 def bench_full(w, device, steps, warmup, flush, peaks, phases=True, fence=None):
@@ -792,7 +792,7 @@ def main():
             "bound": "tensor", "unit": "TFLOP/s", "peak": peaks["bf16_tflops"],
             "ms": sum(x["score_ms"] for x in st_all) + res["score_caches_ms"],
             "work": sum(x["score_flops"] for x in st_all) + res["score_caches_flops"],
-            "calls": n_st + res["score_caches_calls"], "launches": 2 * (n_st + res["score_caches_calls"])},
+            "calls": n_st + res["score_caches_calls"], "launches": 3 * (n_st + res["score_caches_calls"])},
         "lvlm_merge_compact": {
             "bound": "hbm", "unit": "GB/s", "peak": peaks["hbm_gbs"],
             "ms": sum(x["merge_compact_ms"] for x in st_all), "work": sum(x["merge_compact_bytes"] for x in st_all),
