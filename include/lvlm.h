@@ -214,7 +214,8 @@ lvlm_status lvlm_merge_compact(void* hidden, void* hidden_out, void* Kc, void* V
  * but at most budget - (entries outside E); drop the rest of E.  Survivors keep their order;
  * K, V, acc_score and pos are compacted in place and len is updated.
  * The count is exact: scores are taken in integer units of 2^-24 and beta in parts per
- * million; beta >= 1 disables the threshold (keep all, subject to the budget).
+ * million; beta >= 1 disables the threshold (keep all, subject to the budget).  Where a head's scores sum to
+ * 2^39 or more the unit is coarser, 2^-47 of the largest score's power of two (the sums are kept in 63 bits).
  *   Kc, Vc     [B][Hkv][cap][D] bf16 in/out        acc_score [B][Hkv][cap] fp32 in/out
  *   pos        optional [B][Hkv][cap] int32 in/out len [B][Hkv] int32 in/out
  *   e_lo,e_hi  optional [B] int32 (both or neither); NULL = every entry is evictable

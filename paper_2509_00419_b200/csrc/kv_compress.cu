@@ -29,10 +29,11 @@ size_t kv_compress_workspace(const lvlm_dims* d) {
     return kv_layout(d, &L) ? L.total : 0;
 }
 
-// Score in integer units of 2^-24 (negative and non-finite scores count as zero).
-__device__ __forceinline__ long long score_units(float s) {
+// Score in integer units of 1 / per_unit, a power of two (negative and non-finite scores count as zero).
+constexpr float kScoreUnits = 16777216.0f;               // units of 2^-24
+__device__ __forceinline__ long long score_units(float s, float per_unit) {
     if (!(s > 0.f) || (__float_as_uint(s) & 0x7F800000u) == 0x7F800000u) return 0;
-    return __float2ll_rn(s * 16777216.0f);               // exact: a power of two (beyond 2^104 both saturate)
+    return __float2ll_rn(s * per_unit);                  // (saturates at 2^63 - 1)
 }
 
 // ceil(beta_ppm * total / 10^6) for beta_ppm < 10^6, total < 2^63: with total = 10^6 q + r it is beta_ppm q + ceil(beta_ppm r / 10^6).
@@ -50,11 +51,25 @@ __device__ __forceinline__ unsigned long long redux_add_u64(unsigned long long v
     return (unsigned long long)l0 + ((unsigned long long)l1 << 22) + ((unsigned long long)l2 << 44);
 }
 
-// The score units behind a key.
-__device__ __forceinline__ unsigned long long units_of_key(uint32_t dk) {
-    if (dk == 0xFFFFFFFFu) return 0ull;
+// The score behind a key, and its units.
+__device__ __forceinline__ float score_of_key(uint32_t dk) {
     const uint32_t asc = ~dk;
-    return score_units(__uint_as_float((asc & 0x80000000u) ? (asc & 0x7FFFFFFFu) : ~asc));
+    return __uint_as_float((asc & 0x80000000u) ? (asc & 0x7FFFFFFFu) : ~asc);
+}
+__device__ __forceinline__ unsigned long long units_of_key(uint32_t dk, float per_unit) {
+    return dk == 0xFFFFFFFFu ? 0ull : (unsigned long long)score_units(score_of_key(dk), per_unit);
+}
+
+// Scores so large that their sum may not fit 63 bits in units of 2^-24 (an entry of 2^49 units or more: 16384 smaller ones
+// always fit).  A sum that wraps around would name a threshold that the entries do not reach, and survivors that
+// are not there.  lo, hi: the sums of the low and of the high words of the units; if the whole sum does not fit, the unit
+// is taken coarser, so that an entry has at most 2^48 of them.  best: the key of the largest finite score.
+constexpr int kBigUnits = 49;
+constexpr uint32_t kKeyOfInfinity = 0x007FFFFFu;         // the smallest key
+__device__ __forceinline__ float units_that_fit(unsigned long long lo, unsigned long long hi, uint32_t best) {
+    if (hi + (lo >> 32) < (1ull << 31)) return kScoreUnits;
+    const uint32_t e = __float_as_uint(score_of_key(best)) >> 23;            // 127 + exponent, at least 25
+    return __uint_as_float((127u + 47u - (e - 127u)) << 23);
 }
 
 // One CTA per (sequence, KV head).  A warp has 32 * KPT consecutive evictable entries, lane l of it l, l + 32, ..., as 32-bit
@@ -77,7 +92,7 @@ kv_plan_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t* __re
                int32_t* __restrict__ pos_new, int32_t* dev_status) {
     __shared__ __align__(16) uint32_t s_hist[kPlanLimbs][kPlanHist];
     __shared__ unsigned long long s_sum[32], s_before;
-    __shared__ uint32_t s_and[32], s_or[32], s_digit;
+    __shared__ uint32_t s_and[32], s_or[32], s_big[32], s_digit;
     __shared__ int s_first_drop;
 
     pdl_enter();
@@ -117,7 +132,7 @@ kv_plan_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t* __re
     uint32_t key[KPT];
     unsigned long long un[KPT];                          // the scores in integer units
     bool nonfinite = false;
-    uint32_t k_and = ~0u, k_or = 0u;
+    uint32_t k_and = ~0u, k_or = 0u, big = 0u;
 #pragma unroll
     for (int u = 0; u < KPT; ++u) sv[u] = j0 + 32 * u < m ? acc[lo + j0 + 32 * u] : 0.f;
 #pragma unroll
@@ -127,16 +142,19 @@ kv_plan_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t* __re
         if (j0 + 32 * u < m) {
             key[u] = desc_key(sv[u], &nonfinite);
             k_and &= key[u]; k_or |= key[u];
-            un[u] = (unsigned long long)score_units(sv[u]);
+            un[u] = (unsigned long long)score_units(sv[u], kScoreUnits);
+            big |= (uint32_t)(un[u] >> kBigUnits);
         }
     }
     if (nonfinite && dev_status) atomicOr(dev_status, LVLM_DEV_NONFINITE);
     k_and = __reduce_and_sync(0xFFFFFFFFu, k_and);       // bits in which the keys differ
     k_or = __reduce_or_sync(0xFFFFFFFFu, k_or);
-    if (lane == 0) { s_and[warp] = k_and; s_or[warp] = k_or; }
+    big = __reduce_or_sync(0xFFFFFFFFu, big);
+    if (lane == 0) { s_and[warp] = k_and; s_or[warp] = k_or; s_big[warp] = big; }
     sync_active();
     k_and = __reduce_and_sync(0xFFFFFFFFu, lane < nwarp ? s_and[lane] : ~0u);
     k_or = __reduce_or_sync(0xFFFFFFFFu, lane < nwarp ? s_or[lane] : 0u);
+    big = __reduce_or_sync(0xFFFFFFFFu, lane < nwarp ? s_big[lane] : 0u);
     const uint32_t diff = m > 0 ? (k_and ^ k_or) : 0u;
 
     // Exclusive prefix sum over the block's threads, in thread order, and the total.
@@ -223,6 +241,25 @@ kv_plan_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t* __re
     unsigned long long before = 0ull;
     if (beta_ppm < 1000000ull && m > 0) {
         unsigned long long mine = 0ull, total;
+        float per_unit = kScoreUnits;
+        if (big) {
+            unsigned long long lo_w = 0ull, hi_w = 0ull;
+            uint32_t best = ~0u;
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) {
+                lo_w += un[u] & 0xFFFFFFFFull;
+                hi_w += un[u] >> 32;
+                if (un[u]) best = min(best, key[u]);
+            }
+            block_scan(lo_w, &lo_w);
+            block_scan(hi_w, &hi_w);
+            best = __reduce_min_sync(0xFFFFFFFFu, best);
+            if (lane == 0) s_big[warp] = best;           // (the flags were read before the scans)
+            sync_active();
+            per_unit = units_that_fit(lo_w, hi_w, __reduce_min_sync(0xFFFFFFFFu, lane < nwarp ? s_big[lane] : ~0u));
+#pragma unroll
+            for (int u = 0; u < KPT; ++u) un[u] = un[u] ? units_of_key(key[u], per_unit) : 0ull;
+        }
 #pragma unroll
         for (int u = 0; u < KPT; ++u) mine += un[u];
         block_scan(mine, &total);
@@ -231,7 +268,7 @@ kv_plan_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t* __re
         else {
             const int limbs = min(kPlanLimbs, (63 - __clzll((long long)total)) / kPlanLimb + 1);     // (no entry holds more than all)
             T = search(thr, true, limbs, &before);
-            const unsigned long long each = units_of_key(T);             // > 0: the entries of key T are needed
+            const unsigned long long each = units_of_key(T, per_unit);   // > 0: the entries of key T are needed
             need = (int)((thr - before + each - 1ull) / each);
             have_T = true;
         }
@@ -379,6 +416,7 @@ kv_plan_warp_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t*
         k_or |= __shfl_xor_sync(0xFFFFFFFFu, k_or, o);
     }
     const uint32_t diff = m > 0 ? (k_and ^ k_or) : 0u;
+    float per_unit = kScoreUnits;
     // Score units of the entries with key <= cand (or < cand), summed over the warp.
     auto mass_upto = [&](uint32_t cand, bool strict) -> unsigned long long {
         unsigned long long ms = 0;
@@ -386,7 +424,7 @@ kv_plan_warp_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t*
         for (int u = 0; u < KPL; ++u) {
             uint32_t h = hk[u];
             if (KPL > 32) asm volatile("" : "+r"(h));    // worked out again at every use: 64 more registers would not fit
-            if (strict ? h < cand : h <= cand) ms += units_of_key(h);
+            if (strict ? h < cand : h <= cand) ms += units_of_key(h, per_unit);
         }
         return redux_add_u64(ms);
     };
@@ -426,6 +464,20 @@ kv_plan_warp_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t*
     int need = 0;
     bool have_T = false;
     if (MASS && m > 0) {
+        uint32_t best = ~0u;                             // the largest finite score
+#pragma unroll
+        for (int u = 0; u < KPL; ++u) if (hk[u] > kKeyOfInfinity) best = min(best, hk[u]);
+        best = __reduce_min_sync(0xFFFFFFFFu, best);
+        if (units_of_key(best, kScoreUnits) >> kBigUnits) {
+            unsigned long long lo_w = 0ull, hi_w = 0ull;
+#pragma unroll 1
+            for (int j = lane; j < KPL * 32; j += 32) {                      // (the keys are in shared memory still)
+                const unsigned long long x = units_of_key(my_hk[j], kScoreUnits);
+                lo_w += x & 0xFFFFFFFFull;
+                hi_w += x >> 32;
+            }
+            per_unit = units_that_fit(redux_add_u64(lo_w), redux_add_u64(hi_w), best);
+        }
         const unsigned long long total = mass_upto(~0u, false);
         const unsigned long long thr = beta_of_total(beta_ppm, total);
         if (thr == 0) k_beta = 1;
@@ -433,7 +485,7 @@ kv_plan_warp_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t*
             T = search(thr, false);
             const int c = count_below(T);
             const unsigned long long below = mass_upto(T, true);
-            const unsigned long long each = units_of_key(T);                 // > 0: the entries of key T are needed
+            const unsigned long long each = units_of_key(T, per_unit);       // > 0: the entries of key T are needed
             need = (int)((thr - below + each - 1ull) / each);
             k_beta = c + need;
             have_T = true;

@@ -171,6 +171,29 @@ def test_kv_threshold_search(cap, kind):
             assert np.array_equal(f64(Kd)[0, g, :m], want["Kc"][0, g, :m].astype(np.float64)), (beta, budget, g)
 
 
+# the same, scores whose sum in units of 2^-24 needs up to 63 bits, or more: whole multiples of one power of two, so that a coarser
+# unit counts them exactly as well; a CTA per head (few heads) and a warp per head
+@pytest.mark.parametrize("heads,cap", [(2, 7), (3, 1000), (2, 4100), (592, 33)])
+@pytest.mark.parametrize("exponent", [24, 29, 39, 90, 117])
+def test_kv_threshold_of_huge_scores(heads, cap, exponent):
+    r = np.random.default_rng(cap + exponent)
+    acc = (r.integers(0, 1000, size=(1, heads, cap)) * 2.0 ** exponent).astype(np.float32)
+    acc[0, 0] = 2.0 ** exponent                                          # all alike
+    acc[0, 1, cap // 2] = np.inf
+    ln = np.full((1, heads), cap, np.int32)
+    Kc = torch.from_numpy(r.normal(size=(1, heads, cap, 128)).astype(np.float32)).to(torch.bfloat16)
+    for beta in (0.5, 0.97):
+        want = O.kv_compress(f64(Kc), f64(Kc), acc, ln, beta=beta)
+        Kd, Vd, ad, ld = Kc.cuda(), Kc.cuda(), torch.from_numpy(acc).cuda(), torch.from_numpy(ln).cuda()
+        flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+        L.kv_compress(Kd, Vd, ad, ld, beta=beta, dev_status=flag)
+        assert flag.item() == L.DEV_NONFINITE and np.array_equal(i32(ld), want["len"]), beta
+        for g in range(0, heads, max(1, heads // 16)):
+            m = want["len"][0, g]
+            assert np.array_equal(ad[0, g, :m].cpu().numpy(), want["acc_score"][0, g, :m]), (beta, g)
+            assert np.array_equal(f64(Kd)[0, g, :m], want["Kc"][0, g, :m].astype(np.float64)), (beta, g)
+
+
 # selection by bins: 1, 2, 4 and 8 slices, 1, 2 and 4 tokens a thread, last slices that are shorter; bins as deep as they may be
 # and one key deeper, one bin for all but one key, one value
 @pytest.mark.parametrize("B,n", [(1, 511), (1, 512), (1, 1023), (1, 1025), (1, 2049), (1, 14337), (2, 34817), (37, 3001), (140, 1100)])
