@@ -151,7 +151,8 @@ lvlm_status lvlm_score_tokens(const void* Q, const void* K, const float* lse,
  * Reads d: B,H,Hkv,D,N,cap,causal,q_stride_*,kv_stride_*, and with score also i0,n,q_lo,q_hi,head_stride.
  * Errors: INVALID_ARG (NULL Q/K/V/out/lse, N>cap, H%Hkv, scale<=0, score_head without score, a bad window),
  * UNSUPPORTED (D!=128), ALIGNMENT, WORKSPACE.  Contents of the outputs are undefined when a kernel gave up
- * on a wait and set LVLM_DEV_TIMEOUT (the same holds for lvlm_score_tokens and lvlm_merge_compact).
+ * on a wait and set LVLM_DEV_TIMEOUT (the same holds for lvlm_score_tokens, lvlm_merge_compact and out and acc_score
+ * of lvlm_decode_attn, whose appended row and len are as without the timeout).
  */
 lvlm_status lvlm_prefill_attn(const void* Q, const void* K, const void* V, const lvlm_dims* d, float scale,
                               void* out, float* lse, float* score, float* score_head,

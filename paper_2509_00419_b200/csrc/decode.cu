@@ -173,7 +173,18 @@ struct DecodeArgs {
     int32_t* part_len;
     float* ws_s;             // [B*H][cap] scaled logits (log2 domain), only with acc_score and a long run
     int32_t* dev_status;
+#ifdef LVLM_TEST_HOOKS
+    int starve;
+#endif
 };
+
+// The test build can keep the producer from fetching anything, so that the waits for the stages run out.
+#ifdef LVLM_TEST_HOOKS
+static int g_decode_starve = 0;
+__device__ __forceinline__ bool starved(const DecodeArgs& a) { return a.starve != 0; }
+#else
+__device__ __forceinline__ bool starved(const DecodeArgs&) { return false; }
+#endif
 
 // Offset inside a stage of the 16-byte chunk `ch` (0..15) of key row `r` (0..63): K or V half boxes of 64
 // channels, rows of 128 bytes, chunks XOR-swizzled with the row as the TMA copy wrote them.
@@ -263,8 +274,11 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     // the warp of this CTA whose tile takes the appended row, or -1
     const int app_warp = app && ln / kTileKeys >= t_lo && ln / kTileKeys < t_hi ? (ln / kTileKeys - t_lo) % kDecWarps : -1;
     auto store_appended = [&]() {
-        if (warp == app_warp)
-            *reinterpret_cast<uint4*>((lane < 16 ? a.Kc : a.Vc) + (int64_t)b * a.kv_sb + (int64_t)g * a.kv_sh + (int64_t)ln * kHeadDim + (lane & 15) * 8) = s_app[lane];
+        if (warp != app_warp) return;
+        // (a warp whose wait has given up comes here without having patched its tile: the copy of the row is waited for here too,
+        // so that the cache never takes a row that has not landed)
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        *reinterpret_cast<uint4*>((lane < 16 ? a.Kc : a.Vc) + (int64_t)b * a.kv_sb + (int64_t)g * a.kv_sh + (int64_t)ln * kHeadDim + (lane & 15) * 8) = s_app[lane];
     };
 
     if (warp == kDecWarps) {
@@ -278,11 +292,11 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
             tma_load_4d(st + 2 * kBoxBytes, &vmap, &s_full[s % kStagesDec], 0, j0, g, b);
             tma_load_4d(st + 3 * kBoxBytes, &vmap, &s_full[s % kStagesDec], 64, j0, g, b);
         };
-        if (lane == 0) {
+        if (lane == 0 && !starved(a)) {
             for (int s = 0; s < kStagesDec && s < nstage; ++s) issue(s);
         }
         if (a.early) pdl_enter();
-        if (lane == 0) {
+        if (lane == 0 && !starved(a)) {
             for (int s = kStagesDec; s < nstage; ++s) {
                 if (!wait_on(&s_empty[s % kStagesDec], (uint32_t)(s / kStagesDec - 1) & 1u)) break;
                 issue(s);
@@ -684,7 +698,9 @@ static lvlm_status launch_decode(const void* q, void* Kc, void* Vc, int32_t* len
     a.ws_s = acc_score ? reinterpret_cast<float*>(wsb + L.off_s) : nullptr;
     a.logit_keys = logit_keys;
     a.dev_status = dev_status;
-
+#ifdef LVLM_TEST_HOOKS
+    a.starve = g_decode_starve;
+#endif
     a.part_ml = reinterpret_cast<float2*>(wsb + L.off_ml);
     a.part_o = reinterpret_cast<float*>(wsb + L.off_o);
     a.part_len = reinterpret_cast<int32_t*>(wsb + L.off_len);
@@ -724,6 +740,10 @@ static lvlm_status decode_attn(const void* q, void* Kc, void* Vc, int32_t* len, 
 }
 
 }  // namespace lvlm
+
+#ifdef LVLM_TEST_HOOKS
+extern "C" void lvlm_debug_starve_decode(int on) { lvlm::g_decode_starve = on ? 1 : 0; }
+#endif
 
 extern "C" lvlm_status lvlm_decode_attn(const void* q, void* Kc, void* Vc, int32_t* len,
                                          const void* k_new, const void* v_new, float* acc_score,

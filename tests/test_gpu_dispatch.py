@@ -6,6 +6,7 @@ import torch
 
 from oracle import lvlm_oracle as O
 from paper_2509_00419_b200 import binding as L
+from paper_2509_00419_b200 import build as BU
 from tests.util import assert_rows_close, assert_scores_close, f64, i32
 
 pytestmark = pytest.mark.gpu
@@ -57,6 +58,29 @@ def test_decode_in_parts_bad_lengths_are_skipped():
     assert flag.item() == L.DEV_BOUNDS and ln.tolist() == [[cap + 1, -1, cap, 701]]
     assert not out[0, :2].any() and not acc[0, :2].any()
     assert abs(acc[0, 2].sum().item() - 1) < 1e-4 and abs(acc[0, 3, :701].sum().item() - 1) < 1e-4 and not acc[0, 3, 701:].any()
+
+
+# waits that run out (the test build fetches no stage): the call ends and says so, and the appended row and the length are what they
+# are without a timeout, in all three forms (one CTA, a cluster, parts)
+@pytest.mark.parametrize("B,H,Hkv,cap", [(40, 32, 8, 100), (1, 8, 2, 150), (1, 4, 4, 4200)])
+def test_decode_timeout_keeps_the_appended_row(B, H, Hkv, cap):
+    q, kn, vn = (torch.randn(B, h, 128, device="cuda").to(torch.bfloat16) for h in (H, Hkv, Hkv))
+    Kc, Vc = torch.zeros(B, Hkv, cap, 128, device="cuda", dtype=torch.bfloat16), torch.zeros(B, Hkv, cap, 128, device="cuda", dtype=torch.bfloat16)
+    ln = (torch.arange(B * Hkv, device="cuda", dtype=torch.int32) * 37 % 97).view(B, Hkv).contiguous()
+    want, at = ln + 1, ln.long()[..., None, None].expand(B, Hkv, 1, 128)
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    try:
+        L.use_library(BU.build_test())
+        L.lib().lvlm_debug_starve_decode(1)
+        L.decode_attn(q, Kc, Vc, ln, k_new=kn, v_new=vn, dev_status=flag)
+        torch.cuda.synchronize()
+        L.lib().lvlm_debug_starve_decode(0)
+    finally:
+        L.use_library(None)
+    assert flag.item() == L.DEV_TIMEOUT and torch.equal(ln, want)
+    for cache, row in ((Kc, kn), (Vc, vn)):
+        assert torch.equal(cache.gather(2, at)[:, :, 0], row)
+        assert (cache != 0).any(dim=3).sum(dim=2).eq(1).all()                  # and no other row
 
 
 # scoring: few and many tiles (small and large shape of the kernel), heads of a group in one query tile or one each, windows
