@@ -41,7 +41,8 @@ constexpr int kATile = 2 * kAHalf;           // 32 KB
 constexpr int kAStages = 2;                  // K ring and V ring (released separately: K after S, V after O)
 constexpr int kAThreads = 128 + 2 * kAT;     // warp 0 TMA, warp 1 MMA, (2, 3 idle,) four softmax warps for each of the two tiles
 // A softmax thread holds a row of 128 logits: the first warpgroup hands registers over to the other two.  Launched with
-// 168 a thread (65536 / 384, rounded down to 8): 3 * 168 = 104 + 2 * 200.
+// 168 a thread (65536 / 384, rounded down to 8): 3 * 168 = 104 + 2 * 200.  What the kernel is launched with is the compiler's
+// choice; with less, the two would wait for registers that nobody has, so a call looks it up first (attn_registers_fit).
 constexpr int kARegsLaunch = 168, kARegsFew = 104, kARegsMany = 200;
 static_assert(3 * kARegsLaunch >= kARegsFew + 2 * kARegsMany, "the split has to fit the registers the block is launched with");
 constexpr uint32_t kATmemCols = 512;         // S/P of the two tiles | O of the two tiles
@@ -466,12 +467,31 @@ static bool attn_split(int64_t tiles, int64_t pairs, double heads, int nqt, int 
     return estimate((double)tiles, 0.5 * nqt, 3.0) < estimate((double)pairs, nqt, 3.5);
 }
 
+#ifdef LVLM_TEST_HOOKS
+static int g_attn_regs = 0;                  // the test build's idea of the registers a thread, 0 = the kernel's own
+#endif
+
+// The registers that the kernel is launched with cover the split of its warpgroups.
+static lvlm_status attn_registers_fit() {
+    cudaFuncAttributes f;
+    LVLM_RETURN_IF_CUDA(cudaFuncGetAttributes(&f, prefill_attn_kernel));
+    int regs = f.numRegs;
+#ifdef LVLM_TEST_HOOKS
+    if (g_attn_regs) regs = g_attn_regs;
+#endif
+    return 3 * regs >= kARegsFew + 2 * kARegsMany ? LVLM_OK : LVLM_ERR_CUDA;
+}
+
 size_t prefill_attn_workspace(const lvlm_dims* d) {
     ScoreLayout L;
     return score_layout(d, &L) ? L.total : 0;
 }
 
 }  // namespace lvlm
+
+#ifdef LVLM_TEST_HOOKS
+extern "C" void lvlm_debug_set_attn_regs(int n) { lvlm::g_attn_regs = n; }
+#endif
 
 extern "C" lvlm_status lvlm_prefill_attn(const void* Q, const void* K, const void* V, const lvlm_dims* d,
                                           float scale, void* out, float* lse, float* score, float* score_head,
@@ -523,6 +543,8 @@ extern "C" lvlm_status lvlm_prefill_attn(const void* Q, const void* K, const voi
     a.dev_status = dev_status;
     const size_t smem = 1024 + (size_t)kATile * (2 + 2 * kAStages) + sizeof(AttnSmem);
     LVLM_RETURN_IF_CUDA(cudaFuncSetAttribute(prefill_attn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const lvlm_status fits = attn_registers_fit();
+    if (fits != LVLM_OK) return fits;
     const int nqt = (d->N + kAT - 1) / kAT;
     const int64_t groups = (int64_t)d->B * d->Hkv, tiles = (int64_t)d->B * d->H * nqt;
     a.nqt = nqt;

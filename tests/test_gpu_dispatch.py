@@ -139,6 +139,25 @@ def test_attention_shapes(case):
     np.testing.assert_allclose(f64(lse), f64(torch.logsumexp(logits, dim=-1)), rtol=1e-5, atol=1e-5)   # fp32 sums
 
 
+# the warpgroups' registers are shared out anew inside the kernel: launched with too few it would wait for ever, so it is not launched
+def test_attention_refuses_too_few_registers():
+    Q, K = torch.randn(1, 200, 2, 128, device="cuda").bfloat16(), torch.randn(1, 1, 200, 128, device="cuda").bfloat16()
+    out, lse = torch.full_like(Q, 9.0), torch.empty(1, 2, 200, device="cuda")
+    try:
+        L.use_library(BU.build_test())
+        L.lib().lvlm_debug_set_attn_regs(160)
+        with pytest.raises(L.LvlmError) as e:
+            L.prefill_attn(Q, K, K, N=200, out=out, lse=lse)
+        torch.cuda.synchronize()
+        assert e.value.code == L.ERR_CUDA and out.eq(9).all()
+        L.lib().lvlm_debug_set_attn_regs(168)                # ... 3 x 168 = 104 + 2 x 200
+        L.prefill_attn(Q, K, K, N=200, out=out, lse=lse)
+        assert not out.eq(9).any()
+    finally:
+        L.lib().lvlm_debug_set_attn_regs(0)
+        L.use_library(None)
+
+
 # nearest-kept grouping: every dropped token to one kept token (one long segment), segments around a warp's 32 tokens, none
 # at all for most; text rows that are the source of rows before them; runs over several CTAs of the plan's cluster
 @pytest.mark.parametrize("case", [        # B, C, Hkv, i0, n, T, k, kept tokens that attract the dropped ones
