@@ -15,12 +15,12 @@ bool score_layout(const lvlm_dims* d, ScoreLayout* L) {
     const ScoreShape s = L->shape = score_shape(d);
     const size_t groups = (size_t)d->B * d->Hkv;
     size_t off = 0;
-    // (at least a row of n floats per query head: what callers have been asked for, whatever the split)
-    const size_t rows = groups * s.parts * s.nkt * 128, promised = (size_t)d->B * d->H * d->n;
-    L->off_partial = off; off = align_up(off + (rows > promised ? rows : promised) * 4, 256);
+    // (never less for a larger problem; at least a row of n floats per query head: what callers have been asked for)
+    const size_t sums = (size_t)s.part_tiles * 128, promised = (size_t)d->B * d->H * d->n;
+    L->off_partial = off; off = align_up(off + (sums > promised ? sums : promised) * 4, 256);
     L->off_lse = off;     off = align_up(off + (size_t)d->B * d->H * (d->q_hi - d->q_lo) * 4, 256);
     L->off_nlse = off;    off = align_up(off + groups * s.tpg * 128 * 4, 256);
-    L->off_stat = off;    off = align_up(off + (s.ksplit > 1 ? groups * s.tpg * s.ksplit * 128 * 8 : 0), 256);
+    L->off_stat = off;    off = align_up(off + (size_t)s.stat_tiles * 128 * 8, 256);
     L->total = off;
     return true;
 }

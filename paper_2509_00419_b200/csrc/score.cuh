@@ -13,6 +13,7 @@ struct ScoreShape {
     bool small1, small2;       // which shape of the kernel runs the passes
     int ksplit;                // pass 1: work items that share the keys of a query tile
     int parts;                 // pass 2: work items that share the query tiles of a key tile and KV group
+    int64_t part_tiles, stat_tiles;    // tiles of results the workspace has room for: pass 2 (column sums), pass 1 (max, sum)
 };
 
 struct ScoreLayout { ScoreShape shape; size_t off_partial, off_lse, off_nlse, off_stat, total; };

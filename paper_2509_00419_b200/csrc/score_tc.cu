@@ -68,6 +68,10 @@ constexpr int kFirstEpiWarp = 4;
 // call: 672 tiles (4 KV heads of 7, 3008 keys, 128 rows) 27.2 / 28.7, 924 32.0 / 35.5, 512 26.2 / 29.8, 476 25.1 / 25.3, 256
 // 27.7 / 20.5, 40 13.9 / 13.0; pass 2: 1136 tiles 16.9 / 16.4, 896 14.8 / 14.4, 512 14.9 / 12.8, 40 11.8 / 8.2.
 constexpr int64_t kSmallTiles1 = 148 * 3, kSmallTiles2 = 148 * 8;
+// Most parts of an item, and tiles of 128 results of them in the workspace: 4 MB either way.  The second figures bind where
+// there are thousands of items anyhow (an 8 x 48-head window of 5000 rows: five parts instead of six).
+constexpr int kMaxSplit = 32, kMaxParts = 16;
+constexpr int64_t kMaxStatTiles = 4096, kMaxPartTiles = 8192;
 constexpr float kLog2eT = 1.4426950408889634f;
 
 // n / d for 0 <= n < 2^31 by a multiplication: every warp of a CTA takes every work item apart.
@@ -828,10 +832,21 @@ ScoreShape score_shape(const lvlm_dims* d) {
     };
     s.small1 = groups * s.tpg * max_kt <= kSmallTiles1;
     s.small2 = groups * s.nkt * s.tpg <= kSmallTiles2;
+    // Tiles of results in the workspace.  The splits rise and fall with the size, the workspace may not (a program sizes it
+    // once, for its longest prompt and widest batch): it has room for any split up to a limit on the tiles, beyond that
+    // for the results without one, and the splits keep to it.
+    const int64_t key_tiles = groups * s.nkt, query_tiles = groups * s.tpg, per_head = (int64_t)d->B * d->H * d->n / kTile;
+    const int64_t no_split = key_tiles > kMaxPartTiles ? key_tiles : kMaxPartTiles, any_part = key_tiles * (s.tpg < kMaxParts ? s.tpg : kMaxParts);
+    const int64_t any_split = query_tiles * (max_kt < kMaxSplit ? max_kt : kMaxSplit);
+    s.part_tiles = any_part < no_split ? any_part : no_split;
+    s.stat_tiles = any_split < kMaxStatTiles ? any_split : kMaxStatTiles;
+    const int most1 = (int)(s.stat_tiles / query_tiles), most2 = (int)((s.part_tiles > per_head ? s.part_tiles : per_head) / key_tiles);
     // (large shape, pass 1: items that share a query tile need a launch that adds their results, about five tiles' time: 16 x 8 heads
     // of 4 x 1230 keys x 96 rows, whole call, without 59.1 us, with three items a tile 63.4)
-    s.ksplit = s.small1 ? split(s.tpg, max_kt, 16, 2 * kSmCount, 1, 4.0, 0.5, 0.3) : split(s.tpg, max_kt, 32, kSmCount, 2, 1.0, 4.5, 0.02);
-    s.parts = s.small2 ? split(s.nkt, s.tpg, 16, 2 * kSmCount, 1, 4.0, 0.0, 0.02) : split(s.nkt, s.tpg, 16, kSmCount, 2, 1.0, 0.0, 0.02);
+    s.ksplit = s.small1 ? split(s.tpg, max_kt, most1 < 16 ? most1 : 16, 2 * kSmCount, 1, 4.0, 0.5, 0.3)
+                        : split(s.tpg, max_kt, most1 < kMaxSplit ? most1 : kMaxSplit, kSmCount, 2, 1.0, 4.5, 0.02);
+    s.parts = split(s.nkt, s.tpg, most2 < kMaxParts ? most2 : kMaxParts, s.small2 ? 2 * kSmCount : kSmCount, s.small2 ? 1 : 2,
+                    s.small2 ? 4.0 : 1.0, 0.0, 0.02);
     return s;
 }
 

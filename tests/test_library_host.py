@@ -50,6 +50,26 @@ def test_workspace_sizes(lib):
     assert L.workspace_bytes(L.OP_SCORE_TOKENS, d) >= 16 * 32 * 1792 * 4
 
 
+# a program sizes a workspace once, for its widest batch, longest prompt and window: nothing smaller may ask for more
+@pytest.mark.parametrize("op", [L.OP_SCORE_TOKENS, L.OP_PREFILL_ATTN])
+@pytest.mark.parametrize("heads", [(1024, 8, 8), (3584, 28, 4), (4096, 32, 8), (64, 1, 1)])
+def test_workspace_never_shrinks(lib, op, heads):
+    C, H, Hkv = heads
+
+    def size(B, n, T):
+        return L.workspace_bytes(op, L.Dims(B=B, H=H, Hkv=Hkv, D=128, N=n + T, C=C, cap=n + T, n=n, k=n // 2 or 1, q_lo=n,
+                                            q_hi=n + T, causal=1))
+
+    Bs = [1, 2, 3, 4, 5, 7, 8, 9, 10, 16, 32, 74, 75, 149]
+    ns = list(range(1, 1400, 37)) + [2515, 2516, 3072, 3136, 4000, 8000, 10752, 10816, 16000, 32767, 60000]
+    Ts = [1, 17, 64, 127, 128, 129, 300, 1000, 5000]
+    for line in ([[(B, n, T) for n in ns] for B in (1, 4, 16) for T in Ts] + [[(B, n, T) for B in Bs] for n in ns for T in (17, 128)] +
+                 [[(B, n, T) for T in Ts] for B in (1, 4, 16) for n in ns]):
+        sizes = [size(*x) for x in line]
+        for i in range(1, len(line)):
+            assert sizes[i] >= sizes[i - 1], (line[i - 1], line[i])
+
+
 def test_bad_arguments_are_rejected_on_the_host(lib):
     p = ctypes.c_void_p(0x1000)           # never dereferenced: every call below fails validation
     odd = ctypes.c_void_p(0x1008)
