@@ -255,7 +255,8 @@ lvlm_status lvlm_kv_compress(void* Kc, void* Vc, float* acc_score, int32_t* pos,
  * Workspace: used when acc_score is given and the cache is so long that the scaled logits of a CTA's
  * own keys do not fit in its shared memory (they are then parked there between the pass over the keys and
  * the update of acc_score), and for the partial results where few heads with long caches are cut into parts
- * (two launches then); its contents need not be zeroed.
+ * (two launches then); its contents need not be zeroed.  B * H * cap * 4 bytes (rounded up to 256) are needed; with less than
+ * lvlm_workspace_bytes no head is cut.
  * Reads d: B,H,Hkv,D,cap,kv_stride_*.
  * Errors: INVALID_ARG, UNSUPPORTED (D!=128, H/Hkv > 8), ALIGNMENT, WORKSPACE.
  */

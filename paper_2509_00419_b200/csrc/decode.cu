@@ -56,7 +56,9 @@ constexpr int kDecLogitBytes = 12 * 1024;            // scaled logits of a CTA's
 constexpr float kLog2e = 1.4426950408889634f;
 
 // S CTAs a head form a cluster; P > 0: as many independent CTAs a head whose results a second launch adds.
-struct DecodeLayout { int S, P; size_t off_s, off_ml, off_o, off_len, total; };
+// Bytes of workspace: `logits` always, `used` by the form taken, `total` what a caller is told: room for the parts of any number of
+// heads, so that it never shrinks as the problem grows.
+struct DecodeLayout { int S, P; size_t off_s, off_ml, off_o, off_len, logits, used, total; };
 
 // Rows of a cache, in tiles, from which the parts are the faster form where a cluster of 8 a head leaves SMs idle (the
 // lengths are only known on the device).  us per layer as cluster / as parts, inside a chain of layers:
@@ -74,7 +76,7 @@ static int parts_from_tiles(int64_t heads, bool acc) {
     return heads <= 4 ? 64 : heads <= 8 ? 192 : heads <= 20 ? 320 : 800;
 }
 
-// may_split: the caller's workspace has room for the parts (lvlm_decode_attn_static's may not).
+// may_split: the caller's workspace has room for the parts.
 static bool decode_layout(const lvlm_dims* d, DecodeLayout* L, bool may_split = true) {
     if (!d || d->B <= 0 || d->H <= 0 || d->Hkv <= 0 || d->H % d->Hkv || d->cap <= 0) return false;
     // cluster size: the power of two that brings the grid closest to the target without going
@@ -92,13 +94,18 @@ static bool decode_layout(const lvlm_dims* d, DecodeLayout* L, bool may_split = 
     }
     size_t off = 0;
     L->off_s = off; off = align_up(off + (size_t)d->B * d->H * d->cap * 4, 256);
-    L->off_ml = L->off_o = L->off_len = off;
+    L->logits = L->off_ml = L->off_o = L->off_len = off;
     if (L->P > 0) {
         L->off_ml = off;  off = align_up(off + (size_t)d->B * d->H * L->P * 8, 256);
         L->off_o = off;   off = align_up(off + (size_t)d->B * d->H * L->P * kHeadDim * 4, 256);
         L->off_len = off; off = align_up(off + (size_t)heads * 4, 256);
     }
-    L->total = off;
+    L->used = off;
+    // (heads * P <= kDecTargetCtas; shorter caches are never cut)
+    const size_t part_rows = (size_t)(d->H / d->Hkv) * kDecTargetCtas;
+    L->total = L->logits;
+    if (tiles >= kDecMaxCluster * kDecMinTiles)
+        L->total += align_up(part_rows * 8, 256) + align_up(part_rows * kHeadDim * 4, 256) + align_up((size_t)heads * 4, 256);
     return true;
 }
 
@@ -715,9 +722,10 @@ static lvlm_status launch_decode(const void* q, void* Kc, void* Vc, int32_t* len
 }
 
 static lvlm_status decode_attn(const void* q, void* Kc, void* Vc, int32_t* len, const void* k_new, const void* v_new,
-                               float* acc_score, const lvlm_dims* d, const DecodeLayout& L, float scale, void* out,
-                               void* ws, size_t ws_bytes, int32_t* dev_status, cudaStream_t stream) {
-    if (!q || !Kc || !Vc || !len || !out) return LVLM_ERR_INVALID_ARG;
+                               float* acc_score, const lvlm_dims* d, float scale, void* out, void* ws, size_t ws_bytes,
+                               int32_t* dev_status, cudaStream_t stream) {
+    DecodeLayout L;
+    if (!q || !Kc || !Vc || !len || !out || !decode_layout(d, &L)) return LVLM_ERR_INVALID_ARG;
     if ((k_new == nullptr) != (v_new == nullptr)) return LVLM_ERR_INVALID_ARG;
     const int G = d->H / d->Hkv;
     if (d->D != kHeadDim || G > kMaxGroup) return LVLM_ERR_UNSUPPORTED;
@@ -726,7 +734,8 @@ static lvlm_status decode_attn(const void* q, void* Kc, void* Vc, int32_t* len, 
     if (!aligned16(q) || !aligned16(Kc) || !aligned16(Vc) || !aligned16(out) || !aligned16(k_new) ||
         !aligned16(v_new) || kv_sh % 8 || kv_sb % 8)
         return LVLM_ERR_ALIGNMENT;
-    if (!ws || !aligned256(ws) || ws_bytes < L.total) return LVLM_ERR_WORKSPACE;
+    if (!ws || !aligned256(ws) || ws_bytes < L.logits) return LVLM_ERR_WORKSPACE;
+    if (ws_bytes < L.used) decode_layout(d, &L, false);              // without room for parts: no parts
     char* wsb = static_cast<char*>(ws);
 #define LVLM_DEC_CASE(GG)                                                                         \
     case GG: return launch_decode<GG>(q, Kc, Vc, len, k_new, v_new, acc_score, d, scale, out, wsb, \
@@ -749,11 +758,8 @@ extern "C" lvlm_status lvlm_decode_attn(const void* q, void* Kc, void* Vc, int32
                                          const void* k_new, const void* v_new, float* acc_score,
                                          const lvlm_dims* d, float scale, void* out, void* ws,
                                          size_t ws_bytes, int32_t* dev_status, void* stream_) {
-    using namespace lvlm;
-    DecodeLayout L;
-    if (!decode_layout(d, &L)) return LVLM_ERR_INVALID_ARG;
-    return decode_attn(q, Kc, Vc, len, k_new, v_new, acc_score, d, L, scale, out, ws, ws_bytes, dev_status,
-                       (cudaStream_t)stream_);
+    return lvlm::decode_attn(q, Kc, Vc, len, k_new, v_new, acc_score, d, scale, out, ws, ws_bytes, dev_status,
+                             (cudaStream_t)stream_);
 }
 
 // ---- decode attention for callers that cannot allocate ------------------------------------------
@@ -791,11 +797,10 @@ extern "C" lvlm_status lvlm_decode_attn_static(const void* q, void* Kc, void* Vc
     using namespace lvlm;
     DecodeLayout L;
     if (!decode_layout(d, &L)) return LVLM_ERR_INVALID_ARG;
-    if (L.total > (size_t)LVLM_STATIC_SCRATCH_BYTES) decode_layout(d, &L, false);     // without room for parts
-    if (L.total > (size_t)LVLM_STATIC_SCRATCH_BYTES) return LVLM_ERR_WORKSPACE;
+    if (L.logits > (size_t)LVLM_STATIC_SCRATCH_BYTES) return LVLM_ERR_WORKSPACE;
     void* scratch = nullptr;
     const lvlm_status st = static_scratch_address(&scratch);
     if (st != LVLM_OK) return st;
-    return decode_attn(q, Kc, Vc, len, k_new, v_new, acc_score, d, L, scale, out, scratch,
+    return decode_attn(q, Kc, Vc, len, k_new, v_new, acc_score, d, scale, out, scratch,
                        (size_t)LVLM_STATIC_SCRATCH_BYTES, dev_status, (cudaStream_t)stream);
 }

@@ -47,6 +47,25 @@ def test_decode_in_parts(case):
                 assert np.array_equal(ad[b, g, m:].cpu().numpy(), acc[b, g, m:])
 
 
+def test_decode_without_room_for_parts():
+    B, H, Hkv, cap = 1, 28, 4, 5000
+    q, Kc = torch.randn(B, H, 128, device="cuda").bfloat16(), torch.randn(B, Hkv, cap, 128, device="cuda").bfloat16()
+    ln = torch.full((B, Hkv), cap - 3, dtype=torch.int32, device="cuda")
+    d, least = L.kv_dims(Kc, H=H), -(-B * H * cap * 4 // 256) * 256
+    assert L.workspace_bytes(L.OP_DECODE_ATTN, d) > least
+    outs, accs = [], []
+    for n_ws in (L.workspace_bytes(L.OP_DECODE_ATTN, d), least):
+        ws = torch.full((n_ws + 4096,), 0x77, dtype=torch.uint8, device="cuda")
+        accs.append(torch.zeros(B, Hkv, cap, device="cuda"))
+        outs.append(L.decode_attn(q, Kc, Kc, ln, acc_score=accs[-1], ws=ws[:n_ws]))
+        assert ws[n_ws:].eq(0x77).all()
+    with pytest.raises(L.LvlmError) as e:
+        L.decode_attn(q, Kc, Kc, ln, ws=torch.empty(least - 256, dtype=torch.uint8, device="cuda"))
+    assert e.value.code == L.ERR_WORKSPACE
+    assert_rows_close(f64(outs[0]), f64(outs[1]), what="attention output")
+    assert_scores_close(f64(accs[0]), f64(accs[1]), what="acc_score")
+
+
 def test_decode_in_parts_bad_lengths_are_skipped():
     B, H, Hkv, cap = 1, 4, 4, 1100
     q, Kc = torch.randn(B, H, 128, device="cuda").to(torch.bfloat16), torch.randn(B, Hkv, cap, 128, device="cuda").to(torch.bfloat16)
