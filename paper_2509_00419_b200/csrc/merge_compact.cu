@@ -90,18 +90,19 @@ static bool merge_layout(const lvlm_dims* d, MergeLayout* L) {
     L->V = d->C / 8;
     L->grid = hidden_grid(d);
     L->kvP = kv_chunks(d, L->grid);
-    const int cps = L->grid.cps;
+    // Partial rows, as many as any smaller problem may leave (the shape of the launch rises and falls with the size, the
+    // workspace may not): of the hidden states one per CTA at most - up to 148 of them or one a sequence - and up to
+    // kMaxHidPartials a sequence; of K and V four chunks per CTA, rounded up for every sequence, of 64 rows at least.
+    const size_t B = d->B, ctas = d->B > 148 ? d->B : 148, per_seq = d->N < kMaxHidPartials ? d->N : kMaxHidPartials;
+    const size_t kv_seqs = B * (d->Hkv > 0 ? d->Hkv : 0) * 2, kv_dealt = 4 * ctas + kv_seqs, kv_cut = kv_seqs * (d->n < 64 ? 1 : d->n / 64);
     size_t off = 0;
     L->off_src = off;     off = align_up(off + (size_t)d->B * d->N * 4, 256);
     L->off_dst = off;     off = align_up(off + (size_t)d->B * d->N * 4, 256);
     L->off_wgt = off;     off = align_up(off + (size_t)d->B * d->n * 4, 256);
     L->off_meta = off;    off = align_up(off + (size_t)d->B * kMetaInts * 4, 256);
-    // (the launch may settle for smaller clusters than grid.cl, up to kMaxHidPartials partial rows a sequence)
-    const int few = cps < kMaxHidPartials ? cps : kMaxHidPartials;
-    const int prow = cps / L->grid.cl > few ? cps / L->grid.cl : few;
-    L->off_partial = off; off = align_up(off + (size_t)d->B * prow * d->C * 4, 256);
+    L->off_partial = off; off = align_up(off + (ctas < B * per_seq ? ctas : B * per_seq) * d->C * 4, 256);
     L->off_kvpartial = off;
-    if (d->Hkv > 0) off = align_up(off + (size_t)d->B * d->Hkv * 2 * L->kvP * kHeadDim * 4, 256);
+    off = align_up(off + (kv_dealt < kv_cut ? kv_dealt : kv_cut) * kHeadDim * 4, 256);
     L->total = off;
     return true;
 }

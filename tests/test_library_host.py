@@ -51,7 +51,7 @@ def test_workspace_sizes(lib):
 
 
 # a program sizes a workspace once, for its widest batch, longest prompt and window: nothing smaller may ask for more
-@pytest.mark.parametrize("op", [L.OP_SCORE_TOKENS, L.OP_PREFILL_ATTN, L.OP_DECODE_ATTN])
+@pytest.mark.parametrize("op", [L.OP_SCORE_TOKENS, L.OP_PREFILL_ATTN, L.OP_DECODE_ATTN, L.OP_MERGE_COMPACT])
 @pytest.mark.parametrize("heads", [(1024, 8, 8), (3584, 28, 4), (4096, 32, 8), (64, 1, 1)])
 def test_workspace_never_shrinks(lib, op, heads):
     C, H, Hkv = heads
