@@ -55,9 +55,10 @@ static bool nk_layout(const lvlm_dims* d, NkLayout* L) {
     L->off_order = off;   off = align_up(off + B * (r ? r : 1) * 8, 256);
     L->off_seg = off;     off = align_up(off + B * (k + 1) * 4, 256);
     L->off_newmass = off; off = align_up(off + B * (k ? k : 1) * 4, 256);
-    L->off_scratch = off; off = align_up(off + B * (r ? r : 1) * (size_t)d->C * 2, 256);
-    L->off_kvtmp = off;
-    if (d->Hkv > 0) off = align_up(off + B * d->Hkv * 2 * (k + L->rest + 1) * (size_t)kHeadDim * 2, 256);
+    // The dropped hidden rows and, once they are merged, the rows of K and V on their way back into the cache lie in the same
+    // place.  (Of these it is k and those behind the image; counted are N, which does not fall as the image span grows.)
+    const size_t hid = B * (r ? r : 1) * (size_t)d->C * 2, kv = B * (d->Hkv > 0 ? d->Hkv : 0) * 2 * d->N * (size_t)kHeadDim * 2;
+    L->off_scratch = L->off_kvtmp = off; off = align_up(off + (hid > kv ? hid : kv), 256);
     L->total = off;
     return true;
 }

@@ -70,6 +70,14 @@ def test_workspace_never_shrinks(lib, op, heads):
             assert sizes[i] >= sizes[i - 1], (line[i - 1], line[i])
 
 
+def test_nearest_kept_workspace_covers_shorter_image_spans(lib):
+    for C, H, Hkv in [(1024, 8, 8), (3584, 28, 4), (64, 4, 4)]:
+        for N, k in ((640, 100), (4096, 900), (16640, 4096)):
+            sizes = [L.workspace_bytes(L.OP_MERGE_COMPACT, L.Dims(B=2, H=H, Hkv=Hkv, D=128, N=N, C=C, cap=N, n=n, k=k,
+                                                                  merge_mode=L.W_NEAREST_KEPT)) for n in range(k, N + 1, 37)]
+            assert sizes == sorted(sizes), (C, N)
+
+
 def test_bad_arguments_are_rejected_on_the_host(lib):
     p = ctypes.c_void_p(0x1000)           # never dereferenced: every call below fails validation
     odd = ctypes.c_void_p(0x1008)
