@@ -263,6 +263,11 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     if (per >= kDecWarps) per = (per + kDecWarps - 1) / kDecWarps * kDecWarps;   // whole stages where the run is long enough
     const int t_lo = min(nt, rank * per), t_hi = min(nt, t_lo + per);   // my run of tiles
     const int nstage = (t_hi - t_lo + kDecWarps - 1) / kDecWarps;
+    if (MODE == kDecParts && nstage == 0) {                             // a part without keys: no weight, no output
+        if (a.early) pdl_enter();
+        if (tid < G) a.part_ml[((int64_t)hd * S + rank) * G + tid] = make_float2(-INFINITY, 0.f);
+        return;
+    }
     const uint32_t ring = smem_u32(smem);
     volatile int* abort_flag = &s_abort;
     auto wait_on = [&](uint64_t* bar, uint32_t parity) -> bool {
@@ -567,12 +572,15 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     if (CL) cluster_wait();                               // nobody leaves while its shared memory is still read
 }
 
-// Adds the parts of every head.  grid (G + key slices, heads): CTA y < G finishes the output of query head y of the
-// group, the others add the probabilities of a slice of the keys to acc_score.  Latency-bound (0.3 to 1 MB in all): every
+// Adds the parts of every head.  grid (G + CTAs for the keys, heads): CTA x < G finishes the output of query head x of the
+// group, the others add the probabilities of the keys to acc_score, a slice at a time in turn: as many CTAs as fit the GPU
+// beside the others, but eight, not one for every slice of the capacity (us a layer in a capacity of 32898 rows: 36 heads of 216
+// rows 16.3 so, 8.2 now; of 32000 rows 118.8 / 118.0, with four CTAs 122.8; 16 heads of 216 rows 8.2 / 6.2).  Latency-bound (0.3 to 1 MB in all): every
 // weight is worked out first, so that the loads of the parts depend on nothing - a warp takes every 16th part, a lane
 // four channels - and the warps are added in warp order.
 constexpr int kDecCombineThreads = 512;
 constexpr int kDecSliceKeys = 2 * kDecCombineThreads;
+constexpr int kDecLeastSliceCtas = 8;
 
 template <int G>
 __global__ void __launch_bounds__(kDecCombineThreads) decode_combine_kernel(const DecodeArgs a) {
@@ -586,6 +594,10 @@ __global__ void __launch_bounds__(kDecCombineThreads) decode_combine_kernel(cons
     const int app_at = a.part_len[hd];
     // every warp takes one of the query heads this CTA needs: (max, 1/sum) over the parts
     const bool finish = (int)blockIdx.x < G;
+    const int first_key = ((int)blockIdx.x - G) * kDecSliceKeys, key_step = ((int)gridDim.x - G) * kDecSliceKeys;
+    // (a.acc_score) where a row was appended another CTA bumps len meanwhile: part_len tells the keys then
+    const int lne = finish ? 0 : app_at >= 0 ? app_at + 1 : a.len[hd];
+    if (!finish && (lne <= first_key || lne > a.cap)) return;          // no keys for this CTA, or the head was skipped
     const int hh_w = finish ? (int)blockIdx.x : warp;
     if (finish ? warp == 0 : warp < G) {
         float m[(kDecTargetCtas + 31) / 32], l[(kDecTargetCtas + 31) / 32], M = -INFINITY, Ls = 0.f;
@@ -641,27 +653,25 @@ __global__ void __launch_bounds__(kDecCombineThreads) decode_combine_kernel(cons
         if (hh == 0 && tid == 0 && app_at >= 0) a.len[hd] = app_at + 1;
         return;
     }
-    // (a.acc_score) where a row was appended another CTA bumps len meanwhile: part_len tells the keys then
-    const int lne = app_at >= 0 ? app_at + 1 : a.len[hd];
-    if (lne < 0 || lne > a.cap) return;                    // this head was skipped
     float* acc = a.acc_score + (int64_t)hd * a.cap;
-    const int j0 = ((int)blockIdx.x - G) * kDecSliceKeys;
-    float lg[2][G], old[2];
+    for (int j0 = first_key; j0 < lne; j0 += key_step) {
+        float lg[2][G], old[2];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const int j = j0 + u * kDecCombineThreads + tid;
-        old[u] = 0.f;
+        for (int u = 0; u < 2; ++u) {
+            const int j = j0 + u * kDecCombineThreads + tid;
+            old[u] = 0.f;
 #pragma unroll
-        for (int hh = 0; hh < G; ++hh) lg[u][hh] = j < lne ? __ldcg(a.ws_s + (int64_t)(b * a.H + h0 + hh) * a.cap + j) : 0.f;
-        if (j < lne && j != app_at) old[u] = acc[j];       // a new entry starts at zero
-    }
+            for (int hh = 0; hh < G; ++hh) lg[u][hh] = j < lne ? __ldcg(a.ws_s + (int64_t)(b * a.H + h0 + hh) * a.cap + j) : 0.f;
+            if (j < lne && j != app_at) old[u] = acc[j];   // a new entry starts at zero
+        }
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const int j = j0 + u * kDecCombineThreads + tid;
-        float pr = 0.f;
+        for (int u = 0; u < 2; ++u) {
+            const int j = j0 + u * kDecCombineThreads + tid;
+            float pr = 0.f;
 #pragma unroll
-        for (int hh = 0; hh < G; ++hh) pr += exp2f(lg[u][hh] - s_M[hh]) * s_I[hh];
-        if (j < lne) acc[j] = old[u] + pr;
+            for (int hh = 0; hh < G; ++hh) pr += exp2f(lg[u][hh] - s_M[hh]) * s_I[hh];
+            if (j < lne) acc[j] = old[u] + pr;
+        }
     }
 }
 
@@ -716,8 +726,14 @@ static lvlm_status launch_decode(const void* q, void* Kc, void* Vc, int32_t* len
     LVLM_RETURN_IF_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem));
     const lvlm_status st = launch_kernel(kernel, dim3((unsigned)ctas), dim3(kDecThreads), smem, stream, parts ? 1 : S, kmap, vmap, a);
     if (st != LVLM_OK || !parts) return st;
-    const int slices = acc_score ? (d->cap + kDecSliceKeys - 1) / kDecSliceKeys : 0;
-    return launch_kernel(decode_combine_kernel<G>, dim3((unsigned)(G + slices), (unsigned)(d->B * d->Hkv)), dim3(kDecCombineThreads),
+    const int heads = d->B * d->Hkv;                       // (at most kDecTargetCtas / kDecMaxCluster here)
+    int slices = 0;
+    if (acc_score) {
+        const int most = (d->cap + kDecSliceKeys - 1) / kDecSliceKeys, room = kDecTargetCtas / heads - G;
+        slices = room > kDecLeastSliceCtas ? room : kDecLeastSliceCtas;
+        slices = slices < most ? slices : most;
+    }
+    return launch_kernel(decode_combine_kernel<G>, dim3((unsigned)(G + slices), (unsigned)heads), dim3(kDecCombineThreads),
                          0, stream, 1, a);
 }
 

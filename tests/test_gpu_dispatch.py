@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("case", [        # B, H, Hkv, cap, append, acc_score
     (1, 1, 1, 512, True, True), (1, 3, 1, 1037, False, True), (1, 7, 1, 256, True, False), (2, 8, 1, 545, True, False),
     (1, 28, 4, 1024, True, False), (5, 8, 4, 511, True, True), (9, 24, 4, 223, True, True), (8, 16, 4, 224, False, False),
-    (1, 2, 2, 7001, True, True)])
+    (1, 2, 2, 7001, True, True), (9, 4, 4, 9300, True, True)])      # (the last: a CTA has several slices of the keys)
 def test_decode_in_parts(case):
     B, H, Hkv, cap, append, with_acc = case
     r = np.random.default_rng(cap + H)
