@@ -52,7 +52,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 
 def build_test(force: bool = False) -> str:
-    """The library with its test hooks compiled in (switching programmatic dependent launch off)."""
+    """The library with its test hooks compiled in (switching programmatic dependent launch off, letting waits run out)."""
     if not force and not needs_build(TEST_LIB):
         return TEST_LIB
     return _compile(TEST_LIB, ["LVLM_TEST_HOOKS"], False)

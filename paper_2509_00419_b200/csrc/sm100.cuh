@@ -10,7 +10,12 @@
 namespace lvlm {
 namespace sm100 {
 
-constexpr uint32_t kSpinLimit = 1u << 21;        // polls of mbarrier.try_wait before giving up
+// Polls of mbarrier.try_wait before giving up, about 4 us each.  (The test build lets waits run out on purpose, for a moment only.)
+#ifdef LVLM_TEST_HOOKS
+constexpr uint32_t kSpinLimit = 1u << 14;
+#else
+constexpr uint32_t kSpinLimit = 1u << 21;
+#endif
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
