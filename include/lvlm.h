@@ -257,7 +257,10 @@ lvlm_status lvlm_kv_compress(void* Kc, void* Vc, float* acc_score, int32_t* pos,
  * the update of acc_score), and for the partial results where few heads with long caches are cut into parts
  * (two launches then); its contents need not be zeroed.  B * H * cap * 4 bytes (rounded up to 256) are needed; with less than
  * lvlm_workspace_bytes no head is cut.
- * Reads d: B,H,Hkv,D,cap,kv_stride_*.
+ * d->N, optional: how many rows the caller expects a head to hold at most (0 = unknown).  Caches are compacted in
+ * place, so their capacity says little about their length, and the length is only known on the device; with it
+ * the faster form is taken.  It changes no result beyond rounding, and longer heads are handled all the same.
+ * Reads d: B,H,Hkv,D,N,cap,kv_stride_*.
  * Errors: INVALID_ARG, UNSUPPORTED (D!=128, H/Hkv > 8), ALIGNMENT, WORKSPACE.
  */
 lvlm_status lvlm_decode_attn(const void* q, void* Kc, void* Vc, int32_t* len,

@@ -271,9 +271,9 @@ def nearest_assignment(ws: torch.Tensor, B: int, r: int) -> torch.Tensor:
     return ws[:B * r * 4].view(torch.int32).view(B, r)
 
 
-def kv_dims(Kc, *, H=None, recent=0) -> Dims:
+def kv_dims(Kc, *, H=None, recent=0, max_len=None) -> Dims:
     B, Hkv, cap, D = Kc.shape
-    d = Dims(B=B, Hkv=Hkv, H=H if H is not None else Hkv, D=D, cap=cap, recent=recent)
+    d = Dims(B=B, Hkv=Hkv, H=H if H is not None else Hkv, D=D, N=max_len or 0, cap=cap, recent=recent)
     d.kv_stride_b, d.kv_stride_h = Kc.stride(0), Kc.stride(1)
     return d
 
@@ -290,11 +290,12 @@ def kv_compress(Kc, Vc, acc_score, length, *, beta=1.0, budget=0, recent=0, e_lo
 
 
 def decode_attn(q, Kc, Vc, length, *, k_new=None, v_new=None, acc_score=None, scale=None, out=None,
-                ws=None, dev_status=None, stream=None, cache_stable=False):
+                ws=None, dev_status=None, stream=None, cache_stable=False, max_len=None):
     """lvlm_decode_attn.  q [B,H,D]; returns out [B,H,D] bf16.  Kc, Vc, length and acc_score are
-    updated in place when k_new/v_new or acc_score are given."""
+    updated in place when k_new/v_new or acc_score are given.  max_len: rows a head is expected to hold at most, where the
+    caller knows (it decides the form of the kernel, not the result)."""
     B, H, D = q.shape
-    d = kv_dims(Kc, H=H)
+    d = kv_dims(Kc, H=H, max_len=max_len)
     d.cache_stable = int(bool(cache_stable))
     if scale is None:
         scale = 1.0 / math.sqrt(D)
@@ -309,7 +310,7 @@ def decode_attn(q, Kc, Vc, length, *, k_new=None, v_new=None, acc_score=None, sc
 
 
 def decode_attn_static(q, Kc, Vc, length, *, k_new=None, v_new=None, acc_score=None, scale=None,
-                       out=None, dev_status=None, stream=None):
+                       out=None, dev_status=None, stream=None, max_len=None):
     """lvlm_decode_attn_static: lvlm_decode_attn for callers that have no way to get device
     scratch memory (all of it belongs to someone else's pool, or allocating would stall the
     device).  The scratch is a fixed array inside the library, at most STATIC_SCRATCH_BYTES per
@@ -317,7 +318,7 @@ def decode_attn_static(q, Kc, Vc, length, *, k_new=None, v_new=None, acc_score=N
     required to come from the caller as well when nothing may be allocated; it is created here
     only as a convenience when omitted."""
     B, H, D = q.shape
-    d = kv_dims(Kc, H=H)
+    d = kv_dims(Kc, H=H, max_len=max_len)
     if scale is None:
         scale = 1.0 / math.sqrt(D)
     if out is None:

@@ -26,7 +26,7 @@
 // fetched ahead of the cluster barrier (5.2 -> 5.6).
 //
 // Few heads with long caches (a video prompt's first layers: one sequence, 4 KV heads, 32898 rows) leave most of the
-// GPU idle that way: a cluster has at most 8 CTAs.  There the run of a head is cut into as many parts as fill the GPU
+// GPU idle that way: a cluster has at most 8 CTAs.  There (parts_from_tiles) the run of a head is cut into as many parts as fill the GPU
 // twice, without clusters; every part leaves its (max, sum, output) in the workspace, and a second, small launch adds
 // the parts in order, finishes acc_score and bumps len.  HBM-bound either way.  That shape, per layer (67 MB):
 // 53.6 us with 8 CTAs a head, 17.8 us as 74 parts a head
@@ -60,24 +60,32 @@ constexpr float kLog2e = 1.4426950408889634f;
 // heads, so that it never shrinks as the problem grows.
 struct DecodeLayout { int S, P; size_t off_s, off_ml, off_o, off_len, logits, used, total; };
 
-// Rows of a cache, in tiles, from which the parts are the faster form where a cluster of 8 a head leaves SMs idle (the
-// lengths are only known on the device).  us per layer as cluster / as parts, inside a chain of layers:
+// Rows, in tiles, from which the heads are cut into parts where a cluster of 8 a head leaves SMs idle.  us per layer as
+// cluster / as parts, inside a chain of layers:
 //   from 32 heads the clusters of 8 no longer fit the GPU side by side: 36 heads of 216 rows 9.3 / 6.9, 2500 18.0 / 14.0,
 //   9000 45 / 33; 32 heads of 216 rows 6.5 / 5.7, 9000 32 / 29;
-//   without acc_score the cluster's one launch wins while the runs are short: 4 heads of 600 rows 4.8 / 5.4, 1100 5.5 / 5.4,
-//   9000 17.2 / 10.2; 8 heads of 2500 rows 6.9 / 7.3, 4000 9.3 / 8.3; 16 heads of 4000 rows 11.8 / 11.9, 6000 16.0 / 14.0;
-//   28 heads of 9000 rows 26.0 / 26.9;
-//   with it the second launch takes the update of acc_score off the cluster's tail: 4 heads of 400 rows 4.9 / 5.6, 600
-//   5.7 / 5.5, 9000 20 / 9.8; 8 heads of 600 rows 5.2 / 5.0; 16 heads of 2500 rows 9.3 / 10.4, 4000 13.2 / 12.1; 28 heads of
-//   9000 rows 31 / 32.
-static int parts_from_tiles(int64_t heads, bool acc) {
+//   without acc_score the cluster's one launch wins while the runs are short: 4 heads of 600 rows 4.8 / 5.4, 1100 5.4 / 5.5,
+//   2100 7.1 / 5.9, 8200 16.4 / 9.5; 8 heads of 2100 rows 7.1 / 7.0, 4100 10.3 / 9.0; 16 heads of 4100 rows 12.7 / 12.0, 16400 36 / 26;
+//   24 heads of 16400 rows 37.5 / 35.6;
+//   with it the second launch takes the update of acc_score off the cluster's tail: 4 heads of 600 rows 5.8 / 5.7, 1100
+//   6.6 / 5.9; 8 heads of 600 rows 5.7 / 5.3; 16 heads of 2100 rows 9.2 / 8.9, 4100 14.0 / 12.1.
+// The lengths themselves are only known on the device.  Where the caller gives a bound of them, that decides (known).
+// Where only the capacity is known, the cache may be short - after the compaction of a prompt it is - and then the
+// second launch is lost time (4 heads of 216 rows in 33000: 4.1 / 5.6, with acc_score 5.3 / 6.1; 16 heads 4.4 / 6.3, 5.6 / 6.2).  The
+// line lies where a full cache gains in proportion what such a short one loses: without acc_score 4 heads of 6200 rows 13.4 / 8.7,
+// 8 of 8200 16.5 / 11.8, 16 of 25000 52 / 36, more never; with it 4 heads of 2100 rows 8.3 / 6.8, 8 of 4100 11.4 / 9.0, 20 of
+// 4100 16.1 / 14.1.
+static int parts_from_tiles(int64_t heads, bool acc, bool known) {
+    constexpr int kNever = 1 << 28;
     if (heads >= 32) return 14;
-    if (acc) return heads <= 8 ? 36 : heads <= 20 ? 192 : 800;
-    return heads <= 4 ? 64 : heads <= 8 ? 192 : heads <= 20 ? 320 : 800;
+    if (known && acc) return heads <= 8 ? 36 : heads <= 20 ? 192 : 800;
+    if (known) return heads <= 4 ? 96 : heads <= 8 ? 192 : heads <= 20 ? 320 : 800;
+    if (acc) return heads <= 4 ? 128 : heads <= 8 ? 192 : heads <= 20 ? 256 : 800;
+    return heads <= 4 ? 384 : heads <= 8 ? 512 : heads <= 16 ? 1536 : kNever;
 }
 
 // may_split: the caller's workspace has room for the parts.
-static bool decode_layout(const lvlm_dims* d, DecodeLayout* L, bool may_split = true) {
+static bool decode_layout(const lvlm_dims* d, DecodeLayout* L, bool acc, bool may_split) {
     if (!d || d->B <= 0 || d->H <= 0 || d->Hkv <= 0 || d->H % d->Hkv || d->cap <= 0) return false;
     // cluster size: the power of two that brings the grid closest to the target without going
     // over it, as long as a full cache still gives every CTA a few tiles
@@ -87,9 +95,9 @@ static bool decode_layout(const lvlm_dims* d, DecodeLayout* L, bool may_split = 
     while (S < kDecMaxCluster && heads * (2 * S) <= kDecTargetCtas && tiles / (2 * S) >= kDecMinTiles) S *= 2;
     L->S = S;
     L->P = 0;
-    if (may_split && S == kDecMaxCluster &&
-        (tiles >= parts_from_tiles(heads, false) || tiles >= parts_from_tiles(heads, true))) {
-        const int fill = (int)(kDecTargetCtas / heads), most = tiles / kDecPartTiles;
+    const int rows = d->N > 0 && d->N < d->cap ? d->N : d->cap, row_tiles = (rows + kTileKeys - 1) / kTileKeys;
+    if (may_split && S == kDecMaxCluster && row_tiles >= parts_from_tiles(heads, acc, d->N > 0)) {
+        const int fill = (int)(kDecTargetCtas / heads), most = (row_tiles + kDecPartTiles - 1) / kDecPartTiles;   // (a whole stage each)
         L->P = fill < most ? fill : most;
     }
     size_t off = 0;
@@ -111,7 +119,7 @@ static bool decode_layout(const lvlm_dims* d, DecodeLayout* L, bool may_split = 
 
 size_t decode_attn_workspace(const lvlm_dims* d) {
     DecodeLayout L;
-    return decode_layout(d, &L) ? L.total : 0;
+    return decode_layout(d, &L, false, false) ? L.total : 0;
 }
 
 // ---- thread-block cluster primitives ---------------------------------------------------------------
@@ -682,7 +690,7 @@ static lvlm_status launch_decode(const void* q, void* Kc, void* Vc, int32_t* len
                                  int64_t kv_sh, int32_t* dev_status, cudaStream_t stream) {
     // scaled logits of a CTA's own keys stay in shared memory when the longest run fits the budget
     const int nt_max = (d->cap + kTileKeys - 1) / kTileKeys;
-    const bool parts = L.P > 0 && nt_max >= parts_from_tiles((int64_t)d->B * d->Hkv, acc_score != nullptr);
+    const bool parts = L.P > 0;
     const int S = parts ? L.P : L.S;
     int per = (nt_max + S - 1) / S;
     if (per >= kDecWarps) per = (per + kDecWarps - 1) / kDecWarps * kDecWarps;
@@ -741,7 +749,7 @@ static lvlm_status decode_attn(const void* q, void* Kc, void* Vc, int32_t* len, 
                                float* acc_score, const lvlm_dims* d, float scale, void* out, void* ws, size_t ws_bytes,
                                int32_t* dev_status, cudaStream_t stream) {
     DecodeLayout L;
-    if (!q || !Kc || !Vc || !len || !out || !decode_layout(d, &L)) return LVLM_ERR_INVALID_ARG;
+    if (!q || !Kc || !Vc || !len || !out || !decode_layout(d, &L, acc_score != nullptr, true)) return LVLM_ERR_INVALID_ARG;
     if ((k_new == nullptr) != (v_new == nullptr)) return LVLM_ERR_INVALID_ARG;
     const int G = d->H / d->Hkv;
     if (d->D != kHeadDim || G > kMaxGroup) return LVLM_ERR_UNSUPPORTED;
@@ -751,7 +759,7 @@ static lvlm_status decode_attn(const void* q, void* Kc, void* Vc, int32_t* len, 
         !aligned16(v_new) || kv_sh % 8 || kv_sb % 8)
         return LVLM_ERR_ALIGNMENT;
     if (!ws || !aligned256(ws) || ws_bytes < L.logits) return LVLM_ERR_WORKSPACE;
-    if (ws_bytes < L.used) decode_layout(d, &L, false);              // without room for parts: no parts
+    if (ws_bytes < L.used) decode_layout(d, &L, acc_score != nullptr, false);        // without room for parts: no parts
     char* wsb = static_cast<char*>(ws);
 #define LVLM_DEC_CASE(GG)                                                                         \
     case GG: return launch_decode<GG>(q, Kc, Vc, len, k_new, v_new, acc_score, d, scale, out, wsb, \
@@ -812,7 +820,7 @@ extern "C" lvlm_status lvlm_decode_attn_static(const void* q, void* Kc, void* Vc
                                                 void* out, int32_t* dev_status, void* stream) {
     using namespace lvlm;
     DecodeLayout L;
-    if (!decode_layout(d, &L)) return LVLM_ERR_INVALID_ARG;
+    if (!decode_layout(d, &L, false, false)) return LVLM_ERR_INVALID_ARG;
     if (L.logits > (size_t)LVLM_STATIC_SCRATCH_BYTES) return LVLM_ERR_WORKSPACE;
     void* scratch = nullptr;
     const lvlm_status st = static_scratch_address(&scratch);

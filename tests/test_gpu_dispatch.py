@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 # decode attention cut into parts that a second launch adds: few heads with long caches, or more heads than clusters fit
 @pytest.mark.parametrize("case", [        # B, H, Hkv, cap, append, acc_score
     (1, 1, 1, 512, True, True), (1, 3, 1, 1037, False, True), (1, 7, 1, 256, True, False), (2, 8, 1, 545, True, False),
-    (1, 28, 4, 1024, True, False), (5, 8, 4, 511, True, True), (9, 24, 4, 223, True, True), (8, 16, 4, 224, False, False),
+    (1, 28, 4, 1536, True, False), (5, 8, 4, 511, True, True), (9, 24, 4, 223, True, True), (8, 16, 4, 224, False, False),
     (1, 2, 2, 7001, True, True), (9, 4, 4, 9300, True, True)])      # (the last: a CTA has several slices of the keys)
 def test_decode_in_parts(case):
     B, H, Hkv, cap, append, with_acc = case
@@ -32,7 +32,7 @@ def test_decode_in_parts(case):
     ad = torch.from_numpy(acc).cuda() if with_acc else None
     flag = torch.zeros(1, dtype=torch.int32, device="cuda")
     out = L.decode_attn(q.cuda(), Kd, Vd, ld, k_new=kn.cuda() if append else None, v_new=vn.cuda() if append else None,
-                        acc_score=ad, dev_status=flag)
+                        acc_score=ad, dev_status=flag, max_len=cap)
     torch.cuda.synchronize()
     assert flag.item() == 0
     assert_rows_close(f64(out), want["out"], what="attention output")
@@ -45,6 +45,31 @@ def test_decode_in_parts(case):
                 m = want["len"][b, g]
                 assert_scores_close(ad[b, g, :m].cpu().numpy(), want["acc_score"][b, g, :m], what="acc_score")
                 assert np.array_equal(ad[b, g, m:].cpu().numpy(), acc[b, g, m:])
+
+
+# the form follows the rows that the caller expects, not the capacity alone; rows beyond what was expected are attended to as well
+@pytest.mark.parametrize("B,H,Hkv,cap,max_len,rows,acc,parts", [
+    (1, 28, 4, 3072, None, 300, False, False), (1, 28, 4, 3072, 301, 300, False, False), (1, 28, 4, 3072, 2900, 2899, False, True),
+    (1, 28, 4, 3072, 200, 3000, False, False), (1, 28, 4, 33000, None, 300, False, True), (1, 28, 4, 33000, 400, 9000, True, False),
+    (1, 32, 8, 3056, None, 700, True, False), (1, 32, 8, 3072, None, 700, True, True), (9, 28, 4, 300, None, 290, False, True),
+    (1, 28, 4, 2000, 5000, 1999, True, True)])
+def test_decode_form(B, H, Hkv, cap, max_len, rows, acc, parts):
+    from torch.profiler import ProfilerActivity, profile
+    g = torch.Generator(device="cuda").manual_seed(cap + rows)
+    q, kn = (torch.randn(B, h, 128, generator=g, device="cuda").bfloat16() for h in (H, Hkv))
+    Kc = torch.randn(B, Hkv, cap, 128, generator=g, device="cuda").bfloat16()
+    ln = torch.full((B, Hkv), rows, dtype=torch.int32, device="cuda")
+    accs, flag = torch.zeros(B, Hkv, cap, device="cuda") if acc else None, torch.zeros(1, dtype=torch.int32, device="cuda")
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        out = L.decode_attn(q, Kc, Kc, ln, k_new=kn, v_new=kn, acc_score=accs, dev_status=flag, max_len=max_len)
+        torch.cuda.synchronize()
+    assert any("decode_combine" in e.key for e in prof.key_averages()) == parts
+    k = Kc[:, :, :rows + 1].double().repeat_interleave(H // Hkv, dim=1)
+    assert flag.item() == 0 and ln.eq(rows + 1).all() and torch.equal(Kc[:, :, rows], kn)
+    p = torch.softmax(torch.einsum("bhd,bhnd->bhn", q.double(), k) / 128 ** 0.5, dim=-1)
+    assert_rows_close(f64(out), f64(torch.einsum("bhn,bhnd->bhd", p, k)), what="attention output")
+    if acc:
+        assert_scores_close(f64(accs[:, :, :rows + 1]), f64(p.view(B, Hkv, H // Hkv, -1).sum(dim=2)), what="acc_score")
 
 
 def test_decode_without_room_for_parts():
@@ -73,7 +98,7 @@ def test_decode_in_parts_bad_lengths_are_skipped():
     ln = torch.tensor([[cap + 1, -1, cap, 700]], dtype=torch.int32, device="cuda")
     acc = torch.zeros(B, Hkv, cap, device="cuda")
     K0 = Kc.clone()
-    out = L.decode_attn(q, Kc, K0, ln, k_new=kn, v_new=kn, acc_score=acc, dev_status=flag)
+    out = L.decode_attn(q, Kc, K0, ln, k_new=kn, v_new=kn, acc_score=acc, dev_status=flag, max_len=cap)
     assert flag.item() == L.DEV_BOUNDS and ln.tolist() == [[cap + 1, -1, cap, 701]]
     assert not out[0, :2].any() and not acc[0, :2].any()
     assert abs(acc[0, 2].sum().item() - 1) < 1e-4 and abs(acc[0, 3, :701].sum().item() - 1) < 1e-4 and not acc[0, 3, 701:].any()
@@ -91,7 +116,7 @@ def test_decode_timeout_keeps_the_appended_row(B, H, Hkv, cap):
     try:
         L.use_library(BU.build_test())
         L.lib().lvlm_debug_starve_decode(1)
-        L.decode_attn(q, Kc, Vc, ln, k_new=kn, v_new=vn, dev_status=flag)
+        L.decode_attn(q, Kc, Vc, ln, k_new=kn, v_new=vn, dev_status=flag, max_len=cap)
         torch.cuda.synchronize()
         L.lib().lvlm_debug_starve_decode(0)
     finally:
