@@ -14,8 +14,8 @@
 //   merge     every kept row becomes the mass-weighted mean of itself and its segment, in token order
 //   K, V      the same mean per KV head, and the rows behind the image, into scratch; then stored in place
 //   mass      token masses compacted in place
-// us at 16384 + 256 tokens of 6144 channels, 4096 kept, before -> now: plan 39 -> 10, norms 8 -> 0, similarity 523 -> 452 (618
-// GFLOP: 1370 TFLOP/s), group 92 -> 22, K and V 60 -> 35; rows 64 and merge 46 run at the copy rate.
+// us at 16384 + 256 tokens of 6144 channels, 4096 kept: plan 10, similarity 405 (618 GFLOP: 1527 TFLOP/s), group 22, K and V 35;
+// rows 64 and merge 46 run at the copy rate.
 #include "common.cuh"
 #include "merge.cuh"
 #include "sm100.cuh"
@@ -445,25 +445,35 @@ nk_mass_kernel(float* mass, int N, int i0, int k, int r, const float* __restrict
 // S = X_dropped X_kept^T, K = channels in chunks of 64.  The operands come from L2 faster than it can deliver them: a
 // 128x256 tile a time (48 KB a chunk, 424 cycles of MMAs) asked for 30 TB/s over all SMs and got 14.  So a CTA multiplies
 // TWO row tiles of 128 with a column tile of 256 at a time (64 KB for twice the work; the two accumulators fill the
-// tensor memory).  The kernel is persistent: the (column tile, row tile) units are shared out evenly, a CTA takes its run
-// of them in pairs, so that no last wave is left (1536 units on 148 SMs: 11 turns where CTAs of four took 12.75).  Warp 0
-// feeds a ring of shared-memory stages by TMA across units, warp 1 issues the MMAs, eight epilogue warps scale the columns
-// by 1/|x_t| and find the best (value, kept index) of every row.
-constexpr int kSimM = 128, kSimN = 256, kSimK = 64, kSimStages = 3;
+// tensor memory).  The kernel is persistent: an item is two neighbouring row tiles (an odd last one alone) and a column tile, and
+// the CTAs take the items in turn, so that those under way at a time share few rows and columns and lie in L2 (SimItems).
+// The items of a last round that would leave half of the CTAs idle are cut into single row tiles; where that is all there is, the
+// stages of the ring hold single tiles and there is one more of them.
+// us, with one row tile a time and two accumulators in turn / every CTA a run of neighbouring tiles, in twos where it fits / so:
+// 12288 dropped x 4096 kept rows of 6144 channels 522 / 447 / 405; 16 sequences of 732 x 1060 x 4096 115 / 138 / 106; 4 of 1500 x 1500 x
+// 3584 51 / 66 / 48; 1985 x 895 x 3584 25 / 28 / 25; 16 of 500 x 500 x 6144 53 / 69 / 57.
+// Warp 0 feeds a ring of shared-memory stages by TMA
+// across items, warp 1 issues the MMAs, eight epilogue warps scale the columns by 1/|x_t| and find the best (value, kept index)
+// of every row.
+constexpr int kSimM = 128, kSimN = 256, kSimK = 64;
 constexpr int kSimABytes = kSimM * kSimK * 2, kSimBBytes = kSimN * kSimK * 2;
-constexpr int kSimStageBytes = 2 * kSimABytes + kSimBBytes;
+constexpr int kSimRing = 192 * 1024, kSimMaxStages = 4;                  // 3 stages of two row tiles, or 4 of one
+constexpr int kSimCtas = 148, kSimWide = 16;                             // column tiles under way at a time
 constexpr int kSimThreads = 320, kSimEpi = 256;
 constexpr uint32_t kSimTmemCols = 512;
 
 struct SimArgs {
-    int r, k, nkc, nrt, nct, units;
+    int r, k, nkc, nrt, nct;
+    int npr, wide;                  // row tiles two at a time; column tiles of a group
+    int items, whole;               // whole: items taken as they are; those behind go to two CTAs, a row tile each
+    int stages, b_off;              // of the ring; where the column tile lies in a stage
     const float* inv_norm;          // [B][k]
     unsigned long long* best;       // [B][r] (orderable similarity << 32) | ~kept index, zero before
     int32_t* dev_status;
 };
 
 struct SimSmem {
-    uint64_t full[kSimStages], empty[kSimStages], tmem_full, tmem_empty;
+    uint64_t full[kSimMaxStages], empty[kSimMaxStages], tmem_full, tmem_empty;
     uint32_t tmem_base;
     volatile int abort;
     float inv_s[2][kSimN];          // 1/|x_t| of the columns, per column half (written by its warps for themselves)
@@ -471,19 +481,31 @@ struct SimSmem {
     int xt[2][kSimM];
 };
 
-// The units of a CTA: (sequence, column tile, row tile), row tiles fastest; one or two row tiles of a column at a time.
-struct SimUnits {
-    int u, end, b, ct, rt, n;
-    __device__ explicit SimUnits(const SimArgs& a)
-        : u((int)((int64_t)a.units * blockIdx.x / gridDim.x)), end((int)((int64_t)a.units * (blockIdx.x + 1) / gridDim.x)), n(0) {}
+// The items of a CTA: every gridDim.x-th.  In order: sequence, group of up to kSimWide column tiles, pair of row tiles, column
+// tile of the group.  (148 items at a time: 9 pairs of row tiles x 16 column tiles.)
+struct SimItems {
+    int i, b, ct, rt, n;
+    __device__ SimItems() : i((int)blockIdx.x), n(0) {}
     __device__ bool next(const SimArgs& a) {
-        u += n;
-        if (u >= end) return false;
-        rt = u % a.nrt;
-        const int c = u / a.nrt;
-        ct = c % a.nct;
-        b = c / a.nct;
-        n = min(2, min(end - u, a.nrt - rt));
+        int x = i, part = -1;
+        if (x >= a.whole) {
+            if (x - a.whole >= 2 * (a.items - a.whole)) return false;
+            part = (x - a.whole) & 1;
+            x = a.whole + ((x - a.whole) >> 1);
+        }
+        i += (int)gridDim.x;
+        const int per_seq = a.nct * a.npr, per_group = a.wide * a.npr;
+        b = x / per_seq; x -= b * per_seq;
+        const int first = x / per_group * a.wide, width = min(a.wide, a.nct - first);
+        x -= first * a.npr;
+        rt = 2 * (x / width);
+        ct = first + x % width;
+        n = min(2, a.nrt - rt);
+        if (part >= 0) {
+            if (part >= n) return false;                       // (an odd last row tile; nothing follows the items cut in two)
+            rt += part;
+            n = 1;
+        }
         return true;
     }
 };
@@ -501,11 +523,11 @@ nk_sim_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* base = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
-    SimSmem* sm = reinterpret_cast<SimSmem*>(base + kSimStageBytes * kSimStages);
+    SimSmem* sm = reinterpret_cast<SimSmem*>(base + kSimRing);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kSimStages; ++s) { mbar_init(&sm->full[s], 1); mbar_init(&sm->empty[s], 1); }
+        for (int s = 0; s < kSimMaxStages; ++s) { mbar_init(&sm->full[s], 1); mbar_init(&sm->empty[s], 1); }
         mbar_init(&sm->tmem_full, 1);
         mbar_init(&sm->tmem_empty, kSimEpi);
         sm->abort = 0;
@@ -521,7 +543,8 @@ nk_sim_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
     const uint32_t tmem_base = sm->tmem_base;
     pdl_enter();
 
-    SimUnits w(a);
+    SimItems w;
+    const uint32_t stage_bytes = (uint32_t)(a.b_off + kSimBBytes), stages = (uint32_t)a.stages;
     if (warp == 0) {
         if (lane == 0) {
             uint32_t st = 0, phase = 1;                        // (the first lap finds every stage empty)
@@ -529,12 +552,12 @@ nk_sim_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
             while (ok && w.next(a)) {
                 for (int kc = 0; kc < a.nkc; ++kc) {
                     if (!(ok = sim_wait(&sm->empty[st], phase, sm, a.dev_status))) break;
-                    unsigned char* dst = base + st * kSimStageBytes;
+                    unsigned char* dst = base + st * stage_bytes;
                     mbar_arrive_expect_tx(&sm->full[st], (uint32_t)(w.n * kSimABytes + kSimBBytes));
                     for (int i = 0; i < w.n; ++i)
                         tma_load_3d(dst + i * kSimABytes, &amap, &sm->full[st], kc * kSimK, (w.rt + i) * kSimM, w.b);
-                    tma_load_3d(dst + 2 * kSimABytes, &bmap, &sm->full[st], kc * kSimK, w.ct * kSimN, w.b);
-                    if (++st == kSimStages) { st = 0; phase ^= 1u; }
+                    tma_load_3d(dst + a.b_off, &bmap, &sm->full[st], kc * kSimK, w.ct * kSimN, w.b);
+                    if (++st == stages) { st = 0; phase ^= 1u; }
                 }
             }
         }
@@ -547,21 +570,25 @@ nk_sim_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
         while (ok && w.next(a)) {
             if (it > 0) ok = __all_sync(0xFFFFFFFFu, sim_wait(&sm->tmem_empty, (it - 1) & 1, sm, a.dev_status));
             for (int kc = 0; ok && kc < a.nkc; ++kc) {
-                const uint64_t ad = d0 + st * (uint32_t)(kSimStageBytes >> 4), bd = ad + (uint32_t)(2 * kSimABytes >> 4);
+                const uint64_t ad = d0 + st * (stage_bytes >> 4), bd = ad + (uint32_t)(a.b_off >> 4);
                 ok = __all_sync(0xFFFFFFFFu, sim_wait(&sm->full[st], phase, sm, a.dev_status));
                 if (!ok) break;
                 tc_fence_after();
                 if (elect_one()) {
-                    for (int i = 0; i < w.n; ++i)
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        mma_bf16_ss(tmem_base, ad + (uint32_t)(kk * 2), bd + (uint32_t)(kk * 2), idesc, (kc > 0 || kk > 0) ? 1u : 0u);
+                    if (w.n == 2) {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk)
-                            mma_bf16_ss(tmem_base + i * kSimN, ad + (uint32_t)(i * (kSimABytes >> 4) + kk * 2), bd + (uint32_t)(kk * 2), idesc,
+                            mma_bf16_ss(tmem_base + kSimN, ad + (uint32_t)((kSimABytes >> 4) + kk * 2), bd + (uint32_t)(kk * 2), idesc,
                                         (kc > 0 || kk > 0) ? 1u : 0u);
+                    }
                     mma_commit(&sm->empty[st]);
                     if (kc == a.nkc - 1) mma_commit(&sm->tmem_full);
                 }
                 __syncwarp();
-                if (++st == kSimStages) { st = 0; phase ^= 1u; }
+                if (++st == stages) { st = 0; phase ^= 1u; }
             }
             ++it;
         }
@@ -570,12 +597,12 @@ nk_sim_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
         const int row = quarter * 32 + lane;
         const uint32_t my_tmem = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * 128;
         bool ok = true;
-        // (every epilogue thread goes through every unit, also after a wait has given up: the barriers count them all)
+        // (every epilogue thread goes through every item, also after a wait has given up: the barriers count them all)
         for (uint32_t it = 0; w.next(a); ++it) {
-            // 1/|x_t| of my half's columns, while the unit is being multiplied (the four warps write the same values)
+            // 1/|x_t| of my half's columns, while the item is being multiplied (the four warps write the same values)
             const int t0 = w.ct * kSimN + half * 128;
             const float* inv = a.inv_norm + (int64_t)w.b * a.k;
-            asm volatile("bar.sync 1, 256;" ::: "memory");       // the unit before has been read
+            asm volatile("bar.sync 1, 256;" ::: "memory");       // the item before has been read
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int t = t0 + u * 32 + lane;
@@ -587,24 +614,32 @@ nk_sim_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ 
             int best_t[2] = {-1, -1};
             if (ok) {
                 tc_fence_after();
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    if (i >= w.n) break;
-                    // (a chunk is read while the one before is worked on)
-                    float v[2][32];
-                    tmem_ld32(my_tmem + i * kSimN, v[0]);
-#pragma unroll
-                    for (int c4 = 0; c4 < 4; ++c4) {
-                        tmem_ld_wait();
-                        if (c4 < 3) tmem_ld32(my_tmem + i * kSimN + (c4 + 1) * 32, v[(c4 + 1) & 1]);
-                        const int tb = t0 + c4 * 32;
-                        const float* is = &sm->inv_s[half][c4 * 32];
+                // (loops, not straight-line code: a CTA with one item runs through it once, and that is fetched slower than executed)
+#pragma unroll 1
+                for (int i = 0; i < w.n; ++i) {
+                    float bv = -INFINITY, v[2][32];
+                    int bt = -1;
+                    auto pick = [&](const float* x, int c0) {
+                        const float* is = &sm->inv_s[half][c0];
 #pragma unroll
                         for (int c = 0; c < 32; ++c) {
-                            const float val = v[c4 & 1][c] * is[c];
-                            if (tb + c < a.k && val > best_v[i]) { best_v[i] = val; best_t[i] = tb + c; }
+                            const float val = x[c] * is[c];
+                            if (t0 + c0 + c < a.k && val > bv) { bv = val; bt = t0 + c0 + c; }
                         }
+                    };
+                    // (a chunk is read while the one before is worked on)
+                    const uint32_t from = my_tmem + i * kSimN;
+                    tmem_ld32(from, v[0]);
+#pragma unroll 1
+                    for (int c0 = 0; c0 < 128; c0 += 64) {
+                        tmem_ld_wait();
+                        tmem_ld32(from + c0 + 32, v[1]);
+                        pick(v[0], c0);
+                        tmem_ld_wait();
+                        if (c0 == 0) tmem_ld32(from + 64, v[0]);
+                        pick(v[1], c0 + 32);
                     }
+                    if (i == 0) { best_v[0] = bv; best_t[0] = bt; } else { best_v[1] = bv; best_t[1] = bt; }
                 }
                 tc_fence_before();
             }
@@ -706,16 +741,22 @@ lvlm_status launch_nearest_kept(const void* hidden, void* hidden_out, void* Kc, 
         if (!make_tmap_bf16(&bmap, bbase, 3, bdims, bstr, bbox)) return LVLM_ERR_CUDA;
         SimArgs a;
         a.r = L.r; a.k = d->k; a.nkc = (d->C + kSimK - 1) / kSimK; a.nct = (d->k + kSimN - 1) / kSimN;
-        a.nrt = (L.r + kSimM - 1) / kSimM;
-        const int64_t units = (int64_t)d->B * a.nct * a.nrt;
-        if (units > 0x7FFFFFFFll) return LVLM_ERR_UNSUPPORTED;
-        a.units = (int)units;
+        a.nrt = (L.r + kSimM - 1) / kSimM; a.npr = (a.nrt + 1) / 2;
+        const int groups = (a.nct + kSimWide - 1) / kSimWide;
+        a.wide = (a.nct + groups - 1) / groups;
+        const int64_t items = (int64_t)d->B * a.nct * a.npr;
+        if (items > 0x3FFFFFFFll) return LVLM_ERR_UNSUPPORTED;
+        a.items = (int)items;
+        const int rest = a.items % kSimCtas;
+        a.whole = 2 * rest <= kSimCtas ? a.items - rest : a.items;
+        const bool single = a.whole == 0;                        // (then the grid has two CTAs an item)
+        a.stages = single ? 4 : 3; a.b_off = single ? kSimABytes : 2 * kSimABytes;
+        const int ctas = single ? 2 * a.items : a.items < kSimCtas ? a.items : kSimCtas;
         a.inv_norm = inv_norm; a.best = best; a.dev_status = dev_status;
-        const size_t smem = 1024 + (size_t)kSimStageBytes * kSimStages + sizeof(SimSmem);
+        const size_t smem = 1024 + (size_t)kSimRing + sizeof(SimSmem);
         LVLM_RETURN_IF_CUDA(cudaFuncSetAttribute(nk_sim_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)smem));
-        st = launch_kernel(nk_sim_kernel, dim3((unsigned)(units < 148 ? units : 148)), dim3(kSimThreads), smem, stream, 1,
-                           amap, bmap, a);
+        st = launch_kernel(nk_sim_kernel, dim3((unsigned)ctas), dim3(kSimThreads), smem, stream, 1, amap, bmap, a);
         if (st != LVLM_OK) return st;
     }
     st = launch_kernel(nk_count_kernel, dim3((L.r + 255) / 256, d->B), dim3(256), 0, stream, 1, best, L.r, d->k, assign, place, seg);

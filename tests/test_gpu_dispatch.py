@@ -206,7 +206,8 @@ def test_attention_refuses_too_few_registers():
 # at all for most; text rows that are the source of rows before them; runs over several CTAs of the plan's cluster
 @pytest.mark.parametrize("case", [        # B, C, Hkv, i0, n, T, k, kept tokens that attract the dropped ones
     (1, 64, 1, 0, 40, 5, 7, 1), (2, 128, 2, 3, 300, 20, 33, 1), (1, 256, 1, 0, 700, 600, 20, 20), (1, 64, 2, 17, 4500, 31, 2500, 60),
-    (3, 72, 1, 2, 2100, 300, 100, 3), (1, 64, 1, 0, 9000, 10, 1030, 1030)])
+    (3, 72, 1, 2, 2100, 300, 100, 3), (1, 64, 1, 0, 9000, 10, 1030, 1030),
+    (1, 64, 1, 0, 8970, 3, 4500, 700)])    # (similarity: two groups of column tiles, an odd row tile, items cut in two behind whole ones)
 def test_nearest_kept_groups(case):
     B, C, Hkv, i0, n, T, k, attract = case
     r = np.random.default_rng(n + k)
