@@ -14,6 +14,7 @@ collective on the data path) and rank 0 reports the aggregate.
 from __future__ import annotations
 
 import argparse
+import ctypes
 import json
 import os
 import subprocess
@@ -130,6 +131,24 @@ def timed(fn, steps, warmup, flush, between=None):
     return float(np.mean(ts)), ts
 
 
+def count_launches(fn):
+    """Kernels that ``fn`` enqueues: the kernel nodes of a graph it is captured into (not run).  How many a call takes
+    depends on its sizes."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        fn()
+    n, kind = ctypes.c_size_t(0), ctypes.c_int(0)
+    raw = ctypes.c_void_p(g.raw_cuda_graph())
+    assert cu.cuGraphGetNodes(raw, None, ctypes.byref(n)) == 0
+    nodes, kernels = (ctypes.c_void_p * n.value)(), 0
+    assert cu.cuGraphGetNodes(raw, nodes, ctypes.byref(n)) == 0
+    for node in nodes:
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kernels += kind.value == 0                 # CU_GRAPH_NODE_TYPE_KERNEL
+    return kernels
+
+
 # ------------------------------------------------------------------------------------------
 # prefill: pyramid reduction stages
 # ------------------------------------------------------------------------------------------
@@ -139,7 +158,7 @@ def bench_prefill(w, device, steps, warmup, flush, peaks, breakdown=True):
     g = P.capture(run.step)
     ms, _ = timed(g.replay, steps, warmup, flush, between=run.restore)
     res = {"ms_per_step": ms, "tokens_in": run.tokens_in,
-           "tokens_per_s": run.tokens_in / (ms * 1e-3), "launches": run.launches, "stages": []}
+           "tokens_per_s": run.tokens_in / (ms * 1e-3), "launches": count_launches(run.step), "stages": []}
     if breakdown:
         for s, st in enumerate(run.stages):
             hidden_in = run.hidden0 if s == 0 else run.stages[s - 1].hidden_out
@@ -153,6 +172,9 @@ def bench_prefill(w, device, steps, warmup, flush, peaks, breakdown=True):
             t_me, _ = timed(g_me.replay, steps, warmup, flush, between=run.restore)
             by = st.bytes_merge_hidden() + st.bytes_merge_kv()
             res["stages"].append({
+                "score_launches": count_launches(lambda: st.run_score(run.Q[s], run.K[s])),
+                "select_launches": count_launches(st.run_select),
+                "merge_launches": count_launches(lambda: st.run_merge(hidden_in, run.K[s], run.V[s], run.pos[s])),
                 "n_in": st.n, "n_out": st.M, "score_ms": t_sc, "select_ms": t_se,
                 "merge_compact_ms": t_me, "merge_compact_bytes": by, "score_flops": st.flops_score(),
                 "merge_compact_gbs": by / (t_me * 1e6),
@@ -342,13 +364,6 @@ class FullPass:
         self.phase_compress()
         self.phase_decode()
 
-    @property
-    def launches(self):
-        w = self.w
-        # reduction stages; 3 scoring kernels (at least) per group of compressed layers + plan and compaction; one decode
-        # kernel per layer
-        return self.pre.launches + 3 * len(self.groups) + 2 + w.L
-
 
 def bench_full(w, device, steps, warmup, flush, peaks, phases=True, fence=None):
     """``fence`` (a barrier over the ranks plus a device synchronise) brackets the timed steps."""
@@ -364,7 +379,7 @@ def bench_full(w, device, steps, warmup, flush, peaks, phases=True, fence=None):
     if fence is not None:
         fence()
     if not phases:
-        return {"ms_per_step": ms, "launches": fp.launches, "tokens_in": fp.pre.tokens_in}, fp, per_step
+        return {"ms_per_step": ms, "launches": count_launches(fp.step), "tokens_in": fp.pre.tokens_in}, fp, per_step
     # phases, timed one by one (each from the restored state it expects)
     g_red = P.capture(fp.phase_reduce); fp.restore()
     t_red, _ = timed(g_red.replay, steps, warmup, flush, between=fp.restore)
@@ -391,7 +406,9 @@ def bench_full(w, device, steps, warmup, flush, peaks, phases=True, fence=None):
     res = {"ms_per_step": ms, "reduce_ms": t_red, "compress_ms": t_cmp, "decode_ms": t_dec,
            "score_caches_ms": t_scc, "score_caches_flops": scc_flops, "score_caches_calls": len(fp.groups),
            "kv_compress_only_ms": max(t_cmp - t_scc, 0.0), "kv_compress_bytes": int(cmp_bytes),
-           "tokens_in": fp.pre.tokens_in, "launches": fp.launches,
+           "tokens_in": fp.pre.tokens_in, "launches": count_launches(fp.step),
+           "score_caches_launches": count_launches(fp.phase_score_caches), "decode_launches": count_launches(fp.phase_decode),
+           "compress_launches": count_launches(fp.phase_compress),
            "decode_kv_bytes": kv_bytes, "decode_gbs": kv_bytes / (t_dec * 1e6),
            "decode_frac_hbm": kv_bytes / (t_dec * 1e6) / peaks["hbm_gbs"],
            "mean_len_after_compress": kept, "len_before": fp.lens}
@@ -427,6 +444,8 @@ def bench_decode_loop(w, device, flush, peaks, prompt_len, steps_total):
     vb = torch.zeros_like(kb)
     g_step = P.capture(lambda: dec.decode_step(qb, kb, vb, accumulate=True))
     g_cmp = P.capture(lambda: dec.compress(beta=1.0, budget=w.budget, recent=w.recent))
+    per_step = count_launches(lambda: dec.decode_step(qb, kb, vb, accumulate=True))
+    per_compression = count_launches(lambda: dec.compress(beta=1.0, budget=w.budget, recent=w.recent))
     # the captures ran the calls once: start again from the prompt state
     dec.K.copy_(snap[0]); dec.V.copy_(snap[1]); dec.acc.copy_(snap[2]); dec.len.fill_(prompt_len)
     dec.status.zero_()
@@ -478,7 +497,7 @@ def bench_decode_loop(w, device, flush, peaks, prompt_len, steps_total):
            "decode_kv_bytes": bytes_read, "decode_gbs": bytes_read / (t_dec * 1e6),
            "decode_frac_hbm": bytes_read / (t_dec * 1e6) / peaks["hbm_gbs"],
            "compress_us_per_layer": (t_cmp * 1e3 / (n_cmp * w.L)) if n_cmp else None,
-           "final_len": cur_len, "launches": steps_total * w.L + n_cmp * 2}
+           "final_len": cur_len, "launches": steps_total * per_step + n_cmp * per_compression}
     # the same kernel with all layers folded into the batch of ONE call (not how a model decodes - its
     # layers depend on each other - but it shows what the kernel streams when a launch is large)
     nb = w.L * w.B
@@ -792,17 +811,17 @@ def main():
             "bound": "tensor", "unit": "TFLOP/s", "peak": peaks["bf16_tflops"],
             "ms": sum(x["score_ms"] for x in st_all) + res["score_caches_ms"],
             "work": sum(x["score_flops"] for x in st_all) + res["score_caches_flops"],
-            "calls": n_st + res["score_caches_calls"], "launches": 3 * (n_st + res["score_caches_calls"])},
+            "calls": n_st + res["score_caches_calls"], "launches": sum(x["score_launches"] for x in st_all) + res["score_caches_launches"]},
         "lvlm_merge_compact": {
             "bound": "hbm", "unit": "GB/s", "peak": peaks["hbm_gbs"],
             "ms": sum(x["merge_compact_ms"] for x in st_all), "work": sum(x["merge_compact_bytes"] for x in st_all),
-            "calls": n_st, "launches": 3 * n_st},
+            "calls": n_st, "launches": sum(x["merge_launches"] for x in st_all)},
         "lvlm_kv_compress": {
             "bound": "hbm", "unit": "GB/s", "peak": peaks["hbm_gbs"], "ms": res["kv_compress_only_ms"],
-            "work": res["kv_compress_bytes"], "calls": 1, "launches": 2},
+            "work": res["kv_compress_bytes"], "calls": 1, "launches": res["compress_launches"] - res["score_caches_launches"]},
         "lvlm_decode_attn": {
             "bound": "hbm", "unit": "GB/s", "peak": peaks["hbm_gbs"], "ms": res["decode_ms"],
-            "work": res["decode_kv_bytes"], "calls": w.L, "launches": w.L},
+            "work": res["decode_kv_bytes"], "calls": w.L, "launches": res["decode_launches"]},
     }
     rooflines = {}
     for name, kd in kinds.items():
@@ -813,7 +832,7 @@ def main():
                            "launches_per_step": kd["launches"],
                            "algorithmic_work_per_call": kd["work"] / kd["calls"]}
     rooflines["lvlm_select_topk"] = {"bound": "latency", "ms_per_step": sum(x["select_ms"] for x in st_all),
-                                     "calls_per_step": n_st, "launches_per_step": n_st}
+                                     "calls_per_step": n_st, "launches_per_step": sum(x["select_launches"] for x in st_all)}
     # ---- the other configurations (rank 0, one GPU): they carry the launches big enough to be bandwidth-bound ----
     extras = {}
     if rank == 0 and world == 1:

@@ -24,8 +24,8 @@ class ReduceStage:
     """score_tokens -> select_topk -> merge_compact for one layer (Section 3.2.1), with every
     output and workspace allocated once so that the calls can be captured in a CUDA graph."""
 
-    # score (normalisers, column sums, head reduction; on larger shapes one more, which adds up the normalisers, not
-    # counted here), select, merge_compact (plan, hidden, K/V)
+    # at least: score (normalisers, column sums, head reduction; on larger shapes one more, which adds up the normalisers),
+    # select, merge_compact (plan, hidden, K/V)
     LAUNCHES = 3 + 1 + 3
 
     def __init__(self, B, N, C, H, Hkv, cap, i0, n, M, device, want_head=False, mode=L.W_LINEAR_RANK):
