@@ -266,6 +266,7 @@ merge_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int
         }
     }
     if (kept_before != k) bad = true;
+    for (int o = kept_before + me; o < k; o += P * blockDim.x) src[i0 + o] = i0 + o;     // (no permutation: no row without a source)
     // rows outside the image span, shared out over the CTAs
     for (int o = me; o < Nout; o += P * blockDim.x) {
         if (o < i0) { src[o] = o; dst[o] = o; }

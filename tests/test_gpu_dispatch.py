@@ -323,6 +323,24 @@ def test_merge_plan_rounds(case, order):
     assert np.array_equal(f64(out)[0, stay], f64(hid)[0, src[stay]])
 
 
+# a rank that is no permutation is reported, and no map entry that nobody wrote is followed
+@pytest.mark.parametrize("mode", [L.W_LINEAR_RANK, L.W_NEAREST_KEPT])
+@pytest.mark.parametrize("value", [0, 299, -5, 1 << 30])
+def test_merge_of_a_bad_rank(mode, value):
+    N, i0, n, k, C = 2000, 7, 1900, 300, 64
+    hid = torch.randn(1, N, C, device="cuda").bfloat16()
+    K, V = (torch.randn(1, 2, N, 128, device="cuda").bfloat16() for _ in range(2))
+    K0, flag = K.clone(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    rank = torch.full((1, n), value, dtype=torch.int32, device="cuda")
+    if value == 1 << 30:
+        rank[0, :200] = torch.arange(200, device="cuda")              # too few kept tokens
+    ws = torch.full((1 << 22,), 0x7F, dtype=torch.uint8, device="cuda")     # (map entries that nobody writes would point far away)
+    L.merge_compact(hid, rank, i0=i0, k=k, mode=mode, Kc=K, Vc=V, ws=ws, dev_status=flag)
+    torch.cuda.synchronize()
+    assert flag.item() == L.DEV_BOUNDS
+    assert torch.equal(K[:, :, :i0], K0[:, :, :i0])
+
+
 # the merged rows, from few and from many partial sums of the passes over the rows (1 to 16 threads add up a column group), of
 # narrow rows and of rows wider than a column group per thread
 @pytest.mark.parametrize("case", [        # B, N, i0, n, C, Hkv, k
