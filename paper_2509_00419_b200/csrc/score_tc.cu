@@ -20,10 +20,11 @@
 // where the query tiles of a KV group are few, keeps them as B tiles over the items that follow); waiting for
 // normalisers (they come with the tile, by bulk copy) and reading one of them per logit (a TMEM load layout in which
 // a pair of them serves four keys); rows that a query tile does not have.
-// us a call, before -> now: all rows of 8448 x 48 heads, pass 2: 1105 -> 553; 22 layers of 3008 keys x 28 heads x 128 rows,
-// pass 2: 134 -> 91, both: 215 -> 178; 16 sequences of 1888 keys x 32 heads x 96 rows, both: 114 -> 80; 32933 keys x 28 heads
-// x 131 rows, both: 178 -> 100; 640 keys x 8 heads x 64 rows: 12.9 -> 13.0 (start-up and hand-overs).  Of a tile's 1300 to 2000 cycles the special-function unit is busy for 1024; a polynomial on
-// the FMA pipe for a quarter of the exponentials made it 2 to 6 % slower.
+// us a call, with a CTA per tile or two / so: all rows of 8448 x 48 heads, pass 2: 1095 / 521, both: 1643 / 1011; 22 layers of
+// 3008 keys x 28 heads x 128 rows, pass 2: 135 / 90, both: 214 / 178; 16 sequences of 1888 keys x 32 heads x 96 rows, both:
+// 114 / 80; 32933 keys x 28 heads x 131 rows, both: 177 / 100; 640 keys x 8 heads x 64 rows: 12.8 / 13.0 (start-up and
+// hand-overs).  Of a tile's 1300 to 2000 cycles the special-function unit is busy for 1024; a polynomial on the FMA pipe for
+// a quarter of the exponentials made it 2 to 6 % slower.
 // Small launches add the parked sums: normalisers (large shape, where items share a query tile's keys), scores.
 #include <type_traits>
 

@@ -130,7 +130,7 @@ __device__ __forceinline__ void rank_by_bins(KeyFn key_of, int n, int i_lo, int 
         return lo_i;
     };
     auto pair_of = [&](uint32_t k, int i) { return ((uint64_t)k << 32) | (uint32_t)i; };
-    int place[kRankKeys];                                                 // place within the bin (20 bits), bin
+    int place[kRankKeys];                                                 // place within the bin (16 bits), bin
     bool deep = false;
 #pragma unroll
     for (int u = 0; u < kRankKeys; ++u) {
