@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from bench import count_launches
 from oracle import lvlm_oracle as O
 from paper_2509_00419_b200 import binding as L
 from paper_2509_00419_b200 import build as BU
@@ -54,16 +55,17 @@ def test_decode_in_parts(case):
     (1, 32, 8, 3056, None, 700, True, False), (1, 32, 8, 3072, None, 700, True, True), (9, 28, 4, 300, None, 290, False, True),
     (1, 28, 4, 2000, 5000, 1999, True, True)])
 def test_decode_form(B, H, Hkv, cap, max_len, rows, acc, parts):
-    from torch.profiler import ProfilerActivity, profile
     g = torch.Generator(device="cuda").manual_seed(cap + rows)
     q, kn = (torch.randn(B, h, 128, generator=g, device="cuda").bfloat16() for h in (H, Hkv))
     Kc = torch.randn(B, Hkv, cap, 128, generator=g, device="cuda").bfloat16()
     ln = torch.full((B, Hkv), rows, dtype=torch.int32, device="cuda")
     accs, flag = torch.zeros(B, Hkv, cap, device="cuda") if acc else None, torch.zeros(1, dtype=torch.int32, device="cuda")
-    with profile(activities=[ProfilerActivity.CUDA]) as prof:
-        out = L.decode_attn(q, Kc, Kc, ln, k_new=kn, v_new=kn, acc_score=accs, dev_status=flag, max_len=max_len)
-        torch.cuda.synchronize()
-    assert any("decode_combine" in e.key for e in prof.key_averages()) == parts
+
+    def call():
+        return L.decode_attn(q, Kc, Kc, ln, k_new=kn, v_new=kn, acc_score=accs, dev_status=flag, max_len=max_len)
+
+    assert count_launches(call) == (2 if parts else 1)
+    out = call()
     k = Kc[:, :, :rows + 1].double().repeat_interleave(H // Hkv, dim=1)
     assert flag.item() == 0 and ln.eq(rows + 1).all() and torch.equal(Kc[:, :, rows], kn)
     p = torch.softmax(torch.einsum("bhd,bhnd->bhn", q.double(), k) / 128 ** 0.5, dim=-1)
