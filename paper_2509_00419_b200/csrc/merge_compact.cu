@@ -113,34 +113,6 @@ size_t merge_compact_workspace(const lvlm_dims* d) {
     return merge_layout(d, &L) ? L.total : 0;
 }
 
-__device__ __forceinline__ float block_sum_fixed(float v, float* scratch) {
-    // fixed reduction tree: xor shuffles inside a warp, then warp 0 over the warp sums
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
-    __syncthreads();
-    float t = (threadIdx.x < (blockDim.x >> 5)) ? scratch[threadIdx.x] : 0.f;
-    if (threadIdx.x < 32) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
-        if (threadIdx.x == 0) scratch[32] = t;
-    }
-    __syncthreads();
-    return scratch[32];
-}
-
-// Weight of the merged token at place p of the queue (p = 0 most important), normalised.
-__device__ __forceinline__ float merge_weight(int mode, int p, int r1, float inv_sum,
-                                              const float* __restrict__ w_custom) {
-    switch (mode) {
-        case LVLM_W_LINEAR_RANK: return (float)(r1 - p) * inv_sum;
-        case LVLM_W_GEOMETRIC:   return ldexpf(1.0f, -(p < r1 - 1 ? p + 1 : r1 - 1));
-        case LVLM_W_UNIFORM:     return inv_sum;
-        default:                 return w_custom[p] * inv_sum;
-    }
-}
-
 __device__ __forceinline__ uint32_t plan_cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -835,6 +807,12 @@ extern "C" lvlm_status lvlm_merge_compact(void* hidden, void* hidden_out, void* 
     float inv_sum = 1.f;
     if (mode == LVLM_W_LINEAR_RANK) inv_sum = (float)(2.0 / ((double)L.r1 * ((double)L.r1 + 1.0)));
     else if (mode == LVLM_W_UNIFORM) inv_sum = (float)(1.0 / (double)L.r1);
+    const OnceShape once = merge_once_shape(d, Kc != nullptr);
+    if (once.P) {
+        if ((L.V + kHidThreads - 1) / kHidThreads > kHidMaxChunks) return LVLM_ERR_UNSUPPORTED;
+        const MergeOnce m = {hidden, hidden_out, hid_sb, out_sb, Kc, Vc, kv_sb, kv_sh, pos_ids, rank, w_custom, new_len, (int)mode, inv_sum, dev_status};
+        return launch_merge_once(m, d, once, stream);
+    }
     const int plan_threads = d->n >= 1024 ? 1024 : (d->n <= 128 ? 128 : ((d->n + 31) / 32) * 32);
     {
         int P = (d->n + 1023) / 1024;                    // CTAs per sequence: a token a thread while they last

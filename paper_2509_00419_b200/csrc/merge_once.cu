@@ -1,0 +1,315 @@
+// lvlm_merge_compact in one launch, for sequences whose rows fit the shared memory of a CTA or a cluster of them.
+//
+// Everything that moves is cut into columns of 16 P bytes: a K or V sequence is 256 bytes wide, the hidden states 2 C, and a
+// CTA (a cluster, each CTA with a run of consecutive input rows) takes a column over the WHOLE sequence.
+// The rows are brought on chip while every CTA works out for itself, from `rank`, where its rows go and what they weigh; the
+// merged rows are added up; then the CTAs meet in a barrier, and since by then every row of the column is on chip, the kept
+// rows can be written where they belong, also in place, and the partial sums of the merged row are there to be added
+// in rank order.  So no map goes through memory, every row is read once, and nothing is launched behind it.
+//
+// What bounds it: latency (a chain of load, barrier, store) up to about 20 MB, then the waves of CTAs.  A thread loads, adds and
+// stores the same 16-byte pieces of the same rows, so the rows need no block barrier; a row's weight is worked out once.  us of a
+// merge, three launches / this: 640 rows of 2 KB and 8 heads 13.9 / 5.7, 1023 rows of 7 KB and 4 heads 14.9 / 7.3, 3008 rows
+// 22.1 / 13.4 (2.6 TB/s), 16 x 264 rows of 8 KB and 8 heads 28.8 / 19.5, 2 x 3064 rows (75 MB) 38.6 / 32.6 (3.3 TB/s).  The position ids are one more, narrow
+// column.
+#include "common.cuh"
+#include "exp2.cuh"
+#include "merge.cuh"
+
+namespace lvlm {
+
+constexpr int kOnceThreads = 256, kOnceWarps = kOnceThreads / 32;
+constexpr int kOnceMaxCluster = 8;
+constexpr int kOnceGroups = 4;                           // the rows of a CTA land in so many groups
+constexpr int kOnceMaxSmem = 220 * 1024;
+constexpr int kMerged = -1, kFirst = -2;                 // rows that go nowhere
+
+struct OnceArgs {
+    const char* hid; char* out; int64_t hid_sb, out_sb;  // bytes
+    char* K; char* V; int64_t kv_sb, kv_sh;
+    int32_t* pos; const int32_t* rank; const float* w_custom; int32_t* new_len; int32_t* dev_status;
+    int N, i0, n, k, C, Hkv, cols, S, R, mode;           // cols: columns of the hidden states; R: rows of a CTA
+    float inv_sum;
+};
+
+__device__ __forceinline__ uint32_t once_cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ float once_ld_cluster(const float* my_smem, uint32_t rank) {
+    uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
+    return v;
+}
+
+// grid (columns * S, B), clusters of S CTAs along x
+template <int P>
+__global__ void __launch_bounds__(kOnceThreads) merge_once_kernel(const OnceArgs a) {
+    constexpr int kLanes = kOnceThreads / P;                             // rows side by side
+    extern __shared__ __align__(16) uint4 rows[];                        // [R][P]
+    // [R] output row of a kept row, and nothing; kMerged, or kFirst for the first of the queue, and the weight of a merged row
+    int2* s_row = reinterpret_cast<int2*>(rows + (size_t)a.R * P);
+    int* s_pos = reinterpret_cast<int*>(rows);                           // [R] position ids (last column, in the place of rows)
+    __shared__ __align__(16) float s_red[kOnceWarps][P * 8];
+    __shared__ float s_part[P * 8];
+    __shared__ float s_scratch[33];
+    __shared__ int s_before[kOnceWarps], s_warp[kOnceWarps];
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cg = tid % P, rl = tid / P;
+    const int S = a.S, cr = (int)once_cluster_rank(), col = (int)blockIdx.x / S, b = blockIdx.y;
+    const int r1 = a.n - a.k, r = r1 - 1;
+    // my column: where its rows come from and go to
+    const char* from = nullptr; char* to = nullptr; int64_t row_b = 0; int pieces = P;
+    const bool last = col == a.cols + a.Hkv * 2 * (kHeadDim * 2 / (16 * P));     // nothing but position ids and the new length
+    if (last) {
+        pieces = 0;
+    } else if (col < a.cols) {
+        row_b = (int64_t)a.C * 2;
+        from = a.hid + (int64_t)b * a.hid_sb + col * (16 * P);
+        to = a.out + (int64_t)b * a.out_sb + col * (16 * P);
+        pieces = min(P, a.C / 8 - col * P);
+    } else {
+        constexpr int kPer = kHeadDim * 2 / (16 * P);                    // columns of a K or V sequence
+        const int x = (col - a.cols) / kPer, part = (col - a.cols) % kPer;
+        row_b = kHeadDim * 2;
+        to = (x & 1 ? a.V : a.K) + (int64_t)b * a.kv_sb + (int64_t)(x >> 1) * a.kv_sh + part * (16 * P);
+        from = to;
+    }
+    const bool in_place = from == to, with_pos = last && a.pos;
+    const int lo = min(a.N, cr * a.R), cnt = min(a.N, lo + a.R) - lo;    // my input rows
+    const int32_t* rank = a.rank + (int64_t)b * a.n;
+    int32_t* pos = with_pos ? a.pos + (int64_t)b * a.N : nullptr;
+    pdl_enter();
+
+    // ---- my rows start their way ------------------------------------------------------------------------
+    const int rounds = (cnt + kLanes - 1) / kLanes, quarter = (rounds + kOnceGroups - 1) / kOnceGroups;
+    {
+        const char* f = from + (int64_t)(lo + rl) * row_b + cg * 16;
+        uint32_t d = (uint32_t)__cvta_generic_to_shared(&rows[rl * P + cg]);
+        const int64_t step = kLanes * row_b;
+        int e = rl;
+#pragma unroll
+        for (int g = 0; g < kOnceGroups; ++g) {
+            const int end = cg < pieces ? min(cnt, (g + 1) * quarter * kLanes) : 0;
+#pragma unroll 4
+            for (; e < end; e += kLanes, f += step, d += kOnceThreads * 16)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(f) : "memory");
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
+        }
+    }
+    // ---- where they go: ranks of my tokens, and how many tokens ahead of mine are kept ---------------------------
+    // tokens [ja, jb) are mine; a warp has runs of 32 T consecutive ones
+    const int ja = min(max(lo - a.i0, 0), a.n), jb = min(max(lo + cnt - a.i0, 0), a.n);
+    const int T = (jb - ja + kOnceThreads - 1) / kOnceThreads, jw = ja + warp * T * 32 + lane;
+    int mine = 0, before = 0;
+    bool bad = false;
+    for (int t0 = 0; t0 < T; t0 += 4) {
+        int x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = t0 + u < T && jw + (t0 + u) * 32 < jb ? rank[jw + (t0 + u) * 32] : a.n;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = jw + (t0 + u) * 32;
+            if (t0 + u < T && j < jb) {
+                s_row[a.i0 + j - lo].x = x[u];                           // (read again by this very thread)
+                mine += x[u] < a.k;
+                bad |= x[u] < 0 || x[u] >= a.n;
+            }
+        }
+    }
+    for (int j0 = tid; j0 < ja; j0 += 8 * kOnceThreads) {
+        int x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = j0 + u * kOnceThreads < ja ? rank[j0 + u * kOnceThreads] : a.n;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) before += j0 + u * kOnceThreads < ja && x[u] < a.k;
+    }
+    if (with_pos)
+        for (int e = tid; e < cnt; e += kOnceThreads) s_pos[e] = pos[lo + e];
+    float inv_sum = a.inv_sum;
+    if (a.mode == LVLM_W_CUSTOM) {
+        float part = 0.f;
+        for (int p = tid; p < r1; p += kOnceThreads) part += a.w_custom[p];
+        inv_sum = 1.0f / block_sum_fixed(part, s_scratch);
+    }
+    before = __reduce_add_sync(0xFFFFFFFFu, before);
+    mine = __reduce_add_sync(0xFFFFFFFFu, mine);
+    if (lane == 0) { s_before[warp] = before; s_warp[warp] = mine; }
+    __syncthreads();
+    int off = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < kOnceWarps; ++w) {
+        off += s_before[w] + (w < warp ? s_warp[w] : 0);
+        total += s_before[w] + s_warp[w];
+    }
+    const unsigned lt = (1u << lane) - 1u;
+    for (int t = 0; t < T; ++t) {
+        const int j = jw + t * 32, e = a.i0 + j - lo;
+        const bool on = j < jb;
+        const int x = on ? s_row[e].x : a.n;
+        const unsigned kept = __ballot_sync(0xFFFFFFFFu, on && x < a.k);
+        if (on) {
+            const int o = off + __popc(kept & lt);
+            int2 to_w = make_int2(a.i0 + o, 0);
+            if (x >= a.k) {
+                to_w.x = x == a.k ? kFirst : kMerged;
+                to_w.y = __float_as_int(merge_weight(a.mode, min(x - a.k, r1 - 1), r1, inv_sum, a.w_custom));
+            } else if (o >= a.k) {
+                to_w.x = kMerged;                        // (no permutation: too many)
+            }
+            s_row[e] = to_w;
+        }
+        off += __popc(kept);
+    }
+    for (int e = tid; e < cnt; e += kOnceThreads) {      // rows outside the image span
+        const int i = lo + e;
+        if (i < a.i0) s_row[e].x = i; else if (i >= a.i0 + a.n) s_row[e].x = i - r;
+    }
+    if (cr == S - 1 && total != a.k) bad = true;         // (its run ends with the sequence)
+    if (bad && last && a.dev_status) atomicOr(a.dev_status, LVLM_DEV_BOUNDS);
+    if (last && cr == 0 && tid == 0 && a.new_len) a.new_len[b] = a.N - r;
+    __syncthreads();
+
+    // ---- my share of the merged row, as the rows come in -----------------------------------------------------------
+    f32x2 acc2[4] = {both(0.f), both(0.f), both(0.f), both(0.f)};
+    auto add_group = [&](int g) {
+        const int end = cg < pieces ? min(cnt, (g + 1) * quarter * kLanes) : 0;
+#pragma unroll 2
+        for (int e = g * quarter * kLanes + rl; e < end; e += kLanes) {
+            const int2 d = s_row[e];
+            if (d.x >= 0) continue;
+            const f32x2 w = both(__int_as_float(d.y));
+            const uint4 x = rows[e * P + cg];
+            acc2[0] = fma2(w, pack2(bf16_lo(x.x), bf16_hi(x.x)), acc2[0]);
+            acc2[1] = fma2(w, pack2(bf16_lo(x.y), bf16_hi(x.y)), acc2[1]);
+            acc2[2] = fma2(w, pack2(bf16_lo(x.z), bf16_hi(x.z)), acc2[2]);
+            acc2[3] = fma2(w, pack2(bf16_lo(x.w), bf16_hi(x.w)), acc2[3]);
+        }
+    };
+    asm volatile("cp.async.wait_group 3;\n" ::: "memory"); add_group(0);
+    asm volatile("cp.async.wait_group 2;\n" ::: "memory"); add_group(1);
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory"); add_group(2);
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory"); add_group(3);
+    float acc[8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) unpack2(acc2[u], acc[2 * u], acc[2 * u + 1]);
+#pragma unroll
+    for (int o = 16; o >= P; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc[u] += __shfl_xor_sync(0xFFFFFFFFu, acc[u], o);
+    if (lane < P) {
+        *reinterpret_cast<float4*>(&s_red[warp][cg * 8]) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        *reinterpret_cast<float4*>(&s_red[warp][cg * 8 + 4]) = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    }
+    __syncthreads();
+    if (tid < P * 8) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < kOnceWarps; ++w) s += s_red[w][tid];
+        s_part[tid] = s;
+    }
+    // ---- every row of the column is on chip, every share is there ----------------------------------------------
+    if (S > 1) {
+        asm volatile("barrier.cluster.arrive.release.aligned;\n"
+                     "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    } else {
+        __syncthreads();
+    }
+    if (cr == 0 && tid < pieces * 4) {                   // the merged row: two channels a thread
+        float x = 0.f, y = 0.f;
+#pragma unroll
+        for (int q = 0; q < kOnceMaxCluster; ++q) {
+            if (q < S) { x += once_ld_cluster(&s_part[2 * tid], q); y += once_ld_cluster(&s_part[2 * tid + 1], q); }
+        }
+        *reinterpret_cast<uint32_t*>(to + (int64_t)(a.i0 + a.k) * row_b + tid * 4) = pack_bf16(x, y);
+    }
+    if (S > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");      // (the shares have been read)
+    if (cg < pieces) {
+#pragma unroll 4
+        for (int e = rl; e < cnt; e += kLanes) {
+            const int d = s_row[e].x;
+            if (d >= 0 && !(in_place && d == lo + e)) *reinterpret_cast<uint4*>(to + (int64_t)d * row_b + cg * 16) = rows[e * P + cg];
+        }
+    }
+    if (with_pos) {                                      // P_new takes the id of the first of the queue
+        for (int e = tid; e < cnt; e += kOnceThreads) {
+            const int d = s_row[e].x;
+            if (d != kMerged) pos[d == kFirst ? a.i0 + a.k : d] = s_pos[e];
+        }
+    }
+    if (S > 1) asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");     // nobody leaves while its share is still read
+}
+
+static size_t once_smem(int P, int R) { return (size_t)R * (16 * P + 8); }
+static int once_rows(int N, int S) { return ((N + S - 1) / S + 3) / 4 * 4; }
+
+// Column width and cluster size: the smallest estimate of the time in us, a fit (within 10 %) to 400 measurements of 68 sizes
+// (1 to 16 sequences of 214 to 9064 rows, 1024 to 6144 channels, 4 or 8 KV heads).  A wave of CTAs takes a latency and
+// what its SM moves, at a lower rate where an SM has one CTA only; a CTA goes through its tokens; clusters meet, and fewer of them
+// find room.  What decides: one wave where all rows fit the chip at all (up to about 27 MB), two CTAs an SM rather than one
+// (3008 rows of 7 KB and 4 heads, 64-byte columns in clusters of two 13.9 us, 128-byte ones 16.4, 256-byte ones in clusters of eight
+// 20.7), beyond that small CTAs in many waves (8 KB and 8 heads, 5564 rows, 50 KB a CTA 35.4, 100 KB 44.6).
+static double once_estimate(const lvlm_dims* d, int heads, int P, int S) {
+    const int R = once_rows(d->N, S);
+    const size_t smem = once_smem(P, R);
+    if (smem > (size_t)kOnceMaxSmem) return 1e30;
+    const double ctas = (double)d->B * ((d->C / 8 + P - 1) / P + 2 * heads * (16 / P) + 1) * S, kb = (double)R * P / 64;
+    int per_sm = (int)(227 * 1024 / (smem + 1024 + 512 + 288 * P));
+    per_sm = per_sm > 4 ? 4 : per_sm;
+    const double room = 148.0 * per_sm * (S <= 2 ? 1.0 : S == 4 ? 0.91 : 0.95), full = ctas / room;
+    const double waves = full <= 1 ? 1.0 : full + 1.1 / per_sm;
+    const int here = ctas >= 148.0 * per_sm ? per_sm : (int)((ctas + 147) / 148);
+    const double moved = here * kb * 0.039 > kb * 0.0464 ? here * kb * 0.039 : kb * 0.0464;
+    return 0.9 + waves * (2.5 + moved) + 0.0019 * d->n / S + (S > 1 ? 1.8 : 0.0);
+}
+
+// The launches of the general path (plan, row pass, compaction) take over where they are quicker: us so / here, 4 x 1856 rows of 8 KB
+// and 8 heads (91 MB) 40.2 / 42.8, 3 x 2846 of 7 KB and 4 heads (79 MB) 38.0 / 38.4, 9064 rows of 2 KB (56 MB) 37.0 / 39.3, of 7 KB (84 MB)
+// 39.7 / 59.0; but 2 x 4064 rows of 7 KB (75 MB) 39.0 / 36.9, 5964 rows of 8 KB and 8 heads (73 MB) 39.5 / 37.8, and short sequences, in
+// many small CTAs: 16 x 464 of 8 KB (91 MB) 40.7 / 36.1.
+OnceShape merge_once_shape(const lvlm_dims* d, bool with_kv) {
+    OnceShape s = {0, 0};
+    // (Without K and V as if there were eight heads of them: the order in which the merged rows are added follows the shape, and the
+    // hidden states should come out the same bits with and without them.)
+    const int heads = with_kv ? d->Hkv : 8;
+    const double mb = (double)d->B * d->N * (d->C * 2.0 + heads * 512.0) * 1e-6;
+    if (d->N > 6000 || mb > (d->N <= 800 ? 100.0 : 75.0)) return s;
+    double best = 1e29;
+    for (int P = 16; P >= 4; P /= 2) {
+        for (int S = 1; S <= kOnceMaxCluster; S *= 2) {
+            const double t = once_estimate(d, heads, P, S);
+            if (t < best) { best = t; s.P = P; s.S = S; }
+        }
+    }
+    return s;
+}
+
+template <int P>
+static lvlm_status launch_once(OnceArgs& a, int B, cudaStream_t stream) {
+    a.cols = (a.C / 8 + P - 1) / P;
+    const int64_t x = (int64_t)(a.cols + 2 * a.Hkv * (16 / P) + 1) * a.S;
+    LVLM_RETURN_IF_CUDA(cudaFuncSetAttribute(merge_once_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnceMaxSmem));
+    return launch_kernel(merge_once_kernel<P>, dim3((unsigned)x, (unsigned)B), dim3(kOnceThreads), once_smem(P, a.R), stream, a.S, a);
+}
+
+lvlm_status launch_merge_once(const MergeOnce& m, const lvlm_dims* d, OnceShape s, cudaStream_t stream) {
+    OnceArgs a;
+    a.hid = static_cast<const char*>(m.hidden);
+    a.out = static_cast<char*>(m.hidden_out ? m.hidden_out : m.hidden);
+    a.hid_sb = m.hid_sb * 2; a.out_sb = m.out_sb * 2;
+    a.K = static_cast<char*>(m.K); a.V = static_cast<char*>(m.V); a.kv_sb = m.kv_sb * 2; a.kv_sh = m.kv_sh * 2;
+    a.pos = m.pos_ids; a.rank = m.rank; a.w_custom = m.w_custom; a.new_len = m.new_len; a.dev_status = m.dev_status;
+    a.N = d->N; a.i0 = d->i0; a.n = d->n; a.k = d->k; a.C = d->C; a.Hkv = m.K ? d->Hkv : 0;
+    a.S = s.S; a.R = once_rows(d->N, s.S); a.mode = m.mode; a.inv_sum = m.inv_sum;
+    switch (s.P) {
+        case 4: return launch_once<4>(a, d->B, stream);
+        case 8: return launch_once<8>(a, d->B, stream);
+        case 16: return launch_once<16>(a, d->B, stream);
+    }
+    return LVLM_ERR_UNSUPPORTED;
+}
+
+}  // namespace lvlm

@@ -366,3 +366,45 @@ def test_merge_partial_sums(case, in_place):
         assert_rows_close(got[:, :, i0 + k], w[:, :, i0 + k], rtol=2.0 ** -7, atol=1.1e-4, what=what)
         got[:, :, i0 + k] = w[:, :, i0 + k]
         assert np.array_equal(got, w), what
+
+
+# a merge in one launch: columns of 64, 128 and 256 bytes, last ones that are narrower, one to eight CTAs a column, runs that end
+# inside the rows ahead of, in and behind the image; and one row more than it takes (three launches)
+@pytest.mark.parametrize("case", [        # B, N, i0, n, C, Hkv, k, launches
+    (1, 1, 0, 1, 8, 0, 0, None), (1, 40, 3, 33, 72, 1, 5, 1), (1, 257, 0, 255, 8, 2, 253, 1), (1, 3008, 0, 2880, 3584, 4, 300, 1),
+    (3, 900, 60, 800, 200, 3, 0, 1), (1, 1300, 35, 1200, 6144, 8, 600, 1), (16, 264, 0, 200, 1024, 8, 60, 1), (16, 464, 1, 400, 1024, 8, 120, 1),
+    (1, 2000, 1700, 290, 64, 2, 100, 1), (1, 6000, 5, 5990, 64, 1, 2999, 1), (1, 6001, 5, 5990, 64, 1, 2999, 3)])
+@pytest.mark.parametrize("mode,in_place", [(L.W_LINEAR_RANK, False), (L.W_CUSTOM, True)])
+def test_merge_in_one_launch(case, mode, in_place):
+    B, N, i0, n, C, Hkv, k, launches = case
+    r = np.random.default_rng(N + C)
+    bf = lambda *s: torch.from_numpy(r.normal(size=s).astype(np.float32)).to(torch.bfloat16)
+    hid, Kc, Vc = bf(B, N, C), bf(B, max(Hkv, 1), N + 3, 128), bf(B, max(Hkv, 1), N + 3, 128)
+    rank = np.stack([r.permutation(n) for _ in range(B)]).astype(np.int32)
+    custom = (r.random(n - k) + 0.1).astype(np.float32) if mode == L.W_CUSTOM else None
+    pos = r.integers(0, 1 << 30, size=(B, N)).astype(np.int32)
+    want = O.merge_compact(f64(hid), rank, i0, n, k, mode=O.CUSTOM if custom is not None else O.LINEAR_RANK, custom=custom,
+                           Kc=f64(Kc)[:, :, :N], Vc=f64(Vc)[:, :, :N], pos_ids=pos)
+    rd, flag = torch.from_numpy(rank).cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    hd, Kd, Vd, pd = hid.cuda(), Kc.cuda(), Vc.cuda(), torch.from_numpy(pos).cuda()
+    out, new_len, Nout = None if in_place else torch.empty(B, want["hidden"].shape[1], C, dtype=hid.dtype, device="cuda"), torch.empty(B, dtype=torch.int32, device="cuda"), L.merged_rows(N, n, k)
+    ws = torch.empty(1 << 24, dtype=torch.uint8, device="cuda")
+
+    def call():
+        L.merge_compact(hd, rd, i0=i0, k=k, mode=mode, Kc=Kd if Hkv else None, Vc=Vd if Hkv else None, pos_ids=pd, in_place=in_place, out=out,
+                        w_custom=None if custom is None else torch.from_numpy(custom).cuda(), new_len=new_len, ws=ws, dev_status=flag)
+
+    call()
+    assert flag.item() == 0 and new_len.tolist() == [Nout] * B
+    got = [(hd if in_place else out)[:, None, :Nout]] + ([Kd[:, :, :Nout], Vd[:, :, :Nout]] if Hkv else [])
+    for x, w, what in zip(got, (want["hidden"][:, None], want["Kc"], want["Vc"]), ("hidden", "K", "V")):
+        x, w = f64(x), w.astype(np.float64)[:, :, :Nout]
+        if Nout < N:                             # a unit in the last place of bf16, fp32 sums of up to 400 terms in a row: below 1.5e-4
+            assert_rows_close(x[:, :, i0 + k], w[:, :, i0 + k], rtol=2.0 ** -7, atol=1.5e-4, what=what)
+            x[:, :, i0 + k] = w[:, :, i0 + k]
+        assert np.array_equal(x, w), what
+    assert np.array_equal(i32(pd)[:, :Nout], want["pos_ids"][:, :Nout])
+    if Hkv:
+        assert torch.equal(Kd[:, :, N:].cpu(), Kc[:, :, N:]) and torch.equal(Vd[:, :, N:].cpu(), Vc[:, :, N:])
+    if launches and custom is None:
+        assert count_launches(call) == launches
