@@ -1,7 +1,7 @@
 // lvlm_score_tokens: attention mass each image key receives from a window of query rows,
 // averaged over heads (Section 3.2.1, paragraph 3).
 //
-// Argument checks, workspace layout and the entry point; the kernels are in score_tc.cu.
+// Argument checks, workspace layout and the entry point; the kernels are in score_tc.cu and score_once.cu.
 #include "common.cuh"
 #include "score.cuh"
 

@@ -1,4 +1,4 @@
-// Tensor-core scoring kernels (tcgen05 + TMEM + TMA) for lvlm_score_tokens.
+// Tensor-core scoring kernels (tcgen05 + TMEM + TMA) for lvlm_score_tokens, where score_once.cu does not do it in one pass.
 //
 // The score of an image key is a column sum of softmax probabilities (Section 3.2.1,
 // paragraph 3), so two passes over Q K^T are needed when the caller has no row normalisers:
@@ -74,18 +74,6 @@ constexpr int64_t kSmallTiles1 = 148 * 3, kSmallTiles2 = 148 * 8;
 constexpr int kMaxSplit = 32, kMaxParts = 16;
 constexpr int64_t kMaxStatTiles = 4096, kMaxPartTiles = 8192;
 constexpr float kLog2eT = 1.4426950408889634f;
-
-// n / d for 0 <= n < 2^31 by a multiplication: every warp of a CTA takes every work item apart.
-struct FastDiv {
-    uint32_t d, m, sh;
-    FastDiv() = default;
-    explicit FastDiv(int div) : d((uint32_t)div), sh(0) {
-        while ((1u << sh) < d) ++sh;
-        m = (uint32_t)(((((uint64_t)1 << sh) - d) << 32) / d + 1);
-    }
-    __device__ __forceinline__ int div(int n) const { return (int)((__umulhi(m, (uint32_t)n) + (uint32_t)n) >> sh); }
-    __device__ __forceinline__ int divmod(int n, int* rem) const { const int q = div(n); *rem = n - q * (int)d; return q; }
-};
 
 struct ScoreTcArgs {
     int B, H, G, Hkv, N, Nq, i0, n, q_lo, causal;
@@ -176,17 +164,6 @@ __device__ __forceinline__ void colsum_chunk(const float* v, const float* nls, c
             acc[k] = add2(acc[k], pack2(x0, x1));
         }
     }
-}
-
-// 16 TMEM lanes x 32 fp32 columns: thread l has rows l/4 and l/4 + 8, columns 8 i + 2 (l % 4) + {0, 1}.
-__device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, float* v) {
-    uint32_t* r = reinterpret_cast<uint32_t*>(v);
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
 }
 
 __device__ __forceinline__ bool wait_or_abort(uint64_t* bar, uint32_t parity, TcCtl* sm, int32_t* dev_status) {
@@ -869,6 +846,18 @@ lvlm_status launch_score_tc(const void* Q, const void* K, const float* lse, cons
         const uint32_t box[4] = {64, (uint32_t)kTile, 1, 1};
         if (!make_tmap_bf16(&kmap, K, 4, dims, strides, box)) return LVLM_ERR_CUDA;
     }
+    auto add_up = [&](int parts) {
+        return launch_kernel(score_sum_kernel, dim3((unsigned)((d->n + kSumThreads - 1) / kSumThreads), (unsigned)d->B), dim3(kSumThreads), 0,
+                             stream, 1, reinterpret_cast<float*>(ws + L.off_partial), d->n, (int64_t)s.nkt * kTile, d->Hkv, parts,
+                             1.0f / (float)d->H, score, score_head, d->head_stride ? d->head_stride : (int64_t)d->n, dev_status);
+    };
+    if (lse == nullptr && !normalisers_ready) {
+        const OnceScoreShape o = score_once_shape(d, s, scale);
+        if (o.kt) {
+            const lvlm_status r = launch_score_once(qmap, kmap, d, s, o, scale, reinterpret_cast<float*>(ws + L.off_partial), dev_status, stream);
+            return r != LVLM_OK ? r : add_up(o.parts);
+        }
+    }
     ScoreTcArgs a;
     a.B = d->B; a.H = d->H; a.G = d->H / d->Hkv; a.Hkv = d->Hkv; a.N = d->N; a.Nq = Nq; a.i0 = d->i0; a.n = d->n;
     a.q_lo = d->q_lo; a.causal = d->causal; a.scale_log2 = scale * kLog2eT; a.s = s;
@@ -919,9 +908,7 @@ lvlm_status launch_score_tc(const void* Q, const void* K, const float* lse, cons
     r = s.small2 ? launch(std::true_type(), score_tc_kernel<1, true>, s.nkt, s.parts)
                  : launch(std::false_type(), score_tc_kernel<1, false>, s.nkt, s.parts);
     if (r != LVLM_OK) return r;
-    return launch_kernel(score_sum_kernel, dim3((unsigned)((d->n + kSumThreads - 1) / kSumThreads), (unsigned)d->B), dim3(kSumThreads), 0,
-                         stream, 1, a.partial, d->n, (int64_t)s.nkt * kTile, d->Hkv, s.parts, 1.0f / (float)d->H, score, score_head,
-                         d->head_stride ? d->head_stride : (int64_t)d->n, dev_status);
+    return add_up(s.parts);
 }
 
 }  // namespace lvlm

@@ -408,3 +408,14 @@ def test_merge_in_one_launch(case, mode, in_place):
         assert torch.equal(Kd[:, :, N:].cpu(), Kc[:, :, N:]) and torch.equal(Vd[:, :, N:].cpu(), Vc[:, :, N:])
     if launches and custom is None:
         assert count_launches(call) == launches
+
+
+# scoring in one pass over Q K^T: one to four key tiles a CTA, one to eight CTAs a cluster, teams that take turns at one or many
+# query tiles, rows of a query tile that are not there, runs that share a KV group, the last size that takes it and the first that does not
+@pytest.mark.parametrize("case", [        # B, H, Hkv, N, i0, n, T, causal, lse
+    (1, 1, 1, 2, 0, 1, 1, True, False), (1, 3, 3, 128, 1, 100, 27, True, False), (1, 8, 1, 129, 0, 64, 65, True, False),
+    (24, 12, 2, 250, 9, 200, 41, True, False), (40, 16, 8, 700, 0, 600, 100, True, False), (20, 28, 4, 1030, 3, 900, 127, True, False),
+    (9, 32, 8, 1500, 0, 1437, 33, False, False), (30, 7, 7, 2100, 0, 2000, 100, True, False), (3, 48, 8, 2600, 30, 2314, 256, True, False),
+    (2, 24, 4, 3400, 0, 3000, 400, True, False), (1, 28, 4, 4096, 0, 3968, 128, True, False), (1, 4, 2, 4097, 0, 3968, 129, True, False)])
+def test_score_one_pass(case):
+    test_score_shapes(case)
