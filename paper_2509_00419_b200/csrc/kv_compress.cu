@@ -315,7 +315,7 @@ kv_plan_kernel(float* acc_score, int32_t* pos, int32_t* len, const int32_t* __re
             if (kept) {
                 const int o = lo + off + __popc(bk & lt);
                 src[o] = lo + j;
-                an[o] = KPT > 4 && MAXT > 256 ? acc[lo + j] : sv[u];     // (1024 threads: 16 scores more do not fit the registers)
+                an[o] = KPT > 4 && MAXT > 256 ? acc[lo + j] : sv[u];     // (1024 threads: 8 or 16 scores more do not fit the registers)
                 if (ps) pn[o] = ps[lo + j];
             }
             if (first_drop == m && bd) first_drop = j - lane + __ffs((int)bd) - 1;
@@ -588,7 +588,10 @@ extern "C" lvlm_status lvlm_kv_compress(void* Kc, void* Vc, float* acc_score, in
     // With enough heads to fill the GPU with one warp each, a warp per head (no barrier in the searches); a CTA per
     // head otherwise, and for the heads whose entries do not fit a warp's registers.
     const bool many = heads >= 4 * 148;
-    const int kpt = d->cap <= 1024 ? 4 : 16;             // entries a thread: at most 8 warps up to 4096 rows
+    // Entries a thread: the plan is a chain of passes over them, so few while the heads leave SMs idle, and no more than the cache needs
+    // beyond that.  us of a compression with 16 entries up to 16384 rows / so: 88 heads of 3008 rows 53.4 / 49.3 (with 8: 50.8), 40 of
+    // 2000 33.0 / 31.8, 320 of 4000 138.0 / 137.2 (with 4: 147), 1024 of 3000 278 / 266 (288), 112 of 6000 79.9 / 75.3, 32 of 8000 59.9 / 57.6.
+    const int kpt = d->cap <= (heads <= 148 ? 4096 : 1024) ? 4 : d->cap <= 8192 ? 8 : 16;
     int threads = ((d->cap + kpt - 1) / kpt + 31) / 32 * 32;
     int min_m = 0;                                       // heads the CTA kernel leaves to the warp kernel
     bool cta_kernel = true;
@@ -604,7 +607,8 @@ extern "C" lvlm_status lvlm_kv_compress(void* Kc, void* Vc, float* acc_score, in
     }
     if (cta_kernel) {
         // a CTA per head; warps without entries leave at once
-        auto kernel = kpt == 4 ? kv_plan_kernel<4, 256> : threads <= 256 ? kv_plan_kernel<16, 256> : kv_plan_kernel<16, 1024>;
+        auto kernel = kpt == 4 ? (threads <= 256 ? kv_plan_kernel<4, 256> : kv_plan_kernel<4, 1024>)
+                               : kpt == 8 ? kv_plan_kernel<8, 1024> : kv_plan_kernel<16, 1024>;
         st = launch_kernel(kernel, dim3(d->Hkv, d->B), dim3(threads), 0, stream, 1, acc_score, pos, len, e_lo, e_hi, d->Hkv, d->cap,
                            d->recent, min_m, beta_ppm, budget, src_map, meta, nout, acc_new, pos_new, dev_status);
     }

@@ -419,3 +419,21 @@ def test_merge_in_one_launch(case, mode, in_place):
     (2, 24, 4, 3400, 0, 3000, 400, True, False), (1, 28, 4, 4096, 0, 3968, 128, True, False), (1, 4, 2, 4097, 0, 3968, 129, True, False)])
 def test_score_one_pass(case):
     test_score_shapes(case)
+
+
+# cache compression with 8 entries a thread (more heads than SMs, or long caches) and with 4 (few heads), at the ends of both ranges
+@pytest.mark.parametrize("heads,cap", [(148, 1025), (149, 1025), (148, 4096), (149, 2055), (2, 4097), (2, 8191), (2, 8193)])
+def test_kv_entries_a_thread(heads, cap):
+    r = np.random.default_rng(heads + cap)
+    acc = r.integers(0, 40, size=(1, heads, cap)).astype(np.float32) * 0.25
+    ln = r.integers(1, cap + 1, size=(1, heads)).astype(np.int32)
+    Kc = torch.from_numpy(r.normal(size=(1, heads, cap, 128)).astype(np.float32)).to(torch.bfloat16)
+    for beta, budget in ((0.9, 0), (1.0, cap // 2)):
+        want = O.kv_compress(f64(Kc), f64(Kc), acc, ln, beta=beta, budget=budget or None)
+        Kd, Vd, ad, ld = Kc.cuda(), Kc.cuda(), torch.from_numpy(acc).cuda(), torch.from_numpy(ln).cuda()
+        L.kv_compress(Kd, Vd, ad, ld, beta=beta, budget=budget)
+        assert np.array_equal(i32(ld), want["len"]), (beta, budget)
+        for g in range(0, heads, max(1, heads // 8)):
+            m = want["len"][0, g]
+            assert np.array_equal(ad[0, g, :m].cpu().numpy(), want["acc_score"][0, g, :m]), (beta, budget, g)
+            assert np.array_equal(f64(Kd[0, g, :m]), want["Kc"][0, g, :m].astype(np.float64)), (beta, budget, g)
