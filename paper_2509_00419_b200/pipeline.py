@@ -24,9 +24,9 @@ class ReduceStage:
     """score_tokens -> select_topk -> merge_compact for one layer (Section 3.2.1), with every
     output and workspace allocated once so that the calls can be captured in a CUDA graph."""
 
-    # at least: score (normalisers, column sums, head reduction; on larger shapes one more, which adds up the normalisers),
-    # select, merge_compact (with more rows than fit the chip three: plan, hidden, K/V)
-    LAUNCHES = 3 + 1 + 1
+    # at least: score (column sums, head reduction; in two passes one or two more, for the normalisers), select,
+    # merge_compact (with more rows than fit the chip three: plan, hidden, K/V)
+    LAUNCHES = 2 + 1 + 1
 
     def __init__(self, B, N, C, H, Hkv, cap, i0, n, M, device, want_head=False, mode=L.W_LINEAR_RANK):
         self.B, self.N, self.C, self.H, self.Hkv, self.cap = B, N, C, H, Hkv, cap
