@@ -20,6 +20,7 @@
 // 2 KB and 8 heads 21.6 -> 19.7, 16 sequences of 1888 119.3 -> 118.6.  The scratch for it lies in the second buffer: 8 KB of
 // its own made the last of these 128.)
 #include "compact.cuh"
+#include "sm100.cuh"
 
 namespace lvlm {
 
@@ -52,10 +53,7 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 }
 // Execution barrier only: nobody passes before everybody has arrived, but no memory is published.  Enough
 // between "my rows are on chip" and "I overwrite rows": nobody reads what another CTA writes here.
-__device__ __forceinline__ void cluster_barrier_exec() {
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n"
-                 "barrier.cluster.wait.aligned;\n" ::: "memory");
-}
+__device__ __forceinline__ void cluster_barrier_exec() { sm100::cluster_arrive_exec(); sm100::cluster_wait(); }
 
 // Sum of P fp32 partial rows (pp[p*row_floats + c*8 ...]) for 16-byte group c, rounded once.  `lanes` threads (256 /
 // lanes apart) take every lanes-th row, four in flight, and the first of them adds up what they have, in a fixed

@@ -128,20 +128,6 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-// Every thread of every CTA of the cluster arrives and waits; shared-memory writes made before it
-// are visible to the other CTAs after it.
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n"
-                 "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
-// Execution only: what I have read from other CTAs has been used, nothing is published (a releasing arrive would wait for
-// the stores to global memory before it, about 1200 cycles).
-__device__ __forceinline__ void cluster_arrive_exec() {
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
 __device__ __forceinline__ void prefetch_l2(const void* p) {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
@@ -493,7 +479,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     }
 
     // ---- combine the CTAs of the cluster in rank order through distributed shared memory ----------------
-    if (CL) cluster_sync_all(); else __syncthreads();
+    if (CL) cluster_barrier(); else __syncthreads();
     // my slice of the output: pairs of channels rank * kDecThreads + tid (+ S * kDecThreads ...) of the G heads.  A thread fetches
     // what it needs from every CTA in one go (max, sum and its channels) and works out the weights itself, so there is one
     // round trip and no block barrier on this path.

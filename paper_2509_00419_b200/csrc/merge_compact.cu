@@ -118,10 +118,6 @@ __device__ __forceinline__ uint32_t plan_cluster_rank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-__device__ __forceinline__ void plan_cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n"
-                 "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
 __device__ __forceinline__ int plan_ld_cluster(const int* my_smem, uint32_t rank) {
     uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
@@ -200,7 +196,7 @@ merge_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int
             if (on && rj[t] == k) { s_cta[pb][2] = j; is_new = true; pos_new = pv[t]; }     // P_new takes this token's place
         }
         if (lane == 0) { s_warp[pb][warp] = mine; atomicAdd(&s_cta[pb][0], mine); }
-        if (P > 1) plan_cluster_barrier(); else __syncthreads();
+        if (P > 1) sm100::cluster_barrier(); else __syncthreads();
         int c = 0, d = n, m = -1;                         // lane q asks CTA q
         if (lane < P) {
             c = plan_ld_cluster(&s_cta[pb][0], lane);
@@ -251,7 +247,7 @@ merge_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int
         for (int o0 = tail0 + P * (int)blockDim.x; o0 < Nout; o0 += P * (int)blockDim.x) {
             const bool on = o0 + me < Nout;
             if (on) tail_pos = pid[o0 + me + r];
-            plan_cluster_barrier();
+            sm100::cluster_barrier();
             if (on) pid[o0 + me] = tail_pos;
         }
     }
@@ -262,7 +258,7 @@ merge_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int
         if (new_len) new_len[b] = Nout;
     }
     if (bad && dev_status) atomicOr(dev_status, LVLM_DEV_BOUNDS);
-    if (P > 1) plan_cluster_barrier();                   // nobody leaves while its shared memory may still be read
+    if (P > 1) sm100::cluster_barrier();                   // nobody leaves while its shared memory may still be read
 }
 
 __global__ void identity_len_kernel(int32_t* new_len, int B, int N) {
@@ -275,10 +271,6 @@ __device__ __forceinline__ uint32_t hid_cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
-}
-__device__ __forceinline__ void hid_cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n"
-                 "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 __device__ __forceinline__ int hid_ld_cluster_i32(const int* my_smem, uint32_t rank) {
     uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
@@ -621,7 +613,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) row_stream_kernel(const Str
             }
         }
     }
-    hid_cluster_barrier();
+    sm100::cluster_barrier();
     const int Vs = (V + cl - 1) / cl;                         // my slice of the column groups
     const int c_lo = min(V, rank * Vs), c_hi = min(V, c_lo + Vs);
     {
@@ -637,7 +629,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) row_stream_kernel(const Str
             *reinterpret_cast<float4*>(my_partial + c * 8 + half * 4) = t;
         }
     }
-    hid_cluster_barrier();                 // every CTA's sums have been read: nobody leaves before
+    sm100::cluster_barrier();                 // every CTA's sums have been read: nobody leaves before
 }
 
 // Dynamic shared memory of the streaming kernel: always the whole ring budget, so that how many clusters fit on

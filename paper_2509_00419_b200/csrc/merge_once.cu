@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "exp2.cuh"
 #include "merge.cuh"
+#include "sm100.cuh"
 
 namespace lvlm {
 
@@ -213,20 +214,20 @@ __global__ void __launch_bounds__(kOnceThreads) merge_once_kernel(const OnceArgs
     }
     // ---- every row of the column is on chip, every share is there ----------------------------------------------
     if (S > 1) {
-        asm volatile("barrier.cluster.arrive.release.aligned;\n"
-                     "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+        sm100::cluster_barrier();
     } else {
         __syncthreads();
     }
-    if (cr == 0 && tid < pieces * 4) {                   // the merged row: two channels a thread
-        float x = 0.f, y = 0.f;
+    const bool adds = cr == 0 && tid < pieces * 4;       // the merged row: two channels a thread
+    float x = 0.f, y = 0.f;
+    if (adds) {
 #pragma unroll
         for (int q = 0; q < kOnceMaxCluster; ++q) {
             if (q < S) { x += once_ld_cluster(&s_part[2 * tid], q); y += once_ld_cluster(&s_part[2 * tid + 1], q); }
         }
-        *reinterpret_cast<uint32_t*>(to + (int64_t)(a.i0 + a.k) * row_b + tid * 4) = pack_bf16(x, y);
     }
-    if (S > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");      // (the shares have been read)
+    if (S > 1) sm100::cluster_arrive();                  // the shares have been read (and nothing is stored yet)
+    if (adds) *reinterpret_cast<uint32_t*>(to + (int64_t)(a.i0 + a.k) * row_b + tid * 4) = pack_bf16(x, y);
     if (cg < pieces) {
 #pragma unroll 4
         for (int e = rl; e < cnt; e += kLanes) {
@@ -240,7 +241,7 @@ __global__ void __launch_bounds__(kOnceThreads) merge_once_kernel(const OnceArgs
             if (d != kMerged) pos[d == kFirst ? a.i0 + a.k : d] = s_pos[e];
         }
     }
-    if (S > 1) asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");     // nobody leaves while its share is still read
+    if (S > 1) sm100::cluster_wait();                    // nobody leaves while its share is still read
 }
 
 static size_t once_smem(int P, int R) { return (size_t)R * (16 * P + 8); }

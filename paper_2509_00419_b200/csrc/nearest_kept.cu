@@ -74,10 +74,6 @@ __device__ __forceinline__ uint32_t nk_cluster_rank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-__device__ __forceinline__ void nk_cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n"
-                 "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-}
 __device__ __forceinline__ int nk_ld_cluster(const int* my_smem, uint32_t rank) {
     uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
@@ -115,7 +111,7 @@ nk_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int i0
     }
     mine = warp_sum(mine);
     if ((threadIdx.x & 31) == 0 && mine) atomicAdd(&s_total, mine);
-    nk_cluster_barrier();
+    cluster_barrier();
     int kq = 0, all = 0;
     for (int c = 0; c < P; ++c) {
         const int t = nk_ld_cluster(&s_total, c);
@@ -146,18 +142,18 @@ nk_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int i0
     for (int t = first; t <= k; t += step) seg[(int64_t)b * (k + 1) + t] = 0;            // counts, to begin with
     if (bad && dev_status) atomicOr(dev_status, LVLM_DEV_BOUNDS);
     if (cr == 0 && threadIdx.x == 0 && new_len) new_len[b] = Nout;
-    nk_cluster_barrier();                                                               // the kept list is complete
+    cluster_barrier();                                                               // the kept list is complete
     if (pos_ids) {
         int32_t* pid = pos_ids + (int64_t)b * N;
         for (int o0 = i0; o0 < Nout; o0 += step) {
             const int o = o0 + first;
             int val = 0;
             if (o < Nout) val = pid[o < i0 + k ? i0 + (all == k ? kp[o - i0] : o - i0) : o + r];
-            nk_cluster_barrier();
+            cluster_barrier();
             if (o < Nout) pid[o] = val;
         }
     }
-    nk_cluster_barrier();                                  // nobody leaves while its shared memory may still be read
+    cluster_barrier();                                  // nobody leaves while its shared memory may still be read
 }
 
 // ---- group -----------------------------------------------------------------------------------------

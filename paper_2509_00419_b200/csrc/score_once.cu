@@ -199,7 +199,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
     __syncthreads();
     tc_fence_after();
     if (S > 1)                                 // (a CTA's barriers are there before anybody sends to them)
-        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+        cluster_barrier();
     const uint32_t tmem_base = sm->tmem_base;
     pdl_enter();
 
@@ -501,7 +501,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
         for (int i = 0; i < 1000; ++i) __nanosleep(1000);
     }
     if (S > 1)                                    // (nobody leaves while somebody may still send to it)
-        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+        cluster_barrier();
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);

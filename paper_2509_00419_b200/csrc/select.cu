@@ -19,6 +19,7 @@
 // 4.8 -> 4.7, 6000: 12.5 -> 5.8, 32767: 32.6 -> 11.4, 16 sequences of 1792: 16.8 -> 5.1, 4 of 8000: 55.5 -> 6.4.
 // The optional outputs (kept list, near-tie count) come from a second, small kernel.
 #include "common.cuh"
+#include "sm100.cuh"
 
 namespace lvlm {
 
@@ -34,10 +35,6 @@ __device__ __forceinline__ uint32_t rank_cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
-}
-__device__ __forceinline__ void rank_cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n"
-                 "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }
 __device__ __forceinline__ int rank_ld_cluster(const int* my_smem, uint32_t rank) {
     uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
@@ -209,7 +206,7 @@ select_count_kernel(const float* __restrict__ score, int64_t stride, int n, int 
     if (S > 1) {
 #pragma unroll
         for (int u = 0; u < kRankMaxJT; ++u) s_cnt[u * kRankThreads + tid] = cnt[u];
-        rank_cluster_barrier();
+        sm100::cluster_barrier();
     }
     if (s == 0) {
 #pragma unroll
@@ -224,7 +221,7 @@ select_count_kernel(const float* __restrict__ score, int64_t stride, int n, int 
     }
     // every key is looked at by the CTAs of slice 0 as "their own" key: one report is enough
     if (nonfinite && blockIdx.y == 0 && dev_status) atomicOr(dev_status, LVLM_DEV_NONFINITE);
-    if (S > 1) rank_cluster_barrier();                    // nobody leaves while its counts are read
+    if (S > 1) sm100::cluster_barrier();                    // nobody leaves while its counts are read
 }
 
 // One CTA per sequence: the kept tokens in ascending order (prefix sum of rank < k over the index) and

@@ -66,6 +66,26 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     return false;
 }
 
+// ---- thread-block clusters ---------------------------------------------------------------------
+// The barrier of the cluster, in whole or as arrival and wait; every thread of every CTA takes part.  The .aligned forms want a warp's
+// threads to come together, which behind a branch or a loop of theirs is only so if they are brought together.
+// Publishes what I have written, and keeps what I have read from other CTAs ahead of the barrier.  (It waits for my stores
+// to global memory before it, about 1200 cycles.)
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+// Execution only: nothing is published.
+__device__ __forceinline__ void cluster_arrive_exec() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_barrier() { cluster_arrive(); cluster_wait(); }
+
 // ---- TMA -------------------------------------------------------------------------------------
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* m) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(m) : "memory");

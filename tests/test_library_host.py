@@ -141,6 +141,18 @@ def test_bad_arguments_are_rejected_on_the_host(lib):
     assert dec(dd) == L.ERR_UNSUPPORTED
 
 
+# barrier.cluster.*.aligned is undefined for a warp whose lanes come to it apart: the one place that issues it brings them together,
+# and an arrival that lets a CTA leave while its shared memory is still being read releases the reads
+def test_cluster_barriers_are_issued_by_whole_warps():
+    lines = {f: open(os.path.join(B.CSRC, f)).read().splitlines() for f in sorted(os.listdir(B.CSRC))}
+    at = [(f, i) for f, text in lines.items() for i, x in enumerate(text) if "barrier.cluster." in x]
+    assert {f for f, _ in at} == {"sm100.cuh"} and len(at) == 3
+    for f, i in at:
+        assert "__syncwarp();" in lines[f][i - 1]
+    once = "\n".join(lines["merge_once.cu"])
+    assert "cluster_arrive_exec" not in once and once.index("cluster_arrive()") < once.index("pack_bf16(x, y)")
+
+
 def test_binding_refuses_cpu_tensors():
     import torch
     with pytest.raises(TypeError):
