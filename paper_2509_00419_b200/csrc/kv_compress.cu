@@ -588,10 +588,13 @@ extern "C" lvlm_status lvlm_kv_compress(void* Kc, void* Vc, float* acc_score, in
     // With enough heads to fill the GPU with one warp each, a warp per head (no barrier in the searches); a CTA per
     // head otherwise, and for the heads whose entries do not fit a warp's registers.
     const bool many = heads >= 4 * 148;
-    // Entries a thread: the plan is a chain of passes over them, so few while the heads leave SMs idle, and no more than the cache needs
-    // beyond that.  us of a compression with 16 entries up to 16384 rows / so: 88 heads of 3008 rows 53.4 / 49.3 (with 8: 50.8), 40 of
-    // 2000 33.0 / 31.8, 320 of 4000 138.0 / 137.2 (with 4: 147), 1024 of 3000 278 / 266 (288), 112 of 6000 79.9 / 75.3, 32 of 8000 59.9 / 57.6.
-    const int kpt = d->cap <= (heads <= 148 ? 4096 : 1024) ? 4 : d->cap <= 8192 ? 8 : 16;
+    // Entries a thread: the plan is a chain of passes over them, so few while the heads leave SMs idle; with more heads than SMs warps
+    // wait for one another anyhow, and long caches are better off with fewer of them.  us of a compression (beta 0.99) with 16 / 8 / 4
+    // entries, heads x rows: 40 x 3000 31.2 / - / 27.8, 148 x 4096 56.1 / - / 54.0, 100 x 6000 67.2 / 61.2, 148 x 8000 90.9 / 88.0; 149 x 1100
+    // 36.4 / 32.8 / 30.2, 320 x 1100 48.1 / 46.9 / 43.4, 200 x 2048 48.2 / 46.0 / 45.7, 320 x 2048 64.4 / 63.2 / 68.1, 448 x 3000 114.7 / 112.3 / 125.4,
+    // 400 x 3500 116.3 / 114.7 / 122.8, 700 x 3000 172.5 / 162.3 / 175.8; 256 x 4096 78.0 / 79.4, 512 x 4096 145.0 / 146.9, 256 x 5000
+    // 96.3 / 100.3, 560 x 5000 190.8 / 201.2, 300 x 6000 149.8 / 151.5.
+    const int kpt = d->cap <= (heads <= 148 ? 4096 : 1024) ? 4 : d->cap <= (heads <= 148 ? 8192 : 3584) ? 8 : 16;
     int threads = ((d->cap + kpt - 1) / kpt + 31) / 32 * 32;
     int min_m = 0;                                       // heads the CTA kernel leaves to the warp kernel
     bool cta_kernel = true;
@@ -608,7 +611,7 @@ extern "C" lvlm_status lvlm_kv_compress(void* Kc, void* Vc, float* acc_score, in
     if (cta_kernel) {
         // a CTA per head; warps without entries leave at once
         auto kernel = kpt == 4 ? (threads <= 256 ? kv_plan_kernel<4, 256> : kv_plan_kernel<4, 1024>)
-                               : kpt == 8 ? kv_plan_kernel<8, 1024> : kv_plan_kernel<16, 1024>;
+                               : kpt == 8 ? kv_plan_kernel<8, 1024> : threads <= 256 ? kv_plan_kernel<16, 256> : kv_plan_kernel<16, 1024>;
         st = launch_kernel(kernel, dim3(d->Hkv, d->B), dim3(threads), 0, stream, 1, acc_score, pos, len, e_lo, e_hi, d->Hkv, d->cap,
                            d->recent, min_m, beta_ppm, budget, src_map, meta, nout, acc_new, pos_new, dev_status);
     }

@@ -421,8 +421,9 @@ def test_score_one_pass(case):
     test_score_shapes(case)
 
 
-# cache compression with 8 entries a thread (more heads than SMs, or long caches) and with 4 (few heads), at the ends of both ranges
-@pytest.mark.parametrize("heads,cap", [(148, 1025), (149, 1025), (148, 4096), (149, 2055), (2, 4097), (2, 8191), (2, 8193)])
+# cache compression with 4, 8 and 16 entries a thread, few heads and more heads than SMs, at the ends of the ranges of each
+@pytest.mark.parametrize("heads,cap", [(148, 1025), (149, 1025), (148, 4096), (149, 2055), (149, 3584), (149, 3585), (149, 4097),
+                                       (2, 4097), (2, 8191), (2, 8193)])
 def test_kv_entries_a_thread(heads, cap):
     r = np.random.default_rng(heads + cap)
     acc = r.integers(0, 40, size=(1, heads, cap)).astype(np.float32) * 0.25
