@@ -67,7 +67,7 @@ struct MergeOnce {
     void* hidden; void* hidden_out; int64_t hid_sb, out_sb; void* K; void* V; int64_t kv_sb, kv_sh;
     int32_t* pos_ids; const int32_t* rank; const float* w_custom; int32_t* new_len; int mode; float inv_sum; int32_t* dev_status;
 };
-OnceShape merge_once_shape(const lvlm_dims* d, bool with_kv);
+OnceShape merge_once_shape(const lvlm_dims* d);
 lvlm_status launch_merge_once(const MergeOnce& m, const lvlm_dims* d, OnceShape s, cudaStream_t stream);
 
 // lvlm_merge_compact in mode LVLM_W_NEAREST_KEPT (nearest_kept.cu).

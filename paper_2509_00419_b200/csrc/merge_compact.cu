@@ -799,7 +799,7 @@ extern "C" lvlm_status lvlm_merge_compact(void* hidden, void* hidden_out, void* 
     float inv_sum = 1.f;
     if (mode == LVLM_W_LINEAR_RANK) inv_sum = (float)(2.0 / ((double)L.r1 * ((double)L.r1 + 1.0)));
     else if (mode == LVLM_W_UNIFORM) inv_sum = (float)(1.0 / (double)L.r1);
-    const OnceShape once = merge_once_shape(d, Kc != nullptr);
+    const OnceShape once = merge_once_shape(d);
     if (once.P) {
         if ((L.V + kHidThreads - 1) / kHidThreads > kHidMaxChunks) return LVLM_ERR_UNSUPPORTED;
         const MergeOnce m = {hidden, hidden_out, hid_sb, out_sb, Kc, Vc, kv_sb, kv_sh, pos_ids, rank, w_custom, new_len, (int)mode, inv_sum, dev_status};

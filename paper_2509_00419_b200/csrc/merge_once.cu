@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kOnceThreads) merge_once_kernel(const OnceArgs
 static size_t once_smem(int P, int R) { return (size_t)R * (16 * P + 8); }
 static int once_rows(int N, int S) { return ((N + S - 1) / S + 3) / 4 * 4; }
 
-// Column width and cluster size: the smallest estimate of the time in us, a fit (within 10 %) to 400 measurements of 68 sizes
+// Estimate of the time in us by column width and cluster size, a fit (within 10 %) to 400 measurements of 68 sizes
 // (1 to 16 sequences of 214 to 9064 rows, 1024 to 6144 channels, 4 or 8 KV heads).  A wave of CTAs takes a latency and
 // what its SM moves, at a lower rate where an SM has one CTA only; a CTA goes through its tokens; clusters meet, and fewer of them
 // find room.  What decides: one wave where all rows fit the chip at all (up to about 27 MB), two CTAs an SM rather than one
@@ -267,24 +267,36 @@ static double once_estimate(const lvlm_dims* d, int heads, int P, int S) {
     return 0.9 + waves * (2.5 + moved) + 0.0019 * d->n / S + (S > 1 ? 1.8 : 0.0);
 }
 
-// The launches of the general path (plan, row pass, compaction) take over where they are quicker: us so / here, 4 x 1856 rows of 8 KB
-// and 8 heads (91 MB) 40.2 / 42.8, 3 x 2846 of 7 KB and 4 heads (79 MB) 38.0 / 38.4, 9064 rows of 2 KB (56 MB) 37.0 / 39.3, of 7 KB (84 MB)
-// 39.7 / 59.0; but 2 x 4064 rows of 7 KB (75 MB) 39.0 / 36.9, 5964 rows of 8 KB and 8 heads (73 MB) 39.5 / 37.8, and short sequences, in
-// many small CTAs: 16 x 464 of 8 KB (91 MB) 40.7 / 36.1.
-OnceShape merge_once_shape(const lvlm_dims* d, bool with_kv) {
+// Neither the path nor the column width and the cluster size may follow K and V: the merged row of the hidden states is added in an
+// order that these decide, and it should be the same bits whether a call brings K and V, and however many heads of them.  So
+// both rules see batch, rows and channels alone, and take K and V for what GQA models have: 3500 bytes a row for the path; for width and
+// size 8 heads up to 2048 channels and 4 beyond, or, where that leaves two choices close, the one that the other number prefers.  By
+// the estimate that costs 0 to 0.2 % on average against a choice that knows the heads (1024 to 6144 channels, 4 or 8 of them), 3 %
+// with 32 heads or without K and V.
+//
+// The launches of the general path (plan, row pass, compaction) take over where they are quicker.  us so / here: 2 x 3064 rows of 8 KB and
+// 8 heads 38.0 / 36.6, 2 x 3300 39.8 / 43.7; 2 x 3600 of 7 KB and 4 heads 33.9 / 36.9; 4500 of 12 KB and 8 heads 39.0 / 36.5; 2 x 5900 of
+// 2 KB and 8 heads 44.2 / 38.4, 3 x 4500 43.1 / 42.8, 3 x 4900 45.4 / 49.2; 9064 rows of 7 KB and 4 heads 39.7 / 59.0.  Short sequences, in
+// many small CTAs, gain longer: 16 x 560 of 8 KB and 8 heads 45.6 / 41.7, 16 x 400 of 12 KB 47.2 / 44.8, 16 x 640 of 7 KB and 4 heads 38.5 /
+// 37.4.  With 32 heads of 8 KB: 3008 rows 43.1 / 35.6, 2 x 3000 66.2 / 64.5, 5900 67.9 / 70.2.
+OnceShape merge_once_shape(const lvlm_dims* d) {
     OnceShape s = {0, 0};
-    // (Without K and V as if there were eight heads of them: the order in which the merged rows are added follows the shape, and the
-    // hidden states should come out the same bits with and without them.)
-    const int heads = with_kv ? d->Hkv : 8;
-    const double mb = (double)d->B * d->N * (d->C * 2.0 + heads * 512.0) * 1e-6;
-    if (d->N > 6000 || mb > (d->N <= 800 ? 100.0 : 75.0)) return s;
+    const double mb = (double)d->B * d->N * (d->C * 2.0 + 3500.0) * 1e-6;
+    if (d->N > 6000 || mb > (d->N <= 800 ? 110.0 : 73.0)) return s;
+    const int heads[2] = {d->C <= 2048 ? 8 : 4, d->C <= 2048 ? 4 : 8};
+    double t[2][3][4], least[2] = {1e29, 1e29};          // [heads][log2 P - 2][log2 S]
+    for (int h = 0; h < 2; ++h)
+        for (int p = 0; p < 3; ++p)
+            for (int c = 0; c < 4; ++c) {
+                t[h][p][c] = once_estimate(d, heads[h], 4 << p, 1 << c);
+                least[h] = t[h][p][c] < least[h] ? t[h][p][c] : least[h];
+            }
     double best = 1e29;
-    for (int P = 16; P >= 4; P /= 2) {
-        for (int S = 1; S <= kOnceMaxCluster; S *= 2) {
-            const double t = once_estimate(d, heads, P, S);
-            if (t < best) { best = t; s.P = P; s.S = S; }
+    for (int p = 2; p >= 0; --p)
+        for (int c = 0; c < 4; ++c) {
+            const double x = t[0][p][c] / least[0] + 0.1 * t[1][p][c] / least[1];
+            if (x < best) { best = x; s.P = 4 << p; s.S = 1 << c; }
         }
-    }
     return s;
 }
 

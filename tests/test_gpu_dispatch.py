@@ -410,6 +410,22 @@ def test_merge_in_one_launch(case, mode, in_place):
         assert count_launches(call) == launches
 
 
+# the merged row of the hidden states is the same bits without K and V and with any number of heads of them, on both sides of the limit
+# of a merge in one launch and where column widths and cluster sizes change
+@pytest.mark.parametrize("B,N,C", [(1, 640, 1024), (3, 689, 1024), (9, 502, 1024), (2, 5900, 1024), (3, 4500, 1024), (1, 3008, 3584), (2, 3400, 3584), (2, 3500, 3584),
+                                   (2, 1107, 3584), (8, 407, 3584), (2, 4064, 3584), (16, 264, 4096), (1, 6500, 512)])
+def test_hidden_merge_does_not_depend_on_kv(B, N, C):
+    g = torch.Generator(device="cuda").manual_seed(N)
+    n, k = N - 33, N // 5
+    hid = torch.randn(B, N, C, generator=g, device="cuda").bfloat16()
+    rank = torch.argsort(torch.rand(B, n, generator=g, device="cuda"), dim=1).int()
+    want, _ = L.merge_compact(hid, rank, i0=1, k=k)
+    for heads in (1, 2, 4, 8, 16):
+        K = torch.randn(B, heads, N, 128, generator=g, device="cuda").bfloat16()
+        got, _ = L.merge_compact(hid, rank, i0=1, k=k, Kc=K, Vc=K.clone())
+        assert torch.equal(got, want), heads
+
+
 # scoring in one pass over Q K^T: one to four key tiles a CTA, one to eight CTAs a cluster, teams that take turns at one or many
 # query tiles, rows of a query tile that are not there, runs that share a KV group, the last size that takes it and the first that does not
 @pytest.mark.parametrize("case", [        # B, H, Hkv, N, i0, n, T, causal, lse
