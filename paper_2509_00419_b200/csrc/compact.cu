@@ -46,11 +46,6 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 __device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
 // Execution barrier only: nobody passes before everybody has arrived, but no memory is published.  Enough
 // between "my rows are on chip" and "I overwrite rows": nobody reads what another CTA writes here.
 __device__ __forceinline__ void cluster_barrier_exec() { sm100::cluster_arrive_exec(); sm100::cluster_wait(); }
@@ -120,7 +115,7 @@ __global__ void __launch_bounds__(kCompactThreads) inplace_compact_kernel(const 
         return;
     }
     const int S = a.S;
-    const int rank = (int)cluster_rank();
+    const int rank = (int)sm100::cluster_ctarank();
     const int col = blockIdx.x / S;
     const int which = blockIdx.y / a.G, g = blockIdx.y % a.G, b = blockIdx.z;
     char* base = (which ? a.base1 : a.base0) + (int64_t)b * a.stride_b + (int64_t)g * a.stride_g;

@@ -122,25 +122,8 @@ size_t decode_attn_workspace(const lvlm_dims* d) {
     return decode_layout(d, &L, false, false) ? L.total : 0;
 }
 
-// ---- thread-block cluster primitives ---------------------------------------------------------------
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
 __device__ __forceinline__ void prefetch_l2(const void* p) {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-// Address of my shared-memory location `saddr` in the CTA of rank `rank`.
-__device__ __forceinline__ uint32_t dsmem_addr(uint32_t saddr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ float2 dsmem_ld2(uint32_t addr) {
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
-    return v;
 }
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
@@ -485,15 +468,14 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     // round trip and no block barrier on this path.
     for (int idx = rank * kDecThreads + tid; idx < G * (kHeadDim / 2); idx += S * kDecThreads) {
         const int hh = idx >> 6;
-        const uint32_t a_o = (uint32_t)__cvta_generic_to_shared(s_res + idx), a_ml = (uint32_t)__cvta_generic_to_shared(s_ML + hh);
         float2 x[kDecMaxCluster], ml[kDecMaxCluster];
 #pragma unroll
         for (int r = 0; r < kDecMaxCluster; ++r) {
             x[r] = make_float2(0.f, 0.f); ml[r] = make_float2(-INFINITY, 0.f);
             if (r < S) {
                 if (CL) {
-                    x[r] = dsmem_ld2(dsmem_addr(a_o, r));
-                    ml[r] = dsmem_ld2(dsmem_addr(a_ml, r));
+                    x[r] = cluster_ld(s_res + idx, r);
+                    ml[r] = cluster_ld(s_ML + hh, r);
                 } else {                       // a head with one CTA: its own shared memory, read directly
                     x[r] = s_res[idx]; ml[r] = s_ML[hh];
                 }
@@ -516,7 +498,7 @@ decode_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_con
     if (a.acc_score && tid < 64) {             // cluster-wide (max, 1 / sum) of every head: thread = (head, CTA)
         const int hh = tid >> 3, r = tid & 7;
         float2 ml = make_float2(-INFINITY, 0.f);
-        if (hh < G && r < S) ml = CL ? dsmem_ld2(dsmem_addr((uint32_t)__cvta_generic_to_shared(s_ML + hh), r)) : s_ML[hh];
+        if (hh < G && r < S) ml = CL ? cluster_ld(s_ML + hh, r) : s_ML[hh];
         float FM = ml.x;
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) FM = fmaxf(FM, __shfl_xor_sync(0xFFFFFFFFu, FM, o));

@@ -113,18 +113,6 @@ size_t merge_compact_workspace(const lvlm_dims* d) {
     return merge_layout(d, &L) ? L.total : 0;
 }
 
-__device__ __forceinline__ uint32_t plan_cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ int plan_ld_cluster(const int* my_smem, uint32_t rank) {
-    uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
-    int v;
-    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
-    return v;
-}
 
 // A cluster of P CTAs per sequence (grid (P, B)): source map, destination map, weights, position ids, new length.
 // A chain of latencies, so everything is loaded once, at the start, and the CTAs meet once a round: in a round each
@@ -145,7 +133,7 @@ merge_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int
     __shared__ int s_warp[2][32];                         // kept tokens of every warp, of two rounds
     __shared__ int s_cta[2][3];                           // ... of the CTA; first dropped token; the token that gives P_new its place
     pdl_enter();
-    const int b = blockIdx.y, P = (int)gridDim.x, cr = (int)plan_cluster_rank();
+    const int b = blockIdx.y, P = (int)gridDim.x, cr = (int)sm100::cluster_ctarank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const int r1 = n - k, r = r1 - 1, Nout = N - r;
     const int32_t* rk = rank + (int64_t)b * n;
@@ -199,9 +187,9 @@ merge_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int
         if (P > 1) sm100::cluster_barrier(); else __syncthreads();
         int c = 0, d = n, m = -1;                         // lane q asks CTA q
         if (lane < P) {
-            c = plan_ld_cluster(&s_cta[pb][0], lane);
-            d = plan_ld_cluster(&s_cta[pb][1], lane);
-            m = plan_ld_cluster(&s_cta[pb][2], lane);
+            c = sm100::cluster_ld(&s_cta[pb][0], lane);
+            d = sm100::cluster_ld(&s_cta[pb][1], lane);
+            m = sm100::cluster_ld(&s_cta[pb][2], lane);
         }
         first_drop = min(first_drop, __reduce_min_sync(0xFFFFFFFFu, d));
         m = __reduce_max_sync(0xFFFFFFFFu, m);
@@ -267,26 +255,6 @@ __global__ void identity_len_kernel(int32_t* new_len, int B, int N) {
     if (b < B) new_len[b] = N;
 }
 
-__device__ __forceinline__ uint32_t hid_cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ int hid_ld_cluster_i32(const int* my_smem, uint32_t rank) {
-    uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
-    int v;
-    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
-    return v;
-}
-__device__ __forceinline__ float4 hid_ld_cluster_f4(const float* my_smem, uint32_t rank) {
-    uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(remote) : "memory");
-    return v;
-}
 
 // One pass over the rows.  grid (CTAs per sequence, B), clusters of `cl` CTAs along x.  A CTA is eight consumer
 // warps, a loader warp and a storer warp around a ring of shared-memory tiles, each guarded by a "full" mbarrier
@@ -602,7 +570,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) row_stream_kernel(const Str
     const int V = a.V, cl = a.cl;
     const int cluster = cta / cl;
     const int nq = cps / cl;                                   // partials of this sequence, one per cluster
-    const int rank = (int)hid_cluster_rank();
+    const int rank = (int)sm100::cluster_ctarank();
     if (tid < kHidThreads) {
 #pragma unroll
         for (int ci = 0; ci < CH; ++ci) {
@@ -623,7 +591,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) row_stream_kernel(const Str
             const int c = c_lo + (idx >> 1), half = idx & 1;
             float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
             for (int r = 0; r < cl; ++r) {
-                const float4 x = hid_ld_cluster_f4(s_sum + c * 8 + half * 4, r);
+                const float4 x = sm100::cluster_ld(reinterpret_cast<const float4*>(s_sum + c * 8 + half * 4), r);
                 t.x += x.x; t.y += x.y; t.z += x.z; t.w += x.w;
             }
             *reinterpret_cast<float4*>(my_partial + c * 8 + half * 4) = t;

@@ -33,18 +33,6 @@ struct OnceArgs {
     float inv_sum;
 };
 
-__device__ __forceinline__ uint32_t once_cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ float once_ld_cluster(const float* my_smem, uint32_t rank) {
-    uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
-    return v;
-}
 
 // grid (columns * S, B), clusters of S CTAs along x
 template <int P>
@@ -60,7 +48,7 @@ __global__ void __launch_bounds__(kOnceThreads) merge_once_kernel(const OnceArgs
     __shared__ int s_before[kOnceWarps], s_warp[kOnceWarps];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cg = tid % P, rl = tid / P;
-    const int S = a.S, cr = (int)once_cluster_rank(), col = (int)blockIdx.x / S, b = blockIdx.y;
+    const int S = a.S, cr = (int)sm100::cluster_ctarank(), col = (int)blockIdx.x / S, b = blockIdx.y;
     const int r1 = a.n - a.k, r = r1 - 1;
     // my column: where its rows come from and go to
     const char* from = nullptr; char* to = nullptr; int64_t row_b = 0; int pieces = P;
@@ -223,7 +211,7 @@ __global__ void __launch_bounds__(kOnceThreads) merge_once_kernel(const OnceArgs
     if (adds) {
 #pragma unroll
         for (int q = 0; q < kOnceMaxCluster; ++q) {
-            if (q < S) { x += once_ld_cluster(&s_part[2 * tid], q); y += once_ld_cluster(&s_part[2 * tid + 1], q); }
+            if (q < S) { x += sm100::cluster_ld(&s_part[2 * tid], q); y += sm100::cluster_ld(&s_part[2 * tid + 1], q); }
         }
     }
     if (S > 1) sm100::cluster_arrive();                  // the shares have been read (and nothing is stored yet)

@@ -69,18 +69,6 @@ size_t nearest_kept_workspace(const lvlm_dims* d) {
 }
 
 // ---- plan ------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t nk_cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ int nk_ld_cluster(const int* my_smem, uint32_t rank) {
-    uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
-    int v;
-    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
-    return v;
-}
 
 // A cluster of P CTAs per sequence (grid (P, B)), CTA c the c-th run of the image tokens: it counts its kept tokens, learns
 // from the lower ranks how many came before, then writes its run tile by tile (thread = token, coalesced; one CTA with
@@ -94,7 +82,7 @@ nk_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int i0
     __shared__ int scan_scratch[33];
     __shared__ int s_total;
     pdl_enter();
-    const int b = blockIdx.y, r = n - k, Nout = N - r, P = (int)gridDim.x, cr = (int)nk_cluster_rank();
+    const int b = blockIdx.y, r = n - k, Nout = N - r, P = (int)gridDim.x, cr = (int)cluster_ctarank();
     const int32_t* rk = rank + (int64_t)b * n;
     int32_t* dst = dst_map + (int64_t)b * N;
     int32_t* kp = kept + (int64_t)b * k;
@@ -114,7 +102,7 @@ nk_plan_kernel(const int32_t* __restrict__ rank, int32_t* pos_ids, int N, int i0
     cluster_barrier();
     int kq = 0, all = 0;
     for (int c = 0; c < P; ++c) {
-        const int t = nk_ld_cluster(&s_total, c);
+        const int t = cluster_ld(&s_total, c);
         kq += c < cr ? t : 0;
         all += t;
     }

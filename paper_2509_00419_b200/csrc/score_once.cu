@@ -55,34 +55,6 @@ struct OnceCtl {
     volatile int abort;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ uint32_t map_cluster(uint32_t smem, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem), "r"(rank));
-    return r;
-}
-// Eight bytes into the shared memory of a CTA of the cluster, credited to a barrier there.
-__device__ __forceinline__ void st_async8(uint32_t addr, float2 v, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
-                 ::"r"(addr), "l"(pack2(v.x, v.y)), "r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
-#pragma unroll 1
-    for (uint32_t it = 0; it < kSpinLimit; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done) : "r"(smem_u32(bar)), "r"(parity), "r"(64u) : "memory");
-        if (done) return true;
-    }
-    return false;
-}
 __device__ __forceinline__ void tmem_st_16x256b_x4(uint32_t taddr, const float* v) {
     const uint32_t* r = reinterpret_cast<const uint32_t*>(v);
     asm volatile(
@@ -170,7 +142,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
     OnceCtl* sm = reinterpret_cast<OnceCtl*>(s_res + (size_t)res_bufs * kOSets * 4 * kOTile);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cr = (int)cluster_rank(), sets = teams * kt;
+    const int cr = (int)cluster_ctarank(), sets = teams * kt;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kOQSlots; ++s) { mbar_init(&sm->q_full[s], 1); mbar_init(&sm->q_empty[s], 2); }
         for (int s = 0; s < 4; ++s) { mbar_init(&sm->k_full[s], 1); mbar_init(&sm->k_empty[s], 2); }
@@ -424,7 +396,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                         float2* to = s_recv + (size_t)((team * 2 + (z & 1)) * S) * kOTile + row0 + lane;
                         if (tile == 0 && lane == 0) mbar_arrive_expect_tx(bar, (uint32_t)(S * 256));
                         const uint32_t addr = smem_u32(to + cr * kOTile), bar_addr = smem_u32(bar);
-                        for (int d = tile; d < S; d += kt) st_async8(map_cluster(addr, (uint32_t)d), mine, map_cluster(bar_addr, (uint32_t)d));
+                        for (int d = tile; d < S; d += kt) st_async8(cluster_map(addr, (uint32_t)d), mine, cluster_map(bar_addr, (uint32_t)d));
                         ok = sm->abort ? false : mbar_wait_cluster(bar, (z >> 1) & 1) || once_give_up(sm, a.dev_status);
                         ok = __all_sync(0xFFFFFFFFu, ok);
                         if (!ok) break;

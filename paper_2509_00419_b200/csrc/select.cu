@@ -31,18 +31,6 @@ constexpr int kRankBins = 2048, kRankSamples = 1024, kRankDeep = 128;
 constexpr int kRankKeys = kRankMaxSlice / kRankThreads;           // keys a thread puts into bins at most
 constexpr int kRankMaxJT = 4;              // tokens a thread ranks at most
 
-__device__ __forceinline__ uint32_t rank_cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ int rank_ld_cluster(const int* my_smem, uint32_t rank) {
-    uint32_t local = (uint32_t)__cvta_generic_to_shared(my_smem), remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
-    int v;
-    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
-    return v;
-}
 
 struct RankShape { int S, slice_len, jt; };                           // slices, keys of one, tokens a thread ranks
 
@@ -197,7 +185,7 @@ select_count_kernel(const float* __restrict__ score, int64_t stride, int n, int 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_cnt[kRankMaxJT * kRankThreads];
     pdl_enter();
-    const int b = blockIdx.z, s = (int)rank_cluster_rank(), tid = threadIdx.x;
+    const int b = blockIdx.z, s = (int)sm100::cluster_ctarank(), tid = threadIdx.x;
     const float* row = score + (int64_t)b * stride;
     bool nonfinite = false;
     auto key_of = [&](int i) { return desc_key(row[i], &nonfinite); };
@@ -214,7 +202,7 @@ select_count_kernel(const float* __restrict__ score, int64_t stride, int n, int 
             const int j = (blockIdx.x * jt + u) * kRankThreads + tid;
             if (u < jt && j < n) {
                 int tot = cnt[u];
-                for (int r = 1; r < S; ++r) tot += rank_ld_cluster(&s_cnt[u * kRankThreads + tid], r);
+                for (int r = 1; r < S; ++r) tot += sm100::cluster_ld(&s_cnt[u * kRankThreads + tid], r);
                 rank[(int64_t)b * n + j] = tot;
             }
         }

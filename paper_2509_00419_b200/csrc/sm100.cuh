@@ -85,6 +85,59 @@ __device__ __forceinline__ void cluster_wait() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_barrier() { cluster_arrive(); cluster_wait(); }
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Address of my shared-memory location `saddr` in the CTA of rank `rank`, and loads from there.
+__device__ __forceinline__ uint32_t cluster_map(uint32_t saddr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ int cluster_ld(const int* my_smem, uint32_t rank) {
+    int v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_map(smem_u32(my_smem), rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ float cluster_ld(const float* my_smem, uint32_t rank) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_map(smem_u32(my_smem), rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ float2 cluster_ld(const float2* my_smem, uint32_t rank) {
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];"
+                 : "=f"(v.x), "=f"(v.y) : "r"(cluster_map(smem_u32(my_smem), rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 cluster_ld(const float4* my_smem, uint32_t rank) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_map(smem_u32(my_smem), rank)) : "memory");
+    return v;
+}
+// Eight bytes into the shared memory of a CTA of the cluster (both addresses from cluster_map), credited to a barrier there.
+__device__ __forceinline__ void st_async8(uint32_t addr, float2 v, uint32_t bar) {
+    asm volatile("{\n\t.reg .b64 v;\n\tmov.b64 v, {%1, %2};\n\t"
+                 "st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], v, [%3];\n\t}"
+                 ::"r"(addr), "f"(v.x), "f"(v.y), "r"(bar) : "memory");
+}
+// mbar_wait for a barrier that other CTAs of the cluster complete: what they sent is visible.
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
+#pragma unroll 1
+    for (uint32_t it = 0; it < kSpinLimit; ++it) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, %3;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done) : "r"(smem_u32(bar)), "r"(parity), "r"(64u) : "memory");
+        if (done) return true;
+    }
+    return false;
+}
 
 // ---- TMA -------------------------------------------------------------------------------------
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* m) {
