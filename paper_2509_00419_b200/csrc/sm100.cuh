@@ -101,11 +101,6 @@ __device__ __forceinline__ int cluster_ld(const int* my_smem, uint32_t rank) {
     asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_map(smem_u32(my_smem), rank)) : "memory");
     return v;
 }
-__device__ __forceinline__ float cluster_ld(const float* my_smem, uint32_t rank) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_map(smem_u32(my_smem), rank)) : "memory");
-    return v;
-}
 __device__ __forceinline__ float2 cluster_ld(const float2* my_smem, uint32_t rank) {
     float2 v;
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];"

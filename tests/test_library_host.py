@@ -141,8 +141,8 @@ def test_bad_arguments_are_rejected_on_the_host(lib):
     assert dec(dd) == L.ERR_UNSUPPORTED
 
 
-# barrier.cluster.*.aligned is undefined for a warp whose lanes come to it apart: the one place that issues it brings them together,
-# and an arrival that lets a CTA leave while its shared memory is still being read releases the reads
+# barrier.cluster.*.aligned is undefined for a warp whose lanes come to it apart: the one place that issues it brings them together;
+# and what the merge has read from other CTAs lies in its own shared memory before the arrival that lets them leave
 def test_cluster_barriers_are_issued_by_whole_warps():
     lines = {f: open(os.path.join(B.CSRC, f)).read().splitlines() for f in sorted(os.listdir(B.CSRC))}
     at = [(f, i) for f, text in lines.items() for i, x in enumerate(text) if "barrier.cluster." in x]
@@ -150,7 +150,8 @@ def test_cluster_barriers_are_issued_by_whole_warps():
     for f, i in at:
         assert "__syncwarp();" in lines[f][i - 1]
     once = "\n".join(lines["merge_once.cu"])
-    assert "cluster_arrive_exec" not in once and once.index("cluster_arrive()") < once.index("pack_bf16(x, y)")
+    steps = ["cluster_ld(", "s_new[tid] = ", "cluster_arrive_exec()", "reinterpret_cast<const uint4*>(s_new)", "cluster_wait()"]
+    assert [once.count(x) for x in steps] == [1] * 5 and sorted(steps, key=once.index) == steps
 
 
 def test_binding_refuses_cpu_tensors():
