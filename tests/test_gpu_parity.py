@@ -449,11 +449,12 @@ def test_nearest_kept_exact_tie_goes_to_the_lower_kept_index():
 
 
 # ------------------------------------------------------------------ library-internal cross-checks
-def test_results_do_not_depend_on_programmatic_dependent_launch():
+@pytest.mark.parametrize("n", [448, 6200])               # (scores in one pass and a merge in one launch; two passes, three launches)
+def test_results_do_not_depend_on_programmatic_dependent_launch(n):
     """The same chain of calls with and without programmatic dependent launch, bit for bit (no kernel
     may touch its inputs before the kernels ahead of it have finished)."""
     from paper_2509_00419_b200 import build as Bld
-    w = I.shrink(I.CFG1, n=448, T=64, C=512, planted=8)
+    w = I.shrink(I.CFG1, n=n, T=64, C=512, planted=8)
     L.use_library(Bld.build_test())           # the build that carries the switch; the library proper has none
     lib = L.lib()
 
