@@ -11,7 +11,8 @@
 // own but for four shuffles, and a column takes four multiplications and 7/8 of a shuffle.
 //
 // Against sums in 64 bits the scores are off by 6e-8 to 1.2e-7 of their norm (nine sizes of 300 to 4096 keys), those of two passes by 8e-8 to
-// 1.5e-7: an exponential's argument is small where the exponential is not.
+// 1.5e-7: an exponential's argument is small where the exponential is not.  (test_score_one_pass and test_score_two_passes hold both
+// below 2^-21.)
 //
 // Roles as in score_tc.cu: a TMA warp, two MMA-issuing warps, a finisher warp, and sixteen epilogue warps in four sets, each
 // with an accumulator.  With few key tiles a CTA the sets form teams that work on query tiles in turn, so that the exponentials
@@ -44,7 +45,18 @@ struct OnceScoreArgs {
     float scale_log2;
     float* partial; int64_t row_len;   // [B][Hkv * parts][row_len] column sums
     int32_t* dev_status;
+#ifdef LVLM_TEST_HOOKS
+    int starve;
+#endif
 };
+
+// The test build can keep the first CTA of every cluster from sending, so that all of them wait for sums that never come.
+#ifdef LVLM_TEST_HOOKS
+static int g_score_starve = 0;
+__device__ __forceinline__ bool once_starved(const OnceScoreArgs& a, int cr) { return a.starve != 0 && cr == 0; }
+#else
+__device__ __forceinline__ bool once_starved(const OnceScoreArgs&, int) { return false; }
+#endif
 
 struct OnceCtl {
     uint64_t q_full[kOQSlots], q_empty[kOQSlots], k_full[4], k_empty[4], acc_full[kOSets], acc_empty[kOSets];
@@ -396,7 +408,7 @@ score_once_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constan
                         float2* to = s_recv + (size_t)((team * 2 + (z & 1)) * S) * kOTile + row0 + lane;
                         if (tile == 0 && lane == 0) mbar_arrive_expect_tx(bar, (uint32_t)(S * 256));
                         const uint32_t addr = smem_u32(to + cr * kOTile), bar_addr = smem_u32(bar);
-                        for (int d = tile; d < S; d += kt) st_async8(cluster_map(addr, (uint32_t)d), mine, cluster_map(bar_addr, (uint32_t)d));
+                        for (int d = once_starved(a, cr) ? S : tile; d < S; d += kt) st_async8(cluster_map(addr, (uint32_t)d), mine, cluster_map(bar_addr, (uint32_t)d));
                         ok = sm->abort ? false : mbar_wait_cluster(bar, (z >> 1) & 1) || once_give_up(sm, a.dev_status);
                         ok = __all_sync(0xFFFFFFFFu, ok);
                         if (!ok) break;
@@ -522,8 +534,8 @@ static int once_clusters(int S) {
 // cycles a tile and SM.  us measured, two passes / one: 8 heads x 640 keys x 64 rows 12.4 / 9.2, 28 x 406 x 128 15.0 / 10.4, 28 x 1023 x
 // 128 17.2 / 11.6, 28 x 3008 x 128 26.6 / 18.0, 3 sequences of 28 x 2846 x 50 29.1 / 19.9, 16 of 8 x 400 x 17 22.9 / 12.2, 16 of 32 x 1156 x
 // 96 57.5 / 50.0, 2 of 32 x 4000 x 100 43.9 / 39.4; where a cluster has many query tiles the chains lose: 16 of 32 x 1888 x 96 78.9 / 82.6,
-// 16 of 48 x 2000 x 100 125 / 132.  Between other launches clusters find their SMs later than CTAs do (the 57.5 / 50.0 above make a reduction
-// 367 / 370): one pass has to be ahead by 7 %.
+// 16 of 48 x 2000 x 100 125 / 132.  One pass has to be ahead by 7 %: between other launches it gains less than in a loop of its own (the
+// 57.5 / 50.0 above made a whole two-stage reduction of 16 x 1888 rows 367 / 370 us; the reason is not measured).
 OnceScoreShape score_once_shape(const lvlm_dims* d, const ScoreShape& s, float scale) {
     static const double chain[4] = {3700, 5800, 10300, 12000};             // cycles a query tile in a row of them, by key tiles a CTA
     OnceScoreShape best = {0, 0, 0, 0};
@@ -560,6 +572,9 @@ lvlm_status launch_score_once(const CUtensorMap& qmap, const CUtensorMap& kmap, 
     a.runs = (int)runs;
     a.by_nh = FastDiv(s.nh); a.by_box_h = FastDiv(s.box_h); a.by_parts = FastDiv(o.parts); a.by_hkv = FastDiv(d->Hkv);
     a.scale_log2 = scale * kLog2eO;
+#ifdef LVLM_TEST_HOOKS
+    a.starve = g_score_starve;
+#endif
     a.partial = partial; a.row_len = (int64_t)s.nkt * kOTile; a.dev_status = dev_status;
     LVLM_RETURN_IF_CUDA(cudaFuncSetAttribute(score_once_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnceScoreSmem));
     return launch_kernel(score_once_kernel, dim3((unsigned)(o.clusters * o.S)), dim3(kOThreads), once_smem(a.k_slots, a.teams, a.S), stream,
@@ -567,3 +582,7 @@ lvlm_status launch_score_once(const CUtensorMap& qmap, const CUtensorMap& kmap, 
 }
 
 }  // namespace lvlm
+
+#ifdef LVLM_TEST_HOOKS
+extern "C" void lvlm_debug_starve_score(int on) { lvlm::g_score_starve = on ? 1 : 0; }
+#endif

@@ -506,6 +506,26 @@ def test_score_one_pass(case):
     assert _check_scoring(case) == 2
 
 
+# sums of another CTA that never come (the test build keeps the first CTA of a cluster from sending): the call ends and says so, and
+# the next one is as ever; with one, two and four key tiles a CTA
+@pytest.mark.parametrize("case", [(1, 8, 1, 129, 0, 64, 65, True), (4, 64, 8, 1000, 0, 900, 100, True), (1, 28, 4, 4096, 0, 3968, 128, True)])
+def test_score_one_pass_timeout(case):
+    B, H, Hkv, N, i0, n, T, causal = case
+    Q, K, want, _ = _scoring(case)
+    try:
+        L.use_library(BU.build_test())
+        for starve in (1, 0):
+            flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+            L.lib().lvlm_debug_starve_score(starve)
+            score, _ = L.score_tokens(Q, K, N=N, i0=i0, n=n, q_lo=N - T, q_hi=N, causal=causal, dev_status=flag)
+            torch.cuda.synchronize()
+            assert flag.item() & L.DEV_TIMEOUT if starve else flag.item() == 0
+    finally:
+        L.lib().lvlm_debug_starve_score(0)
+        L.use_library(None)
+    assert_scores_close(f64(score), f64(want), what="score")
+
+
 # scoring in two passes: one key more than a cluster holds, windows that begin among the scored keys, shapes where it is quicker; with
 # few rows pass 1 has them two or four times in a query tile, on the small and on the large shape of the kernel
 @pytest.mark.parametrize("case", [
