@@ -16,9 +16,9 @@
 // before this one leaves fp32 partial sums, and the CTA that owns the merged position adds them in
 // a fixed order and writes the row, as soon as the sums are there and while its first rows come in.
 // (One thread a column group waited for up to 80 partial rows, four at a time, at the end of the last super-tile.  us of a whole
-// merge: 32933 rows of 7 KB and 4 heads' K and V 143.8 -> 111.1, 9075 rows 66.8 -> 39.6, 3008 rows 26.6 -> 21.6, 640 rows of
-// 2 KB and 8 heads 21.6 -> 19.7, 16 sequences of 1888 119.3 -> 118.6.  The scratch for it lies in the second buffer: 8 KB of
-// its own made the last of these 128.)
+// merge: 32933 rows of 7 KB and 4 heads' K and V 143.8 -> 111.1, 9075 rows 66.8 -> 39.6,
+// 16 sequences of 1888 rows of 8 KB and 8 heads 119.3 -> 118.6.  The scratch for it lies in the second buffer: 8 KB of its own
+// made the last of these 128.)
 #include "compact.cuh"
 #include "sm100.cuh"
 

@@ -2,7 +2,8 @@
 // (Section 3.2.1, paragraph 4), applied to the hidden states, to that layer's K and V and
 // to the position ids.
 //
-// Launches: (1) a plan kernel, one CTA per sequence, turns `rank` into a source-row map for
+// Where the rows fit the chip, merge_once.cu does all of it in one launch; this file has the entry point and the launches
+// for larger problems (and the row pass of mode NEAREST_KEPT at any size): (1) a plan kernel, a cluster per sequence, turns `rank` into a source-row map for
 // every output row, a destination for every input row and a merge weight for every image token;
 // (2) one streaming kernel reads every input row of the hidden states once, moves it if it is
 // kept and adds it to the weighted sum if it is merged; (3) one kernel compacts K and V in place.
@@ -41,9 +42,9 @@ HiddenGrid hidden_grid(const lvlm_dims* d) {
     int rpt = kStreamTileBytes / rowB;
     rpt = rpt > 32 ? 32 : rpt;
     rpt = rpt < 1 ? 1 : rpt;
-    // Short sequences, where that would leave most SMs without rows: two smaller tiles for every SM (a chain of a dozen tiles in a
-    // few CTAs is the time).  us of a merge, 34 KB tiles / this: 640 rows of 2 KB and 8 heads 19.5 / 13.6, 220 rows 19.9 / 11.4;
-    // 1060 rows of 7 KB, where 132 CTAs have rows, 14.2 / 15.1.
+    // Short sequences (they come here in mode NEAREST_KEPT), where that would leave most SMs without rows: two smaller tiles for every
+    // SM, a chain of a dozen tiles in a few CTAs is slower.  us of such a merge, 34 KB tiles / this: 220 rows of 2 KB and 8 heads 29.0 /
+    // 28.0, 640 rows 29.5 / 29.7, 640 of 7 KB and 4 heads 43.0 / 43.2, 1060 rows 47.0 / 47.0.
     if ((int64_t)d->N * d->B < (int64_t)148 * rpt) {
         const int few = (int)(((int64_t)d->N * d->B) / (2 * 148));
         rpt = few < 1 ? 1 : few;
@@ -68,12 +69,12 @@ HiddenGrid hidden_grid(const lvlm_dims* d) {
 }
 
 // Chunks the image span of every K and V sequence is cut into when the merged rows are summed: about four
-// work items per CTA of the sequence's batch element (the CTAs take them in turn), not shorter than 128 rows
-// (64, a tile, where that makes an item a CTA at most: 330 rows of 7 KB and 4 heads 13.3 -> 12.5 us; with more items it is slower).
+// work items per CTA of the sequence's batch element (the CTAs take them in turn), not shorter than 128 rows.  (With 64 where that
+// makes an item a CTA at most: 6400 rows of 2 KB and 1 head 18.0 -> 19.3 us, 330 image rows of 6400 of 2 KB and 4 heads 22.6 -> 22.7.)
 static int kv_chunks(const lvlm_dims* d, const HiddenGrid& g) {
     if (d->Hkv <= 0) return 1;
     int p = (4 * g.cps + d->Hkv * 2 - 1) / (d->Hkv * 2);
-    const int by_rows = d->n / (d->Hkv * 2 * (int64_t)(d->n / 64) <= g.cps ? 64 : 128);
+    const int by_rows = d->n / 128;
     p = p > by_rows ? by_rows : p;
     p = p < 1 ? 1 : p;
     while (p > 1 && (int64_t)(p - 1) * ((d->n + p - 1) / p) >= d->n) --p;      // no chunk is empty
