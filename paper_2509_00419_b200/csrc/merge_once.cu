@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kOnceThreads) merge_once_kernel(const OnceArgs
 }
 
 static size_t once_smem(int P, int R) { return (size_t)R * (16 * P + 8); }
-static int once_rows(int N, int S) { return ((N + S - 1) / S + 3) / 4 * 4; }
+static int once_rows(int N, int S) { return ((N + S - 1) / S + 3) & ~3; }
 
 // Estimate of the time in us by column width and cluster size, a fit (within 10 %) to 400 measurements of 68 sizes
 // (1 to 16 sequences of 214 to 9064 rows, 1024 to 6144 channels, 4 or 8 KV heads).  A wave of CTAs takes a latency and
@@ -249,18 +249,23 @@ static int once_rows(int N, int S) { return ((N + S - 1) / S + 3) / 4 * 4; }
 // find room.  What decides: one wave where all rows fit the chip at all (up to about 27 MB), two CTAs an SM rather than one
 // (3008 rows of 7 KB and 4 heads, 64-byte columns in clusters of two 13.9 us, 128-byte ones 16.4, 256-byte ones in clusters of eight
 // 20.7), beyond that small CTAs in many waves (8 KB and 8 heads, 5564 rows, 50 KB a CTA 35.4, 100 KB 44.6).
-static double once_estimate(const lvlm_dims* d, int heads, int P, int S) {
-    const int R = once_rows(d->N, S);
-    const size_t smem = once_smem(P, R);
-    if (smem > (size_t)kOnceMaxSmem) return 1e30;
-    const double ctas = (double)d->B * ((d->C / 8 + P - 1) / P + 2 * heads * (16 / P) + 1) * S, kb = (double)R * P / 64;
-    int per_sm = (int)(227 * 1024 / (smem + 1024 + 512 + 288 * P));
+// 16-byte pieces 4 << p, CTAs 1 << c, for two numbers of heads at a time: twelve of these are a tenth of a microsecond of every call.
+static void once_estimate(const lvlm_dims* d, const int (&heads)[2], int p, int c, double (&t)[2]) {
+    static const double kInvCtas[5] = {0.0, 1.0 / 148, 1.0 / 296, 1.0 / 444, 1.0 / 592}, kLast[5] = {0.0, 1.1, 0.55, 1.1 / 3, 0.275};
+    static const double kFewer[4] = {1.0, 1.0, 1.0 / 0.91, 1.0 / 0.95};
+    const int P = 4 << p, S = 1 << c, R = once_rows(d->N, S);
+    const int smem = (int)once_smem(P, R);
+    t[0] = t[1] = 1e30;
+    if (smem > kOnceMaxSmem) return;
+    int per_sm = 227 * 1024 / (smem + 1024 + 512 + 288 * P);
     per_sm = per_sm > 4 ? 4 : per_sm;
-    const double room = 148.0 * per_sm * (S <= 2 ? 1.0 : S == 4 ? 0.91 : 0.95), full = ctas / room;
-    const double waves = full <= 1 ? 1.0 : full + 1.1 / per_sm;
-    const int here = ctas >= 148.0 * per_sm ? per_sm : (int)((ctas + 147) / 148);
-    const double moved = here * kb * 0.039 > kb * 0.0464 ? here * kb * 0.039 : kb * 0.0464;
-    return 0.9 + waves * (2.5 + moved) + 0.0019 * d->n / S + (S > 1 ? 1.8 : 0.0);
+    const double kb = R * P * (1.0 / 64), fixed = 0.9 + 0.0019 * d->n / S + (S > 1 ? 1.8 : 0.0);
+    for (int h = 0; h < 2; ++h) {
+        const int ctas = d->B * (((d->C / 8 + P - 1) >> (p + 2)) + 2 * heads[h] * (4 >> p) + 1) * S;
+        const double full = ctas * kInvCtas[per_sm] * kFewer[c], waves = full <= 1 ? 1.0 : full + kLast[per_sm];
+        const int here = ctas >= 148 * per_sm ? per_sm : (ctas + 147) / 148;
+        t[h] = fixed + waves * (2.5 + kb * (here > 1 ? here * 0.039 : 0.0464));
+    }
 }
 
 // Neither the path nor the column width and the cluster size may follow K and V: the merged row of the hidden states is added in an
@@ -280,17 +285,17 @@ OnceShape merge_once_shape(const lvlm_dims* d) {
     const double mb = (double)d->B * d->N * (d->C * 2.0 + 3500.0) * 1e-6;
     if (d->N > 6000 || mb > (d->N <= 800 ? 110.0 : 73.0)) return s;
     const int heads[2] = {d->C <= 2048 ? 8 : 4, d->C <= 2048 ? 4 : 8};
-    double t[2][3][4], least[2] = {1e29, 1e29};          // [heads][log2 P - 2][log2 S]
-    for (int h = 0; h < 2; ++h)
-        for (int p = 0; p < 3; ++p)
-            for (int c = 0; c < 4; ++c) {
-                t[h][p][c] = once_estimate(d, heads[h], 4 << p, 1 << c);
-                least[h] = t[h][p][c] < least[h] ? t[h][p][c] : least[h];
-            }
+    double t[3][4][2], least[2] = {1e29, 1e29};          // [log2 P - 2][log2 S][heads]
+    for (int p = 0; p < 3; ++p)
+        for (int c = 0; c < 4; ++c) {
+            once_estimate(d, heads, p, c, t[p][c]);
+            for (int h = 0; h < 2; ++h) least[h] = t[p][c][h] < least[h] ? t[p][c][h] : least[h];
+        }
+    const double other = 0.1 * least[0] / least[1];
     double best = 1e29;
     for (int p = 2; p >= 0; --p)
         for (int c = 0; c < 4; ++c) {
-            const double x = t[0][p][c] / least[0] + 0.1 * t[1][p][c] / least[1];
+            const double x = t[p][c][0] + other * t[p][c][1];
             if (x < best) { best = x; s.P = 4 << p; s.S = 1 << c; }
         }
     return s;
